@@ -89,6 +89,9 @@ typedef enum {
                            hi/lo pairs with fp32 accumulation.  d = 128, u = k_hat, no refresh,
                            [B,H,T,d] or [B,T,H,d] tensors, T >= 1; VLA_ERR_UNSUPPORTED otherwise.  AUTO picks it
                            where it applies (and VLA_KERNEL_CHUNK then forces the fp32-FMA form) */
+  ,VLA_KERNEL_PAIR = 5    /* the chunk algebra on warp-level tensor-core products (fp16 hi/lo operands, fp32
+                           accumulation, states in registers), two CTAs per unit; every d, u = k_hat or
+                           explicit, either layout; VLA_ERR_UNSUPPORTED with the refresh */
 } vla_kernel_t;
 
 typedef struct {

@@ -48,7 +48,7 @@ int resolve_opts(const vla_opts_t* opts, vla_opts_t* r) {
                            VLA_FLAG_LINEAR_ATTENTION))
     return VLA_ERR_INVALID_ARG;
   if (r->kernel != VLA_KERNEL_AUTO && r->kernel != VLA_KERNEL_TOKEN && r->kernel != VLA_KERNEL_CHUNK &&
-      r->kernel != VLA_KERNEL_DECODE && r->kernel != VLA_KERNEL_CHUNK_TC)
+      r->kernel != VLA_KERNEL_DECODE && r->kernel != VLA_KERNEL_CHUNK_TC && r->kernel != VLA_KERNEL_PAIR)
     return VLA_ERR_INVALID_ARG;
   if (r->refresh_period > 0 && (r->step_offset < 0 || !(r->refresh_eta == r->refresh_eta)))
     return VLA_ERR_INVALID_ARG;
@@ -63,8 +63,7 @@ bool shape_supported(int d_k, int d_v) {
 // means "done"; ids never repeat within 2^32 launches, so the flags never need clearing).
 std::atomic<unsigned int> g_launch_epoch{0};
 
-// The chunk kernel covers d in {32, 64, 128}; d = 16 runs on the token kernel.  Both are CUDA
-// paths; there is no host fallback.
+// The FMA chunk kernel covers d in {32, 64, 128}.  Every path is CUDA; there is no host fallback.
 bool chunk_covers(const ScanParams&, int d) { return d >= 32; }
 
 // Very short sequences (single-step decode and the like) are bound by reading and writing
@@ -83,6 +82,23 @@ bool chunk_tc_covers(const ScanParams& p, int d) {
   return d == 128 && !p.u && p.refresh_period <= 0 && p.T > 0;
 }
 
+// The pair kernel: every d, u = k_hat or explicit, either layout; no refresh.
+bool pair_covers(const ScanParams& p) { return p.refresh_period <= 0 && p.n_main <= 0 && p.units <= 0x3fffffff; }
+
+// Where it is the library's choice.  Against the token kernel (measured, few units | units beyond one wave
+// of clusters, us at T = 8, 16, 32, 64): d = 64 token 8.4, 13.4, 24.6, 46.9 pair 7.5, 7.6, 10.4, 14.4 | 256
+// units 11.5, 18.6, 33.9, 64.4 and 29.7, 29.9, 40.4, 56.5; d = 32, 16 alike with the second crossing near 24.  At
+// d = 128 the tensor-memory kernel keeps what is short (below seven chunks the clusters' start costs
+// what the shorter chain saves) and, with u = k_hat, more units than SM pairs (one SM per unit there:
+// 48 units x 1777 tokens 0.63 against 0.44 ms, 128 x 2048 0.75 against 1.02 ms).
+bool pair_pays_off(const ScanParams& p, int d) {
+  const long long sms = vla::device_sms();
+  const long long resident = d == 16 ? 6 : d == 32 ? 4 : 1;   // CTAs per SM
+  const bool one_wave = 2LL * p.units <= resident * sms;
+  if (d == 128) return p.T > 96 && (p.u || one_wave);
+  return p.T > (one_wave ? 8 : d == 64 ? 48 : 24);
+}
+
 int launch(const ScanParams& p, int d, int dtype, int kernel, cudaStream_t st) {
   // the linear-attention comparison mode lives in the token kernel (u = k_hat instantiation)
   if (p.flags & VLA_FLAG_LINEAR_ATTENTION) {
@@ -90,11 +106,14 @@ int launch(const ScanParams& p, int d, int dtype, int kernel, cudaStream_t st) {
       return VLA_ERR_UNSUPPORTED;
     return vla::launch_token(d, dtype, p, st);
   }
+  if (kernel == VLA_KERNEL_PAIR)
+    return pair_covers(p) ? vla::launch_pair(d, dtype, p, nullptr, st) : VLA_ERR_UNSUPPORTED;
   if (kernel == VLA_KERNEL_CHUNK_TC)
     return chunk_tc_covers(p, d) ? vla::launch_chunk_tc(d, dtype, p, st) : VLA_ERR_UNSUPPORTED;
   if (kernel == VLA_KERNEL_DECODE && !decode_covers(p, d)) return VLA_ERR_UNSUPPORTED;
   if ((kernel == VLA_KERNEL_DECODE || kernel == VLA_KERNEL_AUTO) && decode_covers(p, d))
     return vla::launch_decode(d, dtype, p, st);
+  if (kernel == VLA_KERNEL_AUTO && pair_covers(p) && pair_pays_off(p, d)) return vla::launch_pair(d, dtype, p, nullptr, st);
   bool chunk = chunk_covers(p, d);
   if (kernel == VLA_KERNEL_CHUNK && !chunk) return VLA_ERR_UNSUPPORTED;
   if (kernel == VLA_KERNEL_AUTO && !chunk_pays_off(p, d)) chunk = false;

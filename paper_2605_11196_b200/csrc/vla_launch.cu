@@ -1,5 +1,7 @@
 // Dispatch from (d, input type) to the translation unit that holds the kernels, the token
 // kernel's launchers, and the helper launches of the sequence-parallel path.
+#include <atomic>
+
 #include "vla.h"
 #include "vla_launch.h"
 #include "vla_backward.cuh"
@@ -54,6 +56,45 @@ int launch_chunk_stash(int d, int dtype, const ScanParams& p, cudaStream_t st) {
 int chunk_resident_ctas(int d, int dtype, bool tri) {
   VLA_CHUNK_DISPATCH(chunk_resident, tri);
   return 0;
+}
+
+int device_sms() {
+  static std::atomic<int> known[64];
+  int dev = -1, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return 0;
+  }
+  n = known[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    known[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
+#define VLA_DECLARE_PAIR_TU(TAG) int launch_pair_##TAG(const ScanParams& p, const PairStash* sh, cudaStream_t st);
+VLA_DECLARE_PAIR_TU(d16_f32)
+VLA_DECLARE_PAIR_TU(d16_bf16)
+VLA_DECLARE_PAIR_TU(d32_f32)
+VLA_DECLARE_PAIR_TU(d32_bf16)
+VLA_DECLARE_PAIR_TU(d64_f32)
+VLA_DECLARE_PAIR_TU(d64_bf16)
+VLA_DECLARE_PAIR_TU(d128_f32)
+VLA_DECLARE_PAIR_TU(d128_bf16)
+#undef VLA_DECLARE_PAIR_TU
+
+int launch_pair(int d, int dtype, const ScanParams& p, const PairStash* sh, cudaStream_t st) {
+  const bool f32 = dtype == VLA_F32;
+  switch (d) {
+    case 16: return f32 ? launch_pair_d16_f32(p, sh, st) : launch_pair_d16_bf16(p, sh, st);
+    default: break;
+  }
+  VLA_CHUNK_DISPATCH(launch_pair, p, sh, st);
+  return VLA_ERR_UNSUPPORTED;
 }
 
 // ---------------------------------------------------------------- token kernel

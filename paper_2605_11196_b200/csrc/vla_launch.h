@@ -12,6 +12,7 @@ namespace vla {
 struct BackwardParams;
 struct BackwardSplitParams;
 struct MakeUParams;
+struct PairStash;
 }
 
 namespace vla {
@@ -21,6 +22,10 @@ int launch_token(int d, int dtype, const ScanParams& p, cudaStream_t st);
 
 // Single-step kernel (T = 1, carried states in and out, u = k_hat, no refresh), d in {32, 64, 128}.
 int launch_decode(int d, int dtype, const ScanParams& p, cudaStream_t st);
+
+// Pair kernel (two CTAs per unit, warp-level tensor-core products), d in {16, 32, 64, 128}, u = k_hat or
+// explicit, no refresh; sh: what a backward pass wants left behind, or nullptr.
+int launch_pair(int d, int dtype, const ScanParams& p, const PairStash* sh, cudaStream_t st);
 
 // Chunk kernel, d in {32, 64, 128}: plain or balanced grid, chosen from the shape.
 int launch_chunk(int d, int dtype, const ScanParams& p, cudaStream_t st);
@@ -69,6 +74,9 @@ void sched_slot_mark(unsigned int epoch, cudaStream_t st);
 
 // What the calling thread launched last (read back by vla_last_launch).
 void note_launch(const char* kernel, int d, int dtype, int grid, int balanced);
+
+// Multiprocessors of the current device (asked once per device); 0 on a failure.
+int device_sms();
 
 // Test kernel of the bounded wait: a barrier that never completes.
 int launch_wait_selftest(unsigned int probe_limit, int* status, cudaStream_t st);

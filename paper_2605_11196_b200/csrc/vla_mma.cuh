@@ -1,0 +1,228 @@
+// Warp-level matrix products in fp32 accuracy, shared by the pair kernel and the backward pass.
+//
+// Operands are split into two fp16 (or tf32) terms, x = hi + lo, and a product is
+// lo*hi + hi*lo + hi*hi: 22+ bits of each factor, the dropped lo*lo below 2^-24 of the product.  fp16
+// needs its operands inside the type's range, so every user scales by powers of two (exact) and
+// says where its bound comes from; in exchange mma.sync runs fp16 at twice the tf32 rate
+// (measured on B200: 1020 against 510 multiply-adds per clock and SM, 8 clk per instruction
+// and scheduler, 21 clk latency).  The small 16 x 16 products, whose range is the data's, use tf32.
+//
+// The tensor core truncates when it accumulates.  Chained over K = 64 same-signed terms that is a
+// one-sided error of 4.7e-7 of the sum (measured; an fp32 FMA chain: 1.2e-7 rms, unbiased), so
+// each K step starts from zero and its result is added in fp32 (6e-8 rms).
+#pragma once
+
+#include <cuda_fp16.h>
+#include <stdint.h>
+
+#include "vla_common.cuh"
+
+namespace vla {
+
+// ---------------------------------------------------------------- instructions
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_f16_zero(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+}
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_tf32_zero(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+}
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+
+// ---------------------------------------------------------------- splitting
+// two values -> packed fp16 pair of their rounded parts and of the remainders (x0 in the low half)
+__device__ __forceinline__ void split_f16(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(x1), "f"(x0));
+  const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hi));
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(x1 - h.y), "f"(x0 - h.x));
+}
+// hi: the upper 19 bits (a NaN stays one); lo: the remainder, rounded where the tensor core cuts it
+__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
+  hi = __float_as_uint(x) & 0xffffe000u;
+  lo = __float_as_uint(x - __uint_as_float(hi)) + 0x1000u;
+}
+// A operand (16 x 16) of an fp16 product from two neighbouring accumulator tiles (16 x 8 each)
+__device__ __forceinline__ void split_frag(const float (&t0)[4], const float (&t1)[4], uint32_t (&hi)[4],
+                                           uint32_t (&lo)[4]) {
+  split_f16(t0[0], t0[1], hi[0], lo[0]);
+  split_f16(t0[2], t0[3], hi[1], lo[1]);
+  split_f16(t1[0], t1[1], hi[2], lo[2]);
+  split_f16(t1[2], t1[3], hi[3], lo[3]);
+}
+// A operand (16 x 8) of a tf32 product from one accumulator tile.  The accumulator holds columns
+// (2c, 2c+1) where the operand wants (c, c+4): the contraction index is permuted accordingly, and
+// the B operand takes its rows 2c and 2c+1 in the same order.
+__device__ __forceinline__ void split_frag_tf32(const float (&t)[4], uint32_t (&hi)[4], uint32_t (&lo)[4]) {
+  split_tf32(t[0], hi[0], lo[0]);
+  split_tf32(t[2], hi[1], lo[1]);
+  split_tf32(t[1], hi[2], lo[2]);
+  split_tf32(t[3], hi[3], lo[3]);
+}
+
+// N independent products of one K step, acc[i] += A[i] B[i] as lo*hi + hi*lo + hi*hi from zero, added
+// in fp32.  A warp issues in order and an mma's result takes 21 clk, so the three dependent
+// instructions of one product are spread over the others' (at 8 clk apiece three products hide it).
+// a: index of the A operand of product i, b: its four B registers (hi 0, hi 1, lo 0, lo 1).
+template <int N, typename FA, typename FB, typename FC>
+__device__ __forceinline__ void mma3_f16_many(FA a, FB b, FC acc) {
+  float x[N][4];
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_f16_zero(x[i], a(i, 1), b(i, 0), b(i, 1));
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_f16(x[i], a(i, 0), b(i, 2), b(i, 3));
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_f16(x[i], a(i, 0), b(i, 0), b(i, 1));
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc(i)[e] += x[i][e];
+}
+// out (16 x 16 as two tiles) += X M^T for a small row-major M[n][k] (16 x 16 fp32, row stride LD) and
+// X in accumulator tiles (16 x 16).  M[n][k] is taken as 0 for n < 8 <= k (lower triangular matrices).
+template <int LD>
+__device__ __forceinline__ void small_product(float (&out)[2][4], const float (&x)[2][4], const float* M, int lane) {
+  const int g = lane >> 2, c = lane & 3;
+  // products (k half, n tile): (0, 0), (0, 1), (1, 1)
+  uint32_t ah[2][4], al[2][4], bh[3][2], bl[3][2];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int j = i >> 1, nt = (i + 1) >> 1;
+    const float2 b = *reinterpret_cast<const float2*>(M + (8 * nt + g) * LD + 8 * j + 2 * c);
+    split_tf32(b.x, bh[i][0], bl[i][0]);
+    split_tf32(b.y, bh[i][1], bl[i][1]);
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) split_frag_tf32(x[j], ah[j], al[j]);
+  float y[3][4];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) mma_tf32_zero(y[i], al[i >> 1], bl[i][0], bl[i][1]);   // (remainders up to 2^-10: kept)
+#pragma unroll
+  for (int i = 0; i < 3; ++i) mma_tf32(y[i], al[i >> 1], bh[i][0], bh[i][1]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) mma_tf32(y[i], ah[i >> 1], bl[i][0], bl[i][1]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) mma_tf32(y[i], ah[i >> 1], bh[i][0], bh[i][1]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    out[0][e] += y[0][e];
+    out[1][e] += y[1][e] + y[2][e];
+  }
+}
+
+// ---------------------------------------------------------------- operand arrays in shared memory
+// Token rows: [tokens][D fp16 hi | D fp16 lo], and vector rows: [index][16 tokens fp16 hi | lo].  A row is
+// an odd number of 16-byte pieces long (one of padding), so the eight rows an ldmatrix reads lie in
+// different banks while every address is a lane's base plus a constant.
+template <int D> constexpr uint32_t kTokRow = 4 * D + 16;
+constexpr uint32_t kVecRow = 80;
+
+// The lane's share of the ldmatrix address of each operand kind (add the array's base):
+// A operand, rows = tokens: matrices (rows 0-7, k 0-7), (8-15, 0-7), (0-7, 8-15), (8-15, 8-15)
+template <int D>
+__device__ __forceinline__ uint32_t tok_lane_a(int lane) {
+  return uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * kTokRow<D> + (lane >> 4) * 16;
+}
+// B operand, columns = tokens: r[0], r[1] for tokens 0-7, r[2], r[3] for tokens 8-15
+template <int D>
+__device__ __forceinline__ uint32_t tok_lane_b(int lane) {
+  return uint32_t((lane & 7) + (lane >> 4) * 8) * kTokRow<D> + ((lane >> 3) & 1) * 16;
+}
+// B operand with K = the 16 tokens, N = eight vector rows: hi in r[0], r[1], lo in r[2], r[3]
+__device__ __forceinline__ uint32_t vec_lane_b(int lane) { return uint32_t(lane & 7) * kVecRow + (lane >> 3) * 16; }
+// B operand with K = 16 vector rows, N = tokens (transposed load): r[0], r[1] for tokens 0-7, r[2], r[3] for 8-15
+__device__ __forceinline__ uint32_t vec_lane_bt(int lane) {
+  return uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * kVecRow + (lane >> 4) * 16;
+}
+// ... of one tile of eight tokens: hi in r[0], r[1], lo in r[2], r[3]
+__device__ __forceinline__ uint32_t vec_lane_bt1(int lane) {
+  return uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * kVecRow + (lane >> 4) * 32;
+}
+// K step ks of a token-row operand (hi, or the remainders)
+template <int D>
+__device__ __forceinline__ void tok_frag(uint32_t (&r)[4], uint32_t lane_base, int ks, bool lo) {
+  ldsm_x4(r, lane_base + 32 * ks + (lo ? 2 * D : 0));
+}
+// N tile nt of a vector-row operand (tokens contracted)
+__device__ __forceinline__ void vec_frag_b(uint32_t (&r)[4], uint32_t lane_base, int nt) { ldsm_x4(r, lane_base + nt * 8 * kVecRow); }
+// K step ks of a vector-row operand (tokens as columns)
+__device__ __forceinline__ void vec_frag_bt(uint32_t (&r)[4], uint32_t lane_base, int ks, bool lo) {
+  ldsm_x4_t(r, lane_base + ks * 16 * kVecRow + (lo ? 32 : 0));
+}
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts64(uint32_t addr, uint32_t v0, uint32_t v1) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(v0), "r"(v1) : "memory");
+}
+// a warp's 16 x 16 accumulator (rows g, g + 8; columns = tokens) into vector rows; base: row g's address + 4 c4
+__device__ __forceinline__ void vec_store(uint32_t base, const float (&x)[2][4]) {
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      uint32_t hi, lo;
+      split_f16(x[nt][2 * r], x[nt][2 * r + 1], hi, lo);
+      sts32(base + r * 8 * kVecRow + nt * 16, hi);
+      sts32(base + r * 8 * kVecRow + nt * 16 + 32, lo);
+    }
+}
+
+// ---------------------------------------------------------------- scales
+// the largest value over the warp of a non-negative float
+__device__ __forceinline__ float warp_max_nonneg(float x) {
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
+}
+// 2^k that brings a positive m into [2^target, 2^(target+1)); 1 for zero; k is kept within +-100
+__device__ __forceinline__ float pow2_scale(float m, int target) {
+  const int e = int(__float_as_uint(m) >> 23) - 127;
+  int k = target - e;
+  k = k > 100 ? 100 : (k < -100 ? -100 : k);
+  return m > 0.0f ? __uint_as_float(uint32_t(127 + k) << 23) : 1.0f;
+}
+// its inverse
+__device__ __forceinline__ float pow2_inverse(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
+
+// ---------------------------------------------------------------- cluster of two CTAs
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// own shared memory -> the other CTA's, completion counted in bytes on a barrier over there
+__device__ __forceinline__ void bulk_to_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "r"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+// "no longer read" to the other CTA (nothing is written before it that the other side reads; a
+// cluster-scope release here costs some 800 clk)
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+}  // namespace vla

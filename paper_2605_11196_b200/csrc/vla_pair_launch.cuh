@@ -1,0 +1,40 @@
+// Launchers of the pair kernel for one (d, input type); each vla_pair_d*.cu instantiates them.
+#pragma once
+
+#include "vla.h"
+#include "vla_launch.h"
+#include "vla_scan_pair.cuh"
+
+namespace vla {
+
+template <int D, typename TIn, bool UT, bool STASH>
+int launch_pair_t(const ScanParams& p, const PairStash& sh, cudaStream_t st) {
+  using Cfg = PairCfg<D, TIn, UT>;
+  static_assert(Cfg::smem_bytes <= 227 * 1024, "pair kernel exceeds the shared memory of one CTA");
+  if (p.units > 0x3fffffff) return VLA_ERR_INVALID_ARG;
+  auto kern = vla_scan_pair_kernel<D, TIn, UT, STASH>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Cfg::smem_bytes)) != cudaSuccess) {
+    cudaGetLastError();
+    return VLA_ERR_CUDA;
+  }
+  kern<<<2 * p.units, Cfg::NT, Cfg::smem_bytes, st>>>(p, sh);
+  note_launch(STASH ? "vla_scan_pair_kernel(stash)" : "vla_scan_pair_kernel", D, sizeof(TIn) == 2 ? VLA_BF16 : VLA_F32,
+              2 * p.units, 0);
+  return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
+}
+
+template <int D, typename TIn>
+int launch_pair_any(const ScanParams& p, const PairStash* sh, cudaStream_t st) {
+  const PairStash none = {};
+  if (sh) return p.u ? launch_pair_t<D, TIn, true, true>(p, *sh, st) : launch_pair_t<D, TIn, false, true>(p, *sh, st);
+  return p.u ? launch_pair_t<D, TIn, true, false>(p, none, st) : launch_pair_t<D, TIn, false, false>(p, none, st);
+}
+
+}  // namespace vla
+
+#define VLA_DEFINE_PAIR_TU(D, TIN, TAG)                                                          \
+  namespace vla {                                                                                \
+  int launch_pair_##TAG(const ScanParams& p, const PairStash* sh, cudaStream_t st) {             \
+    return launch_pair_any<D, TIN>(p, sh, st);                                                   \
+  }                                                                                              \
+  }

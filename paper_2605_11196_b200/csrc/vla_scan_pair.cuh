@@ -1,0 +1,993 @@
+// VLA forward scan, "pair" kernel: the 16-token chunk algebra of the recurrence (Eqs. "sm",
+// "s-update", "output") with every d x d product on warp-level tensor-core instructions and the
+// states in registers.  A cluster of two CTAs works on one (batch, head) unit:
+//
+//   rank 0 carries A.   Z0^T = A K^T;  W = K Z0 + I = L diag(delta) L^T;  Z = L^-1 Z0;
+//                       A <- A - Z^T diag(1/delta) Z;  alpha_t = sc_t z_t -> rank 1
+//   rank 1 carries S.   P = S K^T, R = S Q^T;  E = Tm (V - P), Tm = (I + stril(K alpha^T))^-1;
+//                       O = R + tril(Q alpha^T) E;  S <- S + E^T alpha
+//
+// (explicit u: Z0 = A U^T, W = U Z0, W0 = A K^T, N = L^-1 (U W0), a = W0 - tril(N^T diag(1/delta)) Z,
+// alpha = a / ||a||.)  A warp owns 16 rows of a state as accumulator tiles; an accumulator tile is also
+// the A operand of the next product, so a chunk's chain K -> Z0 -> Z -> A stays in one warp's
+// registers except for two exchanges over shared memory (Z0 for W, Z for the update); every
+// S row is independent of the others.  Beside the D / 16 state warps a CTA has one warp for the
+// 16 x 16 algebra and one or two that widen the inputs (phi, k_hat, hi/lo operand rows) one chunk ahead.
+//
+// What bounds it: at one unit per SM pair the serial chain of rank 0 (state split, Z0, W, the
+// 16 x 16 elimination, Z, update), with many units the tensor pipe (8 clk per instruction and
+// scheduler).  Two CTAs because at d = 128 both states and their operands do not fit one SM's
+// registers, and below because small batches then use twice the SMs.
+//
+// Ranges of the fp16 operands (vla_mma.cuh): k_hat and alpha are unit vectors, scaled by 2^8; A <= its
+// largest diagonal entry elementwise, which never grows, scaled to 2^7 (||A k|| then stays below 2^15 at
+// d = 128) and rescaled by powers of two as it shrinks; rows of Q and u by their own power of two;
+// S and E by powers of two per warp that follow their size.
+#pragma once
+
+#include "vla_mma.cuh"
+
+namespace vla {
+
+// What the forward leaves for the backward pass (STASH instantiations).  Per token: alpha_t, e_t
+// [units, T, D], zeta_t = z_t / sqrt(delta_t) (explicit u only), and scalars [units, T]:
+// delta_t, an_t = max(||a_t||, eps), 1 / den_t.  Per block of
+// `ck` chunks: the states and the key sum at its start, [units, blocks, ...].
+struct PairStash {
+  float *alpha, *zeta, *e, *delta, *an, *iden, *Ack, *Sck, *zck;
+  int ck;
+};
+
+template <int D, typename TIn, bool UT>
+struct PairCfg {
+  static constexpr int C = 16;
+  static constexpr int NW = D / 16;                         // state warps
+  static constexpr int NPREP = D == 128 ? 3 : D == 64 ? 2 : 1;   // widening warps
+  static constexpr int NT = (NW + 1 + NPREP) * 32;
+  static constexpr int LPT = D / 4;                         // lanes per token in the widening pass
+  static constexpr int TPW = 32 / LPT;                      // tokens per warp pass
+  static constexpr int NP = (C + TPW * NPREP - 1) / (TPW * NPREP);   // passes per chunk
+  static constexpr uint32_t piece = 4 * sizeof(TIn);        // bytes of a lane's four columns
+  static constexpr uint32_t raw_stage = 2 * NPREP * NP * 32 * piece;   // both tensors of a chunk as the lanes take them
+  static constexpr int RK = 2, RA = 4;                      // input and alpha slots
+  static constexpr int LD = 20;                             // row of a small matrix
+  static constexpr int SM = C * LD;
+  static constexpr int NJOB = UT ? 4 : 2;                   // 16 x 8 tiles of W [and X]
+  static constexpr int PARTS = NW > NJOB ? NW / NJOB : 1;   // contraction split over warps
+  static constexpr uint32_t kslot = 16 * kTokRow<D>;        // token rows of a chunk
+  static constexpr uint32_t aslot = kVecRow * D;            // vector rows of a chunk
+  // rank 0
+  static constexpr uint32_t a_K = 0, a_U = RK * kslot, a_Z0 = a_U + (UT ? RK * kslot : 0), a_W0 = a_Z0 + aslot,
+                            a_Z = a_W0 + (UT ? aslot : 0), a_A = a_Z + aslot, a_f = a_A + RA * aslot;
+  static constexpr int af_W = 0, af_Li = af_W + (UT ? 3 : 1) * PARTS * SM, af_PT = af_Li + SM, af_dl = af_PT + (UT ? 2 * SM : 0),
+                       af_n = af_dl + 32, af_mx = af_n + 2 * NW * 16, af_us = af_mx + 16, af_pv = af_us + RK * 16, af_end = af_pv + 64;
+  // rank 1
+  static constexpr uint32_t s_K = 0, s_Q = RK * kslot, s_A = 2 * RK * kslot, s_f = s_A + RA * aslot;
+  static constexpr int sf_N = 0, sf_T = SM, sf_H = sf_T + 2 * SM, sf_osc = sf_H + 2 * SM, sf_nrm = sf_osc + 32,
+                       sf_qs = sf_nrm + RK * 16, sf_dq = sf_qs + RK * 16, sf_zp = sf_dq + RK * 16, sf_end = sf_zp + 2 * NPREP * D;
+  static constexpr uint32_t f_end = (a_f + 4 * af_end > s_f + 4 * sf_end ? a_f + 4 * af_end : s_f + 4 * sf_end);
+  static constexpr uint32_t raw = (f_end + 15) / 16 * 16;
+  static constexpr uint32_t bars = raw + 2 * raw_stage;
+  static constexpr int NBAR = 2 * RK + 2 * RA + 6;
+  static constexpr size_t smem_bytes = bars + NBAR * 8 + 16;
+};
+
+// global -> shared, 16 or 8 bytes, zeros when !act (each lane reads back only what it copied itself)
+template <int BYTES>
+__device__ __forceinline__ void copy_piece(uint32_t dst, const void* src, bool act) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(BYTES), "r"(act ? BYTES : 0) : "memory");
+}
+__device__ __forceinline__ float4 piece_f32(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 piece_f32(const uint16_t* p) { return load4(p, 0); }
+
+// four consecutive columns of a token row, scaled, as hi/lo operand entries
+template <int D>
+__device__ __forceinline__ void tok_store4(uint32_t base, int row, int pl, float4 x, float s) {
+  uint32_t h0, l0, h1, l1;
+  split_f16(x.x * s, x.y * s, h0, l0);
+  split_f16(x.z * s, x.w * s, h1, l1);
+  const uint32_t at = base + uint32_t(row) * kTokRow<D> + 8 * pl;
+  sts64(at, h0, h1);
+  sts64(at + 2 * D, l0, l1);
+}
+
+template <int D, typename TIn, bool UT, bool STASH>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((PairCfg<D, TIn, UT>::NT), 1)
+vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
+  using Cfg = PairCfg<D, TIn, UT>;
+  constexpr int C = Cfg::C, NW = Cfg::NW, NPREP = Cfg::NPREP, LPT = Cfg::LPT, TPW = Cfg::TPW, NP = Cfg::NP;
+  constexpr int RK = Cfg::RK, RA = Cfg::RA, LD = Cfg::LD, SM = Cfg::SM, PARTS = Cfg::PARTS, NJOB = Cfg::NJOB;
+  constexpr int NTILE = D / 8, KS = D / 16, NB = NTILE < 4 ? NTILE : 4;
+  constexpr float kUnit = 256.0f, kUnitInv = 1.0f / 256.0f;   // scale of unit-vector operands
+
+  extern __shared__ __align__(1024) unsigned char smem[];
+  const uint32_t sb = smem_u32(smem);
+  const uint32_t rank = blockIdx.x & 1u;   // (of the cluster; from the block index, which the compiler knows to be uniform)
+  const int unit = int(blockIdx.x >> 1);
+  const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
+  // read from lane 0 so that the compiler takes the roles as uniform over a warp
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const bool ident = (p.flags & VLA_FLAG_IDENTITY_MAP) != 0;
+  const float eps = p.eps;
+  const int T = p.T;
+  const int nch = (T + C - 1) / C;
+
+  // barriers (both CTAs lay them out alike)
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::bars);
+  uint64_t* kfull = bars;             // [RK] a chunk's operand rows are written
+  uint64_t* kfree = kfull + RK;       // [RK] ... and no longer read
+  uint64_t* pfull = kfree + RK;       // [2] rank 0, explicit u: the coefficients of a are written
+  uint64_t* afull = pfull + 2;        // [RA] rank 1: alpha has arrived
+  uint64_t* aempty = afull + RA;      // [RA] rank 0: rank 1 no longer reads that slot
+  uint64_t* gfull = aempty + RA;      // [2] rank 1: Tm, H, output scales are written
+  uint64_t* gfree = gfull + 2;        // [2] ... and no longer read
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + Cfg::NBAR);
+
+  // Bounded wait; a limit that runs out is reported when the CTA ends.
+  const uint32_t probes = p.wait_limit == 0 ? kWaitProbeLimit : p.wait_limit;
+  auto wait = [&](uint64_t* bar, int parity) {
+    uint32_t it = 0;
+    while (!mbar_try_wait(bar, uint32_t(parity))) {
+      if (++it > probes || *abort_flag) {
+        *abort_flag = 1;
+        break;
+      }
+    }
+  };
+  auto arrive = [&](uint64_t* bar) {   // one arrival per warp
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
+  };
+  auto arrive_cl = [&](uint64_t* bar, uint32_t to) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(bar), to));
+  };
+
+  if (tid == 0) {
+    *abort_flag = 0;
+    for (int i = 0; i < RK; ++i) {
+      mbar_init(&kfull[i], NPREP);
+      mbar_init(&kfree[i], rank == 0 ? NW : NW + 1);
+    }
+    mbar_init(&pfull[0], 1);
+    mbar_init(&pfull[1], 1);
+    for (int i = 0; i < RA; ++i) {
+      mbar_init(&afull[i], 1);
+      mbar_init(&aempty[i], NW + 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&gfull[i], 1);
+      mbar_init(&gfree[i], NW);
+    }
+    mbar_init_fence();
+  }
+  __syncthreads();
+  cluster_sync();   // the other CTA's barriers exist before anything arrives on them
+
+  const uint32_t lane_ta = tok_lane_a<D>(lane), lane_tb = tok_lane_b<D>(lane), lane_vb = vec_lane_b(lane), lane_vt = vec_lane_bt(lane), lane_vn = vec_lane_bt1(lane);
+  const size_t tok0 = token_offset(p, unit, 0, D), tstride = token_stride(p, D);
+
+  if (warp > NW) {
+    // ===================================================================== widening warps
+    // A lane takes four columns of a token at a time, through a staging ring that only it reads; the
+    // copies of chunk c + 1 are in flight while chunk c is widened.  (Rolled loops: all warps' code
+    // together has to stay inside the SM's instruction cache.)
+    const int pw = warp - NW - 1, sub = lane / LPT, pl = lane % LPT;
+    const TIn* src0 = static_cast<const TIn*>(p.k) + tok0 + 4 * pl;
+    const bool two = UT || rank == 1;
+    const TIn* src1 = two ? static_cast<const TIn*>(rank ? p.q : p.u) + tok0 + 4 * pl : src0;
+    float* fs = reinterpret_cast<float*>(smem + (rank ? Cfg::s_f : Cfg::a_f));
+    const uint32_t base0 = sb + (rank ? Cfg::s_K : Cfg::a_K), base1 = sb + (rank ? Cfg::s_Q : Cfg::a_U);
+    auto stage = [&](int c, int ps) {   // byte offset of this lane's pieces (the second tensor's follows at + 32 pieces)
+      return Cfg::raw + (c & 1) * Cfg::raw_stage + uint32_t((ps * NPREP + pw) * 64 + lane) * Cfg::piece;
+    };
+    auto fetch = [&](int c) {
+#pragma unroll 1
+      for (int ps = 0; ps < NP; ++ps) {
+        const int t = c * C + (ps * NPREP + pw) * TPW + sub;
+        const bool act = t < T && (C % (TPW * NPREP) == 0 || (ps * NPREP + pw) * TPW < C);
+        const size_t off = act ? size_t(t) * tstride : 0;
+        copy_piece<Cfg::piece>(sb + stage(c, ps), src0 + off, act);
+        if (two) copy_piece<Cfg::piece>(sb + stage(c, ps) + 32 * Cfg::piece, src1 + off, act);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float zk[4] = {0.f, 0.f, 0.f, 0.f};
+    if (rank == 1 && p.z0) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) zk[e] = p.z0[size_t(unit) * D + 4 * pl + e];
+    }
+    if (nch > 0) fetch(0);
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) {
+      const int slot = c % RK;
+      fetch(c + 1);   // (past the end: zeros)
+      if (STASH && rank == 1 && c % sh.ck == 0 && pw == 0 && sub == 0) {
+        const size_t nblk = (nch + sh.ck - 1) / sh.ck;
+        *reinterpret_cast<float4*>(sh.zck + (size_t(unit) * nblk + c / sh.ck) * D + 4 * pl) = make_float4(zk[0], zk[1], zk[2], zk[3]);
+      }
+      if (c >= RK) wait(&kfree[slot], (c / RK - 1) & 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      float ks[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+      for (int ps = 0; ps < NP; ++ps) {
+        const int tt = (ps * NPREP + pw) * TPW + sub;
+        if (C % (TPW * NPREP) != 0 && tt >= C) break;   // (uniform over the warp: one token a pass there)
+        const bool act = c * C + tt < T;
+        const TIn* raw = reinterpret_cast<const TIn*>(smem + stage(c, ps));
+        float4 k = piece_f32(raw), x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (two) x = piece_f32(raw + 128);
+        if (!ident) {
+          k.x = phi_fast(k.x); k.y = phi_fast(k.y); k.z = phi_fast(k.z); k.w = phi_fast(k.w);
+          if (rank == 1) {
+            x.x = phi_fast(x.x); x.y = phi_fast(x.y); x.z = phi_fast(x.z); x.w = phi_fast(x.w);
+          }
+        }
+        if (!act) k = x = make_float4(0.f, 0.f, 0.f, 0.f);
+        float ss = fmaf(k.x, k.x, fmaf(k.y, k.y, fmaf(k.z, k.z, k.w * k.w)));
+        float qq = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
+        float dn = fmaf(x.x, zk[0], fmaf(x.y, zk[1], fmaf(x.z, zk[2], x.w * zk[3])));
+        ks[0] += k.x; ks[1] += k.y; ks[2] += k.z; ks[3] += k.w;
+#pragma unroll
+        for (int off = LPT / 2; off >= 1; off >>= 1) {
+          ss += __shfl_xor_sync(0xffffffffu, ss, off);
+          qq += __shfl_xor_sync(0xffffffffu, qq, off);
+          dn += __shfl_xor_sync(0xffffffffu, dn, off);
+        }
+        const float nr = fmaxf(sqrt_ftz(ss), eps);   // max(||phi(k)||, eps)
+        tok_store4<D>(base0 + slot * Cfg::kslot, tt, pl, k, rcp_ftz_nr(nr) * kUnit);
+        if (two) {
+          const float s = pow2_scale(sqrt_ftz(qq), 8);
+          tok_store4<D>(base1 + slot * Cfg::kslot, tt, pl, x, s);
+          if (pl == 0) fs[(rank ? Cfg::sf_qs : Cfg::af_us) + slot * 16 + tt] = pow2_inverse(s);
+        }
+        if (rank == 1 && pl == 0) {
+          fs[Cfg::sf_nrm + slot * 16 + tt] = act ? nr : 0.f;
+          fs[Cfg::sf_dq + slot * 16 + tt] = dn;
+        }
+      }
+      if (rank == 1 && !ident) {   // the key sum after this chunk
+#pragma unroll
+        for (int off = LPT; off < 32; off <<= 1)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) ks[e] += __shfl_xor_sync(0xffffffffu, ks[e], off);
+        if constexpr (NPREP > 1) {
+          float* zp = fs + Cfg::sf_zp + (c & 1) * NPREP * D;
+          if (sub == 0) *reinterpret_cast<float4*>(zp + pw * D + 4 * pl) = make_float4(ks[0], ks[1], ks[2], ks[3]);
+          named_sync(2, NPREP * 32);
+          ks[0] = ks[1] = ks[2] = ks[3] = 0.f;
+#pragma unroll
+          for (int w = 0; w < NPREP; ++w) {
+            const float4 y = *reinterpret_cast<const float4*>(zp + w * D + 4 * pl);
+            ks[0] += y.x; ks[1] += y.y; ks[2] += y.z; ks[3] += y.w;
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) zk[e] += ks[e];
+      }
+      arrive(&kfull[slot]);
+    }
+    if (rank == 1 && p.zT && pw == 0 && sub == 0)
+      *reinterpret_cast<float4*>(p.zT + size_t(unit) * D + 4 * pl) = make_float4(zk[0], zk[1], zk[2], zk[3]);
+  } else if (rank == 0 && warp == NW) {
+    // ===================================================================== rank 0: elimination
+    // I + W = L diag(delta) L^T in place, two columns a step: lane (r, h) holds row r, columns
+    // 8 h .. 8 h + 7; the slots of eliminated columns fill with L^-1 (the same row operations on the
+    // identity).  A step's latency is one shuffle, the 2 x 2 determinant's reciprocal and two FMAs.
+    float* fs = reinterpret_cast<float*>(smem + Cfg::a_f);
+    float* Li = fs + Cfg::af_Li;
+    float* dl = fs + Cfg::af_dl;
+    float* piv = fs + Cfg::af_pv;
+    const int r = lane & 15, h = lane >> 4;
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) {
+      named_sync(3, (NW + 1) * 32);   // W is written
+      float m[8];
+      {
+        const float4* w4 = reinterpret_cast<const float4*>(fs + Cfg::af_W + r * LD + 8 * h);
+        float4 x = w4[0], y = w4[1];
+#pragma unroll
+        for (int q = 1; q < PARTS; ++q) {
+          const float4 x2 = w4[q * SM / 4], y2 = w4[q * SM / 4 + 1];
+          x.x += x2.x; x.y += x2.y; x.z += x2.z; x.w += x2.w;
+          y.x += y2.x; y.y += y2.y; y.z += y2.z; y.w += y2.w;
+        }
+        m[0] = x.x; m[1] = x.y; m[2] = x.z; m[3] = x.w;
+        m[4] = y.x; m[5] = y.y; m[6] = y.z; m[7] = y.w;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) m[j] += (8 * h + j == r) ? 1.0f : 0.0f;
+      float delta = 1.0f;
+      // (an all but rolled loop: the registers rotate by two a step, so that columns s, s + 1 are always m[0], m[1]
+      // of the half that holds them; eight steps bring them back)
+#pragma unroll 2
+      for (int s = 0; s < 16; s += 2) {
+        constexpr unsigned full = 0xffffffffu;
+        const int hs = s >> 3;
+        float* rows = piv + (s & 2) * 16;
+        const float a0 = __shfl_sync(full, m[0], s + 16 * hs);
+        const float b = __shfl_sync(full, m[0], s + 1 + 16 * hs);
+        const float d = __shfl_sync(full, m[1], s + 1 + 16 * hs);
+        const float ms0 = __shfl_sync(full, m[0], r + 16 * hs);
+        const float ms1 = __shfl_sync(full, m[1], r + 16 * hs);
+        if ((r | 1) == s + 1) {
+          float4* o = reinterpret_cast<float4*>(rows + (r & 1) * 16 + 8 * h);
+          o[0] = make_float4(m[0], m[1], m[2], m[3]);
+          o[1] = make_float4(m[4], m[5], m[6], m[7]);
+        }
+        __syncwarp();
+        const float4 x0 = *reinterpret_cast<const float4*>(rows + 8 * h), x1 = *reinterpret_cast<const float4*>(rows + 8 * h + 4);
+        const float4 y0 = *reinterpret_cast<const float4*>(rows + 16 + 8 * h), y1 = *reinterpret_cast<const float4*>(rows + 20 + 8 * h);
+        const float r0[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+        const float r1[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+        // Algorithm 1 clamps delta at eps (delta >= 1 whenever A is positive definite)
+        const float a = fmaxf(a0, eps);
+        const float det = fmaxf(fmaf(a, d, -b * b), eps * a);
+        const float idet = rcp_ftz(det), ia = rcp_ftz(a);
+        const float n0 = fmaf(d, ms0, -b * ms1), n1 = fmaf(a, ms1, -b * ms0);
+        const float q = r == s + 1 ? b * ia : 0.0f;     // row s + 1 loses its multiple of row s
+        const float im = r > s + 1 ? idet : 0.0f;
+        delta = r == s ? a : delta;
+        delta = r == s + 1 ? det * ia : delta;
+        const float w0 = fmaf(n0, im, q), w1 = n1 * im;
+        float t[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          // in the slots of columns s, s + 1 the identity's entries take the raw ones' place
+          const bool mine = h == hs;
+          const float c0 = j == 0 ? (mine ? 1.0f : r0[0]) : (mine && r > s + 1 ? 0.0f : r0[1]);
+          const float c1 = mine ? (j == 0 ? 0.0f : 1.0f) : r1[j];
+          const float mj = mine && r > s + j ? 0.0f : m[j];
+          t[j] = fmaf(-w0, c0, fmaf(-w1, c1, mj));
+        }
+#pragma unroll
+        for (int j = 0; j < 6; ++j) m[j] = fmaf(-w0, r0[j + 2], fmaf(-w1, r1[j + 2], m[j + 2]));
+        m[6] = t[0];
+        m[7] = t[1];
+      }
+      {
+        float x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = 8 * h + j < r ? m[j] : (8 * h + j == r ? 1.0f : 0.0f);
+        float4* o = reinterpret_cast<float4*>(Li + r * LD + 8 * h);
+        o[0] = make_float4(x[0], x[1], x[2], x[3]);
+        o[1] = make_float4(x[4], x[5], x[6], x[7]);
+        if (h == 0) {
+          dl[r] = delta;
+          dl[16 + r] = rcp_ftz_nr(delta);
+        }
+      }
+      named_arrive(4, (NW + 1) * 32);   // L^-1 and delta are written
+      if (STASH && h == 0 && c * C + r < T) sh.delta[size_t(unit) * T + c * C + r] = delta;
+      if constexpr (UT) {
+        // N = L^-1 X, X[s][t] = u_s . A k_t;  PT[t][s] = N[s][t] / delta_s for s <= t
+        // (X and PT alternate between two buffers: the state warps may be a chunk ahead here)
+        const float* X = fs + Cfg::af_W + (1 + (c & 1)) * PARTS * SM;
+        float* PT = fs + Cfg::af_PT + (c & 1) * SM;
+        float n[2][4] = {};
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const float2 la = *reinterpret_cast<const float2*>(Li + g * LD + 8 * j + 2 * c4);
+          const float2 lb = *reinterpret_cast<const float2*>(Li + (g + 8) * LD + 8 * j + 2 * c4);
+          const float lt[4] = {la.x, la.y, lb.x, lb.y};
+          uint32_t ah[4], al[4];
+          split_frag_tf32(lt, ah, al);
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) {
+            float b0 = 0.f, b1 = 0.f;
+#pragma unroll
+            for (int q = 0; q < PARTS; ++q) {
+              b0 += X[q * SM + (8 * j + 2 * c4) * LD + 8 * nt + g];
+              b1 += X[q * SM + (8 * j + 2 * c4 + 1) * LD + 8 * nt + g];
+            }
+            uint32_t bh0, bl0, bh1, bl1;
+            split_tf32(b0, bh0, bl0);
+            split_tf32(b1, bh1, bl1);
+            float x[4];
+            mma_tf32_zero(x, al, bl0, bl1);
+            mma_tf32(x, al, bh0, bh1);
+            mma_tf32(x, ah, bl0, bl1);
+            mma_tf32(x, ah, bh0, bh1);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) n[nt][e] += x[e];
+          }
+        }
+        const float i0 = dl[16 + g], i1 = dl[24 + g];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int t = 8 * nt + 2 * c4 + e;
+            PT[t * LD + g] = g <= t ? n[nt][e] * i0 : 0.0f;
+            PT[t * LD + g + 8] = g + 8 <= t ? n[nt][2 + e] * i1 : 0.0f;
+          }
+        arrive(&pfull[c & 1]);
+      }
+    }
+  } else if (rank == 0) {
+    // ===================================================================== rank 0: state warps
+    float* fs = reinterpret_cast<float*>(smem + Cfg::a_f);
+    float* Wp = fs + Cfg::af_W;
+    const float* Li = fs + Cfg::af_Li;
+    const float* dl = fs + Cfg::af_dl;
+    float* mxs = fs + Cfg::af_mx;
+    const int row0 = 16 * warp;
+    const uint32_t my_rows = uint32_t(row0 + g) * kVecRow + 4 * c4;
+    const uint32_t remote_A = map_to_rank(sb + Cfg::s_A, 1);
+    float st[NTILE][4];
+    float sA, sAi;                   // st = sA * A
+    {
+      float dm = 0.f;
+      if (p.A0) {
+        for (int i = lane; i < D; i += 32) dm = fmaxf(dm, fabsf(p.A0[(size_t(unit) * D + i) * D + i]));
+        dm = warp_max_nonneg(dm);
+      } else {
+        dm = 1.0f / p.lambda;
+      }
+      sA = pow2_scale(dm, 7);
+      sAi = pow2_inverse(sA);
+#pragma unroll
+      for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          const int row = row0 + g + 8 * hf, col = 8 * nt + 2 * c4;
+          float2 x;
+          if (p.A0) x = *reinterpret_cast<const float2*>(p.A0 + (size_t(unit) * D + row) * D + col);
+          else x = make_float2(row == col ? dm : 0.f, row == col + 1 ? dm : 0.f);
+          st[nt][2 * hf] = x.x * sA;
+          st[nt][2 * hf + 1] = x.y * sA;
+        }
+    }
+    // Off the serial chain, while the other warp eliminates chunk c: the squared norms of the rows a_t of
+    // chunk c - 1 (a_t = A_t k_hat_t in true units), and alpha of chunk c - 2 to rank 1.
+    float a1[2][4], a2[2][4] = {};   // a of chunks c - 1 and c - 2
+    float w1[2][4] = {}, z1[2][4] = {};   // explicit u: W0 and Z of chunk c - 1
+    auto between = [&](int c, float sz1) {
+      const int c1 = c - 1, c2 = c - 2;
+      float* np = fs + Cfg::af_n;
+      if (c2 >= 0 && c2 < nch) {
+        float al[2][4];
+        bool bad = false;
+        const float* q = np + (c2 & 1) * NW * 16;
+        const int as = c2 % RA;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            float n2 = 0.f;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) n2 += q[w * 16 + 8 * nt + 2 * c4 + e];
+            const float an = fmaxf(sqrt_ftz(n2), eps), sc = rcp_ftz_nr(an);
+            al[nt][e] = a2[nt][e] * sc;
+            al[nt][2 + e] = a2[nt][2 + e] * sc;
+            const int t = c2 * C + 8 * nt + 2 * c4 + e;
+            if constexpr (STASH) {
+              if (t < T) {
+                float* o = sh.alpha + (size_t(unit) * T + t) * D + row0 + g;
+                o[0] = al[nt][e];
+                o[8] = al[nt][2 + e];
+                if (warp == 0 && g == 0) sh.an[size_t(unit) * T + t] = an;
+              }
+            }
+            bad |= !isfinite(n2);
+            al[nt][e] *= kUnit;
+            al[nt][2 + e] *= kUnit;
+          }
+        if (bad && (p.flags & VLA_FLAG_CHECK_FINITE) && p.status) atomicCAS(p.status, 0, int(VLA_ERR_NONFINITE));
+        if (c2 >= RA) wait(&aempty[as], (c2 / RA - 1) & 1);   // (the staged rows have been copied too, then)
+        const uint32_t stage = sb + Cfg::a_A + as * Cfg::aslot;
+        vec_store(stage + my_rows, al);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0 && !*abort_flag)
+          bulk_to_cluster(remote_A + as * Cfg::aslot + row0 * kVecRow, stage + row0 * kVecRow, 16 * kVecRow,
+                          map_to_rank(smem_u32(&afull[as]), 1));
+      }
+      if (c1 < nch && c1 >= 0) {
+        if constexpr (UT) {
+          // a^T = (A K^T) - Z^T PT^T of the chunk, both scaled by sA
+          wait(&pfull[c1 & 1], (c1 >> 1) & 1);   // (the elimination may be a chunk ahead: two barriers)
+          float t[2][4] = {};
+          small_product<LD>(t, z1, fs + Cfg::af_PT + (c1 & 1) * SM, lane);
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a1[nt][e] = (w1[nt][e] - t[nt][e]) * sz1;
+        }
+        float n2[4];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) n2[2 * nt + e] = fmaf(a1[nt][e], a1[nt][e], a1[nt][2 + e] * a1[nt][2 + e]);
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) n2[i] += __shfl_xor_sync(0xffffffffu, n2[i], off);
+        if (g == 0) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) np[(c1 & 1) * NW * 16 + warp * 16 + 8 * (i >> 1) + 2 * c4 + (i & 1)] = n2[i];
+        }
+      }
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) a2[nt][e] = a1[nt][e];
+    };
+    float sz1 = 0.f;
+    if (nch > 0) wait(&kfull[0], 0);
+#pragma unroll 1
+    for (int c = 0; c < nch + 2; ++c) {   // (the last two rounds only pass on the last two chunks' alpha)
+      const bool live = c < nch;
+      const int slot = c % RK;
+      const uint32_t Kop = sb + Cfg::a_K + slot * Cfg::kslot, Uop = UT ? sb + Cfg::a_U + slot * Cfg::kslot : Kop;
+      if (STASH && live && c % sh.ck == 0) {
+        const size_t nblk = (nch + sh.ck - 1) / sh.ck;
+        float* dst = sh.Ack + (size_t(unit) * nblk + c / sh.ck) * D * D;
+#pragma unroll
+        for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf)
+            *reinterpret_cast<float2*>(dst + size_t(row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
+                make_float2(st[nt][2 * hf] * sAi, st[nt][2 * hf + 1] * sAi);
+      }
+      // ---- Z0^T = A U^T (rows: this warp's state rows, columns: tokens), with an explicit u also A K^T
+      float z0[2][4] = {}, w0[2][4] = {};
+      if (live) {
+      constexpr int KB = (KS >= 2 && !UT) ? 2 : 1;   // K steps whose products are interleaved
+#pragma unroll
+      for (int ks = 0; ks < KS; ks += KB) {
+        uint32_t ah[KB][4], al[KB][4], bh[2][4], bl[2][4];   // UT: operand 0 is U, 1 is K; else K step
+#pragma unroll
+        for (int i = 0; i < KB; ++i) split_frag(st[2 * (ks + i)], st[2 * (ks + i) + 1], ah[i], al[i]);
+#pragma unroll
+        for (int i = 0; i < (UT ? 2 : KB); ++i) {
+          tok_frag<D>(bh[i], (i == 0 || !UT ? Uop : Kop) + lane_tb, ks + (UT ? 0 : i), false);
+          tok_frag<D>(bl[i], (i == 0 || !UT ? Uop : Kop) + lane_tb, ks + (UT ? 0 : i), true);
+        }
+        // product i: operand (K step, or U / K) i >> 1, token tile i & 1
+        mma3_f16_many<UT ? 4 : 2 * KB>(
+            [&](int i, int lo) -> const uint32_t(&)[4] { return lo ? al[UT ? 0 : i >> 1] : ah[UT ? 0 : i >> 1]; },
+            [&](int i, int r) { return (r & 2) ? bl[i >> 1][2 * (i & 1) + (r & 1)] : bh[i >> 1][2 * (i & 1) + (r & 1)]; },
+            [&](int i) -> float* { return UT && i >= 2 ? w0[i & 1] : z0[i & 1]; });
+      }
+      const float* us = fs + Cfg::af_us + slot * 16;
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          z0[nt][e] *= UT ? us[8 * nt + 2 * c4 + (e & 1)] : kUnitInv;
+          w0[nt][e] *= kUnitInv;
+        }
+      vec_store(sb + Cfg::a_Z0 + my_rows, z0);
+      if (UT) vec_store(sb + Cfg::a_W0 + my_rows, w0);
+      named_sync(1, NW * 32);
+      // ---- W = U Z0 [and X = U W0], one 16 x 8 tile a job, the contraction split over PARTS warps
+      const int part = NW > NJOB ? warp / NJOB : 0;
+#pragma unroll 1
+      for (int job = NW >= NJOB ? warp % NJOB : warp; job < NJOB; job += NW) {
+        float acc[4] = {};
+        constexpr int K2 = KS / PARTS < 2 ? 1 : 2;
+        const uint32_t src = sb + (job >= 2 ? Cfg::a_W0 : Cfg::a_Z0) + lane_vn + (job & 1) * 16 + part * (KS / PARTS) * 16 * kVecRow;
+        const uint32_t rows = Uop + lane_ta + part * (KS / PARTS) * 32;
+#pragma unroll
+        for (int k2 = 0; k2 < KS / PARTS; k2 += K2) {
+          uint32_t ah[K2][4], al[K2][4], b[K2][4];
+#pragma unroll
+          for (int i = 0; i < K2; ++i) {
+            tok_frag<D>(ah[i], rows, k2 + i, false);
+            tok_frag<D>(al[i], rows, k2 + i, true);
+            vec_frag_bt(b[i], src, k2 + i, false);
+          }
+          mma3_f16_many<K2>([&](int i, int lo) -> const uint32_t(&)[4] { return lo ? al[i] : ah[i]; },
+                            [&](int i, int r) { return b[i][r]; }, [&](int) -> float* { return acc; });
+        }
+        const float s0 = sAi * (UT ? us[g] : kUnitInv), s1 = sAi * (UT ? us[g + 8] : kUnitInv);
+        float* dst = Wp + ((job >= 2 ? 1 + (c & 1) : 0) * PARTS + part) * SM + 8 * (job & 1) + 2 * c4;
+        *reinterpret_cast<float2*>(dst + g * LD) = make_float2(acc[0] * s0, acc[1] * s0);
+        *reinterpret_cast<float2*>(dst + (g + 8) * LD) = make_float2(acc[2] * s1, acc[3] * s1);
+      }
+      named_arrive(3, (NW + 1) * 32);
+      arrive(&kfree[slot]);
+      }
+      // ---- while the elimination runs
+      between(c, sz1);
+      if (!live) {
+        named_sync(1, NW * 32);
+        continue;
+      }
+      if (c + 1 < nch) wait(&kfull[(c + 1) % RK], ((c + 1) / RK) & 1);
+      const bool look = (c & 7) == 7;
+      if (look) {   // A shrinks as tokens come: keep its operands inside fp16's range
+        float mx = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fabsf(st[nt][e]));
+        mx = warp_max_nonneg(mx);
+        if (lane == 0) mxs[warp] = mx;
+      }
+      named_sync(4, (NW + 1) * 32);   // L^-1
+      // ---- Z^T = Z0^T L^-T
+      float z[2][4] = {};
+      small_product<LD>(z, z0, Li, lane);
+      vec_store(sb + Cfg::a_Z + my_rows, z);
+      uint32_t yh[4], yl[4];
+      {
+        float y[2][4];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float idl = dl[16 + 8 * nt + 2 * c4 + (e & 1)];
+            y[nt][e] = -z[nt][e] * idl;
+            if (!UT) a1[nt][e] = -y[nt][e] * sAi;   // u = k_hat: a_t = z_t / delta_t
+            else { z1[nt][e] = z[nt][e]; w1[nt][e] = w0[nt][e]; }
+            if (STASH && UT) {
+              const int t = c * C + 8 * nt + 2 * c4 + (e & 1);
+              if (t < T) sh.zeta[(size_t(unit) * T + t) * D + row0 + g + 8 * (e >> 1)] = z[nt][e] * sAi * sqrt_ftz(idl);
+            }
+          }
+        sz1 = sAi;
+        split_frag(y[0], y[1], yh, yl);
+      }
+      named_sync(1, NW * 32);
+      // ---- A <- A - Z^T diag(1/delta) Z
+#pragma unroll
+      for (int nt = 0; nt < NTILE; nt += NB) {
+        uint32_t b[NB][4];
+        float x[NB][4];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) vec_frag_b(b[i], sb + Cfg::a_Z + lane_vb, nt + i);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) mma_f16_zero(x[i], yl, b[i][0], b[i][1]);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) mma_f16(x[i], yh, b[i][2], b[i][3]);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) mma_f16(x[i], yh, b[i][0], b[i][1]);
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) st[nt + i][e] = fmaf(x[i][e], sAi, st[nt + i][e]);
+      }
+      if (look) {
+        float mx = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) mx = fmaxf(mx, mxs[w]);
+        if (mx < 8.0f) {
+          const float f = pow2_scale(mx, 7);
+#pragma unroll
+          for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) st[nt][e] *= f;
+          sA *= f;
+          sAi = pow2_inverse(sA);
+        }
+      }
+    }
+    // rank 1's arrivals on this CTA's barriers must have landed before the CTA may leave (the cluster
+    // barrier at the end does not order them): wait for the last use of every slot
+    for (int c = nch > RA ? nch - RA : 0; c < nch; ++c) wait(&aempty[c % RA], (c / RA) & 1);
+    if (p.A_T) {
+#pragma unroll
+      for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+          *reinterpret_cast<float2*>(p.A_T + (size_t(unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
+              make_float2(st[nt][2 * hf] * sAi, st[nt][2 * hf + 1] * sAi);
+    }
+  } else if (warp == NW) {
+    // ===================================================================== rank 1: small matrices
+    // N = K alpha^T, H = Q alpha^T, Q K^T; Tm = (I + stril(N))^-1; output scales 1 / (den_t * scale of q_t)
+    float* fs = reinterpret_cast<float*>(smem + Cfg::s_f);
+    float* Nb = fs + Cfg::sf_N;
+    if (lane == 0) {
+      for (int i = 0; i < RA && i < nch; ++i) mbar_arrive_expect_tx(&afull[i], Cfg::aslot);
+    }
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) {
+      const int slot = c % RK, as = c % RA, gs = c & 1;
+      const uint32_t Kop = sb + Cfg::s_K + slot * Cfg::kslot, Qop = sb + Cfg::s_Q + slot * Cfg::kslot;
+      const uint32_t Aop = sb + Cfg::s_A + as * Cfg::aslot;
+      float* Tm = fs + Cfg::sf_T + gs * SM;
+      float* H = fs + Cfg::sf_H + gs * SM;
+      float* osc = fs + Cfg::sf_osc + gs * 16;
+      wait(&kfull[slot], (c / RK) & 1);
+      float qk[2][4] = {};
+      constexpr int K2 = KS >= 2 ? 2 : 1;
+      if (!ident) {
+#pragma unroll 1
+        for (int ks = 0; ks < KS; ks += K2) {
+          uint32_t ah[K2][4], al[K2][4], bh[K2][4], bl[K2][4];
+#pragma unroll
+          for (int i = 0; i < K2; ++i) {
+            tok_frag<D>(ah[i], Qop + lane_ta, ks + i, false);
+            tok_frag<D>(al[i], Qop + lane_ta, ks + i, true);
+            tok_frag<D>(bh[i], (Kop) + lane_tb, ks + i, false);
+            tok_frag<D>(bl[i], (Kop) + lane_tb, ks + i, true);
+          }
+          mma3_f16_many<2 * K2>([&](int i, int lo) -> const uint32_t(&)[4] { return lo ? al[i >> 1] : ah[i >> 1]; },
+                                [&](int i, int r) { return (r & 2) ? bl[i >> 1][2 * (i & 1) + (r & 1)] : bh[i >> 1][2 * (i & 1) + (r & 1)]; },
+                                [&](int i) -> float* { return qk[i & 1]; });
+        }
+      }
+      const float* nrm = fs + Cfg::sf_nrm + slot * 16;
+      const float qsi[2] = {fs[Cfg::sf_qs + slot * 16 + g], fs[Cfg::sf_qs + slot * 16 + g + 8]};
+      const float* dq = fs + Cfg::sf_dq + slot * 16;
+      float den[2] = {0.f, 0.f};
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int t = g + 8 * hf;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int s = 8 * nt + 2 * c4 + e;
+            if (s <= t) den[hf] = fmaf(nrm[s], qk[nt][2 * hf + e], den[hf]);
+          }
+        den[hf] += __shfl_xor_sync(0xffffffffu, den[hf], 1);
+        den[hf] += __shfl_xor_sync(0xffffffffu, den[hf], 2);
+        den[hf] = fmaf(den[hf], qsi[hf] * kUnitInv, dq[t]);
+      }
+      wait(&afull[as], (c / RA) & 1);
+      __syncwarp();
+      if (lane == 0 && c + RA < nch) mbar_arrive_expect_tx(&afull[as], Cfg::aslot);   // arm the slot's next use
+      float n[2][4] = {}, hh[2][4] = {};
+#pragma unroll 1
+      for (int ks = 0; ks < KS; ++ks) {
+        uint32_t ah[2][4], al[2][4], bh[4], bl[4];
+        vec_frag_bt(bh, Aop + lane_vt, ks, false);
+        vec_frag_bt(bl, Aop + lane_vt, ks, true);
+        tok_frag<D>(ah[0], Kop + lane_ta, ks, false);
+        tok_frag<D>(al[0], Kop + lane_ta, ks, true);
+        tok_frag<D>(ah[1], Qop + lane_ta, ks, false);
+        tok_frag<D>(al[1], Qop + lane_ta, ks, true);
+        mma3_f16_many<4>([&](int i, int lo) -> const uint32_t(&)[4] { return lo ? al[i >> 1] : ah[i >> 1]; },
+                         [&](int i, int r) { return (r & 2) ? bl[2 * (i & 1) + (r & 1)] : bh[2 * (i & 1) + (r & 1)]; },
+                         [&](int i) -> float* { return i >= 2 ? hh[i & 1] : n[i & 1]; });
+      }
+      __syncwarp();
+      arrive(&kfree[slot]);
+      arrive_cl(&aempty[as], 0);
+      if (c >= 2) wait(&gfree[gs], (c / 2 - 1) & 1);
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int t = g + 8 * hf;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          const int s = 8 * nt + 2 * c4;
+          constexpr float f = kUnitInv * kUnitInv;
+          *reinterpret_cast<float2*>(Nb + t * LD + s) = make_float2(n[nt][2 * hf] * f, n[nt][2 * hf + 1] * f);
+          *reinterpret_cast<float2*>(H + t * LD + s) =
+              make_float2(s <= t ? hh[nt][2 * hf] * kUnitInv : 0.f, s + 1 <= t ? hh[nt][2 * hf + 1] * kUnitInv : 0.f);
+        }
+        if (c4 == 0) {
+          const float id = ident ? 1.0f : rcp_ftz_nr(fmaxf(den[hf], eps));
+          osc[t] = id * qsi[hf];
+          if (STASH && c * C + t < T) sh.iden[size_t(unit) * T + c * C + t] = id;
+        }
+      }
+      __syncwarp();
+      // Tm = (I + stril(N))^-1 by 8 x 8 blocks: the two on the diagonal by forward substitution (lane j + 8 b:
+      // column j of block b; the upper lanes repeat it), then -T22 N21 T11
+      {
+        const int j = lane & 7, b8 = lane & 8;
+        const float* Nd = Nb + b8 * LD + b8;
+        float x[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          float a0 = t == j ? 1.0f : 0.0f, a1 = 0.f;
+#pragma unroll
+          for (int s4 = 0; 4 * s4 < t; ++s4) {
+            const float4 y = *reinterpret_cast<const float4*>(Nd + t * LD + 4 * s4);
+            a0 = fmaf(-y.x, x[4 * s4], a0);
+            if (4 * s4 + 1 < t) a1 = fmaf(-y.y, x[4 * s4 + 1], a1);
+            if (4 * s4 + 2 < t) a0 = fmaf(-y.z, x[4 * s4 + 2], a0);
+            if (4 * s4 + 3 < t) a1 = fmaf(-y.w, x[4 * s4 + 3], a1);
+          }
+          x[t] = a0 + a1;
+        }
+        if (lane < 16) {
+#pragma unroll
+          for (int t = 0; t < 8; ++t) Tm[(b8 + t) * LD + b8 + j] = x[t];
+          // (the consumers skip the upper right block)
+        }
+        __syncwarp();
+        // lane: row r of the block, columns 2 c4, 2 c4 + 1
+        float2 y = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const float nk = Nb[(8 + g) * LD + k];
+          const float2 tk = *reinterpret_cast<const float2*>(Tm + k * LD + 2 * c4);
+          y.x = fmaf(nk, tk.x, y.x);
+          y.y = fmaf(nk, tk.y, y.y);
+        }
+        float2* Y = reinterpret_cast<float2*>(Nb + 8) ;   // (the block of N above the diagonal is free)
+        Y[(g * LD + 2 * c4) / 2] = y;
+        __syncwarp();
+        float2 z = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const float tk = Tm[(8 + g) * LD + 8 + k];
+          const float2 yk = Y[(k * LD + 2 * c4) / 2];
+          z.x = fmaf(-tk, yk.x, z.x);
+          z.y = fmaf(-tk, yk.y, z.y);
+        }
+        *reinterpret_cast<float2*>(Tm + (8 + g) * LD + 2 * c4) = z;
+      }
+      arrive(&gfull[gs]);
+    }
+  } else {
+    // ===================================================================== rank 1: state warps
+    float* fs = reinterpret_cast<float*>(smem + Cfg::s_f);
+    const int row0 = 16 * warp;
+    float st[NTILE][4];
+    float sS = 1.0f, sSi = 1.0f;     // st = sS * S
+    float bound = 0.0f;              // largest entry of st, from above
+    auto true_max = [&]() {
+      float mx = 0.f;
+#pragma unroll
+      for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fabsf(st[nt][e]));
+      return warp_max_nonneg(mx);
+    };
+    auto rescale = [&](float mx) {
+      bound = mx;
+      if (mx > 0.0f && (mx > 512.0f || mx < 1.0f)) {
+        // (sS itself stays within 2^+-100)
+        float f = pow2_scale(mx, 5);
+        const float ns = fminf(fmaxf(sS * f, 7.888609e-31f), 1.2676506e30f);
+        f = ns * sSi;
+#pragma unroll
+        for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) st[nt][e] *= f;
+        sS = ns;
+        sSi = pow2_inverse(ns);
+        bound = mx * f;
+      }
+    };
+#pragma unroll
+    for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        float2 x = make_float2(0.f, 0.f);
+        if (p.S0) x = *reinterpret_cast<const float2*>(p.S0 + (size_t(unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4);
+        st[nt][2 * hf] = x.x;
+        st[nt][2 * hf + 1] = x.y;
+      }
+    bool look = p.S0 != nullptr;
+    // this lane's four tokens of a chunk: 2 c4, 2 c4 + 1, and 8 further
+    const size_t my0 = tok0 + size_t(2 * c4) * tstride + row0 + g;
+    const TIn* vsrc = static_cast<const TIn*>(p.v) + my0;
+    float* odst = p.out + my0;
+    float* edst = STASH ? sh.e + (size_t(unit) * T + 2 * c4) * D + row0 + g : nullptr;
+    float vn[8];
+    auto fetch_v = [&](int c) {   // v^T in accumulator order: [token tile][row half * 2 + token]
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const TIn* q = vsrc + (k & 1 ? tstride : 0) + (k & 2 ? 8 * tstride : 0);
+        const bool act = c * C + 2 * c4 + (k & 1) + 4 * (k & 2) < T;
+        vn[2 * (k & 2) + (k & 1)] = act ? load1<TIn>(q, 0) : 0.0f;
+        vn[2 * (k & 2) + 2 + (k & 1)] = act ? load1<TIn>(q, 8) : 0.0f;
+      }
+      vsrc += 16 * tstride;
+    };
+    if (nch > 0) fetch_v(0);
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) {
+      const int slot = c % RK, as = c % RA, gs = c & 1;
+      const uint32_t Kop = sb + Cfg::s_K + slot * Cfg::kslot, Qop = sb + Cfg::s_Q + slot * Cfg::kslot;
+      const uint32_t Aop = sb + Cfg::s_A + as * Cfg::aslot;
+      if (look) rescale(true_max());
+      if (STASH && c % sh.ck == 0) {
+        const size_t nblk = (nch + sh.ck - 1) / sh.ck;
+        float* dst = sh.Sck + (size_t(unit) * nblk + c / sh.ck) * D * D;
+#pragma unroll
+        for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf)
+            *reinterpret_cast<float2*>(dst + size_t(row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
+                make_float2(st[nt][2 * hf] * sSi, st[nt][2 * hf + 1] * sSi);
+      }
+      wait(&kfull[slot], (c / RK) & 1);
+      // ---- P = S K^T and R = S Q^T (rows: this warp's, columns: tokens)
+      float pk[2][4] = {}, rq[2][4] = {};
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) {
+        uint32_t ah[4], al[4], bh[2][4], bl[2][4];
+        split_frag(st[2 * ks], st[2 * ks + 1], ah, al);
+        tok_frag<D>(bh[0], (Kop) + lane_tb, ks, false);
+        tok_frag<D>(bl[0], (Kop) + lane_tb, ks, true);
+        tok_frag<D>(bh[1], (Qop) + lane_tb, ks, false);
+        tok_frag<D>(bl[1], (Qop) + lane_tb, ks, true);
+        mma3_f16_many<4>([&](int, int lo) -> const uint32_t(&)[4] { return lo ? al : ah; },
+                         [&](int i, int r) { return (r & 2) ? bl[i >> 1][2 * (i & 1) + (r & 1)] : bh[i >> 1][2 * (i & 1) + (r & 1)]; },
+                         [&](int i) -> float* { return i >= 2 ? rq[i & 1] : pk[i & 1]; });
+      }
+      arrive(&kfree[slot]);
+      float b[2][4], ev[2][4] = {};
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) b[nt][e] = fmaf(vn[4 * nt + e], sS, -pk[nt][e] * kUnitInv);
+      if (c + 1 < nch) fetch_v(c + 1);
+      wait(&gfull[gs], (c >> 1) & 1);
+      // ---- E^T = (V - P) Tm^T;  O^T = R + E^T H^T
+      small_product<LD>(ev, b, fs + Cfg::sf_T + gs * SM, lane);
+      small_product<LD>(rq, ev, fs + Cfg::sf_H + gs * SM, lane);
+      {
+        const float* osc = fs + Cfg::sf_osc + gs * 16;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int nt = k >> 1, e = k & 1;
+          const float f = osc[8 * nt + 2 * c4 + e] * sSi;
+          if (c * C + 2 * c4 + e + 8 * nt < T) {
+            float* q = odst + (e ? tstride : 0) + (nt ? 8 * tstride : 0);
+            if (!STASH || p.out) {
+              q[0] = rq[nt][e] * f;
+              q[8] = rq[nt][2 + e] * f;
+            }
+            if (STASH) {
+              edst[(8 * nt + e) * D] = ev[nt][e] * sSi;
+              edst[(8 * nt + e) * D + 8] = ev[nt][2 + e] * sSi;
+            }
+          }
+        }
+        odst += 16 * tstride;
+        if (STASH) edst += 16 * D;
+      }
+      arrive(&gfree[gs]);
+      // ---- S <- S + E^T alpha
+      float me = 0.f;
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) me = fmaxf(me, fabsf(ev[nt][e]));
+      me = warp_max_nonneg(me);
+      const float se = pow2_scale(me, 8), sei = pow2_inverse(se) * kUnitInv;
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) ev[nt][e] *= se;
+      {
+        uint32_t ah[4], al[4];
+        split_frag(ev[0], ev[1], ah, al);
+        wait(&afull[as], (c / RA) & 1);   // (complete: the small matrices came from it)
+#pragma unroll
+      for (int nt = 0; nt < NTILE; nt += NB) {
+        uint32_t b[NB][4];
+        float x[NB][4];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) vec_frag_b(b[i], Aop + lane_vb, nt + i);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) mma_f16_zero(x[i], al, b[i][0], b[i][1]);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) mma_f16(x[i], ah, b[i][2], b[i][3]);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) mma_f16(x[i], ah, b[i][0], b[i][1]);
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) st[nt + i][e] = fmaf(x[i][e], sei, st[nt + i][e]);
+      }
+      }
+      arrive_cl(&aempty[as], 0);
+      bound += 16.0f * me;
+      look = !(bound <= 16384.0f) || bound < 1.0f;
+    }
+    if (p.S_T) {
+#pragma unroll
+      for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+          *reinterpret_cast<float2*>(p.S_T + (size_t(unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
+              make_float2(st[nt][2 * hf] * sSi, st[nt][2 * hf + 1] * sSi);
+    }
+  }
+  __syncthreads();
+  if (tid == 0 && *abort_flag && p.status) atomicCAS(p.status, 0, int(VLA_ERR_DEVICE_TIMEOUT));
+  cluster_sync();   // neither CTA leaves while the other may still write to its shared memory
+}
+
+}  // namespace vla

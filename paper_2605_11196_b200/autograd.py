@@ -57,7 +57,7 @@ class _VlaScan(torch.autograd.Function):
             d_out = torch.zeros(v.shape, dtype=torch.float32, device=v.device)
         g = _b.vla_backward(q, k, v, lam, f32c(d_out), u=u, S0=S0, A0=A0, z0=z0, dS_T=f32c(dS_T),
                             dA_T=f32c(dA_T), dz_T=f32c(dz_T), flags=flags, eps=eps, refresh=refresh,
-                            status=_status_word(q.device))
+                            status=_status_word(q.device), want_dA0=ctx.needs_input_grad[5])
         need = ctx.needs_input_grad
         pick = lambda i, x, like: x.to(like.dtype) if (need[i] and x is not None and like is not None) else None
         return (pick(0, g.dq, q), pick(1, g.dk, k), pick(2, g.dv, v), pick(3, g.du, u), pick(4, g.dS0, S0),

@@ -293,10 +293,11 @@ class VlaGrads(NamedTuple):
 def vla_backward(q, k, v, lam: float, d_out, *, u=None, S0=None, A0=None, z0=None, dS_T=None, dA_T=None,
                  dz_T=None, flags: int = 0, eps: float = 1e-4, workspace=None, status=None,
                  stream: Optional[torch.cuda.Stream] = None, want_status: bool = True,
-                 refresh=None) -> VlaGrads:
+                 refresh=None, want_dA0: bool = True) -> VlaGrads:
     """Gradients of the forward scan for CUDA tensors (u = k_hat: d in {16, 32, 64, 128}; explicit
     ``u`` (its gradient is returned as ``du``) and / or the periodic ``refresh`` = (period, eta,
-    step_offset): d in {32, 64, 128}); the forward is recomputed inside.  ``d_out`` is dL/d(out); ``dS_T, dA_T, dz_T`` default to zero."""
+    step_offset): d in {32, 64, 128}); the forward is recomputed inside.  ``d_out`` is dL/d(out); ``dS_T, dA_T, dz_T`` default to zero.
+    ``want_dA0=False`` leaves the gradient of ``A0`` out, which lets the chunked form run (several times faster)."""
     lib = load_library()
     if flags & VLA_FLAG_TOKEN_MAJOR:      # sequence tensors and their gradients as [B, T, H, d]
         B, T, H, dk = q.shape
@@ -318,7 +319,7 @@ def vla_backward(q, k, v, lam: float, d_out, *, u=None, S0=None, A0=None, z0=Non
     dkk = torch.empty(tok(dk), dtype=f32, device=dev)
     dvv = torch.empty(tok(dv_), dtype=f32, device=dev)
     dS0 = torch.empty((B, H, dv_, dk), dtype=f32, device=dev)
-    dA0 = torch.empty((B, H, dk, dk), dtype=f32, device=dev)
+    dA0 = torch.empty((B, H, dk, dk), dtype=f32, device=dev) if want_dA0 else None
     dz0 = torch.empty((B, H, dk), dtype=f32, device=dev)
     if status is None and want_status:
         status = torch.zeros((), dtype=torch.int32, device=dev)

@@ -16,6 +16,7 @@
 #include "vla.h"
 #include "vla_launch.h"
 #include "vla_backward_params.h"
+#include "vla_bwd_chunk_params.h"
 #include "vla_make_u_params.h"
 
 namespace {
@@ -217,14 +218,122 @@ int seqpar_choose_segments(int units, int T, int d, int dtype) {
   return best;
 }
 
+// ---- backward pass: workspace of the two token-level reverse scans
+// z, e, dalpha, dk_hat (S part), key-sum gradient per token; delta per token; S_T, A_T, key sum; the key sum
+// after every 16 tokens; a_t per token (explicit u); the forward's readout; progress words
+size_t backward_scans_bytes(size_t units, size_t T, size_t d) {
+  const size_t vec = round256(units * T * d * sizeof(float)), mat = round256(units * d * d * sizeof(float));
+  const size_t ck = round256(units * ((T + 15) / 16) * d * sizeof(float));
+  return 7 * vec + round256(units * T * sizeof(float)) + 2 * mat + round256(units * d * sizeof(float)) + ck +
+         round256((units + 1) * sizeof(int)) + 256;
+}
+
+// ---- ... and of the chunked form: bytes per unit (every array of `n` units is n times its unit's part)
+struct BwdLayout {
+  size_t alpha, zeta, e, g, zkc, scal, opK, opQ, opA, small, Aimg, Simg, Dimg, sc, X, Y, A_T, XT, XT2, total;
+};
+BwdLayout bwd_layout(size_t T, size_t d) {
+  const size_t nch = (T + 15) / 16, NB = (nch + 1) / 2, row = 4 * d + 16;   // row: an operand row of the kernels
+  BwdLayout L;
+  size_t off = 0;
+  auto take = [&](size_t bytes) { const size_t at = off; off += round256(bytes); return at; };
+  L.alpha = take(T * d * 4);
+  L.zeta = take(T * d * 4);
+  L.e = take(T * d * 4);
+  L.g = take(T * d * 4);
+  L.zkc = take(nch * d * 4);
+  L.scal = take(6 * round256(T * 4));   // delta, an, qsi, iden, nrm, dden
+  L.opK = take(nch * 16 * row);
+  L.opQ = take(nch * 16 * row);
+  L.opA = take(nch * 16 * row);
+  L.small = take(nch * 2 * 320 * 4);
+  L.Aimg = take(NB * d * row);
+  L.Simg = take(NB * d * row);
+  L.Dimg = take(NB * d * row);
+  L.sc = take(3 * round256(NB * (d / 16) * 4));   // scales of the images: A, S, D
+  L.X = take(NB * d * d * 4);
+  L.Y = take(NB * d * 4);
+  L.A_T = take(d * d * 4);
+  L.XT = take(d * d * 4);
+  L.XT2 = take(d * d * 4);
+  L.total = off;
+  return L;
+}
+size_t bwd_unit_bytes(size_t T, size_t d) { return bwd_layout(T, d).total; }
+// Units per pass.  The chains of a pass run one CTA per unit, so all units go at once while the workspace stays
+// below 4 GiB; beyond that groups of at least one unit per SM take turns in it ([B,T,H,d] tensors: whole
+// batch entries).
+size_t bwd_group(size_t units, size_t H, size_t T, size_t d) {
+  const size_t fits = (size_t(4) << 30) / bwd_unit_bytes(T, d), want = fits > 148 ? fits : 148;
+  if (units <= want) return units;
+  return H >= want ? H : want / H * H;
+}
+
 // One event per (device, flag slot) of the balanced schedule, recorded behind the launch that
 // used the slot last.  Created on first use; they live until the process exits.
 constexpr int kSlotCount = 16;   // == kSchedSlots of the chunk kernel
 std::mutex g_slot_mutex;
 cudaEvent_t g_slot_event[kMaxDevices][kSlotCount] = {};
 
-struct LaunchNote { char kernel[48]; int d, dtype, grid, balanced; };
+struct LaunchNote { const char* kernel; int d, dtype, grid, balanced; };   // kernel: a literal
 thread_local LaunchNote g_last_launch = {"", 0, 0, 0, 0};
+
+// The chunked backward pass, a group of units at a time through one workspace.
+int backward_chunked(const void* q, const void* k, const void* v, float lambda_, int H, int T, int d, int units,
+                     const float* S0, const float* A0, const float* d_out, const float* dS_T, const float* dA_T,
+                     const float* dz_T, float* dq, float* dk, float* dv, float* dS0, float* dz0, const vla_opts_t& o,
+                     unsigned char* w, cudaStream_t st) {
+  const size_t es = o.qkv_dtype == VLA_F32 ? 4 : 2, Tz = size_t(T), dd = size_t(d);
+  const BwdLayout L = bwd_layout(Tz, dd);
+  const size_t group = bwd_group(size_t(units), size_t(H), Tz, dd);
+  for (size_t u0 = 0; u0 < size_t(units); u0 += group) {
+    const size_t n = size_t(units) - u0 < group ? size_t(units) - u0 : group;
+    // (a [B,T,H,d] group starts at a batch entry, so unit u0's tokens start at u0 T d in both layouts)
+    const size_t tok = u0 * Tz * dd, sq = u0 * dd * dd;
+    auto in = [&](const void* p) { return p ? static_cast<const void*>(static_cast<const unsigned char*>(p) + tok * es) : nullptr; };
+    auto at = [](auto* p, size_t off) { return p ? p + off : p; };
+    auto ws = [&](size_t off) { return w + off * n; };
+    auto wf = [&](size_t off) { return reinterpret_cast<float*>(w + off * n); };
+    const size_t scal = round256(Tz * 4) / 4 * n;
+    const int nch = (T + 15) / 16;
+
+    vla::PairStash sh;
+    sh.alpha = wf(L.alpha); sh.zeta = wf(L.zeta); sh.zkc = wf(L.zkc);
+    sh.delta = wf(L.scal); sh.an = sh.delta + scal;
+    sh.Aimg = ws(L.Aimg); sh.Asc = wf(L.sc); sh.ck = 2;
+    ScanParams f = {};
+    f.q = in(q); f.k = in(k); f.v = in(v); f.u = in(o.u);
+    f.A0 = at(A0, sq); f.z0 = at(o.z0, u0 * dd);
+    f.A_T = wf(L.A_T);
+    f.status = o.status; f.lambda = lambda_; f.eps = o.eps;
+    f.T = T; f.units = int(n); f.flags = o.flags; f.heads = H; f.wait_limit = o.wait_probe_limit;
+    int rc = vla::launch_pair(d, o.qkv_dtype, f, &sh, st);
+    if (rc != VLA_OK) return rc;
+
+    vla::BwdChunkParams p = {};
+    p.q = f.q; p.k = f.k; p.v = f.v; p.u = f.u;
+    p.S0 = at(S0, sq); p.d_out = d_out + tok;
+    p.dS_T = at(dS_T, sq); p.dA_T = at(dA_T, sq); p.dz_T = at(dz_T, u0 * dd);
+    p.dq = dq + tok; p.dk = dk + tok; p.dv = dv + tok; p.du = at(o.du, tok);
+    p.dS0 = at(dS0, sq); p.dz0 = at(dz0, u0 * dd);
+    p.alpha = sh.alpha; p.zeta = sh.zeta; p.delta = sh.delta; p.an = sh.an; p.zkc = sh.zkc;
+    p.qsi = sh.an + scal; p.iden = p.qsi + scal; p.nrm = p.iden + scal; p.dden = p.nrm + scal;
+    p.Aimg = sh.Aimg; p.Asc = sh.Asc; p.A_T = f.A_T;
+    p.opK = ws(L.opK); p.opQ = ws(L.opQ); p.opA = ws(L.opA); p.small = wf(L.small);
+    p.e = wf(L.e); p.g = wf(L.g);
+    p.NB = (nch + 1) / 2;
+    const size_t scs = round256(size_t(p.NB) * (dd / 16) * 4) / 4 * n;
+    p.Ssc = sh.Asc + scs; p.Dsc = p.Ssc + scs;
+    p.Simg = ws(L.Simg); p.Dimg = ws(L.Dimg);
+    p.X = wf(L.X); p.Y = wf(L.Y); p.XT = wf(L.XT); p.XT2 = wf(L.XT2);
+    p.status = o.status;
+    p.T = T; p.units = int(n); p.nch = nch; p.heads = H;
+    p.flags = o.flags; p.wait_limit = o.wait_probe_limit; p.eps = o.eps;
+    rc = vla::launch_bwd_chunk(d, o.qkv_dtype, p, st);
+    if (rc != VLA_OK) return rc;
+  }
+  return VLA_OK;
+}
 
 }  // namespace
 
@@ -269,7 +378,7 @@ void sched_slot_mark(unsigned int epoch, cudaStream_t st) {
 }
 
 void note_launch(const char* kernel, int d, int dtype, int grid, int balanced) {
-  std::snprintf(g_last_launch.kernel, sizeof(g_last_launch.kernel), "%s", kernel);
+  g_last_launch.kernel = kernel;
   g_last_launch.d = d; g_last_launch.dtype = dtype; g_last_launch.grid = grid; g_last_launch.balanced = balanced;
 }
 }  // namespace vla
@@ -594,13 +703,9 @@ int vla_forward_seqpar(const void* q, const void* k, const void* v, float lambda
 size_t vla_backward_workspace_bytes(int B, int H, int T, int d_k) {
   if (B < 0 || H < 0 || T < 0 || d_k <= 0) return 0;
   const size_t units = size_t(B) * size_t(H);
-  const size_t vec = round256(units * T * d_k * sizeof(float));
-  const size_t mat = round256(units * d_k * d_k * sizeof(float));
-  // z, e, dalpha, dk_hat (S part), key-sum gradient per token; delta per token; S_T, A_T, key sum;
-  // the key sum after every 16 tokens; a_t per token (explicit u); the forward's readout; progress words
-  const size_t ck = round256(units * ((size_t(T) + 15) / 16) * d_k * sizeof(float));
-  return 7 * vec + round256(units * T * sizeof(float)) + 2 * mat + round256(units * d_k * sizeof(float)) + ck +
-         round256((units + 1) * sizeof(int)) + 256;
+  const size_t one = bwd_unit_bytes(size_t(T), size_t(d_k)), group = bwd_group(units, size_t(H), size_t(T), size_t(d_k));
+  const size_t scans = backward_scans_bytes(units, size_t(T), size_t(d_k));
+  return one * group + 256 > scans ? one * group + 256 : scans;
 }
 
 int vla_backward(const void* q, const void* k, const void* v, float lambda_, int B, int H, int T,
@@ -614,7 +719,7 @@ int vla_backward(const void* q, const void* k, const void* v, float lambda_, int
   if (rc != VLA_OK) return rc;
   rc = check_common(q, k, v, lambda_, B, H, T, d_k, d_v, A0, d_out);
   if (rc != VLA_OK) return rc;
-  // explicit u, the refresh, token-major tensors: the two reverse scans only
+  // explicit u, the refresh, token-major tensors: d >= 32
   const bool general = o.u || o.refresh_period > 0;
   if ((general || (o.flags & VLA_FLAG_TOKEN_MAJOR)) && d_k < 32) return VLA_ERR_UNSUPPORTED;
   if (o.flags & VLA_FLAG_LINEAR_ATTENTION) return VLA_ERR_UNSUPPORTED;   // a forward-only comparison mode
@@ -628,6 +733,11 @@ int vla_backward(const void* q, const void* k, const void* v, float lambda_, int
   if (!workspace || workspace_bytes < vla_backward_workspace_bytes(B, H, T, d_k)) return VLA_ERR_INVALID_ARG;
   unsigned char* w = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(workspace) + 255) & ~uintptr_t(255));
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // The chunked form: everything but the refresh (M_t is no longer a plain sum there) and the gradient of A0,
+  // which is taken entry by entry through the recurrence and needs its adjoint of A
+  if (T > 0 && o.refresh_period <= 0 && !dA0)
+    return backward_chunked(q, k, v, lambda_, H, T, d_k, units, S0, A0, d_out, dS_T, dA_T, dz_T, dq, dk, dv, dS0, dz0, o, w, st);
   const size_t vec = round256(size_t(units) * T * d_k * sizeof(float));
   const size_t mat = round256(size_t(units) * d_k * d_k * sizeof(float));
   const size_t sca = round256(size_t(units) * T * sizeof(float));
@@ -640,7 +750,6 @@ int vla_backward(const void* q, const void* k, const void* v, float lambda_, int
   int* progw = reinterpret_cast<int*>(w + 6 * vec + sca + 2 * mat + round256(size_t(units) * d_k * sizeof(float)) + ckb);
   float* outw = reinterpret_cast<float*>(w + 6 * vec + sca + 2 * mat + round256(size_t(units) * d_k * sizeof(float)) + ckb +
                                          round256((size_t(units) + 1) * sizeof(int)));
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (d_k == 16) {
     // d = 16 has no chunk kernel: the single kernel runs its own token-level forward sweep
     vla::BackwardParams p;

@@ -1,0 +1,1258 @@
+// Backward pass, chunked (u = k_hat or explicit u, no refresh): gradients of the scan without a
+// token-level reverse sweep.
+//
+//   Memory side.  D_t, the adjoint of S_t, obeys D_{t-1} = D_t - de_t k_t^T (+ dy_t q_t^T), the mirror image of
+//   S_t = S_{t-1} + e_t alpha_t^T, row by row independent.  Per 16-token chunk, with dY = dO / den:
+//       E  = Tm (V - K S^T)                   S <- S + E^T alpha            (forward chain)
+//       dE = Tm^T (alpha D^T + H^T dY)        D <- D + dY^T Q - dE^T K      (reverse chain)
+//   (Tm = (I + stril(K alpha^T))^-1, H = tril(Q alpha^T), both independent of S and D), and dv = de.
+//   Penalty side.  A_t = M_t^-1 with M_t = M_{t-1} + u_t u_t^T (Eq. "penalty"), so the adjoint of M_t is a plain
+//   suffix sum: with g_t = A_t da_t, a_t = A_t k_t,
+//       X_t = sum_{s >= t} (g_s a_s^T + a_s g_s^T) + A_T (dA_T + dA_T^T) A_T
+//       dk_hat_t += g_t,   du_t = -X_t u_t   (u = k_hat: dk_hat_t += du_t as well).
+//   No adjoint of A is carried and no state is walked back.
+//
+// Launches: rank 0's part of the pair kernel (alpha, checkpoints of A), then
+//   bwd_prep    per chunk: operand images of K, Q, alpha; Tm, H; denominators
+//   bwd_chains  the two chains of the memory side, each warp 16 rows, checkpoints of S and D
+//   bwd_block   per block of 32 tokens: dq, the S part of dk_hat, dalpha -> da -> g, the block's sums
+//   bwd_scan    suffix sums over the blocks
+//   bwd_finish  per block: du, dk_hat -> dk, dq through the feature map and the norms
+// Everything between the chains is parallel over chunks or blocks.  fp16 hi/lo operands with fp32 sums
+// as in the pair kernel (vla_mma.cuh); block arrays are scaled by a power of two from their largest entry
+// (absolute error below 2^-38 of it).
+#pragma once
+
+#include <type_traits>
+
+#include "vla_bwd_chunk_params.h"
+#include "vla_mma.cuh"
+
+namespace vla {
+
+constexpr int kBwdBlock = 32;   // tokens per block (checkpoints of A, S, D every two chunks)
+constexpr int kBwdLD = 20, kBwdSM = 16 * kBwdLD;
+
+template <int D>
+struct BwdGeom {
+  static constexpr uint32_t kslot = 16 * kTokRow<D>;   // image of a chunk's token rows
+  static constexpr uint32_t mat = D * kTokRow<D>;      // image of a D x D matrix
+  static constexpr uint32_t tb = kBwdBlock * kTokRow<D>;
+};
+
+// where a token of a unit lies in the caller's tensors
+__device__ __forceinline__ size_t bwd_tok(const BwdChunkParams& p, int unit, int t, int D) {
+  if (p.flags & VLA_FLAG_TOKEN_MAJOR) {
+    const int b = unit / p.heads, h = unit - b * p.heads;
+    return ((size_t(b) * p.T + t) * p.heads + h) * D;
+  }
+  return (size_t(unit) * p.T + t) * D;
+}
+__device__ __forceinline__ size_t bwd_stride(const BwdChunkParams& p, int D) {
+  return (p.flags & VLA_FLAG_TOKEN_MAJOR) ? size_t(p.heads) * D : size_t(D);
+}
+__device__ __forceinline__ float4 gload4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 gload4(const uint16_t* p) {
+  const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(bf16_bits_to_f32(r.x & 0xffffu), bf16_bits_to_f32(r.x >> 16), bf16_bits_to_f32(r.y & 0xffffu),
+                     bf16_bits_to_f32(r.y >> 16));
+}
+// four consecutive columns of a row image
+template <int D>
+__device__ __forceinline__ void row_store4(uint32_t base, int row, int pl, float4 x, float s) {
+  uint32_t h0, l0, h1, l1;
+  split_f16(x.x * s, x.y * s, h0, l0);
+  split_f16(x.z * s, x.w * s, h1, l1);
+  const uint32_t at = base + uint32_t(row) * kTokRow<D> + 8 * pl;
+  sts64(at, h0, h1);
+  sts64(at + 2 * D, l0, l1);
+}
+// columns (c, c + 1) of a row image as fp32 (still scaled)
+template <int D>
+__device__ __forceinline__ float2 row_pair(const unsigned char* base, int row, int col) {
+  const unsigned char* at = base + size_t(row) * kTokRow<D> + 2 * col;
+  const float2 h = __half22float2(*reinterpret_cast<const __half2*>(at));
+  const float2 l = __half22float2(*reinterpret_cast<const __half2*>(at + 2 * D));
+  return make_float2(h.x + l.x, h.y + l.y);
+}
+template <int D>
+__device__ __forceinline__ float row_one(const unsigned char* base, int row, int col) {
+  const unsigned char* at = base + size_t(row) * kTokRow<D> + 2 * col;
+  return __half2float(*reinterpret_cast<const __half*>(at)) + __half2float(*reinterpret_cast<const __half*>(at + 2 * D));
+}
+template <int D>
+__device__ __forceinline__ void row_pair_store(uint32_t base, int row, int col, float x0, float x1) {
+  uint32_t hi, lo;
+  split_f16(x0, x1, hi, lo);
+  const uint32_t at = base + uint32_t(row) * kTokRow<D> + 2 * col;
+  sts32(at, hi);
+  sts32(at + 2 * D, lo);
+}
+
+// ---------------------------------------------------------------- per chunk: operands and small matrices
+template <int D> struct BwdPrepCfg {
+  static constexpr int WPC = D == 128 ? 2 : 4;   // chunks (warps) per CTA
+  static constexpr uint32_t small = 3 * BwdGeom<D>::kslot;
+  static constexpr uint32_t per_warp = small + (3 * kBwdSM + 64) * 4;
+  static constexpr uint32_t smem_bytes = WPC * per_warp;
+};
+
+template <int D, typename TIn>
+__global__ void __launch_bounds__(BwdPrepCfg<D>::WPC * 32) bwd_prep_kernel(const BwdChunkParams p) {
+  using Cfg = BwdPrepCfg<D>;
+  using G = BwdGeom<D>;
+  constexpr int LPT = D / 4, TPW = 32 / LPT, NP = 16 / TPW, KS = D / 16, LD = kBwdLD, SM = kBwdSM;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, c4 = lane & 3;
+  const long long id = (long long)blockIdx.x * Cfg::WPC + warp;
+  if (id >= (long long)p.units * p.nch) return;
+  const int unit = int(id / p.nch), c = int(id % p.nch), T = p.T;
+  const bool ident = (p.flags & VLA_FLAG_IDENTITY_MAP) != 0;
+  unsigned char* mem = smem + warp * Cfg::per_warp;
+  const uint32_t Kop = smem_u32(mem), Qop = Kop + G::kslot, Aop = Qop + G::kslot;
+  float* Nb = reinterpret_cast<float*>(mem + Cfg::small);
+  float* Tm = Nb + SM;
+  float* H = Tm + SM;
+  float* nrm = H + SM;      // [16], then 1 / q scale, q . key sum at the chunk's start
+  float* qsi = nrm + 16;
+  float* dq = qsi + 16;
+  const int sub = lane / LPT, pl = lane % LPT;
+  const size_t tok = bwd_tok(p, unit, c * 16, D) + 4 * pl, ts = bwd_stride(p, D);
+  const float4 zk = *reinterpret_cast<const float4*>(p.zkc + (size_t(unit) * p.nch + c) * D + 4 * pl);
+#pragma unroll (NP < 4 ? NP : 4)
+  for (int ps = 0; ps < NP; ++ps) {
+    const int tt = ps * TPW + sub, t = c * 16 + tt;
+    const bool act = t < T;
+    float4 k = make_float4(0.f, 0.f, 0.f, 0.f), q = k, a = k;
+    if (act) {
+      const size_t o = tok + tt * ts;
+      k = gload4(static_cast<const TIn*>(p.k) + o);
+      q = gload4(static_cast<const TIn*>(p.q) + o);
+      a = gload4(p.alpha + (size_t(unit) * T + t) * D + 4 * pl);
+      if (!ident) {
+        k.x = phi_fast(k.x); k.y = phi_fast(k.y); k.z = phi_fast(k.z); k.w = phi_fast(k.w);
+        q.x = phi_fast(q.x); q.y = phi_fast(q.y); q.z = phi_fast(q.z); q.w = phi_fast(q.w);
+      }
+    }
+    float ss = fmaf(k.x, k.x, fmaf(k.y, k.y, fmaf(k.z, k.z, k.w * k.w)));
+    float qq = fmaf(q.x, q.x, fmaf(q.y, q.y, fmaf(q.z, q.z, q.w * q.w)));
+    float dn = fmaf(q.x, zk.x, fmaf(q.y, zk.y, fmaf(q.z, zk.z, q.w * zk.w)));
+#pragma unroll
+    for (int off = LPT / 2; off >= 1; off >>= 1) {
+      ss += __shfl_xor_sync(0xffffffffu, ss, off);
+      qq += __shfl_xor_sync(0xffffffffu, qq, off);
+      dn += __shfl_xor_sync(0xffffffffu, dn, off);
+    }
+    const float n = sqrt_ftz(ss), nr = fmaxf(n, p.eps), s = pow2_scale(sqrt_ftz(qq), 8);
+    row_store4<D>(Kop, tt, pl, k, rcp_ftz_nr(nr) * 256.0f);
+    row_store4<D>(Qop, tt, pl, q, s);
+    row_store4<D>(Aop, tt, pl, a, 256.0f);
+    if (pl == 0) {
+      nrm[tt] = act ? nr : 0.f;
+      qsi[tt] = pow2_inverse(s);
+      dq[tt] = dn;
+      if (act) {
+        const size_t o = size_t(unit) * T + t;
+        p.nrm[o] = n > p.eps ? nr : -nr;   // negative: the floor holds
+        p.qsi[o] = pow2_inverse(s);
+      }
+    }
+  }
+  __syncwarp();
+  const uint32_t la = tok_lane_a<D>(lane), lb = tok_lane_b<D>(lane);
+  float n[2][4] = {}, hh[2][4] = {}, qk[2][4] = {};
+#pragma unroll 1
+  for (int ks = 0; ks < KS; ++ks) {
+    uint32_t ah[2][4], al[2][4], bh[2][4], bl[2][4];   // A: K, Q rows; B: alpha, K as columns
+    tok_frag<D>(ah[0], Kop + la, ks, false);
+    tok_frag<D>(al[0], Kop + la, ks, true);
+    tok_frag<D>(ah[1], Qop + la, ks, false);
+    tok_frag<D>(al[1], Qop + la, ks, true);
+    tok_frag<D>(bh[0], Aop + lb, ks, false);
+    tok_frag<D>(bl[0], Aop + lb, ks, true);
+    tok_frag<D>(bh[1], Kop + lb, ks, false);
+    tok_frag<D>(bl[1], Kop + lb, ks, true);
+    // products: K alpha^T, Q alpha^T, Q K^T, two token tiles each
+    mma3_f16_many<6>([&](int i, int lo) -> const uint32_t(&)[4] { return lo ? al[i >= 2] : ah[i >= 2]; },
+                     [&](int i, int r) { return (r & 2) ? bl[i >= 4][2 * (i & 1) + (r & 1)] : bh[i >= 4][2 * (i & 1) + (r & 1)]; },
+                     [&](int i) -> float* { return i < 2 ? n[i] : i < 4 ? hh[i - 2] : qk[i - 4]; });
+  }
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf) {
+    const int t = g + 8 * hf;
+    float den = 0.f;
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      const int s = 8 * nt + 2 * c4;
+      constexpr float f = 1.0f / 65536.0f;
+      const float fh = qsi[t] * (1.0f / 256.0f);
+      *reinterpret_cast<float2*>(Nb + t * LD + s) = make_float2(n[nt][2 * hf] * f, n[nt][2 * hf + 1] * f);
+      *reinterpret_cast<float2*>(H + t * LD + s) =
+          make_float2(s <= t ? hh[nt][2 * hf] * fh : 0.f, s + 1 <= t ? hh[nt][2 * hf + 1] * fh : 0.f);
+      if (s <= t) den = fmaf(nrm[s], qk[nt][2 * hf], den);
+      if (s + 1 <= t) den = fmaf(nrm[s + 1], qk[nt][2 * hf + 1], den);
+    }
+    den += __shfl_xor_sync(0xffffffffu, den, 1);
+    den += __shfl_xor_sync(0xffffffffu, den, 2);
+    den = fmaf(den, qsi[t] * (1.0f / 256.0f), dq[t]);
+    if (c4 == 0 && c * 16 + t < T) {
+      const float id = ident ? 1.0f : rcp_ftz_nr(fmaxf(den, p.eps));
+      p.iden[size_t(unit) * T + c * 16 + t] = den > p.eps || ident ? id : -id;   // negative: the floor holds
+    }
+  }
+  __syncwarp();
+  unit_lower_inverse16<LD>(Tm, Nb, lane);
+  fence_async_smem();
+  __syncwarp();
+  if (lane == 0) {
+    const size_t at = size_t(id) * G::kslot;
+    bulk_store(p.opK + at, mem, G::kslot);
+    bulk_store(p.opQ + at, mem + G::kslot, G::kslot);
+    bulk_store(p.opA + at, mem + 2 * G::kslot, G::kslot);
+    bulk_store(p.small + size_t(id) * 2 * SM, Tm, 2 * SM * 4);   // Tm, H
+    bulk_commit();
+    bulk_wait_all<0>();
+  }
+}
+
+// ---------------------------------------------------------------- the two chains of the memory side
+template <int D> struct BwdChainCfg {
+  static constexpr int NW = D / 16;
+  static constexpr int NT = NW * 32 + 32;            // + the copying warp
+  static constexpr int NS = D == 128 ? 3 : 4;        // chunks in flight
+  static constexpr uint32_t stage = 3 * BwdGeom<D>::kslot + 2 * kBwdSM * 4;
+  static constexpr uint32_t smem_bytes = NS * stage + 2 * NS * 8 + 16;
+};
+
+template <int D, typename TIn>
+__global__ void __launch_bounds__(BwdChainCfg<D>::NT) bwd_chains_kernel(const BwdChunkParams p) {
+  using Cfg = BwdChainCfg<D>;
+  using G = BwdGeom<D>;
+  constexpr int NW = Cfg::NW, NS = Cfg::NS, KS = D / 16, NTILE = D / 8, LD = kBwdLD, SM = kBwdSM;
+  constexpr int NB = NTILE < 4 ? NTILE : 4;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int unit = blockIdx.x >> 1;
+  const bool rev = blockIdx.x & 1;
+  const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int nch = p.nch, T = p.T;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + NS * Cfg::stage);
+  uint64_t* empty = full + NS;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + NS);
+  auto wait = [&](uint64_t* bar, int parity) {
+    uint32_t it = 0;
+    const uint32_t probes = p.wait_limit ? p.wait_limit : kWaitProbeLimit;
+    while (!mbar_try_wait(bar, uint32_t(parity))) {
+      if (++it > probes || *abort_flag) {
+        *abort_flag = 1;
+        break;
+      }
+    }
+  };
+  if (tid == 0) {
+    *abort_flag = 0;
+    for (int i = 0; i < NS; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], NW);
+    }
+    mbar_init_fence();
+  }
+  __syncthreads();
+  // chunk taken in step i
+  auto chunk_of = [&](int i) { return rev ? nch - 1 - i : i; };
+  if (warp == NW) {
+    if (lane == 0) {
+      for (int i = 0; i < nch && !*abort_flag; ++i) {
+        const int s = i % NS;
+        if (i >= NS) wait(&empty[s], (i / NS - 1) & 1);
+        const size_t id = size_t(unit) * nch + chunk_of(i);
+        unsigned char* dst = smem + s * Cfg::stage;
+        mbar_arrive_expect_tx(&full[s], (rev ? 3 : 2) * G::kslot + (rev ? 2 : 1) * SM * 4);
+        bulk_load(dst, p.opK + id * G::kslot, G::kslot, &full[s]);
+        bulk_load(dst + G::kslot, p.opA + id * G::kslot, G::kslot, &full[s]);
+        if (rev) bulk_load(dst + 2 * G::kslot, p.opQ + id * G::kslot, G::kslot, &full[s]);
+        bulk_load(dst + 3 * G::kslot, p.small + id * 2 * SM, (rev ? 2 : 1) * SM * 4, &full[s]);
+      }
+    }
+  } else {
+    // a warp's 16 rows of S (or of its adjoint D), scaled by a power of two that follows their size
+    const int row0 = 16 * warp;
+    const float* init = rev ? p.dS_T : p.S0;
+    float st[NTILE][4], sc = 1.0f, sci = 1.0f, bound = 0.0f;
+    bool look = init != nullptr;
+#pragma unroll
+    for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        float2 x = make_float2(0.f, 0.f);
+        if (init) x = *reinterpret_cast<const float2*>(init + (size_t(unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4);
+        st[nt][2 * hf] = x.x;
+        st[nt][2 * hf + 1] = x.y;
+      }
+    const uint32_t lb = tok_lane_b<D>(lane), lk = tok_lane_k<D>(lane);
+    const size_t ts = bwd_stride(p, D);
+    const size_t my0 = bwd_tok(p, unit, 0, D) + row0 + g;
+    // this lane's four tokens of a chunk: 2 c4, 2 c4 + 1 and 8 further.  x: v, or dO (bits as loaded: whatever
+    // touched a value here would wait for it), f: scale of q_t, id: 1 / den_t
+    uint32_t x[8];
+    float f[4], id[4];
+    auto fetch = [&](int c) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int t = c * 16 + 2 * c4 + (k & 1) + 4 * (k & 2), i = 2 * (k & 2) + (k & 1);
+        x[i] = x[i + 2] = 0u;
+        f[k] = id[k] = 0.f;
+        if (t < T) {
+          const size_t o = my0 + size_t(t) * ts;
+          if (!rev) {
+            const TIn* v = static_cast<const TIn*>(p.v) + o;
+            if constexpr (sizeof(TIn) == 2) { x[i] = v[0]; x[i + 2] = v[8]; }
+            else { x[i] = __float_as_uint(v[0]); x[i + 2] = __float_as_uint(v[8]); }
+          } else {
+            x[i] = __float_as_uint(p.d_out[o]);
+            x[i + 2] = __float_as_uint(p.d_out[o + 8]);
+            f[k] = p.qsi[size_t(unit) * T + t];
+            id[k] = p.iden[size_t(unit) * T + t];
+          }
+        }
+      }
+    };
+    if (nch > 0) fetch(chunk_of(0));
+    float* res = rev ? p.dv + my0 : p.e + size_t(unit) * T * D + row0 + g;   // de = dv, or e
+    const size_t rs = rev ? ts : size_t(D);
+#pragma unroll 1
+    for (int i = 0; i < nch; ++i) {
+      const int c = chunk_of(i), s = i % NS;
+      if (look) {
+        float mx = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fabsf(st[nt][e]));
+        mx = warp_max_nonneg(mx);
+        bound = mx;
+        if (mx > 0.0f && (mx > 512.0f || mx < 1.0f)) {
+          const float ns = fminf(fmaxf(sc * pow2_scale(mx, 5), 7.888609e-31f), 1.2676506e30f), r = ns * sci;
+#pragma unroll
+          for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) st[nt][e] *= r;
+          sc = ns;
+          sci = pow2_inverse(ns);
+          bound = mx * r;
+        }
+      }
+      // ---- checkpoint: S at a block's start, D at its end
+      if (rev ? (i == 0 || (c & 1) == 1) : (c & 1) == 0) {
+        const size_t blk = size_t(unit) * p.NB + (c >> 1);
+        unsigned char* dst = (rev ? p.Dimg : p.Simg) + blk * G::mat + size_t(row0 + g) * kTokRow<D> + 4 * c4;
+#pragma unroll
+        for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            uint32_t hi, lo;
+            split_f16(st[nt][2 * hf], st[nt][2 * hf + 1], hi, lo);
+            *reinterpret_cast<uint32_t*>(dst + hf * 8 * kTokRow<D> + 16 * nt) = hi;
+            *reinterpret_cast<uint32_t*>(dst + hf * 8 * kTokRow<D> + 16 * nt + 2 * D) = lo;
+          }
+        if (lane == 0) (rev ? p.Dsc : p.Ssc)[blk * (D / 16) + warp] = sci;
+      }
+      wait(&full[s], (i / NS) & 1);
+      const uint32_t Kop = smem_u32(smem + s * Cfg::stage), Aop = Kop + G::kslot, Qop = Aop + G::kslot;
+      const float* Tm = reinterpret_cast<const float*>(smem + s * Cfg::stage + 3 * G::kslot);
+      // ---- P = S K^T, or X = D alpha^T
+      float pr[2][4] = {};
+      const uint32_t Bop = (rev ? Aop : Kop) + lb;
+      constexpr int KB = KS >= 2 ? 2 : 1;
+#pragma unroll
+      for (int ks = 0; ks < KS; ks += KB) {
+        uint32_t ah[KB][4], al[KB][4], bh[KB][4], bl[KB][4];
+#pragma unroll
+        for (int j = 0; j < KB; ++j) {
+          split_frag(st[2 * (ks + j)], st[2 * (ks + j) + 1], ah[j], al[j]);
+          tok_frag<D>(bh[j], Bop, ks + j, false);
+          tok_frag<D>(bl[j], Bop, ks + j, true);
+        }
+        mma3_f16_many<2 * KB>([&](int q, int lo) -> const uint32_t(&)[4] { return lo ? al[q >> 1] : ah[q >> 1]; },
+                              [&](int q, int r) { return (r & 2) ? bl[q >> 1][2 * (q & 1) + (r & 1)] : bh[q >> 1][2 * (q & 1) + (r & 1)]; },
+                              [&](int q) -> float* { return pr[q & 1]; });
+      }
+      // ---- E^T = (V - P) Tm^T, or dE^T = (X + dY^T H) Tm
+      float y[2][4], ev[2][4] = {};
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const uint32_t raw = x[4 * nt + e];
+          const float val = __uint_as_float(sizeof(TIn) == 2 && !rev ? raw << 16 : raw);
+          y[nt][e] = val * (rev ? sc * fabsf(id[2 * nt + (e & 1)]) : sc);
+          pr[nt][e] *= 1.0f / 256.0f;
+        }
+      if (!rev) {
+        float b[2][4];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) b[nt][e] = y[nt][e] - pr[nt][e];
+        small_product<LD>(ev, b, Tm, lane);
+      } else {
+        small_product_t<LD>(pr, y, Tm + SM, lane);
+        small_product_t<LD>(ev, pr, Tm, lane);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int nt = k >> 1, e = k & 1, t = c * 16 + 2 * c4 + e + 8 * nt;
+        if (t < T) {
+          res[size_t(t) * rs] = ev[nt][e] * sci;
+          res[size_t(t) * rs + 8] = ev[nt][2 + e] * sci;
+        }
+        if (rev) {   // coefficients of the stored q rows
+          y[nt][e] *= f[k];
+          y[nt][2 + e] *= f[k];
+        }
+      }
+      if (i + 1 < nch) fetch(chunk_of(i + 1));
+      // ---- S += E^T alpha, or D += dY^T Q - dE^T K
+      auto update = [&](float (&co)[2][4], uint32_t op, float unit_scale, float reach) {
+        float m = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) m = fmaxf(m, fabsf(co[nt][e]));
+        m = warp_max_nonneg(m);
+        bound += 16.0f * m * reach;
+        const float sx = pow2_scale(m, 8), so = pow2_inverse(sx) * unit_scale;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) co[nt][e] *= sx;
+        uint32_t ah[4], al[4];
+        split_frag(co[0], co[1], ah, al);
+#pragma unroll
+        for (int nt = 0; nt < NTILE; nt += NB) {
+          uint32_t b[NB][4];
+          float w[NB][4];
+#pragma unroll
+          for (int j = 0; j < NB; ++j) tok_frag_k<D>(b[j], op + lk, 0, nt + j);
+#pragma unroll
+          for (int j = 0; j < NB; ++j) mma_f16_zero(w[j], al, b[j][0], b[j][1]);
+#pragma unroll
+          for (int j = 0; j < NB; ++j) mma_f16(w[j], ah, b[j][2], b[j][3]);
+#pragma unroll
+          for (int j = 0; j < NB; ++j) mma_f16(w[j], ah, b[j][0], b[j][1]);
+#pragma unroll
+          for (int j = 0; j < NB; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) st[nt + j][e] = fmaf(w[j][e], so, st[nt + j][e]);
+        }
+      };
+      // (one copy of the update's code: the reverse chain goes through it twice)
+#pragma unroll 1
+      for (int pass = 0; pass < (rev ? 2 : 1); ++pass) {
+        float co[2][4];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) co[nt][e] = pass ? y[nt][e] : ev[nt][e];
+        update(co, pass ? Qop : rev ? Kop : Aop, pass ? 1.0f : (rev ? -1.0f : 1.0f) / 256.0f, pass ? 512.0f : 1.0f);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[s]);
+      look = !(bound <= 16384.0f) || bound < 1.0f;
+    }
+    float* fin = rev ? p.dS0 : nullptr;
+    if (fin) {
+#pragma unroll
+      for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+          *reinterpret_cast<float2*>(fin + (size_t(unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
+              make_float2(st[nt][2 * hf] * sci, st[nt][2 * hf + 1] * sci);
+    }
+  }
+  __syncthreads();
+  if (*abort_flag) {
+    settle_copies();
+    if (tid == 0 && p.status) atomicCAS(p.status, 0, int(VLA_ERR_DEVICE_TIMEOUT));
+  }
+}
+
+// ---------------------------------------------------------------- per block: everything that needs S, D, A of the block
+template <int D> struct BwdBlockCfg {
+  static constexpr uint32_t tb = BwdGeom<D>::tb;
+  static constexpr uint32_t mat = 6 * tb;
+  static constexpr uint32_t fl = mat + BwdGeom<D>::mat;
+  static constexpr int f_red = 0, f_dot = 64, f_dqd = f_dot + 64, f_ddn = f_dqd + 64, f_an = f_ddn + 32, f_rho = f_an + 32,
+                       f_qsi = f_rho + 32, f_id = f_qsi + 32, f_end = f_id + 32;
+  static constexpr uint32_t smem_bytes = fl + f_end * 4 + 32;
+};
+
+// largest of N per-thread values over a CTA of 8 warps, through red[8 * N]; the caller synchronises between
+// cta_max_put and cta_max_get
+__device__ __forceinline__ void cta_max_put(float* red, int slot, float m, int warp, int lane) {
+  m = warp_max_nonneg(m);
+  if (lane == 0) red[slot * 8 + warp] = m;
+}
+__device__ __forceinline__ float cta_max_get(const float* red, int slot) {
+  float m = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) m = fmaxf(m, red[slot * 8 + w]);
+  return m;
+}
+__device__ __forceinline__ float max4(float m, float4 x) {
+  return fmaxf(fmaxf(m, fmaxf(fabsf(x.x), fabsf(x.y))), fmaxf(fabsf(x.z), fabsf(x.w)));
+}
+
+template <int D, typename TIn, bool UT>
+__global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) {
+  using Cfg = BwdBlockCfg<D>;
+  using G = BwdGeom<D>;
+  constexpr int BC = kBwdBlock, KS = D / 16, NH = D / 16;   // NH: n tiles of half the columns
+  constexpr float kInv = 1.0f / 256.0f;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int blk = blockIdx.x, unit = blockIdx.y;
+  const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int tg = warp & 1, h = (warp >> 1) & 1, role = warp >> 2;
+  const int t0 = blk * BC, T = p.T, nt_valid = min(BC, T - t0), nchv = min(2, p.nch - 2 * blk);
+  const size_t ub = size_t(unit) * p.NB + blk, ut0 = size_t(unit) * T + t0;
+  const size_t tok = bwd_tok(p, unit, t0, D), ts = bwd_stride(p, D);   // the block's first token, distance between tokens
+  const uint32_t sb = smem_u32(smem);
+  const uint32_t tE = sb, tDE = sb + Cfg::tb, tDY = sb + 2 * Cfg::tb, tA = sb + 3 * Cfg::tb, tQ = sb + 4 * Cfg::tb,
+                 tK = sb + 5 * Cfg::tb, mat = sb + Cfg::mat;
+  float* fs = reinterpret_cast<float*>(smem + Cfg::fl);
+  float* red = fs + Cfg::f_red;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(fs + Cfg::f_end);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar + 1);
+  auto wait = [&](int parity) {
+    uint32_t it = 0;
+    const uint32_t probes = p.wait_limit ? p.wait_limit : kWaitProbeLimit;
+    while (!mbar_try_wait(bar, uint32_t(parity)))
+      if (++it > probes) { *abort_flag = 1; break; }
+  };
+  if (tid == 0) {
+    *abort_flag = 0;
+    mbar_init(bar, 1);
+    mbar_init_fence();
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const size_t id = size_t(unit) * p.nch + 2 * blk;
+    const uint32_t n = nchv * G::kslot;
+    mbar_arrive_expect_tx(bar, 3 * n + G::mat);
+    bulk_load(smem + 3 * Cfg::tb, p.opA + id * G::kslot, n, bar);
+    bulk_load(smem + 4 * Cfg::tb, p.opQ + id * G::kslot, n, bar);
+    bulk_load(smem + 5 * Cfg::tb, p.opK + id * G::kslot, n, bar);
+    bulk_load(smem + Cfg::mat, p.Simg + ub * G::mat, G::mat, bar);
+  }
+  if (nchv < 2)   // the chunk that is not there reads as zeros
+    for (uint32_t i = tid; i < G::kslot / 4; i += 256)
+#pragma unroll
+      for (int a = 3; a < 6; ++a) sts32(sb + a * Cfg::tb + G::kslot + 4 * i, 0u);
+  if (tid < BC) {
+    const bool act = tid < nt_valid;
+    const float an = act ? p.an[ut0 + tid] : 1.0f;
+    fs[Cfg::f_an + tid] = an;
+    fs[Cfg::f_rho + tid] = act ? an * an * p.delta[ut0 + tid] : 0.f;   // z z^T / delta = rho alpha alpha^T
+    fs[Cfg::f_qsi + tid] = act ? p.qsi[ut0 + tid] : 0.f;
+    fs[Cfg::f_id + tid] = act ? p.iden[ut0 + tid] : 0.f;
+  }
+  __syncthreads();
+  // ---- E, dE, dY as operand rows, scaled by their largest entry
+  constexpr int NG = BC * D / 4, NPT = (NG + 255) / 256;   // groups of four columns, per thread
+  float sE = 1.f, sDE = 1.f, sDY = 1.f, sZ = 1.0f;
+  {
+    float4 xe[NPT], xd[NPT], xy[NPT];
+    float me = 0.f, md = 0.f, my = 0.f;
+#pragma unroll
+    for (int i = 0; i < NPT; ++i) {
+      const int j = tid + 256 * i, t = j / (D / 4), c = j % (D / 4);
+      xe[i] = xd[i] = xy[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (j < NG && t < nt_valid) {
+        const size_t o = tok + t * ts + 4 * c;
+        xe[i] = gload4(p.e + (ut0 + t) * D + 4 * c);
+        xd[i] = *reinterpret_cast<const float4*>(p.dv + o);
+        xy[i] = gload4(p.d_out + o);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NPT; ++i) {
+      const int t = (tid + 256 * i) / (D / 4);
+      const float id = t < BC ? fabsf(fs[Cfg::f_id + t]) : 0.f;
+      xy[i] = make_float4(xy[i].x * id, xy[i].y * id, xy[i].z * id, xy[i].w * id);
+      me = max4(me, xe[i]); md = max4(md, xd[i]); my = max4(my, xy[i]);
+    }
+    cta_max_put(red, 0, me, warp, lane);
+    cta_max_put(red, 1, md, warp, lane);
+    cta_max_put(red, 2, my, warp, lane);
+    __syncthreads();
+    sE = pow2_scale(cta_max_get(red, 0), 10);
+    sDE = pow2_scale(cta_max_get(red, 1), 10);
+    sDY = pow2_scale(cta_max_get(red, 2), 10);
+#pragma unroll
+    for (int i = 0; i < NPT; ++i) {
+      const int j = tid + 256 * i, t = j / (D / 4), c = j % (D / 4);
+      if (j < NG) {
+        row_store4<D>(tE, t, c, xe[i], sE);
+        row_store4<D>(tDE, t, c, xd[i], sDE);
+        row_store4<D>(tDY, t, c, xy[i], sDY);
+      }
+    }
+  }
+  __syncthreads();
+  wait(0);
+  const uint32_t la = tok_lane_a<D>(lane), lb = tok_lane_b<D>(lane), lk = tok_lane_k<D>(lane);
+  const uint32_t own = uint32_t(tg * 16) * kTokRow<D>;   // this warp's 16 tokens
+  const int tr = tg * 16 + g;                            // ... and the lane's first token row
+  // acc0: dq (role 0) or dalpha (role 1); acc1: -(S part of dk_hat); of this warp's tokens and half of the columns
+  float acc0[NH][4] = {}, acc1[NH][4] = {};
+  // (Code size is what limits this kernel first: every helper below is expanded once, two accumulators
+  // take turns in acc0.)
+  auto swap = [&]() {
+#pragma unroll
+    for (int nt = 0; nt < NH; ++nt)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float x = acc0[nt][e];
+        acc0[nt][e] = acc1[nt][e];
+        acc1[nt][e] = x;
+      }
+  };
+  // acc0 += rows x (block matrix with a scale per 16 rows)
+  auto product = [&](uint32_t rows, const float* scale) {
+#pragma unroll 1
+    for (int ks = 0; ks < KS; ++ks) {
+      uint32_t ah[4], al[4];
+      tok_frag<D>(ah, rows + own + la, ks, false);
+      tok_frag<D>(al, rows + own + la, ks, true);
+      const float s = scale[ks];
+      constexpr int NQ = NH < 4 ? NH : 4;
+#pragma unroll
+      for (int nt = 0; nt < NH; nt += NQ) {
+        uint32_t b[NQ][4];
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) tok_frag_k<D>(b[i], mat + lk, 16 * ks, h * NH + nt + i);
+        mma3_f16_scaled<NQ>([&](int, int lo) -> const uint32_t(&)[4] { return lo ? al : ah; }, [&](int i, int r) { return b[i][r]; },
+                            [&](int i) -> float* { return acc0[nt + i]; }, s);
+      }
+    }
+  };
+  // coef (16 own tokens x the 16 tokens of chunk sc, true factors folded in) times token rows -> acc
+  auto apply = [&](const float (&coef)[2][4], uint32_t rows, int sc, int n0, auto& acc, auto ntiles) {
+    float m = 0.f;
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) m = fmaxf(m, fabsf(coef[nt][e]));
+    m = warp_max_nonneg(m);
+    const float s = pow2_scale(m, 8), si = pow2_inverse(s);
+    float x[2][4];
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[nt][e] = coef[nt][e] * s;
+    uint32_t ah[4], al[4];
+    split_frag(x[0], x[1], ah, al);
+    constexpr int NN = decltype(ntiles)::value, NQ = NN < 4 ? NN : 4;
+#pragma unroll
+    for (int nt = 0; nt < NN; nt += NQ) {
+      uint32_t b[NQ][4];
+#pragma unroll
+      for (int i = 0; i < NQ; ++i) tok_frag_k<D>(b[i], rows + lk, 16 * sc, n0 + nt + i);
+      mma3_f16_scaled<NQ>([&](int, int lo) -> const uint32_t(&)[4] { return lo ? al : ah; }, [&](int i, int r) { return b[i][r]; },
+                          [&](int i) -> float* { return acc[nt + i]; }, si);
+    }
+  };
+  // own rows of rows0 [and rows1] against the tokens of chunk sc of cols0 [cols1]: two 16 x 16 Gram matrices
+  auto gram2 = [&](uint32_t rows0, uint32_t rows1, uint32_t cols0, uint32_t cols1, int sc, float (&x)[2][4], float (&y)[2][4]) {
+    const uint32_t oc = uint32_t(sc * 16) * kTokRow<D> + lb;
+#pragma unroll 1
+    for (int ks = 0; ks < KS; ++ks) {
+      uint32_t ah[2][4], al[2][4], bh[2][4], bl[2][4];
+      tok_frag<D>(ah[0], rows0 + own + la, ks, false);
+      tok_frag<D>(al[0], rows0 + own + la, ks, true);
+      tok_frag<D>(ah[1], rows1 + own + la, ks, false);
+      tok_frag<D>(al[1], rows1 + own + la, ks, true);
+      tok_frag<D>(bh[0], cols0 + oc, ks, false);
+      tok_frag<D>(bl[0], cols0 + oc, ks, true);
+      tok_frag<D>(bh[1], cols1 + oc, ks, false);
+      tok_frag<D>(bl[1], cols1 + oc, ks, true);
+      mma3_f16_many<4>([&](int i, int lo) -> const uint32_t(&)[4] { return lo ? al[i >> 1] : ah[i >> 1]; },
+                       [&](int i, int r) { return (r & 2) ? bl[i >> 1][2 * (i & 1) + (r & 1)] : bh[i >> 1][2 * (i & 1) + (r & 1)]; },
+                       [&](int i) -> float* { return i >= 2 ? y[i & 1] : x[i & 1]; });
+    }
+  };
+  using NHc = std::integral_constant<int, NH>;
+  auto grams = [&]() {
+    // role 0: dq += tril(dY E^T) alpha,     -dkS += stril(dE E^T) alpha     (chunks up to the own one)
+    // role 1: dalpha += triu(E dY^T) Q - striu(E dE^T) K                     (chunks from the own one on)
+    const int lo_c = role ? tg : 0, hi_c = role ? 2 : tg + 1;
+#pragma unroll 1
+    for (int sc = lo_c; sc < hi_c; ++sc) {
+      float x[2][4] = {}, y[2][4] = {};
+      gram2(role ? tE : tDY, role ? tE : tDE, role ? tDY : tE, role ? tDE : tE, sc, x, y);
+      const float fx = role ? pow2_inverse(sDY) : pow2_inverse(sE) * kInv, fy = role ? -pow2_inverse(sDE) * kInv : pow2_inverse(sE) * kInv;
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int t = tr + 8 * (e >> 1), s = sc * 16 + 8 * nt + 2 * c4 + (e & 1);
+          const bool kx = role ? s >= t : s <= t, ky = role ? s > t : s < t;
+          x[nt][e] = kx ? x[nt][e] * fx * (role ? fs[Cfg::f_qsi + s] : 1.0f) : 0.f;
+          y[nt][e] = ky ? y[nt][e] * fy : 0.f;
+        }
+#pragma unroll 1
+      for (int w = 0; w < 2; ++w) {   // role 0: into dq, then (acc1) dkS; role 1: both into dalpha
+        float co[2][4];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) co[nt][e] = w ? y[nt][e] : x[nt][e];
+        apply(co, role ? (w ? tK : tQ) : tA, sc, h * NH, acc0, NHc{});
+        if (role == 0) swap();
+      }
+    }
+  };
+#pragma unroll 1
+  for (int phase = 0; phase < 2; ++phase) {
+    if (phase == 1) {
+      __syncthreads();
+      if (tid == 0) {
+        mbar_arrive_expect_tx(bar, G::mat);
+        bulk_load(smem + Cfg::mat, p.Dimg + ub * G::mat, G::mat, bar);
+      }
+    }
+    if (role == phase) {
+      if (role == 1) wait(1);
+#pragma unroll 1
+      for (int w = 0; w < 2 - role; ++w) {
+        product(role ? tE : w ? tDE : tDY, (role ? p.Dsc : p.Ssc) + ub * KS);
+        if (role == 0) swap();
+      }
+    } else {
+      grams();
+    }
+  }
+  // ---- row dots: alpha . dalpha (role 1), q . dq (role 0)
+  {
+    const float f = role ? pow2_inverse(sE) : pow2_inverse(sDY), fk = -pow2_inverse(sDE);
+    float dot[2] = {0.f, 0.f};
+    const size_t row_o[2] = {tok + tr * ts + h * NH * 8 + 2 * c4, tok + (tr + 8) * ts + h * NH * 8 + 2 * c4};
+#pragma unroll
+    for (int nt = 0; nt < NH; ++nt)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int col = (h * NH + nt) * 8 + 2 * c4, t = tr + 8 * hf;
+        const float2 r = row_pair<D>(smem + (role ? 3 : 4) * Cfg::tb, t, col);
+        acc0[nt][2 * hf] *= f;
+        acc0[nt][2 * hf + 1] *= f;
+        dot[hf] = fmaf(r.x, acc0[nt][2 * hf], fmaf(r.y, acc0[nt][2 * hf + 1], dot[hf]));
+        if (role == 0 && t < nt_valid) {   // (dq and dk are completed by the last launch)
+          const size_t o = row_o[hf] + 8 * nt;
+          *reinterpret_cast<float2*>(p.dq + o) = make_float2(acc0[nt][2 * hf], acc0[nt][2 * hf + 1]);
+          *reinterpret_cast<float2*>(p.dk + o) = make_float2(acc1[nt][2 * hf] * fk, acc1[nt][2 * hf + 1] * fk);
+        }
+      }
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      dot[hf] += __shfl_xor_sync(0xffffffffu, dot[hf], 1);
+      dot[hf] += __shfl_xor_sync(0xffffffffu, dot[hf], 2);
+      if (c4 == 0) fs[(role ? Cfg::f_dot : Cfg::f_dqd) + h * 32 + tr + 8 * hf] = dot[hf];
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    mbar_arrive_expect_tx(bar, G::mat);
+    bulk_load(smem + Cfg::mat, p.Aimg + ub * G::mat, G::mat, bar);
+  }
+  // ---- da = (dalpha - alpha (alpha . dalpha)) / ||a||;  gradient of the denominators and its sum with q
+  float mx = 0.f;
+  if (role == 1) {
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      const int t = tr + 8 * hf;
+      const float an = fs[Cfg::f_an + t];
+      const bool floored = !(an > p.eps);
+      const float dot = floored ? 0.f : (fs[Cfg::f_dot + t] + fs[Cfg::f_dot + 32 + t]) * kInv * kInv;
+      const float ia = rcp_ftz_nr(an);
+#pragma unroll
+      for (int nt = 0; nt < NH; ++nt) {
+        const float2 r = row_pair<D>(smem + 3 * Cfg::tb, t, (h * NH + nt) * 8 + 2 * c4);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          float& x = acc0[nt][2 * hf + e];
+          x = (x - (e ? r.y : r.x) * dot) * ia;
+          mx = fmaxf(mx, fabsf(x));
+        }
+      }
+    }
+  } else if (tid < BC) {
+    const float id = fs[Cfg::f_id + tid];
+    float dd = (fs[Cfg::f_dqd + tid] + fs[Cfg::f_dqd + 32 + tid]) * fs[Cfg::f_qsi + tid];
+    dd = id > 0.f && !(p.flags & VLA_FLAG_IDENTITY_MAP) ? -dd * id : 0.f;
+    fs[Cfg::f_ddn + tid] = dd;
+    if (tid < nt_valid) p.dden[ut0 + tid] = dd;
+  }
+  float4 xz[UT ? NPT : 1];
+  float mz = 0.f;
+  if constexpr (UT) {
+#pragma unroll
+    for (int i = 0; i < NPT; ++i) {
+      const int j = tid + 256 * i, t = j / (D / 4), c = j % (D / 4);
+      xz[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (j < NG && t < nt_valid) xz[i] = gload4(p.zeta + (ut0 + t) * D + 4 * c);
+      mz = max4(mz, xz[i]);
+    }
+    cta_max_put(red, 4, mz, warp, lane);
+  }
+  cta_max_put(red, 3, mx, warp, lane);
+  __syncthreads();
+  const float sDA = pow2_scale(cta_max_get(red, 3), 10);
+  if (role == 1) {   // da over dY's rows
+#pragma unroll
+    for (int nt = 0; nt < NH; ++nt)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf)
+        row_pair_store<D>(tDY, tr + 8 * hf, (h * NH + nt) * 8 + 2 * c4, acc0[nt][2 * hf] * sDA, acc0[nt][2 * hf + 1] * sDA);
+  } else if (tid < D) {
+    float y = 0.f;
+#pragma unroll 2
+    for (int t = 0; t < nt_valid; ++t) y = fmaf(fs[Cfg::f_ddn + t] * fs[Cfg::f_qsi + t], row_one<D>(smem + 4 * Cfg::tb, t, tid), y);
+    p.Y[ub * D + tid] = y;
+  }
+  if constexpr (UT) {   // zeta over E's rows
+    sZ = pow2_scale(cta_max_get(red, 4), 10);
+#pragma unroll
+    for (int i = 0; i < NPT; ++i) {
+      const int j = tid + 256 * i;
+      if (j < NG) row_store4<D>(tE, j / (D / 4), j % (D / 4), xz[i], sZ);
+    }
+  }
+  __syncthreads();
+  // ---- g = A_t da_t = da A - tril(da zeta^T) zeta, columns split over up to four warps per 16 tokens
+  constexpr int NCG = D >= 32 ? 4 : 2, N3 = D / NCG / 8;
+  using N3c = std::integral_constant<int, N3>;
+  const int cg = warp >> 1;
+  float ga[N3][4] = {};
+  wait(0);
+  if (cg < NCG) {
+    const float as = p.Asc[ub];
+#pragma unroll 1
+    for (int ks = 0; ks < KS; ++ks) {
+      uint32_t ah[4], al[4];
+      tok_frag<D>(ah, tDY + own + la, ks, false);
+      tok_frag<D>(al, tDY + own + la, ks, true);
+      uint32_t b[N3][4];
+#pragma unroll
+      for (int i = 0; i < N3; ++i) tok_frag_k<D>(b[i], mat + lk, 16 * ks, cg * N3 + i);
+      mma3_f16_scaled<N3>([&](int, int lo) -> const uint32_t(&)[4] { return lo ? al : ah; }, [&](int i, int r) { return b[i][r]; },
+                          [&](int i) -> float* { return ga[i]; }, as);
+    }
+    const uint32_t zr = UT ? tE : tA;
+    const float zf = UT ? -pow2_inverse(sZ) * pow2_inverse(sZ) : -kInv * kInv;
+#pragma unroll 1
+    for (int sc = 0; sc <= tg; ++sc) {
+      float x[2][4] = {};
+      const uint32_t oc = uint32_t(sc * 16) * kTokRow<D> + lb;
+#pragma unroll 1
+      for (int ks = 0; ks < KS; ++ks) {
+        uint32_t ah[4], al[4], bh[4], bl[4];
+        tok_frag<D>(ah, tDY + own + la, ks, false);
+        tok_frag<D>(al, tDY + own + la, ks, true);
+        tok_frag<D>(bh, zr + oc, ks, false);
+        tok_frag<D>(bl, zr + oc, ks, true);
+        mma3_f16_many<2>([&](int, int lo) -> const uint32_t(&)[4] { return lo ? al : ah; },
+                         [&](int i, int r) { return (r & 2) ? bl[2 * i + (r & 1)] : bh[2 * i + (r & 1)]; },
+                         [&](int i) -> float* { return x[i]; });
+      }
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int t = tr + 8 * (e >> 1), s = sc * 16 + 8 * nt + 2 * c4 + (e & 1);
+          x[nt][e] = s <= t ? x[nt][e] * zf * (UT ? 1.0f : fs[Cfg::f_rho + s]) : 0.f;
+        }
+      apply(x, zr, sc, cg * N3, ga, N3c{});
+    }
+  }
+  float mg = 0.f;
+#pragma unroll
+  for (int nt = 0; nt < N3; ++nt)
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      const int t = tr + 8 * hf, col = (cg * N3 + nt) * 8 + 2 * c4;
+      float2 x = make_float2(ga[nt][2 * hf] * pow2_inverse(sDA), ga[nt][2 * hf + 1] * pow2_inverse(sDA));
+      if (cg < NCG && t < nt_valid) *reinterpret_cast<float2*>(p.g + (ut0 + t) * D + col) = x;
+      const float an = fs[Cfg::f_an + t];
+      ga[nt][2 * hf] = x.x * an;        // g_s a_s^T = (an g) alpha^T
+      ga[nt][2 * hf + 1] = x.y * an;
+      mg = fmaxf(mg, fmaxf(fabsf(ga[nt][2 * hf]), fabsf(ga[nt][2 * hf + 1])));
+    }
+  cta_max_put(red, 5, mg, warp, lane);
+  __syncthreads();
+  const float sG = pow2_scale(cta_max_get(red, 5), 10);
+  if (cg < NCG) {   // an g over dE's rows
+#pragma unroll
+    for (int nt = 0; nt < N3; ++nt)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf)
+        row_pair_store<D>(tDE, tr + 8 * hf, (cg * N3 + nt) * 8 + 2 * c4, ga[nt][2 * hf] * sG, ga[nt][2 * hf + 1] * sG);
+  }
+  __syncthreads();
+  // ---- the block's sum of (an g) alpha^T + alpha (an g)^T
+  constexpr int MT = D / 16, PP = 8 / MT > D / 8 ? D / 8 : 8 / MT, N4 = D / 8 / PP;   // m tiles, warps per m tile, n tiles a warp
+  const int mt = warp % MT, part = warp / MT;
+  if (part < PP) {
+    const uint32_t lm = tok_lane_m<D>(lane);
+    uint32_t gh[2][4], gl[2][4], ah[2][4], al[2][4];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      tok_frag_m<D>(gh[k], tDE + lm, 16 * k, mt, false);
+      tok_frag_m<D>(gl[k], tDE + lm, 16 * k, mt, true);
+      tok_frag_m<D>(ah[k], tA + lm, 16 * k, mt, false);
+      tok_frag_m<D>(al[k], tA + lm, 16 * k, mt, true);
+    }
+    const float f = pow2_inverse(sG) * kInv;
+    float* dst = p.X + ub * D * D + size_t(mt * 16 + g) * D + 2 * c4;
+#pragma unroll 1
+    for (int n = 0; n < N4; ++n) {
+      const int nt = part * N4 + n;
+      uint32_t b[4][4];   // alpha, an g; two K steps each
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        tok_frag_k<D>(b[k], tA + lk, 16 * k, nt);
+        tok_frag_k<D>(b[2 + k], tDE + lk, 16 * k, nt);
+      }
+      float x[4] = {};
+      mma3_f16_many<4>([&](int i, int lo) -> const uint32_t(&)[4] { return i < 2 ? (lo ? gl[i & 1] : gh[i & 1]) : (lo ? al[i & 1] : ah[i & 1]); },
+                       [&](int i, int r) { return b[i][r]; }, [&](int) -> float* { return x; });
+      *reinterpret_cast<float2*>(dst + 8 * nt) = make_float2(x[0] * f, x[1] * f);
+      *reinterpret_cast<float2*>(dst + 8 * D + 8 * nt) = make_float2(x[2] * f, x[3] * f);
+    }
+  }
+  if (*abort_flag) {
+    settle_copies();
+    if (tid == 0 && p.status) atomicCAS(p.status, 0, int(VLA_ERR_DEVICE_TIMEOUT));
+  }
+}
+
+// ---------------------------------------------------------------- suffix sums over the blocks
+// Replaces every block's sum by what the later blocks (and the final state's gradient) add up to.
+template <int D>
+__global__ void __launch_bounds__(256) bwd_scan_kernel(const BwdChunkParams p) {
+  const int unit = blockIdx.y, i = blockIdx.x * 256 + threadIdx.x;
+  constexpr int N = D * D / 4;
+  if (i < N) {
+    float4* x = reinterpret_cast<float4*>(p.X + size_t(unit) * p.NB * D * D) + i;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p.dA_T) acc = reinterpret_cast<const float4*>(p.XT + size_t(unit) * D * D)[i];
+    for (int b = p.NB - 1; b >= 0; b -= 8) {
+      float4 v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (b - j >= 0) v[j] = x[size_t(b - j) * N];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (b - j >= 0) {
+          x[size_t(b - j) * N] = acc;
+          acc.x += v[j].x; acc.y += v[j].y; acc.z += v[j].z; acc.w += v[j].w;
+        }
+    }
+  } else if (i < N + D) {
+    const int c = i - N;
+    float* y = p.Y + size_t(unit) * p.NB * D + c;
+    float acc = p.dz_T ? p.dz_T[size_t(unit) * D + c] : 0.f;
+    for (int b = p.NB - 1; b >= 0; --b) {
+      const float v = y[size_t(b) * D];
+      y[size_t(b) * D] = acc;
+      acc += v;
+    }
+    if (p.dz0) p.dz0[size_t(unit) * D + c] = acc;
+  }
+}
+
+// X beyond the last token: A_T (dA_T + dA_T^T) A_T (only when the final A has a gradient)
+template <int D>
+__global__ void __launch_bounds__(256) bwd_final_state_kernel(const BwdChunkParams p) {
+  const size_t at = size_t(blockIdx.x) * D * D;
+  const float *A = p.A_T + at, *dA = p.dA_T + at;
+  float *W = p.XT2 + at, *X = p.XT + at;
+  for (int i = threadIdx.x; i < D * D; i += 256) {
+    const int r = i / D, c = i % D;
+    float s = 0.f;
+    for (int k = 0; k < D; ++k) s = fmaf(dA[r * D + k] + dA[k * D + r], A[k * D + c], s);
+    W[i] = s;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < D * D; i += 256) {
+    const int r = i / D, c = i % D;
+    float s = 0.f;
+    for (int k = 0; k < D; ++k) s = fmaf(A[r * D + k], W[k * D + c], s);
+    X[i] = s;
+  }
+}
+
+// ---------------------------------------------------------------- per block: du, and dq, dk through norms and feature map
+template <int D, bool UT> struct BwdFinishCfg {
+  static constexpr uint32_t tb = BwdGeom<D>::tb;
+  static constexpr uint32_t mat = (UT ? 5 : 4) * tb;   // K, alpha, Q, an g [, u]
+  static constexpr uint32_t zz = mat + BwdGeom<D>::mat;                      // key sums, their gradients: [32][D] each
+  static constexpr uint32_t fl = zz + 2 * kBwdBlock * D * 4;
+  static constexpr int f_red = 0, f_an = 64, f_qsi = 96, f_nrm = 128, f_ddn = 160, f_kd = 192, f_end = 192 + 4 * 32;
+  static constexpr uint32_t smem_bytes = fl + f_end * 4 + 32;
+};
+
+template <int D, typename TIn, bool UT>
+__global__ void __launch_bounds__(256) bwd_finish_kernel(const BwdChunkParams p) {
+  using Cfg = BwdFinishCfg<D, UT>;
+  using G = BwdGeom<D>;
+  constexpr int BC = kBwdBlock, KS = D / 16;
+  constexpr float kInv = 1.0f / 256.0f;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int blk = blockIdx.x, unit = blockIdx.y;
+  const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int t0 = blk * BC, T = p.T, nt_valid = min(BC, T - t0), nchv = min(2, p.nch - 2 * blk);
+  const bool ident = (p.flags & VLA_FLAG_IDENTITY_MAP) != 0;
+  const size_t ub = size_t(unit) * p.NB + blk, ut0 = size_t(unit) * T + t0;
+  const size_t tok = bwd_tok(p, unit, t0, D), ts = bwd_stride(p, D);   // the block's first token, distance between tokens
+  const uint32_t sb = smem_u32(smem);
+  const uint32_t tK = sb, tA = sb + Cfg::tb, tG = sb + 3 * Cfg::tb, tU = UT ? sb + 4 * Cfg::tb : tK, mat = sb + Cfg::mat;
+  float* zp = reinterpret_cast<float*>(smem + Cfg::zz);
+  float* zg = zp + BC * D;
+  float* fs = reinterpret_cast<float*>(smem + Cfg::fl);
+  float* red = fs + Cfg::f_red;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(fs + Cfg::f_end);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar + 1);
+  if (tid == 0) {
+    *abort_flag = 0;
+    mbar_init(bar, 1);
+    mbar_init_fence();
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const size_t id = size_t(unit) * p.nch + 2 * blk;
+    const uint32_t n = nchv * G::kslot;
+    mbar_arrive_expect_tx(bar, 3 * n);
+    bulk_load(smem, p.opK + id * G::kslot, n, bar);
+    bulk_load(smem + Cfg::tb, p.opA + id * G::kslot, n, bar);
+    bulk_load(smem + 2 * Cfg::tb, p.opQ + id * G::kslot, n, bar);
+  }
+  if (nchv < 2)
+    for (uint32_t i = tid; i < G::kslot / 4; i += 256)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) sts32(sb + a * Cfg::tb + G::kslot + 4 * i, 0u);
+  if (tid < BC) {
+    const bool act = tid < nt_valid;
+    fs[Cfg::f_an + tid] = act ? p.an[ut0 + tid] : 0.f;
+    fs[Cfg::f_qsi + tid] = act ? p.qsi[ut0 + tid] : 0.f;
+    fs[Cfg::f_nrm + tid] = act ? p.nrm[ut0 + tid] : 1.f;
+    fs[Cfg::f_ddn + tid] = act ? p.dden[ut0 + tid] : 0.f;
+  }
+  __syncthreads();
+  // ---- X beyond this block, an g and u as operand images
+  constexpr int NG = BC * D / 4, NPT = (NG + 255) / 256, NM = (D * D / 4 + 255) / 256;
+  float sX, sG, sU = 256.0f;
+  {
+    float4 xg[NPT], xu[UT ? NPT : 1];
+    float mm = 0.f, mg = 0.f, mu = 0.f;
+#pragma unroll 4
+    for (int i = 0; i < NM; ++i) {
+      const int j = tid + 256 * i;
+      if (j < D * D / 4) mm = max4(mm, gload4(p.X + ub * D * D + 4 * j));
+    }
+#pragma unroll
+    for (int i = 0; i < NPT; ++i) {
+      const int j = tid + 256 * i, t = j / (D / 4), c = j % (D / 4);
+      xg[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (UT) xu[i] = xg[i];
+      if (j < NG && t < nt_valid) {
+        const float an = fs[Cfg::f_an + t];
+        const float4 x = gload4(p.g + (ut0 + t) * D + 4 * c);
+        xg[i] = make_float4(x.x * an, x.y * an, x.z * an, x.w * an);
+        if (UT) xu[i] = gload4(static_cast<const TIn*>(p.u) + tok + t * ts + 4 * c);
+      }
+      mg = max4(mg, xg[i]);
+      if (UT) mu = max4(mu, xu[i]);
+    }
+    cta_max_put(red, 0, mm, warp, lane);
+    cta_max_put(red, 1, mg, warp, lane);
+    if (UT) cta_max_put(red, 2, mu, warp, lane);
+    __syncthreads();
+    sX = pow2_scale(cta_max_get(red, 0), 10);
+    sG = pow2_scale(cta_max_get(red, 1), 10);
+    if (UT) sU = pow2_scale(cta_max_get(red, 2), 10);
+#pragma unroll 2
+    for (int i = 0; i < NM; ++i) {   // (read a second time, from L2)
+      const int j = tid + 256 * i;
+      if (j < D * D / 4) row_store4<D>(mat, j / (D / 4), j % (D / 4), gload4(p.X + ub * D * D + 4 * j), sX);
+    }
+#pragma unroll
+    for (int i = 0; i < NPT; ++i) {
+      const int j = tid + 256 * i;
+      if (j < NG) {
+        row_store4<D>(tG, j / (D / 4), j % (D / 4), xg[i], sG);
+        if (UT) row_store4<D>(tU, j / (D / 4), j % (D / 4), xu[i], sU);
+      }
+    }
+  }
+  {
+    uint32_t it = 0;
+    const uint32_t probes = p.wait_limit ? p.wait_limit : kWaitProbeLimit;
+    while (!mbar_try_wait(bar, 0))
+      if (++it > probes) { *abort_flag = 1; break; }
+  }
+  __syncthreads();
+  // ---- key sums up to each token, and the sums of dden q from each token on (thread = column)
+  if (!ident) {
+    if (tid < D) {
+      float z = 0.f;
+#pragma unroll 2
+      for (int t = 0; t < nt_valid; ++t) {
+        if ((t & 15) == 0) z = p.zkc[(size_t(unit) * p.nch + 2 * blk + (t >> 4)) * D + tid];
+        z = fmaf(row_one<D>(smem, t, tid), fabsf(fs[Cfg::f_nrm + t]) * kInv, z);
+        zp[t * D + tid] = z;
+      }
+    } else if (tid >= 128 && tid - 128 < D) {
+      const int c = tid - 128;
+      float y = p.Y[ub * D + c];
+#pragma unroll 2
+      for (int t = nt_valid - 1; t >= 0; --t) {
+        y = fmaf(fs[Cfg::f_ddn + t] * fs[Cfg::f_qsi + t], row_one<D>(smem + 2 * Cfg::tb, t, c), y);
+        zg[t * D + c] = y;
+      }
+    }
+  }
+  // ---- du = -U X - triu(U alpha^T) (an g) - triu(U (an g)^T) alpha
+  constexpr int NCG = D >= 32 ? 4 : 2, N3 = D / NCG / 8;
+  const int tg = warp & 1, cg = warp >> 1;
+  const uint32_t la = tok_lane_a<D>(lane), lb = tok_lane_b<D>(lane), lk = tok_lane_k<D>(lane);
+  const uint32_t own = uint32_t(tg * 16) * kTokRow<D>;
+  const int tr = tg * 16 + g;
+  float du[N3][4] = {};
+  if (cg < NCG) {
+    const float fx = -pow2_inverse(sX);
+#pragma unroll 1
+    for (int ks = 0; ks < KS; ++ks) {
+      uint32_t ah[4], al[4];
+      tok_frag<D>(ah, tU + own + la, ks, false);
+      tok_frag<D>(al, tU + own + la, ks, true);
+      uint32_t b[N3][4];
+#pragma unroll
+      for (int i = 0; i < N3; ++i) tok_frag_k<D>(b[i], mat + lk, 16 * ks, cg * N3 + i);
+      mma3_f16_scaled<N3>([&](int, int lo) -> const uint32_t(&)[4] { return lo ? al : ah; }, [&](int i, int r) { return b[i][r]; },
+                          [&](int i) -> float* { return du[i]; }, fx);
+    }
+#pragma unroll 1
+    for (int sc = tg; sc < 2; ++sc) {
+      float x[2][2][4] = {};   // U alpha^T, U (an g)^T
+      const uint32_t oc = uint32_t(sc * 16) * kTokRow<D> + lb;
+#pragma unroll 1
+      for (int ks = 0; ks < KS; ++ks) {
+        uint32_t ah[4], al[4], bh[2][4], bl[2][4];
+        tok_frag<D>(ah, tU + own + la, ks, false);
+        tok_frag<D>(al, tU + own + la, ks, true);
+        tok_frag<D>(bh[0], tA + oc, ks, false);
+        tok_frag<D>(bl[0], tA + oc, ks, true);
+        tok_frag<D>(bh[1], tG + oc, ks, false);
+        tok_frag<D>(bl[1], tG + oc, ks, true);
+        mma3_f16_many<4>([&](int, int lo) -> const uint32_t(&)[4] { return lo ? al : ah; },
+                         [&](int i, int r) { return (r & 2) ? bl[i >> 1][2 * (i & 1) + (r & 1)] : bh[i >> 1][2 * (i & 1) + (r & 1)]; },
+                         [&](int i) -> float* { return x[i >> 1][i & 1]; });
+      }
+#pragma unroll 1
+      for (int w = 0; w < 2; ++w) {
+        const float f = -kInv * pow2_inverse(sG);
+        float co[2][4], m = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int t = tr + 8 * (e >> 1), s = sc * 16 + 8 * nt + 2 * c4 + (e & 1);
+            co[nt][e] = s >= t ? (w ? x[1][nt][e] : x[0][nt][e]) * f : 0.f;
+            m = fmaxf(m, fabsf(co[nt][e]));
+          }
+        m = warp_max_nonneg(m);
+        const float s = pow2_scale(m, 8), si = pow2_inverse(s);
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) co[nt][e] *= s;
+        uint32_t ah[4], al[4];
+        split_frag(co[0], co[1], ah, al);
+        uint32_t b[N3][4];
+#pragma unroll
+        for (int i = 0; i < N3; ++i) tok_frag_k<D>(b[i], (w ? tA : tG) + lk, 16 * sc, cg * N3 + i);
+        mma3_f16_scaled<N3>([&](int, int lo) -> const uint32_t(&)[4] { return lo ? al : ah; }, [&](int i, int r) { return b[i][r]; },
+                            [&](int i) -> float* { return du[i]; }, si);
+      }
+    }
+  }
+  // ---- dk_hat and its projection on k_hat
+  const float fu = pow2_inverse(sU);
+  float dk[N3][4], kd[2] = {0.f, 0.f};
+  const size_t row_o[2] = {tok + tr * ts + cg * N3 * 8 + 2 * c4, tok + (tr + 8) * ts + cg * N3 * 8 + 2 * c4};
+#pragma unroll
+  for (int nt = 0; nt < N3; ++nt)
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      const int t = tr + 8 * hf, col = (cg * N3 + nt) * 8 + 2 * c4;
+      float2 x = make_float2(0.f, 0.f);
+      if (cg < NCG && t < nt_valid) {
+        const size_t o = row_o[hf] + 8 * nt;
+        const float2 u2 = make_float2(du[nt][2 * hf] * fu, du[nt][2 * hf + 1] * fu);
+        const float2 a = *reinterpret_cast<const float2*>(p.dk + o), b = *reinterpret_cast<const float2*>(p.g + (ut0 + t) * D + col);
+        x = make_float2(a.x + b.x, a.y + b.y);
+        if (UT) *reinterpret_cast<float2*>(p.du + o) = u2;
+        else { x.x += u2.x; x.y += u2.y; }
+        const float2 k2 = row_pair<D>(smem, t, col);
+        kd[hf] = fmaf(k2.x, x.x, fmaf(k2.y, x.y, kd[hf]));
+      }
+      dk[nt][2 * hf] = x.x;
+      dk[nt][2 * hf + 1] = x.y;
+    }
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf) {
+    kd[hf] += __shfl_xor_sync(0xffffffffu, kd[hf], 1);
+    kd[hf] += __shfl_xor_sync(0xffffffffu, kd[hf], 2);
+    if (c4 == 0) fs[Cfg::f_kd + cg * 32 + tr + 8 * hf] = kd[hf];
+  }
+  __syncthreads();
+  if (cg < NCG) {
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      const int t = tr + 8 * hf;
+      if (t >= nt_valid) continue;
+      float d = 0.f;
+#pragma unroll
+      for (int w = 0; w < NCG; ++w) d += fs[Cfg::f_kd + w * 32 + t];
+      const float nr = fs[Cfg::f_nrm + t], anr = fabsf(nr), inr = rcp_ftz_nr(anr), dd = fs[Cfg::f_ddn + t], qs = fs[Cfg::f_qsi + t];
+      d = nr > 0.f ? d * kInv * kInv : 0.f;
+#pragma unroll
+      for (int nt = 0; nt < N3; ++nt) {
+        const int col = (cg * N3 + nt) * 8 + 2 * c4;
+        const size_t o = row_o[hf] + 8 * nt;
+        const float2 k2 = row_pair<D>(smem, t, col);
+        float2 r = make_float2((dk[nt][2 * hf] - k2.x * d) * inr, (dk[nt][2 * hf + 1] - k2.y * d) * inr);
+        float2 y = *reinterpret_cast<const float2*>(p.dq + o);
+        if (!ident) {
+          // phi'(x) = 1 for x > 0, else exp(x) = phi(x): the smaller of phi(x) and 1
+          const float2 a = *reinterpret_cast<const float2*>(zg + t * D + col), z = *reinterpret_cast<const float2*>(zp + t * D + col);
+          const float2 q2 = row_pair<D>(smem + 2 * Cfg::tb, t, col);
+          r.x = (r.x + a.x) * fminf(k2.x * kInv * anr, 1.0f);
+          r.y = (r.y + a.y) * fminf(k2.y * kInv * anr, 1.0f);
+          y.x = fmaf(dd, z.x, y.x) * fminf(q2.x * qs, 1.0f);
+          y.y = fmaf(dd, z.y, y.y) * fminf(q2.y * qs, 1.0f);
+          *reinterpret_cast<float2*>(p.dq + o) = y;
+        }
+        *reinterpret_cast<float2*>(p.dk + o) = r;
+      }
+    }
+  }
+  if (*abort_flag) {
+    settle_copies();
+    if (tid == 0 && p.status) atomicCAS(p.status, 0, int(VLA_ERR_DEVICE_TIMEOUT));
+  }
+}
+
+}  // namespace vla

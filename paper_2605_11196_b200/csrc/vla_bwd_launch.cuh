@@ -1,0 +1,48 @@
+// Launcher of the chunked backward pass for one (d, input type); each vla_bwd_d*.cu instantiates it.
+#pragma once
+
+#include "vla.h"
+#include "vla_bwd_chunk.cuh"
+#include "vla_launch.h"
+
+namespace vla {
+
+template <int D, typename TIn, bool UT>
+int launch_bwd_chunk_t(const BwdChunkParams& p, cudaStream_t st) {
+  using Prep = BwdPrepCfg<D>;
+  using Chain = BwdChainCfg<D>;
+  using Block = BwdBlockCfg<D>;
+  using Fin = BwdFinishCfg<D, UT>;
+  static_assert(Block::smem_bytes <= 227 * 1024 && Fin::smem_bytes <= 227 * 1024, "a CTA's shared memory");
+  auto prep = bwd_prep_kernel<D, TIn>;
+  auto chains = bwd_chains_kernel<D, TIn>;
+  auto block = bwd_block_kernel<D, TIn, UT>;
+  auto fin = bwd_finish_kernel<D, TIn, UT>;
+  static std::atomic<unsigned long long> done[4] = {};
+  if (!set_smem_once(done[0], reinterpret_cast<const void*>(prep), Prep::smem_bytes) ||
+      !set_smem_once(done[1], reinterpret_cast<const void*>(chains), Chain::smem_bytes) ||
+      !set_smem_once(done[2], reinterpret_cast<const void*>(block), Block::smem_bytes) ||
+      !set_smem_once(done[3], reinterpret_cast<const void*>(fin), Fin::smem_bytes))
+    return VLA_ERR_CUDA;
+  const long long chunks = (long long)p.units * p.nch;
+  const dim3 blocks(p.NB, p.units);
+  prep<<<unsigned((chunks + Prep::WPC - 1) / Prep::WPC), Prep::WPC * 32, Prep::smem_bytes, st>>>(p);
+  chains<<<2 * p.units, Chain::NT, Chain::smem_bytes, st>>>(p);
+  if (p.dA_T) bwd_final_state_kernel<D><<<p.units, 256, 0, st>>>(p);
+  block<<<blocks, 256, Block::smem_bytes, st>>>(p);
+  bwd_scan_kernel<D><<<dim3((D * D / 4 + D + 255) / 256, p.units), 256, 0, st>>>(p);
+  fin<<<blocks, 256, Fin::smem_bytes, st>>>(p);
+  return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
+}
+
+template <int D, typename TIn>
+int launch_bwd_chunk_any(const BwdChunkParams& p, cudaStream_t st) {
+  return p.u ? launch_bwd_chunk_t<D, TIn, true>(p, st) : launch_bwd_chunk_t<D, TIn, false>(p, st);
+}
+
+}  // namespace vla
+
+#define VLA_DEFINE_BWD_TU(D, TIN, TAG)                                                       \
+  namespace vla {                                                                            \
+  int launch_bwd_chunk_##TAG(const BwdChunkParams& p, cudaStream_t st) { return launch_bwd_chunk_any<D, TIN>(p, st); } \
+  }

@@ -58,6 +58,22 @@ int chunk_resident_ctas(int d, int dtype, bool tri) {
   return 0;
 }
 
+bool set_smem_once(std::atomic<unsigned long long>& done, const void* kern, size_t bytes) {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (dev < 64 && (done.load(std::memory_order_acquire) & bit)) return true;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (dev < 64) done.fetch_or(bit, std::memory_order_release);
+  return true;
+}
+
 int device_sms() {
   static std::atomic<int> known[64];
   int dev = -1, n = 0;
@@ -87,6 +103,23 @@ VLA_DECLARE_PAIR_TU(d128_f32)
 VLA_DECLARE_PAIR_TU(d128_bf16)
 #undef VLA_DECLARE_PAIR_TU
 
+#define VLA_DECLARE_BWD_TU(TAG) int launch_bwd_chunk_##TAG(const BwdChunkParams& p, cudaStream_t st);
+VLA_DECLARE_BWD_TU(d16_f32)
+VLA_DECLARE_BWD_TU(d16_bf16)
+VLA_DECLARE_BWD_TU(d32_f32)
+VLA_DECLARE_BWD_TU(d32_bf16)
+VLA_DECLARE_BWD_TU(d64_f32)
+VLA_DECLARE_BWD_TU(d64_bf16)
+VLA_DECLARE_BWD_TU(d128_f32)
+VLA_DECLARE_BWD_TU(d128_bf16)
+#undef VLA_DECLARE_BWD_TU
+
+int launch_bwd_chunk(int d, int dtype, const BwdChunkParams& p, cudaStream_t st) {
+  if (d == 16) return dtype == VLA_F32 ? launch_bwd_chunk_d16_f32(p, st) : launch_bwd_chunk_d16_bf16(p, st);
+  VLA_CHUNK_DISPATCH(launch_bwd_chunk, p, st);
+  return VLA_ERR_UNSUPPORTED;
+}
+
 int launch_pair(int d, int dtype, const ScanParams& p, const PairStash* sh, cudaStream_t st) {
   const bool f32 = dtype == VLA_F32;
   switch (d) {
@@ -104,12 +137,8 @@ template <int D, typename TIn, bool HAS_U>
 int launch_token_t(const ScanParams& p, cudaStream_t st) {
   using Cfg = TokenCfg<D, TIn, HAS_U>;
   auto kern = vla_scan_token_kernel<D, TIn, HAS_U>;
-  // Idempotent; needed once per device and cheap enough to repeat (no global state kept).
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(Cfg::smem_bytes)) != cudaSuccess) {
-    cudaGetLastError();
-    return VLA_ERR_CUDA;
-  }
+  static std::atomic<unsigned long long> done{0};
+  if (!set_smem_once(done, reinterpret_cast<const void*>(kern), Cfg::smem_bytes)) return VLA_ERR_CUDA;
   kern<<<p.units, Cfg::NT, Cfg::smem_bytes, st>>>(p);
   note_launch("vla_scan_token_kernel", D, sizeof(TIn) == 2 ? VLA_BF16 : VLA_F32, p.units, 0);
   return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
@@ -344,18 +373,21 @@ int launch_decode_t(const ScanParams& p, cudaStream_t st) {
   using Cfg = DecodeCfg<D, TIn>;
   static_assert(Cfg::smem_bytes <= 227 * 1024, "decode kernel exceeds the shared memory of one CTA");
   auto kern = vla_decode_kernel<D, TIn>;
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(Cfg::smem_bytes)) != cudaSuccess ||
-      cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Cfg::NT, Cfg::smem_bytes) !=
-          cudaSuccess ||
-      per_sm < 1) {
-    cudaGetLastError();
-    return VLA_ERR_CUDA;
+  // (the register and shared memory budgets are the same on every device this code runs on)
+  static std::atomic<unsigned long long> done{0};
+  static std::atomic<int> resident{0};
+  if (!set_smem_once(done, reinterpret_cast<const void*>(kern), Cfg::smem_bytes)) return VLA_ERR_CUDA;
+  int per_sm = resident.load(std::memory_order_relaxed);
+  if (per_sm < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Cfg::NT, Cfg::smem_bytes) != cudaSuccess || per_sm < 1) {
+      cudaGetLastError();
+      return VLA_ERR_CUDA;
+    }
+    resident.store(per_sm, std::memory_order_relaxed);
   }
-  const int grid = p.units < sms * per_sm ? p.units : sms * per_sm;   // persistent CTAs
+  const int slots = device_sms() * per_sm;
+  if (slots < 1) return VLA_ERR_CUDA;
+  const int grid = p.units < slots ? p.units : slots;   // persistent CTAs
   kern<<<grid, Cfg::NT, Cfg::smem_bytes, st>>>(p);
   note_launch("vla_decode_kernel", D, sizeof(TIn) == 2 ? VLA_BF16 : VLA_F32, grid, 0);
   return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;

@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "vla_common.cuh"
 #include "vla_seqpar_params.h"
 
@@ -12,7 +14,17 @@ namespace vla {
 struct BackwardParams;
 struct BackwardSplitParams;
 struct MakeUParams;
-struct PairStash;
+struct BwdChunkParams;
+
+// What the backward pass asks the pair kernel's rank 0 for (STASH instantiations: one CTA per unit, no
+// rank 1).  Per token: alpha_t [units, T, D], zeta_t = z_t / sqrt(delta_t) (explicit u only), delta_t and
+// an_t = max(||a_t||, eps) [units, T].  Per chunk: the key sum at its start [units, chunks, D].  Per block of
+// `ck` chunks: A at its start as an operand image (token-row layout, D rows) and the image's scale.
+struct PairStash {
+  float *alpha, *zeta, *delta, *an, *zkc, *Asc;
+  unsigned char* Aimg;
+  int ck;
+};
 }
 
 namespace vla {
@@ -50,7 +62,10 @@ int seqpar_before_scan(int d, int dtype, const SeqParParams& sp, cudaStream_t st
 int seqpar_after_scan(int d, const SeqParParams& sp, float* A_T, float* zT, const float* AT2,
                       const float* zT2, cudaStream_t st);
 
-// Backward pass, token kernel, d in {16, 32, 64}, u = k_hat.
+// Chunked backward pass after the A pass (launch_pair with a stash), d in {16, 32, 64, 128}, no refresh.
+int launch_bwd_chunk(int d, int dtype, const BwdChunkParams& p, cudaStream_t st);
+
+// Backward pass, token kernel, d = 16, u = k_hat.
 int launch_backward(int d, int dtype, const BackwardParams& p, cudaStream_t st);
 
 // Backward pass as two reverse scans over the chunk kernel's stash, d in {32, 64, 128}, u = k_hat.
@@ -74,6 +89,9 @@ void sched_slot_mark(unsigned int epoch, cudaStream_t st);
 
 // What the calling thread launched last (read back by vla_last_launch).
 void note_launch(const char* kernel, int d, int dtype, int grid, int balanced);
+
+// Raises a kernel's dynamic shared memory limit once per device (`done`: a bit per device, one word per kernel).
+bool set_smem_once(std::atomic<unsigned long long>& done, const void* kern, size_t bytes);
 
 // Multiprocessors of the current device (asked once per device); 0 on a failure.
 int device_sms();

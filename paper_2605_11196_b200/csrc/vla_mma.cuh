@@ -99,6 +99,21 @@ __device__ __forceinline__ void mma3_f16_many(FA a, FB b, FC acc) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc(i)[e] += x[i][e];
 }
+// ... with the result scaled: acc[i] += s A[i] B[i]
+template <int N, typename FA, typename FB, typename FC>
+__device__ __forceinline__ void mma3_f16_scaled(FA a, FB b, FC acc, float s) {
+  float x[N][4];
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_f16_zero(x[i], a(i, 1), b(i, 0), b(i, 1));
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_f16(x[i], a(i, 0), b(i, 2), b(i, 3));
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_f16(x[i], a(i, 0), b(i, 0), b(i, 1));
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc(i)[e] = fmaf(x[i][e], s, acc(i)[e]);
+}
 // out (16 x 16 as two tiles) += X M^T for a small row-major M[n][k] (16 x 16 fp32, row stride LD) and
 // X in accumulator tiles (16 x 16).  M[n][k] is taken as 0 for n < 8 <= k (lower triangular matrices).
 template <int LD>
@@ -131,6 +146,84 @@ __device__ __forceinline__ void small_product(float (&out)[2][4], const float (&
   }
 }
 
+// out += X M for a lower triangular M[k][n] (the block k < 8 <= n is taken as 0)
+template <int LD>
+__device__ __forceinline__ void small_product_t(float (&out)[2][4], const float (&x)[2][4], const float* M, int lane) {
+  const int g = lane >> 2, c = lane & 3;
+  // products (k half, n tile): (0, 0), (1, 0), (1, 1)
+  uint32_t ah[2][4], al[2][4], bh[3][2], bl[3][2];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int j = (i + 1) >> 1, nt = i >> 1;
+    split_tf32(M[(8 * j + 2 * c) * LD + 8 * nt + g], bh[i][0], bl[i][0]);
+    split_tf32(M[(8 * j + 2 * c + 1) * LD + 8 * nt + g], bh[i][1], bl[i][1]);
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) split_frag_tf32(x[j], ah[j], al[j]);
+  float y[3][4];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) mma_tf32_zero(y[i], al[(i + 1) >> 1], bl[i][0], bl[i][1]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) mma_tf32(y[i], al[(i + 1) >> 1], bh[i][0], bh[i][1]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) mma_tf32(y[i], ah[(i + 1) >> 1], bl[i][0], bl[i][1]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) mma_tf32(y[i], ah[(i + 1) >> 1], bh[i][0], bh[i][1]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    out[0][e] += y[0][e] + y[1][e];
+    out[1][e] += y[2][e];
+  }
+}
+
+// Tm = (I + stril(N))^-1 of a 16 x 16 N by 8 x 8 blocks, one warp: the two blocks on the diagonal by forward
+// substitution (lane j + 8 b: column j of block b; the upper lanes repeat it), then -T22 N21 T11.  The
+// upper right block of Tm is not written (its users skip it); N's is overwritten.
+template <int LD>
+__device__ __forceinline__ void unit_lower_inverse16(float* Tm, float* N, int lane) {
+  const int g = lane >> 2, c = lane & 3, j = lane & 7, b8 = lane & 8;
+  const float* Nd = N + b8 * LD + b8;
+  float x[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    float a0 = t == j ? 1.0f : 0.0f, a1 = 0.f;
+#pragma unroll
+    for (int s4 = 0; 4 * s4 < t; ++s4) {
+      const float4 y = *reinterpret_cast<const float4*>(Nd + t * LD + 4 * s4);
+      a0 = fmaf(-y.x, x[4 * s4], a0);
+      if (4 * s4 + 1 < t) a1 = fmaf(-y.y, x[4 * s4 + 1], a1);
+      if (4 * s4 + 2 < t) a0 = fmaf(-y.z, x[4 * s4 + 2], a0);
+      if (4 * s4 + 3 < t) a1 = fmaf(-y.w, x[4 * s4 + 3], a1);
+    }
+    x[t] = a0 + a1;
+  }
+  if (lane < 16) {
+#pragma unroll
+    for (int t = 0; t < 8; ++t) Tm[(b8 + t) * LD + b8 + j] = x[t];
+  }
+  __syncwarp();
+  // lane: row g of the lower left block, columns 2 c, 2 c + 1
+  float2 y = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float nk = N[(8 + g) * LD + k];
+    const float2 tk = *reinterpret_cast<const float2*>(Tm + k * LD + 2 * c);
+    y.x = fmaf(nk, tk.x, y.x);
+    y.y = fmaf(nk, tk.y, y.y);
+  }
+  *reinterpret_cast<float2*>(N + 8 + g * LD + 2 * c) = y;
+  __syncwarp();
+  float2 z = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float tk = Tm[(8 + g) * LD + 8 + k];
+    const float2 yk = *reinterpret_cast<const float2*>(N + 8 + k * LD + 2 * c);
+    z.x = fmaf(-tk, yk.x, z.x);
+    z.y = fmaf(-tk, yk.y, z.y);
+  }
+  *reinterpret_cast<float2*>(Tm + (8 + g) * LD + 2 * c) = z;
+}
+
 // ---------------------------------------------------------------- operand arrays in shared memory
 // Token rows: [tokens][D fp16 hi | D fp16 lo], and vector rows: [index][16 tokens fp16 hi | lo].  A row is
 // an odd number of 16-byte pieces long (one of padding), so the eight rows an ldmatrix reads lie in
@@ -158,6 +251,24 @@ __device__ __forceinline__ uint32_t vec_lane_bt(int lane) {
 // ... of one tile of eight tokens: hi in r[0], r[1], lo in r[2], r[3]
 __device__ __forceinline__ uint32_t vec_lane_bt1(int lane) {
   return uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * kVecRow + (lane >> 4) * 32;
+}
+// B operand with K = 16 token rows (or rows of a matrix image), N = eight columns: hi in r[0], r[1], lo in r[2], r[3]
+template <int D>
+__device__ __forceinline__ uint32_t tok_lane_k(int lane) {
+  return uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * kTokRow<D> + (lane >> 4) * (2 * D);
+}
+template <int D>
+__device__ __forceinline__ void tok_frag_k(uint32_t (&r)[4], uint32_t lane_base, int row0, int nt) {
+  ldsm_x4_t(r, lane_base + row0 * kTokRow<D> + nt * 16);
+}
+// A operand with M = 16 columns (tile mt), K = 16 token rows
+template <int D>
+__device__ __forceinline__ uint32_t tok_lane_m(int lane) {
+  return uint32_t((lane & 7) + (lane >> 4) * 8) * kTokRow<D> + ((lane >> 3) & 1) * 16;
+}
+template <int D>
+__device__ __forceinline__ void tok_frag_m(uint32_t (&r)[4], uint32_t lane_base, int row0, int mt, bool lo) {
+  ldsm_x4_t(r, lane_base + row0 * kTokRow<D> + mt * 32 + (lo ? 2 * D : 0));
 }
 // K step ks of a token-row operand (hi, or the remainders)
 template <int D>
@@ -203,6 +314,14 @@ __device__ __forceinline__ float pow2_scale(float m, int target) {
 }
 // its inverse
 __device__ __forceinline__ float pow2_inverse(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
+
+// Held back before a CTA that has given up a wait ends: its copies in flight (a few microseconds at
+// most) must land before its shared memory is handed on, and the barriers that count them are no longer
+// followed.  About 50 us.
+__device__ __forceinline__ void settle_copies() {
+  const long long until = clock64() + 100000;
+  while (clock64() < until) {}
+}
 
 // ---------------------------------------------------------------- cluster of two CTAs
 __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {

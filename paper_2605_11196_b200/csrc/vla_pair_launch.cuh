@@ -13,13 +13,12 @@ int launch_pair_t(const ScanParams& p, const PairStash& sh, cudaStream_t st) {
   static_assert(Cfg::smem_bytes <= 227 * 1024, "pair kernel exceeds the shared memory of one CTA");
   if (p.units > 0x3fffffff) return VLA_ERR_INVALID_ARG;
   auto kern = vla_scan_pair_kernel<D, TIn, UT, STASH>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Cfg::smem_bytes)) != cudaSuccess) {
-    cudaGetLastError();
-    return VLA_ERR_CUDA;
-  }
-  kern<<<2 * p.units, Cfg::NT, Cfg::smem_bytes, st>>>(p, sh);
+  static std::atomic<unsigned long long> done{0};
+  if (!set_smem_once(done, reinterpret_cast<const void*>(kern), Cfg::smem_bytes)) return VLA_ERR_CUDA;
+  const int grid = STASH ? p.units : 2 * p.units;
+  kern<<<grid, Cfg::NT, Cfg::smem_bytes, st>>>(p, sh);
   note_launch(STASH ? "vla_scan_pair_kernel(stash)" : "vla_scan_pair_kernel", D, sizeof(TIn) == 2 ? VLA_BF16 : VLA_F32,
-              2 * p.units, 0);
+              grid, 0);
   return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
 }
 

@@ -25,18 +25,10 @@
 // S and E by powers of two per warp that follow their size.
 #pragma once
 
+#include "vla_launch.h"
 #include "vla_mma.cuh"
 
 namespace vla {
-
-// What the forward leaves for the backward pass (STASH instantiations).  Per token: alpha_t, e_t
-// [units, T, D], zeta_t = z_t / sqrt(delta_t) (explicit u only), and scalars [units, T]:
-// delta_t, an_t = max(||a_t||, eps), 1 / den_t.  Per block of
-// `ck` chunks: the states and the key sum at its start, [units, blocks, ...].
-struct PairStash {
-  float *alpha, *zeta, *e, *delta, *an, *iden, *Ack, *Sck, *zck;
-  int ck;
-};
 
 template <int D, typename TIn, bool UT>
 struct PairCfg {
@@ -60,7 +52,7 @@ struct PairCfg {
   static constexpr uint32_t a_K = 0, a_U = RK * kslot, a_Z0 = a_U + (UT ? RK * kslot : 0), a_W0 = a_Z0 + aslot,
                             a_Z = a_W0 + (UT ? aslot : 0), a_A = a_Z + aslot, a_f = a_A + RA * aslot;
   static constexpr int af_W = 0, af_Li = af_W + (UT ? 3 : 1) * PARTS * SM, af_PT = af_Li + SM, af_dl = af_PT + (UT ? 2 * SM : 0),
-                       af_n = af_dl + 32, af_mx = af_n + 2 * NW * 16, af_us = af_mx + 16, af_pv = af_us + RK * 16, af_end = af_pv + 64;
+                       af_n = af_dl + 32, af_mx = af_n + 2 * NW * 16, af_us = af_mx + 16, af_pv = af_us + RK * 16, af_zp = af_pv + 64, af_end = af_zp + 2 * NPREP * D;
   // rank 1
   static constexpr uint32_t s_K = 0, s_Q = RK * kslot, s_A = 2 * RK * kslot, s_f = s_A + RA * aslot;
   static constexpr int sf_N = 0, sf_T = SM, sf_H = sf_T + 2 * SM, sf_osc = sf_H + 2 * SM, sf_nrm = sf_osc + 32,
@@ -92,7 +84,7 @@ __device__ __forceinline__ void tok_store4(uint32_t base, int row, int pl, float
 }
 
 template <int D, typename TIn, bool UT, bool STASH>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((PairCfg<D, TIn, UT>::NT), 1)
+__global__ void __cluster_dims__(STASH ? 1 : 2, 1, 1) __launch_bounds__((PairCfg<D, TIn, UT>::NT), 1)
 vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
   using Cfg = PairCfg<D, TIn, UT>;
   constexpr int C = Cfg::C, NW = Cfg::NW, NPREP = Cfg::NPREP, LPT = Cfg::LPT, TPW = Cfg::TPW, NP = Cfg::NP;
@@ -102,8 +94,8 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
 
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t sb = smem_u32(smem);
-  const uint32_t rank = blockIdx.x & 1u;   // (of the cluster; from the block index, which the compiler knows to be uniform)
-  const int unit = int(blockIdx.x >> 1);
+  const uint32_t rank = STASH ? 0u : blockIdx.x & 1u;   // (of the cluster; from the block index, which the compiler knows to be uniform)
+  const int unit = int(STASH ? blockIdx.x : blockIdx.x >> 1);
   const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
   // read from lane 0 so that the compiler takes the roles as uniform over a warp
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -162,7 +154,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     mbar_init_fence();
   }
   __syncthreads();
-  cluster_sync();   // the other CTA's barriers exist before anything arrives on them
+  if (!STASH) cluster_sync();   // the other CTA's barriers exist before anything arrives on them
 
   const uint32_t lane_ta = tok_lane_a<D>(lane), lane_tb = tok_lane_b<D>(lane), lane_vb = vec_lane_b(lane), lane_vt = vec_lane_bt(lane), lane_vn = vec_lane_bt1(lane);
   const size_t tok0 = token_offset(p, unit, 0, D), tstride = token_stride(p, D);
@@ -174,7 +166,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     // together has to stay inside the SM's instruction cache.)
     const int pw = warp - NW - 1, sub = lane / LPT, pl = lane % LPT;
     const TIn* src0 = static_cast<const TIn*>(p.k) + tok0 + 4 * pl;
-    const bool two = UT || rank == 1;
+    const bool two = UT || rank == 1, sums = STASH || rank == 1;   // sums: this side carries the key sum
     const TIn* src1 = two ? static_cast<const TIn*>(rank ? p.q : p.u) + tok0 + 4 * pl : src0;
     float* fs = reinterpret_cast<float*>(smem + (rank ? Cfg::s_f : Cfg::a_f));
     const uint32_t base0 = sb + (rank ? Cfg::s_K : Cfg::a_K), base1 = sb + (rank ? Cfg::s_Q : Cfg::a_U);
@@ -193,7 +185,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
     float zk[4] = {0.f, 0.f, 0.f, 0.f};
-    if (rank == 1 && p.z0) {
+    if (sums && p.z0) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) zk[e] = p.z0[size_t(unit) * D + 4 * pl + e];
     }
@@ -202,10 +194,8 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     for (int c = 0; c < nch; ++c) {
       const int slot = c % RK;
       fetch(c + 1);   // (past the end: zeros)
-      if (STASH && rank == 1 && c % sh.ck == 0 && pw == 0 && sub == 0) {
-        const size_t nblk = (nch + sh.ck - 1) / sh.ck;
-        *reinterpret_cast<float4*>(sh.zck + (size_t(unit) * nblk + c / sh.ck) * D + 4 * pl) = make_float4(zk[0], zk[1], zk[2], zk[3]);
-      }
+      if (STASH && pw == 0 && sub == 0)
+        *reinterpret_cast<float4*>(sh.zkc + (size_t(unit) * nch + c) * D + 4 * pl) = make_float4(zk[0], zk[1], zk[2], zk[3]);
       if (c >= RK) wait(&kfree[slot], (c / RK - 1) & 1);
       asm volatile("cp.async.wait_group 1;" ::: "memory");
       float ks[4] = {0.f, 0.f, 0.f, 0.f};
@@ -246,13 +236,13 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           fs[Cfg::sf_dq + slot * 16 + tt] = dn;
         }
       }
-      if (rank == 1 && !ident) {   // the key sum after this chunk
+      if (sums && !ident) {   // the key sum after this chunk
 #pragma unroll
         for (int off = LPT; off < 32; off <<= 1)
 #pragma unroll
           for (int e = 0; e < 4; ++e) ks[e] += __shfl_xor_sync(0xffffffffu, ks[e], off);
         if constexpr (NPREP > 1) {
-          float* zp = fs + Cfg::sf_zp + (c & 1) * NPREP * D;
+          float* zp = fs + (STASH ? Cfg::af_zp : Cfg::sf_zp) + (c & 1) * NPREP * D;
           if (sub == 0) *reinterpret_cast<float4*>(zp + pw * D + 4 * pl) = make_float4(ks[0], ks[1], ks[2], ks[3]);
           named_sync(2, NPREP * 32);
           ks[0] = ks[1] = ks[2] = ks[3] = 0.f;
@@ -267,7 +257,8 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       }
       arrive(&kfull[slot]);
     }
-    if (rank == 1 && p.zT && pw == 0 && sub == 0)
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (sums && p.zT && pw == 0 && sub == 0)
       *reinterpret_cast<float4*>(p.zT + size_t(unit) * D + 4 * pl) = make_float4(zk[0], zk[1], zk[2], zk[3]);
   } else if (rank == 0 && warp == NW) {
     // ===================================================================== rank 0: elimination
@@ -413,7 +404,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     float* mxs = fs + Cfg::af_mx;
     const int row0 = 16 * warp;
     const uint32_t my_rows = uint32_t(row0 + g) * kVecRow + 4 * c4;
-    const uint32_t remote_A = map_to_rank(sb + Cfg::s_A, 1);
+    const uint32_t remote_A = STASH ? 0u : map_to_rank(sb + Cfg::s_A, 1);
     float st[NTILE][4];
     float sA, sAi;                   // st = sA * A
     {
@@ -474,14 +465,16 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
             al[nt][2 + e] *= kUnit;
           }
         if (bad && (p.flags & VLA_FLAG_CHECK_FINITE) && p.status) atomicCAS(p.status, 0, int(VLA_ERR_NONFINITE));
-        if (c2 >= RA) wait(&aempty[as], (c2 / RA - 1) & 1);   // (the staged rows have been copied too, then)
-        const uint32_t stage = sb + Cfg::a_A + as * Cfg::aslot;
-        vec_store(stage + my_rows, al);
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0 && !*abort_flag)
-          bulk_to_cluster(remote_A + as * Cfg::aslot + row0 * kVecRow, stage + row0 * kVecRow, 16 * kVecRow,
-                          map_to_rank(smem_u32(&afull[as]), 1));
+        if constexpr (!STASH) {
+          if (c2 >= RA) wait(&aempty[as], (c2 / RA - 1) & 1);   // (the staged rows have been copied too, then)
+          const uint32_t stage = sb + Cfg::a_A + as * Cfg::aslot;
+          vec_store(stage + my_rows, al);
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0 && !*abort_flag)
+            bulk_to_cluster(remote_A + as * Cfg::aslot + row0 * kVecRow, stage + row0 * kVecRow, 16 * kVecRow,
+                            map_to_rank(smem_u32(&afull[as]), 1));
+        }
       }
       if (c1 < nch && c1 >= 0) {
         if constexpr (UT) {
@@ -514,6 +507,15 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         for (int e = 0; e < 4; ++e) a2[nt][e] = a1[nt][e];
     };
     float sz1 = 0.f;
+    // scale of z / delta in the update of A: 2^10 / sqrt(sA), rounded to a power of two
+    float sy, sAy;
+    auto set_sy = [&]() {
+      const int e = 127 - int(__float_as_uint(sA) >> 23);   // sA = 2^-e
+      const int k = 10 + (e >> 1);
+      sy = __uint_as_float(uint32_t(127 + k) << 23);
+      sAy = sAi * pow2_inverse(sy);
+    };
+    set_sy();
     if (nch > 0) wait(&kfull[0], 0);
 #pragma unroll 1
     for (int c = 0; c < nch + 2; ++c) {   // (the last two rounds only pass on the last two chunks' alpha)
@@ -521,14 +523,18 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       const int slot = c % RK;
       const uint32_t Kop = sb + Cfg::a_K + slot * Cfg::kslot, Uop = UT ? sb + Cfg::a_U + slot * Cfg::kslot : Kop;
       if (STASH && live && c % sh.ck == 0) {
-        const size_t nblk = (nch + sh.ck - 1) / sh.ck;
-        float* dst = sh.Ack + (size_t(unit) * nblk + c / sh.ck) * D * D;
+        const size_t blk = size_t(unit) * ((nch + sh.ck - 1) / sh.ck) + c / sh.ck;
+        unsigned char* dst = sh.Aimg + blk * (D * kTokRow<D>) + size_t(row0 + g) * kTokRow<D> + 4 * c4;
 #pragma unroll
         for (int nt = 0; nt < NTILE; ++nt)
 #pragma unroll
-          for (int hf = 0; hf < 2; ++hf)
-            *reinterpret_cast<float2*>(dst + size_t(row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
-                make_float2(st[nt][2 * hf] * sAi, st[nt][2 * hf + 1] * sAi);
+          for (int hf = 0; hf < 2; ++hf) {
+            uint32_t hi, lo;
+            split_f16(st[nt][2 * hf], st[nt][2 * hf + 1], hi, lo);
+            *reinterpret_cast<uint32_t*>(dst + hf * 8 * kTokRow<D> + 16 * nt) = hi;
+            *reinterpret_cast<uint32_t*>(dst + hf * 8 * kTokRow<D> + 16 * nt + 2 * D) = lo;
+          }
+        if (tid == 0) sh.Asc[blk] = sAi;
       }
       // ---- Z0^T = A U^T (rows: this warp's state rows, columns: tokens), with an explicit u also A K^T
       float z0[2][4] = {}, w0[2][4] = {};
@@ -596,8 +602,10 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         continue;
       }
       if (c + 1 < nch) wait(&kfull[(c + 1) % RK], ((c + 1) / RK) & 1);
-      const bool look = (c & 7) == 7;
-      if (look) {   // A shrinks as tokens come: keep its operands inside fp16's range
+      // A shrinks as tokens come, by up to 1 / lambda within the first d of them, by 1 / t later: its operands are
+      // kept near the top of fp16's range, or the remainders would run into its subnormals
+      const bool look = (c & 7) == 7 || c < D / 4;
+      if (look) {
         float mx = 0.f;
 #pragma unroll
         for (int nt = 0; nt < NTILE; ++nt)
@@ -628,6 +636,12 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
             }
           }
         sz1 = sAi;
+        // z / delta may lie far below z: scaled up on its own, or its remainders would be fp16 subnormals
+        // (|z / delta| <= sqrt(max A) / 2 whatever u is, so sy * y stays below 2^14)
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) y[nt][e] *= sy;
         split_frag(y[0], y[1], yh, yl);
       }
       named_sync(1, NW * 32);
@@ -647,13 +661,13 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
 #pragma unroll
         for (int i = 0; i < NB; ++i)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) st[nt + i][e] = fmaf(x[i][e], sAi, st[nt + i][e]);
+          for (int e = 0; e < 4; ++e) st[nt + i][e] = fmaf(x[i][e], sAy, st[nt + i][e]);
       }
       if (look) {
         float mx = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) mx = fmaxf(mx, mxs[w]);
-        if (mx < 8.0f) {
+        if (mx < 32.0f) {
           const float f = pow2_scale(mx, 7);
 #pragma unroll
           for (int nt = 0; nt < NTILE; ++nt)
@@ -661,12 +675,13 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
             for (int e = 0; e < 4; ++e) st[nt][e] *= f;
           sA *= f;
           sAi = pow2_inverse(sA);
+          set_sy();
         }
       }
     }
     // rank 1's arrivals on this CTA's barriers must have landed before the CTA may leave (the cluster
     // barrier at the end does not order them): wait for the last use of every slot
-    for (int c = nch > RA ? nch - RA : 0; c < nch; ++c) wait(&aempty[c % RA], (c / RA) & 1);
+    for (int c = STASH ? nch : nch > RA ? nch - RA : 0; c < nch; ++c) wait(&aempty[c % RA], (c / RA) & 1);
     if (p.A_T) {
 #pragma unroll
       for (int nt = 0; nt < NTILE; ++nt)
@@ -675,6 +690,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           *reinterpret_cast<float2*>(p.A_T + (size_t(unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
               make_float2(st[nt][2 * hf] * sAi, st[nt][2 * hf + 1] * sAi);
     }
+  } else if constexpr (STASH) {
   } else if (warp == NW) {
     // ===================================================================== rank 1: small matrices
     // N = K alpha^T, H = Q alpha^T, Q K^T; Tm = (I + stril(N))^-1; output scales 1 / (den_t * scale of q_t)
@@ -763,57 +779,10 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         if (c4 == 0) {
           const float id = ident ? 1.0f : rcp_ftz_nr(fmaxf(den[hf], eps));
           osc[t] = id * qsi[hf];
-          if (STASH && c * C + t < T) sh.iden[size_t(unit) * T + c * C + t] = id;
         }
       }
       __syncwarp();
-      // Tm = (I + stril(N))^-1 by 8 x 8 blocks: the two on the diagonal by forward substitution (lane j + 8 b:
-      // column j of block b; the upper lanes repeat it), then -T22 N21 T11
-      {
-        const int j = lane & 7, b8 = lane & 8;
-        const float* Nd = Nb + b8 * LD + b8;
-        float x[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          float a0 = t == j ? 1.0f : 0.0f, a1 = 0.f;
-#pragma unroll
-          for (int s4 = 0; 4 * s4 < t; ++s4) {
-            const float4 y = *reinterpret_cast<const float4*>(Nd + t * LD + 4 * s4);
-            a0 = fmaf(-y.x, x[4 * s4], a0);
-            if (4 * s4 + 1 < t) a1 = fmaf(-y.y, x[4 * s4 + 1], a1);
-            if (4 * s4 + 2 < t) a0 = fmaf(-y.z, x[4 * s4 + 2], a0);
-            if (4 * s4 + 3 < t) a1 = fmaf(-y.w, x[4 * s4 + 3], a1);
-          }
-          x[t] = a0 + a1;
-        }
-        if (lane < 16) {
-#pragma unroll
-          for (int t = 0; t < 8; ++t) Tm[(b8 + t) * LD + b8 + j] = x[t];
-          // (the consumers skip the upper right block)
-        }
-        __syncwarp();
-        // lane: row r of the block, columns 2 c4, 2 c4 + 1
-        float2 y = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float nk = Nb[(8 + g) * LD + k];
-          const float2 tk = *reinterpret_cast<const float2*>(Tm + k * LD + 2 * c4);
-          y.x = fmaf(nk, tk.x, y.x);
-          y.y = fmaf(nk, tk.y, y.y);
-        }
-        float2* Y = reinterpret_cast<float2*>(Nb + 8) ;   // (the block of N above the diagonal is free)
-        Y[(g * LD + 2 * c4) / 2] = y;
-        __syncwarp();
-        float2 z = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float tk = Tm[(8 + g) * LD + 8 + k];
-          const float2 yk = Y[(k * LD + 2 * c4) / 2];
-          z.x = fmaf(-tk, yk.x, z.x);
-          z.y = fmaf(-tk, yk.y, z.y);
-        }
-        *reinterpret_cast<float2*>(Tm + (8 + g) * LD + 2 * c4) = z;
-      }
+      unit_lower_inverse16<LD>(Tm, Nb, lane);
       arrive(&gfull[gs]);
     }
   } else {
@@ -861,7 +830,6 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     const size_t my0 = tok0 + size_t(2 * c4) * tstride + row0 + g;
     const TIn* vsrc = static_cast<const TIn*>(p.v) + my0;
     float* odst = p.out + my0;
-    float* edst = STASH ? sh.e + (size_t(unit) * T + 2 * c4) * D + row0 + g : nullptr;
     float vn[8];
     auto fetch_v = [&](int c) {   // v^T in accumulator order: [token tile][row half * 2 + token]
 #pragma unroll
@@ -880,16 +848,6 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       const uint32_t Kop = sb + Cfg::s_K + slot * Cfg::kslot, Qop = sb + Cfg::s_Q + slot * Cfg::kslot;
       const uint32_t Aop = sb + Cfg::s_A + as * Cfg::aslot;
       if (look) rescale(true_max());
-      if (STASH && c % sh.ck == 0) {
-        const size_t nblk = (nch + sh.ck - 1) / sh.ck;
-        float* dst = sh.Sck + (size_t(unit) * nblk + c / sh.ck) * D * D;
-#pragma unroll
-        for (int nt = 0; nt < NTILE; ++nt)
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf)
-            *reinterpret_cast<float2*>(dst + size_t(row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
-                make_float2(st[nt][2 * hf] * sSi, st[nt][2 * hf + 1] * sSi);
-      }
       wait(&kfull[slot], (c / RK) & 1);
       // ---- P = S K^T and R = S Q^T (rows: this warp's, columns: tokens)
       float pk[2][4] = {}, rq[2][4] = {};
@@ -924,18 +882,11 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           const float f = osc[8 * nt + 2 * c4 + e] * sSi;
           if (c * C + 2 * c4 + e + 8 * nt < T) {
             float* q = odst + (e ? tstride : 0) + (nt ? 8 * tstride : 0);
-            if (!STASH || p.out) {
-              q[0] = rq[nt][e] * f;
-              q[8] = rq[nt][2 + e] * f;
-            }
-            if (STASH) {
-              edst[(8 * nt + e) * D] = ev[nt][e] * sSi;
-              edst[(8 * nt + e) * D + 8] = ev[nt][2 + e] * sSi;
-            }
+            q[0] = rq[nt][e] * f;
+            q[8] = rq[nt][2 + e] * f;
           }
         }
         odst += 16 * tstride;
-        if (STASH) edst += 16 * D;
       }
       arrive(&gfree[gs]);
       // ---- S <- S + E^T alpha
@@ -987,7 +938,14 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
   }
   __syncthreads();
   if (tid == 0 && *abort_flag && p.status) atomicCAS(p.status, 0, int(VLA_ERR_DEVICE_TIMEOUT));
-  cluster_sync();   // neither CTA leaves while the other may still write to its shared memory
+  if (!STASH) {
+    // Neither CTA leaves while the other may still write to its shared memory.  In a run without a
+    // timeout every such write has been waited for; after one, the copies issued before the first barrier get
+    // time to land.
+    cluster_sync();
+    if (*abort_flag) settle_copies();
+    cluster_sync();
+  }
 }
 
 }  // namespace vla

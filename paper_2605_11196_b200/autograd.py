@@ -1,5 +1,7 @@
 """``torch.autograd`` face of the scan: ``vla_scan`` runs ``vla_forward`` and, under autograd,
-``vla_backward``.  Marshalling only; every step of both passes runs in the CUDA library.
+``vla_backward``.  Marshalling only; every step of both passes runs in the CUDA library.  (The ordinary
+call is a native autograd node, csrc_torch/vla_torch.cpp; the class below takes the refresh and what the
+native one leaves to it.)
 
 Differentiable inputs: ``q, k, v``, explicit penalty directions ``u`` (so a learned
 ``u = L2norm(W_u k) / sqrt(d)`` built with torch ops, or with ``vla_make_u`` outside autograd,
@@ -69,4 +71,10 @@ def vla_scan(q, k, v, lam: float, *, u: Optional[torch.Tensor] = None, S0=None, 
     """``(out, S_T, A_T, z_T)`` of the VLA forward scan for CUDA tensors, differentiable with
     respect to ``q, k, v, u, S0, A0, z0``.  Device-side problems of either pass land in a status
     word that ``check_status()`` reads (the calls themselves never synchronise)."""
+    if refresh is None and q.is_cuda:
+        r = _b.native().scan(q, k, v, lam, u, S0, A0, z0, flags, eps, _status_word(q.device))
+        if r.__class__ is tuple:
+            return r
+        if r is not None:
+            raise _b.VlaError(r, "vla_forward")
     return _VlaScan.apply(q, k, v, u, S0, A0, z0, float(lam), int(flags), float(eps), refresh)

@@ -7,6 +7,7 @@ PyTorch is used for device memory and streams only.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 import threading
 from dataclasses import dataclass
@@ -106,6 +107,25 @@ def load_library():
             lib.vla_last_launch.argtypes = [ctypes.c_char_p, ctypes.c_size_t]
             _lib = lib
     return _lib
+
+
+_ext = None
+
+
+def native():
+    """The native marshalling module (built with the library; there is no fallback for a missing build)."""
+    global _ext
+    if _ext is None:
+        load_library()
+        with _lock:
+            if _ext is None:
+                if not os.path.exists(_build.EXT):
+                    raise RuntimeError("%s is missing: run paper_2605_11196_b200.build.build()" % _build.EXT)
+                spec = importlib.util.spec_from_file_location("_vla_torch", _build.EXT)
+                mod = importlib.util.module_from_spec(spec)
+                spec.loader.exec_module(mod)
+                _ext = mod
+    return _ext
 
 
 def last_launch() -> str:
@@ -229,6 +249,14 @@ def vla_forward(q, k, v, lam: float, *, u=None, S0=None, A0=None, z0=None, flags
     units into concurrently scanned segments (``opts->workspace``); ``True`` allocates what the
     library asks for with torch, ``None`` / ``False`` passes none.
     """
+    if stream is None and refresh is None:
+        # well-formed calls are marshalled natively; anything else comes back as None and is told apart below
+        r = (_ext or native()).forward(q, k, v, lam, u, S0, A0, z0, flags, eps, out, S_T, A_T, z_T, status, want_status, kernel,
+                                       workspace, wait_probe_limit)
+        if r.__class__ is tuple:
+            return VlaResult(*r)
+        if r is not None:
+            raise VlaError(r, "vla_forward")
     lib = load_library()
     if q.dim() != 4:
         raise ValueError("q must be [B,H,T,d_k]")

@@ -1,21 +1,26 @@
-"""Builds the C-ABI CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU).
+"""Builds the C-ABI CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the
+native torch marshalling on top of it.
 
 Every csrc/*.cu is compiled to an object file under _build/ (in parallel, only when stale) and
-the objects are linked into libvla.so next to this file.
+the objects are linked into libvla.so next to this file; csrc_torch/vla_torch.cpp becomes _vla_torch.so.
 """
 from __future__ import annotations
 
 import concurrent.futures
 import glob
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libvla.so")
+EXT_SRC = os.path.join(PKG, "csrc_torch", "vla_torch.cpp")
+EXT = os.path.join(PKG, "_vla_torch.so")
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -51,9 +56,26 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in sources() + _headers())
 
 
+def _build_ext(force: bool) -> None:
+    """The marshalling module: links against libvla.so beside it and the torch this interpreter has."""
+    deps = [EXT_SRC, os.path.join(ROOT, "include", "vla.h"), os.path.abspath(__file__)]
+    if not force and os.path.exists(EXT) and all(os.path.getmtime(d) <= os.path.getmtime(EXT) for d in deps):
+        return
+    t = os.path.dirname(importlib.util.find_spec("torch").origin)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    tmp = EXT + ".tmp.%d" % os.getpid()
+    inc = [os.path.join(ROOT, "include"), t + "/include", t + "/include/torch/csrc/api/include",
+           sysconfig.get_paths()["include"], cuda + "/include"]
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-w", "-o", tmp, EXT_SRC] + ["-I" + i for i in inc] +
+                          ["-L" + PKG, "-l:libvla.so", "-L" + t + "/lib", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda",
+                           "-ltorch", "-ltorch_python", "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, EXT)
+
+
 def build(force: bool = False, verbose: bool = False, jobs: int = 0) -> str:
-    """Compile csrc/*.cu and link libvla.so next to this file; returns its path."""
+    """Compile csrc/*.cu, link libvla.so and _vla_torch.so next to this file; returns the library's path."""
     if not force and not _stale():
+        _build_ext(False)
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     os.makedirs(OBJ, exist_ok=True)
@@ -78,6 +100,7 @@ def build(force: bool = False, verbose: bool = False, jobs: int = 0) -> str:
     subprocess.check_call([nvcc, "-shared", "-Xcompiler", "-fPIC", "-gencode",
                            "arch=compute_100a,code=sm_100a", "-o", tmp] + [_obj(s) for s in sources()])
     os.replace(tmp, LIB)
+    _build_ext(force)
     return LIB
 
 

@@ -1,0 +1,318 @@
+// Native marshalling of the hot Python calls (binding.py, autograd.py): argument checks, output
+// allocation and the C-ABI call for vla_forward, and the scan as a torch autograd function.  A single
+// decode step spent 31 us on the host in Python (the library's own part is 3 us) with 10 us of GPU work
+// behind it.
+//
+// Every entry returns None for anything but well-formed CUDA arguments on the ordinary path; the caller
+// then takes the Python path, which raises the proper errors.  A library status other than VLA_OK comes back as
+// an int.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <ATen/ATen.h>
+#include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDAGuard.h>
+#include <c10/cuda/CUDAGraphsC10Utils.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/custom_function.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <map>
+#include <mutex>
+#include <optional>
+
+#include "vla.h"
+
+namespace {
+
+using at::Tensor;
+using OptTensor = std::optional<Tensor>;
+constexpr auto kF32 = at::kFloat;
+
+// Status words, zeroed a block at a time on the stream that uses them (a fill kernel per call costs more
+// than the rest of a small call).  A word is handed out once; a block lives as long as any of its words; at
+// most 64 (device, stream) pairs keep a block in use here.  During a graph capture every call gets a word
+// that the graph itself zeroes.
+class StatusPool {
+ public:
+  Tensor take(const c10::cuda::CUDAStream& st) {
+    const auto opt = at::TensorOptions().dtype(at::kInt).device(at::kCUDA, st.device_index());
+    if (c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None) return at::zeros({}, opt);
+    std::lock_guard<std::mutex> lock(m_);
+    const auto key = std::make_pair(int(st.device_index()), st.stream());
+    auto it = blocks_.find(key);
+    if (it == blocks_.end()) {
+      if (blocks_.size() >= 64) blocks_.clear();
+      it = blocks_.emplace(key, Block{}).first;
+    }
+    Block& b = it->second;
+    if (!b.words.defined() || b.next == kWords) {
+      b.words = at::zeros({kWords}, opt);
+      b.next = 0;
+    }
+    return b.words.select(0, b.next++);
+  }
+
+ private:
+  static constexpr int64_t kWords = 512;
+  struct Block {
+    Tensor words;
+    int64_t next = 0;
+  };
+  std::mutex m_;
+  std::map<std::pair<int, cudaStream_t>, Block> blocks_;
+};
+StatusPool& status_pool() {
+  static auto* p = new StatusPool;   // never destroyed: tensors must not outlive the CUDA context's end
+  return *p;
+}
+
+struct Shape {
+  int64_t B, H, T, d;
+  bool token_major;
+  std::array<int64_t, 4> seq() const {
+    return token_major ? std::array<int64_t, 4>{B, T, H, d} : std::array<int64_t, 4>{B, H, T, d};
+  }
+  std::array<int64_t, 4> state() const { return {B, H, d, d}; }
+  std::array<int64_t, 3> vec() const { return {B, H, d}; }
+};
+
+bool is(const Tensor& t, at::IntArrayRef sizes, at::ScalarType dt, const at::Device& dev) {
+  return t.scalar_type() == dt && t.device() == dev && t.sizes() == sizes && t.is_contiguous();
+}
+bool is_or_none(const Tensor& t, at::IntArrayRef sizes, at::ScalarType dt, const at::Device& dev) {
+  return !t.defined() || is(t, sizes, dt, dev);
+}
+Tensor empty(at::IntArrayRef sizes, const at::Device& dev, at::ScalarType dt = kF32) {
+  return Tensor(at::detail::empty_cuda(sizes, dt, dev, std::nullopt));
+}
+float* f32(const Tensor& t) { return t.defined() ? static_cast<float*>(t.data_ptr()) : nullptr; }
+const void* raw(const Tensor& t) { return t.defined() ? t.data_ptr() : nullptr; }
+
+// q's layout and the checks common to both directions
+bool describe(const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& u, int64_t flags, Shape* s) {
+  if (!q.is_cuda() || q.dim() != 4 || !(q.scalar_type() == kF32 || q.scalar_type() == at::kBFloat16)) return false;
+  s->token_major = (flags & VLA_FLAG_TOKEN_MAJOR) != 0;
+  s->B = q.size(0);
+  s->H = q.size(s->token_major ? 2 : 1);
+  s->T = q.size(s->token_major ? 1 : 2);
+  s->d = q.size(3);
+  const auto seq = s->seq();
+  const auto dt = q.scalar_type();
+  const auto dev = q.device();
+  return is(q, seq, dt, dev) && is(k, seq, dt, dev) && is(v, seq, dt, dev) && is_or_none(u, seq, dt, dev);
+}
+vla_opts_t options(const Tensor& q, const Tensor& u, int64_t flags, double eps, const Tensor& z0, const Tensor& zT,
+                   const Tensor& status, int64_t kernel) {
+  vla_opts_t o = {};
+  o.struct_size = sizeof(o);
+  o.qkv_dtype = q.scalar_type() == kF32 ? VLA_F32 : VLA_BF16;
+  o.u = raw(u);
+  o.flags = uint32_t(flags);
+  o.eps = float(eps);
+  o.z0 = f32(z0);
+  o.zT = f32(zT);
+  o.status = status.defined() ? static_cast<int32_t*>(status.data_ptr()) : nullptr;
+  o.kernel = int32_t(kernel);
+  return o;
+}
+
+// ---------------------------------------------------------------- Python helpers
+bool tensor_arg(PyObject* o, Tensor* t) {
+  if (o == Py_None) return true;
+  if (!THPVariable_Check(o)) return false;
+  *t = THPVariable_Unpack(o);
+  return true;
+}
+bool int_arg(PyObject* o, int64_t* x) {
+  if (!PyLong_Check(o)) return false;
+  int overflow = 0;
+  *x = PyLong_AsLongLongAndOverflow(o, &overflow);
+  return overflow == 0;
+}
+bool real_arg(PyObject* o, double* x) {
+  if (PyFloat_Check(o)) { *x = PyFloat_AS_DOUBLE(o); return true; }
+  if (PyLong_Check(o)) {
+    *x = PyLong_AsDouble(o);
+    if (!PyErr_Occurred()) return true;
+    PyErr_Clear();
+  }
+  return false;
+}
+PyObject* wrap(const Tensor& t) {
+  if (!t.defined()) Py_RETURN_NONE;
+  return THPVariable_Wrap(t);
+}
+
+// forward(q, k, v, lam, u, S0, A0, z0, flags, eps, out, S_T, A_T, z_T, status, want_status, kernel, workspace, probes)
+// -> (out, S_T, A_T, z_T, status) | None | status code
+PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  Tensor q, k, v, u, S0, A0, z0, out, S_T, A_T, z_T, status, ws;
+  double lam = 0, eps = 0;
+  int64_t flags = 0, kernel = 0, probes = 0;
+  if (n != 19 || !tensor_arg(a[0], &q) || !tensor_arg(a[1], &k) || !tensor_arg(a[2], &v) || !real_arg(a[3], &lam) ||
+      !tensor_arg(a[4], &u) || !tensor_arg(a[5], &S0) || !tensor_arg(a[6], &A0) || !tensor_arg(a[7], &z0) ||
+      !int_arg(a[8], &flags) || !real_arg(a[9], &eps) || !tensor_arg(a[10], &out) || !tensor_arg(a[11], &S_T) ||
+      !tensor_arg(a[12], &A_T) || !tensor_arg(a[13], &z_T) || !tensor_arg(a[14], &status) || !int_arg(a[16], &kernel) ||
+      !int_arg(a[18], &probes))
+    Py_RETURN_NONE;
+  const bool want_status = a[15] == Py_True;
+  const bool auto_ws = a[17] == Py_True;
+  if (!auto_ws && a[17] != Py_None && a[17] != Py_False && !(tensor_arg(a[17], &ws) && ws.is_cuda())) Py_RETURN_NONE;
+  Shape s;
+  if (!q.defined() || !k.defined() || !v.defined() || flags < 0 || flags > 0xffffffffLL || probes < 0 || probes > 0xffffffffLL ||
+      !describe(q, k, v, u, flags, &s))
+    Py_RETURN_NONE;
+  const auto dev = q.device();
+  const auto seq = s.seq(), st4 = s.state();
+  const auto vec = s.vec();
+  if (!is_or_none(S0, st4, kF32, dev) || !is_or_none(A0, st4, kF32, dev) || !is_or_none(z0, vec, kF32, dev) ||
+      !is_or_none(out, seq, kF32, dev) || !is_or_none(S_T, st4, kF32, dev) || !is_or_none(A_T, st4, kF32, dev) ||
+      !is_or_none(z_T, vec, kF32, dev) || (status.defined() && !(status.is_cuda() && status.scalar_type() == at::kInt)))
+    Py_RETURN_NONE;
+  try {
+    at::AutoDispatchBelowADInplaceOrView guard;
+    c10::cuda::OptionalCUDAGuard on;
+    if (c10::cuda::current_device() != dev.index()) on.set_device(dev);
+    const auto stream = c10::cuda::getCurrentCUDAStream(dev.index());
+    if (!out.defined()) out = empty(seq, dev);
+    if (!S_T.defined()) S_T = empty(st4, dev);
+    if (!A_T.defined()) A_T = empty(st4, dev);
+    if (!z_T.defined()) z_T = empty(vec, dev);
+    if (!status.defined() && want_status) status = status_pool().take(stream);
+    vla_opts_t o = options(q, u, flags, eps, z0, z_T, status, kernel);
+    o.wait_probe_limit = uint32_t(probes);
+    if (auto_ws && kernel == VLA_KERNEL_AUTO) {
+      const int P = vla_seqpar_segments(int(s.B), int(s.H), int(s.T), int(s.d), o.qkv_dtype);
+      if (P > 1) ws = empty({int64_t(vla_seqpar_workspace_bytes(int(s.B), int(s.H), int(s.T), int(s.d), P))}, dev, at::kByte);
+    }
+    if (ws.defined()) {
+      o.workspace = ws.data_ptr();
+      o.workspace_bytes = size_t(ws.numel());
+    }
+    const int rc = vla_forward(raw(q), raw(k), raw(v), float(lam), int(s.B), int(s.H), int(s.T), int(s.d), int(s.d), f32(S0),
+                               f32(A0), f32(out), f32(S_T), f32(A_T), &o, stream.stream());
+    if (rc != VLA_OK) return PyLong_FromLong(rc);
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+  PyObject* r = PyTuple_New(5);
+  if (!r) return nullptr;
+  PyTuple_SET_ITEM(r, 0, wrap(out));
+  PyTuple_SET_ITEM(r, 1, wrap(S_T));
+  PyTuple_SET_ITEM(r, 2, wrap(A_T));
+  PyTuple_SET_ITEM(r, 3, wrap(z_T));
+  PyTuple_SET_ITEM(r, 4, wrap(status));
+  return r;
+}
+
+// ---------------------------------------------------------------- the scan under autograd
+struct Failed {
+  int code;
+};
+
+struct Scan : public torch::autograd::Function<Scan> {
+  static torch::autograd::variable_list forward(torch::autograd::AutogradContext* ctx, const Tensor& q, const Tensor& k,
+                                                const Tensor& v, const OptTensor& u_, const OptTensor& S0_, const OptTensor& A0_,
+                                                const OptTensor& z0_, const Tensor& status, double lam, int64_t flags, double eps) {
+    const Tensor u = u_.value_or(Tensor()), S0 = S0_.value_or(Tensor()), A0 = A0_.value_or(Tensor()), z0 = z0_.value_or(Tensor());
+    Shape s;
+    describe(q, k, v, u, flags, &s);   // (checked by the caller)
+    const auto dev = q.device();
+    c10::cuda::OptionalCUDAGuard on;
+    if (c10::cuda::current_device() != dev.index()) on.set_device(dev);
+    Tensor out = empty(s.seq(), dev), S_T = empty(s.state(), dev), A_T = empty(s.state(), dev), z_T = empty(s.vec(), dev);
+    const vla_opts_t o = options(q, u, flags, eps, z0, z_T, status, VLA_KERNEL_AUTO);
+    const int rc = vla_forward(raw(q), raw(k), raw(v), float(lam), int(s.B), int(s.H), int(s.T), int(s.d), int(s.d), f32(S0),
+                               f32(A0), f32(out), f32(S_T), f32(A_T), &o, c10::cuda::getCurrentCUDAStream(dev.index()).stream());
+    if (rc != VLA_OK) throw Failed{rc};
+    ctx->save_for_backward({q, k, v, u, S0, A0, z0});
+    ctx->saved_data["status"] = status;   // (not a saved variable: check_status() clears the word in between)
+    ctx->saved_data["lam"] = lam;
+    ctx->saved_data["flags"] = flags;
+    ctx->saved_data["eps"] = eps;
+    ctx->saved_data["need"] = int64_t(q.requires_grad()) | int64_t(k.requires_grad()) << 1 | int64_t(v.requires_grad()) << 2 |
+                              int64_t(u.defined() && u.requires_grad()) << 3 | int64_t(S0.defined() && S0.requires_grad()) << 4 |
+                              int64_t(A0.defined() && A0.requires_grad()) << 5 | int64_t(z0.defined() && z0.requires_grad()) << 6;
+    ctx->set_materialize_grads(false);
+    return {out, S_T, A_T, z_T};
+  }
+
+  static torch::autograd::variable_list backward(torch::autograd::AutogradContext* ctx, torch::autograd::variable_list g) {
+    const auto saved = ctx->get_saved_variables();
+    const Tensor &q = saved[0], &k = saved[1], &v = saved[2], &u = saved[3], &S0 = saved[4], &A0 = saved[5], &z0 = saved[6];
+    const Tensor status = ctx->saved_data["status"].toTensor();
+    const double lam = ctx->saved_data["lam"].toDouble(), eps = ctx->saved_data["eps"].toDouble();
+    const int64_t flags = ctx->saved_data["flags"].toInt(), need = ctx->saved_data["need"].toInt();
+    at::AutoDispatchBelowADInplaceOrView guard;
+    Shape s;
+    describe(q, k, v, u, flags, &s);
+    const auto dev = q.device();
+    const auto seq = s.seq();
+    c10::cuda::OptionalCUDAGuard on;
+    if (c10::cuda::current_device() != dev.index()) on.set_device(dev);
+    auto plain = [](const Tensor& x) { return x.defined() ? x.to(kF32).contiguous() : x; };
+    Tensor d_out = g[0].defined() ? plain(g[0]) : at::zeros(seq, q.options().dtype(kF32));
+    const Tensor dS_T = plain(g[1]), dA_T = plain(g[2]), dz_T = plain(g[3]);
+    Tensor dq = empty(seq, dev), dk = empty(seq, dev), dv = empty(seq, dev), du, dS0, dA0, dz0;
+    if (u.defined()) du = empty(seq, dev);
+    if (need >> 4 & 1) dS0 = empty(s.state(), dev);
+    if (need >> 5 & 1) dA0 = empty(s.state(), dev);
+    if (need >> 6 & 1) dz0 = empty(s.vec(), dev);
+    const size_t bytes = vla_backward_workspace_bytes(int(s.B), int(s.H), int(s.T), int(s.d));
+    const Tensor ws = empty({int64_t(bytes)}, dev, at::kByte);
+    vla_opts_t o = options(q, u, flags, eps, z0, Tensor(), status, VLA_KERNEL_AUTO);
+    o.du = f32(du);
+    const int rc = vla_backward(raw(q), raw(k), raw(v), float(lam), int(s.B), int(s.H), int(s.T), int(s.d), int(s.d), f32(S0),
+                                f32(A0), f32(d_out), f32(dS_T), f32(dA_T), f32(dz_T), f32(dq), f32(dk), f32(dv), f32(dS0),
+                                f32(dA0), f32(dz0), &o, ws.data_ptr(), bytes,
+                                c10::cuda::getCurrentCUDAStream(dev.index()).stream());
+    TORCH_CHECK(rc == VLA_OK, "vla_backward: ", vla_status_string(rc), " (", rc, ")");
+    auto give = [&](int bit, const Tensor& x) { return need >> bit & 1 ? (x.scalar_type() == q.scalar_type() ? x : x.to(q.scalar_type())) : Tensor(); };
+    return {give(0, dq), give(1, dk), give(2, dv), give(3, du), dS0, dA0, dz0, Tensor(), Tensor(), Tensor(), Tensor()};
+  }
+};
+
+// scan(q, k, v, lam, u, S0, A0, z0, flags, eps, status) -> (out, S_T, A_T, z_T) | None | status code
+PyObject* scan(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  Tensor q, k, v, u, S0, A0, z0, status;
+  double lam = 0, eps = 0;
+  int64_t flags = 0;
+  if (n != 11 || !tensor_arg(a[0], &q) || !tensor_arg(a[1], &k) || !tensor_arg(a[2], &v) || !real_arg(a[3], &lam) ||
+      !tensor_arg(a[4], &u) || !tensor_arg(a[5], &S0) || !tensor_arg(a[6], &A0) || !tensor_arg(a[7], &z0) ||
+      !int_arg(a[8], &flags) || !real_arg(a[9], &eps) || !tensor_arg(a[10], &status))
+    Py_RETURN_NONE;
+  Shape s;
+  if (!q.defined() || !k.defined() || !v.defined() || flags < 0 || flags > 0xffffffffLL || !describe(q, k, v, u, flags, &s))
+    Py_RETURN_NONE;
+  const auto dev = q.device();
+  if (!is_or_none(S0, s.state(), kF32, dev) || !is_or_none(A0, s.state(), kF32, dev) || !is_or_none(z0, s.vec(), kF32, dev)) Py_RETURN_NONE;
+  // (what vla_backward does not cover is left to the Python path and its exceptions)
+  if (s.d < 32 && (u.defined() || s.token_major)) Py_RETURN_NONE;
+  if (flags & VLA_FLAG_LINEAR_ATTENTION) Py_RETURN_NONE;
+  torch::autograd::variable_list r;
+  try {
+    auto opt = [](const Tensor& t) { return t.defined() ? OptTensor(t) : OptTensor(); };
+    r = Scan::apply(q, k, v, opt(u), opt(S0), opt(A0), opt(z0), status, lam, flags, eps);
+  } catch (const Failed& f) {
+    return PyLong_FromLong(f.code);
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+  PyObject* t = PyTuple_New(4);
+  if (!t) return nullptr;
+  for (int i = 0; i < 4; ++i) PyTuple_SET_ITEM(t, i, wrap(r[i]));
+  return t;
+}
+
+PyMethodDef methods[] = {
+    {"forward", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(forward)), METH_FASTCALL, "vla_forward"},
+    {"scan", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(scan)), METH_FASTCALL, "vla_scan"},
+    {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_vla_torch", "native marshalling of the VLA calls", -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__vla_torch(void) { return PyModule_Create(&module); }

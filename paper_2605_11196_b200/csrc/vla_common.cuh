@@ -330,6 +330,66 @@ __device__ __forceinline__ void tile16_store(float* G, int i0, int j0, const flo
   }
 }
 
+// ---------------------------------------------------------------- 16 x 16 elimination, one warp
+// M = L diag(delta) L^T of a symmetric positive definite 16 x 16 M by elimination in place, two columns a step.
+// Lane (r = lane & 15, h = lane >> 4) holds row r, columns 8 h .. 8 h + 7, and returns delta_r.  On return m holds
+// L^-1 left of the diagonal (the row operations applied to the identity, in the slots that elimination
+// frees) and delta_r L[c][r] right of it.  piv: 64 floats of shared memory, 16-byte aligned.
+// A step's latency is one shuffle, the 2 x 2 determinant's reciprocal and two FMAs: the pivot entries and the
+// row's own two travel by shuffle while the two pivot rows go through shared memory (1050 clk alone; one column
+// a step with the row by shuffles: 1530).  The registers rotate by two a step, so that columns s, s + 1 are always
+// m[0], m[1] of the half that holds them and the loop stays small; eight steps bring them back.
+__device__ __forceinline__ float eliminate16(float (&m)[8], int lane, float* piv, float eps) {
+  const int r = lane & 15, h = lane >> 4;
+  float delta = 1.0f;
+#pragma unroll 2
+  for (int s = 0; s < 16; s += 2) {
+    constexpr unsigned full = 0xffffffffu;
+    const int hs = s >> 3;
+    float* rows = piv + (s & 2) * 16;   // (two buffers: one barrier a step is enough)
+    const float a0 = __shfl_sync(full, m[0], s + 16 * hs);
+    const float b = __shfl_sync(full, m[0], s + 1 + 16 * hs);
+    const float d = __shfl_sync(full, m[1], s + 1 + 16 * hs);
+    const float ms0 = __shfl_sync(full, m[0], r + 16 * hs);
+    const float ms1 = __shfl_sync(full, m[1], r + 16 * hs);
+    if ((r | 1) == s + 1) {
+      float4* o = reinterpret_cast<float4*>(rows + (r & 1) * 16 + 8 * h);
+      o[0] = make_float4(m[0], m[1], m[2], m[3]);
+      o[1] = make_float4(m[4], m[5], m[6], m[7]);
+    }
+    __syncwarp();
+    const float4 x0 = *reinterpret_cast<const float4*>(rows + 8 * h), x1 = *reinterpret_cast<const float4*>(rows + 8 * h + 4);
+    const float4 y0 = *reinterpret_cast<const float4*>(rows + 16 + 8 * h), y1 = *reinterpret_cast<const float4*>(rows + 20 + 8 * h);
+    const float r0[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+    const float r1[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+    // Algorithm 1 clamps delta at eps (delta >= 1 whenever A is positive definite)
+    const float a = fmaxf(a0, eps);
+    const float det = fmaxf(fmaf(a, d, -b * b), eps * a);
+    const float idet = rcp_ftz(det), ia = rcp_ftz(a);
+    const float n0 = fmaf(d, ms0, -b * ms1), n1 = fmaf(a, ms1, -b * ms0);
+    const float q = r == s + 1 ? b * ia : 0.0f;     // row s + 1 loses its multiple of row s
+    const float im = r > s + 1 ? idet : 0.0f;
+    delta = r == s ? a : delta;
+    delta = r == s + 1 ? det * ia : delta;
+    const float w0 = fmaf(n0, im, q), w1 = n1 * im;
+    float t[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      // in the slots of columns s, s + 1 the identity's entries take the raw ones' place
+      const bool mine = h == hs;
+      const float c0 = j == 0 ? (mine ? 1.0f : r0[0]) : (mine && r > s + 1 ? 0.0f : r0[1]);
+      const float c1 = mine ? (j == 0 ? 0.0f : 1.0f) : r1[j];
+      const float mj = mine && r > s + j ? 0.0f : m[j];
+      t[j] = fmaf(-w0, c0, fmaf(-w1, c1, mj));
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) m[j] = fmaf(-w0, r0[j + 2], fmaf(-w1, r1[j + 2], m[j + 2]));
+    m[6] = t[0];
+    m[7] = t[1];
+  }
+  return delta;
+}
+
 // Reduce-scatter of 16 values over a full warp: lanes 2t and 2t+1 end with the sum of v[t].
 __device__ __forceinline__ float warp_reduce_scatter16(float (&v)[16], int lane) {
 #pragma unroll

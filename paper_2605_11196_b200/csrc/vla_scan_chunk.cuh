@@ -289,7 +289,7 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
   float* W0s = UT ? Z0s + C * D : Z0s;             // [C][D]  A K^T (== A U^T unless u is a tensor)
   float* Ufs = Z0s + 2 * C * D;                    // [2][C][D] widened u      (u tensor only)
   float* Ws = abase + Cfg::a_big * C * D;          // [C][CP] U A U^T (K A K^T when u = k_hat)
-  float* Ls = Ws + C * CP;                         // [C][CP] unit lower factor
+  float* Ls = Ws + C * CP;                         // [C][CP] the factors of I + W: L^-1 below the diagonal, delta_s L[t][s] above
   float* PTs = Ls + C * CP;                        // [C][CP] PT[t][s] = (z_s.k_t)/delta_s (general path)
   float* Guu = PTs + C * CP;                       // [C][CP] U U^T, refresh only (general path)
   float* Xs = UT ? Guu + C * CP : Ws;              // [C][CP] U A K^T (== W unless u is a tensor)
@@ -663,47 +663,40 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
           for (int j = 0; j < 8; ++j)
             m[j] = fmaf(nrs[min(r, h * 8 + j)], Guu[r * CP + h * 8 + j], m[j]);
         }
-#pragma unroll
-        for (int s2 = 0; s2 < 16; ++s2) {
-          const int hs = s2 >> 3, js = s2 & 7;
-          // Algorithm 1 clamps delta at eps; delta >= 1 whenever A is positive definite
-          const float piv = fmaxf(__shfl_sync(0xffffffffu, m[js], s2 + 16 * hs), eps);
-          const float mrs = __shfl_sync(0xffffffffu, m[js], r + 16 * hs);
-          const float ipiv = rcp_nr(piv);
-          const float l = (r > s2) ? mrs * ipiv : 0.0f;  // L[r][s2]
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float msj = __shfl_sync(0xffffffffu, m[j], s2 + 16 * h);
-            m[j] = fmaf(-l, msj, m[j]);
-          }
-          if (h == hs) Ls[r * CP + s2] = l;
-          if (lane == 0) {
-            dlt[s2] = piv; idl[s2] = ipiv; nidl[s2] = -ipiv;
-            if (STASH && p.stash_delta && s2 < nv)
-              p.stash_delta[size_t(unit) * size_t(p.T) + size_t(t_begin) + size_t(c) * C + s2] = piv;
-          }
+        __syncwarp();
+        // (the pivot rows pass through an array that is free by now)
+        const float delta = eliminate16(m, lane, HAS_U ? PTs : Ws, eps);
+        *reinterpret_cast<float4*>(Ls + r * CP + h * 8) = make_float4(m[0], m[1], m[2], m[3]);
+        *reinterpret_cast<float4*>(Ls + r * CP + h * 8 + 4) = make_float4(m[4], m[5], m[6], m[7]);
+        if (h == 0) {
+          const float id = rcp_nr(delta);
+          dlt[r] = delta; idl[r] = id; nidl[r] = -id;
+          if (STASH && p.stash_delta && r < nv)
+            p.stash_delta[size_t(unit) * size_t(p.T) + size_t(t_begin) + size_t(c) * C + r] = delta;
         }
         if (HAS_U) {
-          // N[s][t] = z_s . k_hat_t (s <= t) from X by the same elimination:
-          //   N[s][t] = X[s][t] - sum_{r<s} L[s][r] N[r][t];  PT[t][s] = N[s][t] / delta_s.
+          // N[s][t] = z_s . k_hat_t (s <= t): N = L^-1 X;  PT[t][s] = N[s][t] / delta_s.
           // Lane t < 16 owns column t (both halves of the warp compute the same thing).
           __syncwarp();
           const int t = lane & 15;
-          float nn[16];
+          float x[16];
 #pragma unroll
           for (int s2 = 0; s2 < 16; ++s2) {
-            float a0 = Xs[s2 * CP + t], a1 = 0.f;
-            if (rf_chunk) a0 = fmaf(nrs[s2], Guk[s2 * CP + t], a0);
+            x[s2] = Xs[s2 * CP + t];
+            if (rf_chunk) x[s2] = fmaf(nrs[s2], Guk[s2 * CP + t], x[s2]);
+          }
+#pragma unroll
+          for (int s2 = 0; s2 < 16; ++s2) {
+            float a0 = x[s2], a1 = 0.f;
 #pragma unroll
             for (int r4 = 0; r4 * 4 < s2; ++r4) {
               const float4 l4 = reinterpret_cast<const float4*>(Ls + s2 * CP)[r4];
-              if (4 * r4 + 0 < s2) a0 = fmaf(-l4.x, nn[4 * r4 + 0], a0);
-              if (4 * r4 + 1 < s2) a1 = fmaf(-l4.y, nn[4 * r4 + 1], a1);
-              if (4 * r4 + 2 < s2) a0 = fmaf(-l4.z, nn[4 * r4 + 2], a0);
-              if (4 * r4 + 3 < s2) a1 = fmaf(-l4.w, nn[4 * r4 + 3], a1);
+              if (4 * r4 + 0 < s2) a0 = fmaf(l4.x, x[4 * r4 + 0], a0);
+              if (4 * r4 + 1 < s2) a1 = fmaf(l4.y, x[4 * r4 + 1], a1);
+              if (4 * r4 + 2 < s2) a0 = fmaf(l4.z, x[4 * r4 + 2], a0);
+              if (4 * r4 + 3 < s2) a1 = fmaf(l4.w, x[4 * r4 + 3], a1);
             }
-            nn[s2] = a0 + a1;
-            if (h == 0) PTs[t * CP + s2] = (s2 <= t) ? nn[s2] * idl[s2] : 0.0f;
+            if (h == 0) PTs[t * CP + s2] = (s2 <= t) ? (a0 + a1) * idl[s2] : 0.0f;
           }
         }
         VLA_MARK(8)
@@ -725,21 +718,25 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
       }
       VLA_MARK(4)
 
-      // ---- row g of Z by forward substitution: z_t = z0_t - sum_{s<t} L[t][s] z_s
+      // ---- row g of Z = Z0 L^-T: z_t = z0_t + sum_{s<t} (L^-1)[t][s] z0_s, sixteen independent sums
       const float rf_tot = rf_chunk ? nrs[nv] : 0.0f;   // eta * refreshes in this chunk
       {
-        float z[16];
+        float z0[16], z[16];
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
-          float a0 = Z0s[t * D + g], a1 = 0.f;
-          if (rf_chunk) a0 = fmaf(nrs[t], Uf[t * D + g], a0);
+          z0[t] = Z0s[t * D + g];
+          if (rf_chunk) z0[t] = fmaf(nrs[t], Uf[t * D + g], z0[t]);
+        }
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          float a0 = z0[t], a1 = 0.f;
 #pragma unroll
           for (int s4 = 0; s4 * 4 < t; ++s4) {
             const float4 l4 = reinterpret_cast<const float4*>(Ls + t * CP)[s4];
-            if (4 * s4 + 0 < t) a0 = fmaf(-l4.x, z[4 * s4 + 0], a0);
-            if (4 * s4 + 1 < t) a1 = fmaf(-l4.y, z[4 * s4 + 1], a1);
-            if (4 * s4 + 2 < t) a0 = fmaf(-l4.z, z[4 * s4 + 2], a0);
-            if (4 * s4 + 3 < t) a1 = fmaf(-l4.w, z[4 * s4 + 3], a1);
+            if (4 * s4 + 0 < t) a0 = fmaf(l4.x, z0[4 * s4 + 0], a0);
+            if (4 * s4 + 1 < t) a1 = fmaf(l4.y, z0[4 * s4 + 1], a1);
+            if (4 * s4 + 2 < t) a0 = fmaf(l4.z, z0[4 * s4 + 2], a0);
+            if (4 * s4 + 3 < t) a1 = fmaf(l4.w, z0[4 * s4 + 3], a1);
           }
           z[t] = a0 + a1;
         }
@@ -804,16 +801,15 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
           atomicCAS(p.status, 0, int(VLA_ERR_NONFINITE));
         if (h == 0) scs[r] = sc_r;
         if (!HAS_U) {
-          const float scd = sc_r * d_r;   // multiplies column r of L
-          // lane (r, h) writes GuT[r][h*8 .. h*8+7]: GuT[r][s] = scd_s L[r][s]
+          // lane (r, h) writes GuT[r][h*8 .. h*8+7]: GuT[r][s] = sc_s delta_s L[r][s]
           float lr[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) lr[j] = Ls[r * CP + h * 8 + j];
+          for (int j = 0; j < 8; ++j) lr[j] = Ls[(h * 8 + j) * CP + r];
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const int s2 = h * 8 + j;
-            const float scd_s = __shfl_sync(0xffffffffu, scd, s2);
-            GuT[r * CP + s2] = (s2 < r) ? scd_s * lr[j] : 0.0f;
+            const float sc_s = __shfl_sync(0xffffffffu, sc_r, s2);
+            GuT[r * CP + s2] = (s2 < r) ? sc_s * lr[j] : 0.0f;
           }
         }
       }

@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(TcCfg<TIn>::NT, 1) vla_scan_tc_kernel(
     float* Zsl = Zsf + D * C;                                // its lo part
     float* Zp = Zsl + D * C;                                 // [C][D] rows: Z0, then Z
     float* Ws = Zp + C * D;                                  // [C][CP] K A K^T, then its factors
-    float* Ls = Ws + C * CP;                                 // [C][CP] unit lower factor
+    float* Ls = Ws + C * CP;                                 // [C][CP] the elimination's pivot rows
     float* N2p = Ls + C * CP;                                // [4][C]
     float* ZSp = N2p + 4 * C;                                // [4][C] per-warp sums of the entries of z_t
     float* dlt = ZSp + 4 * C;                                // [C]
@@ -429,33 +429,20 @@ __global__ void __launch_bounds__(TcCfg<TIn>::NT, 1) vla_scan_tc_kernel(
       group_bar(1, NG);
       VLA_MARK(4)
 
-      // ---- warp 0: I + W = L diag(delta) L^T by elimination, in place: once column s is
-      // eliminated its slots below the diagonal are free, and the row operations applied to the
-      // identity fill them with L^-1.  At the end the row holds L^-1 (left of the diagonal),
-      // delta (on it) and delta_s L[t][s] (right of it).
+      // ---- warp 0: I + W = L diag(delta) L^T by elimination in place (eliminate16).  At the end the row holds
+      // L^-1 (left of the diagonal) and delta_s L[t][s] (right of it)
       if (gw == 0) {
         const int r = lane & 15, h = lane >> 4;
         float m[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) m[j] = Ws[r * CP + h * 8 + j] + ((h * 8 + j == r) ? 1.0f : 0.0f);
-#pragma unroll
-        for (int s2 = 0; s2 < 16; ++s2) {
-          const int hs = s2 >> 3, js = s2 & 7;
-          const float piv = fmaxf(__shfl_sync(0xffffffffu, m[js], s2 + 16 * hs), eps);
-          const float mrs = __shfl_sync(0xffffffffu, m[js], r + 16 * hs);
-          const float ipiv = rcp_nr(piv);
-          const float l = (r > s2) ? mrs * ipiv : 0.0f;  // L[r][s2]
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float msj = __shfl_sync(0xffffffffu, m[j], s2 + 16 * h);
-            m[j] = fmaf(-l, msj, m[j]);
-          }
-          if (h == hs && r > s2) m[js] = -l;             // (row r of the identity) -= l (row s2 of it)
-          if (lane == 0) { dlt[s2] = piv; idl[s2] = ipiv; nidl[s2] = -ipiv; }
-        }
-        __syncwarp();
+        const float delta = eliminate16(m, lane, Ls, eps);
         *reinterpret_cast<float4*>(Ws + r * CP + h * 8) = make_float4(m[0], m[1], m[2], m[3]);
         *reinterpret_cast<float4*>(Ws + r * CP + h * 8 + 4) = make_float4(m[4], m[5], m[6], m[7]);
+        if (h == 0) {
+          const float id = rcp_nr(delta);
+          dlt[r] = delta; idl[r] = id; nidl[r] = -id;
+        }
       }
       group_bar(1, NG);
       VLA_MARK(5)

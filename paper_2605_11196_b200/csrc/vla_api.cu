@@ -86,18 +86,18 @@ bool chunk_tc_covers(const ScanParams& p, int d) {
 // The pair kernel: every d, u = k_hat or explicit, either layout; no refresh.
 bool pair_covers(const ScanParams& p) { return p.refresh_period <= 0 && p.n_main <= 0 && p.units <= 0x3fffffff; }
 
-// Where it is the library's choice.  Against the token kernel (measured, few units | units beyond one wave
-// of clusters, us at T = 8, 16, 32, 64): d = 64 token 8.4, 13.4, 24.6, 46.9 pair 7.5, 7.6, 10.4, 14.4 | 256
-// units 11.5, 18.6, 33.9, 64.4 and 29.7, 29.9, 40.4, 56.5; d = 32, 16 alike with the second crossing near 24.  At
+// Where it is the library's choice.  Below d = 128 everywhere but for very short sequences, which the token
+// kernel does without a cluster's start: few units, us at T = 8, 16, 32 (d = 64): token 8.4, 13.4, 24.6, pair
+// 8.2, 8.2, 11.1; more units than fit at once (1024): 33, 57, 107 and 63, 63, 90; d = 32: 12, 19, 35 and 31, 31, 43.  At
 // d = 128 the tensor-memory kernel keeps what is short (below seven chunks the clusters' start costs
 // what the shorter chain saves) and, with u = k_hat, more units than SM pairs (one SM per unit there:
-// 48 units x 1777 tokens 0.63 against 0.44 ms, 128 x 2048 0.75 against 1.02 ms).
+// 48 units x 1777 tokens 0.59 against 0.44 ms, 128 x 2048 0.69 against 1.02 ms).
 bool pair_pays_off(const ScanParams& p, int d) {
   const long long sms = vla::device_sms();
-  const long long resident = d == 16 ? 6 : d == 32 ? 4 : 1;   // CTAs per SM
+  const long long resident = d == 16 ? 6 : d == 32 ? 4 : d == 64 ? 2 : 1;   // CTAs per SM
   const bool one_wave = 2LL * p.units <= resident * sms;
   if (d == 128) return p.T > 96 && (p.u || one_wave);
-  return p.T > (one_wave ? 8 : d == 64 ? 48 : 24);
+  return p.T > (one_wave ? 8 : d == 64 ? 24 : 36);
 }
 
 int launch(const ScanParams& p, int d, int dtype, int kernel, cudaStream_t st) {
@@ -117,7 +117,8 @@ int launch(const ScanParams& p, int d, int dtype, int kernel, cudaStream_t st) {
   if (kernel == VLA_KERNEL_AUTO && pair_covers(p) && pair_pays_off(p, d)) return vla::launch_pair(d, dtype, p, nullptr, st);
   bool chunk = chunk_covers(p, d);
   if (kernel == VLA_KERNEL_CHUNK && !chunk) return VLA_ERR_UNSUPPORTED;
-  if (kernel == VLA_KERNEL_AUTO && !chunk_pays_off(p, d)) chunk = false;
+  // (below d = 128 the FMA chunk kernel is left with the refresh: the pair kernel is faster wherever it covers)
+  if (kernel == VLA_KERNEL_AUTO && (!chunk_pays_off(p, d) || (d < 128 && pair_covers(p)))) chunk = false;
   if (kernel == VLA_KERNEL_TOKEN) chunk = false;
   // d = 128: the same chunk algebra runs faster with the d x d products on the tensor cores
   if (chunk && kernel == VLA_KERNEL_AUTO && chunk_tc_covers(p, d)) return vla::launch_chunk_tc(d, dtype, p, st);
@@ -215,6 +216,15 @@ int seqpar_choose_segments(int units, int T, int d, int dtype) {
   int best = 1;
   for (int P = 2; P <= target && P <= nch; ++P)
     if (nch % P == 0 && T / P >= kSeqparMinTokens) best = P;
+  // Uncut, the pair kernel takes 1.6, 2.0, 3.9 us per 16 tokens (d = 32, 64, 128) whatever the number of units here.  Cut,
+  // the Gram matrices, inversions and corrections cost a start and a share per token, and a segment with its
+  // transfer scan 5.8 us (9.9) per 16 tokens, 12 with two CTAs on an SM.  (d = 64, 16 units x 4096 tokens: 517 us
+  // uncut, 413 in 8; 32 units: 521 and 625 in 4; 8 units x 1024: 136 and 206; 16 units x 65536: 8100 and 3790.)
+  const double uncut = nch * (d == 32 ? 1.6 : d == 64 ? 2.0 : 3.9);
+  const bool shared_sm = (seqpar_tri(d) ? 1LL : 2LL) * units * best > vla::device_sms();
+  const double cut = (d == 128 ? 590.0 : 180.0) + (d == 128 ? 9.9 : shared_sm ? 12.0 : 5.8) * nch / best +
+                     (d == 128 ? 4e-3 : 1.2e-3) * double(units) * T;
+  if (cut >= uncut) return 1;
   return best;
 }
 

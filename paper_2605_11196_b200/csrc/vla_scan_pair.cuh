@@ -36,6 +36,9 @@ struct PairCfg {
   static constexpr int NW = D / 16;                         // state warps
   static constexpr int NPREP = D == 128 ? 3 : D == 64 ? 2 : 1;   // widening warps
   static constexpr int NT = (NW + 1 + NPREP) * 32;
+  // CTAs per SM the registers are cut for.  d = 64: two hide one another's chains (128 units x 1024 tokens 355 -> 203 us,
+  // 256 units 657 -> 392) and cost one unit 2 % (128 registers instead of 192)
+  static constexpr int MINB = D == 64 ? 2 : 1;
   static constexpr int LPT = D / 4;                         // lanes per token in the widening pass
   static constexpr int TPW = 32 / LPT;                      // tokens per warp pass
   static constexpr int NP = (C + TPW * NPREP - 1) / (TPW * NPREP);   // passes per chunk
@@ -84,7 +87,7 @@ __device__ __forceinline__ void tok_store4(uint32_t base, int row, int pl, float
 }
 
 template <int D, typename TIn, bool UT, bool STASH>
-__global__ void __cluster_dims__(STASH ? 1 : 2, 1, 1) __launch_bounds__((PairCfg<D, TIn, UT>::NT), 1)
+__global__ void __cluster_dims__(STASH ? 1 : 2, 1, 1) __launch_bounds__((PairCfg<D, TIn, UT>::NT), (PairCfg<D, TIn, UT>::MINB))
 vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
   using Cfg = PairCfg<D, TIn, UT>;
   constexpr int C = Cfg::C, NW = Cfg::NW, NPREP = Cfg::NPREP, LPT = Cfg::LPT, TPW = Cfg::TPW, NP = Cfg::NP;
@@ -262,9 +265,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       *reinterpret_cast<float4*>(p.zT + size_t(unit) * D + 4 * pl) = make_float4(zk[0], zk[1], zk[2], zk[3]);
   } else if (rank == 0 && warp == NW) {
     // ===================================================================== rank 0: elimination
-    // I + W = L diag(delta) L^T in place, two columns a step: lane (r, h) holds row r, columns
-    // 8 h .. 8 h + 7; the slots of eliminated columns fill with L^-1 (the same row operations on the
-    // identity).  A step's latency is one shuffle, the 2 x 2 determinant's reciprocal and two FMAs.
+    // I + W = L diag(delta) L^T in place (eliminate16): lane (r, h) holds row r, columns 8 h .. 8 h + 7.
     float* fs = reinterpret_cast<float*>(smem + Cfg::a_f);
     float* Li = fs + Cfg::af_Li;
     float* dl = fs + Cfg::af_dl;
@@ -288,54 +289,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       }
 #pragma unroll
       for (int j = 0; j < 8; ++j) m[j] += (8 * h + j == r) ? 1.0f : 0.0f;
-      float delta = 1.0f;
-      // (an all but rolled loop: the registers rotate by two a step, so that columns s, s + 1 are always m[0], m[1]
-      // of the half that holds them; eight steps bring them back)
-#pragma unroll 2
-      for (int s = 0; s < 16; s += 2) {
-        constexpr unsigned full = 0xffffffffu;
-        const int hs = s >> 3;
-        float* rows = piv + (s & 2) * 16;
-        const float a0 = __shfl_sync(full, m[0], s + 16 * hs);
-        const float b = __shfl_sync(full, m[0], s + 1 + 16 * hs);
-        const float d = __shfl_sync(full, m[1], s + 1 + 16 * hs);
-        const float ms0 = __shfl_sync(full, m[0], r + 16 * hs);
-        const float ms1 = __shfl_sync(full, m[1], r + 16 * hs);
-        if ((r | 1) == s + 1) {
-          float4* o = reinterpret_cast<float4*>(rows + (r & 1) * 16 + 8 * h);
-          o[0] = make_float4(m[0], m[1], m[2], m[3]);
-          o[1] = make_float4(m[4], m[5], m[6], m[7]);
-        }
-        __syncwarp();
-        const float4 x0 = *reinterpret_cast<const float4*>(rows + 8 * h), x1 = *reinterpret_cast<const float4*>(rows + 8 * h + 4);
-        const float4 y0 = *reinterpret_cast<const float4*>(rows + 16 + 8 * h), y1 = *reinterpret_cast<const float4*>(rows + 20 + 8 * h);
-        const float r0[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-        const float r1[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
-        // Algorithm 1 clamps delta at eps (delta >= 1 whenever A is positive definite)
-        const float a = fmaxf(a0, eps);
-        const float det = fmaxf(fmaf(a, d, -b * b), eps * a);
-        const float idet = rcp_ftz(det), ia = rcp_ftz(a);
-        const float n0 = fmaf(d, ms0, -b * ms1), n1 = fmaf(a, ms1, -b * ms0);
-        const float q = r == s + 1 ? b * ia : 0.0f;     // row s + 1 loses its multiple of row s
-        const float im = r > s + 1 ? idet : 0.0f;
-        delta = r == s ? a : delta;
-        delta = r == s + 1 ? det * ia : delta;
-        const float w0 = fmaf(n0, im, q), w1 = n1 * im;
-        float t[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          // in the slots of columns s, s + 1 the identity's entries take the raw ones' place
-          const bool mine = h == hs;
-          const float c0 = j == 0 ? (mine ? 1.0f : r0[0]) : (mine && r > s + 1 ? 0.0f : r0[1]);
-          const float c1 = mine ? (j == 0 ? 0.0f : 1.0f) : r1[j];
-          const float mj = mine && r > s + j ? 0.0f : m[j];
-          t[j] = fmaf(-w0, c0, fmaf(-w1, c1, mj));
-        }
-#pragma unroll
-        for (int j = 0; j < 6; ++j) m[j] = fmaf(-w0, r0[j + 2], fmaf(-w1, r1[j + 2], m[j + 2]));
-        m[6] = t[0];
-        m[7] = t[1];
-      }
+      const float delta = eliminate16(m, lane, piv, eps);
       {
         float x[8];
 #pragma unroll

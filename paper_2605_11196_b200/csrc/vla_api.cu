@@ -240,7 +240,7 @@ size_t backward_scans_bytes(size_t units, size_t T, size_t d) {
 
 // ---- ... and of the chunked form: bytes per unit (every array of `n` units is n times its unit's part)
 struct BwdLayout {
-  size_t alpha, zeta, e, g, zkc, scal, opK, opQ, opA, small, Aimg, Simg, Dimg, sc, X, Y, A_T, XT, XT2, total;
+  size_t alpha, zeta, e, g, zkc, scal, opK, opQ, opA, small, Aimg, Simg, Dimg, sc, X, Y, A_T, XT, XT2, Xm, total;
 };
 BwdLayout bwd_layout(size_t T, size_t d) {
   const size_t nch = (T + 15) / 16, NB = (nch + 1) / 2, row = 4 * d + 16;   // row: an operand row of the kernels
@@ -266,6 +266,7 @@ BwdLayout bwd_layout(size_t T, size_t d) {
   L.A_T = take(d * d * 4);
   L.XT = take(d * d * 4);
   L.XT2 = take(d * d * 4);
+  L.Xm = take(2 * round256(NB * 4) + 256);   // Xmax, Xsc, XTmax
   L.total = off;
   return L;
 }
@@ -336,6 +337,8 @@ int backward_chunked(const void* q, const void* k, const void* v, float lambda_,
     p.Ssc = sh.Asc + scs; p.Dsc = p.Ssc + scs;
     p.Simg = ws(L.Simg); p.Dimg = ws(L.Dimg);
     p.X = wf(L.X); p.Y = wf(L.Y); p.XT = wf(L.XT); p.XT2 = wf(L.XT2);
+    const size_t xm = round256(size_t(p.NB) * 4) / 4 * n;
+    p.Xmax = wf(L.Xm); p.Xsc = p.Xmax + xm; p.XTmax = p.Xsc + xm;
     p.status = o.status;
     p.T = T; p.units = int(n); p.nch = nch; p.heads = H;
     p.flags = o.flags; p.wait_limit = o.wait_probe_limit; p.eps = o.eps;

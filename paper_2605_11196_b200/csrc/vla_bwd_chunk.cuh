@@ -478,25 +478,33 @@ __global__ void __launch_bounds__(BwdChainCfg<D>::NT) bwd_chains_kernel(const Bw
 }
 
 // ---------------------------------------------------------------- per block: everything that needs S, D, A of the block
+// Warps: two groups of 16 tokens x CS column groups x two roles.  (CS = 4 at d >= 64 was slower, 1.33 -> 1.49 ms at d = 128:
+// the barriers between the phases cost more than the shorter ones save.)
 template <int D> struct BwdBlockCfg {
+  static constexpr int CS = D >= 64 ? 2 : 1, NWB = 4 * CS, NT = 32 * NWB;
   static constexpr uint32_t tb = BwdGeom<D>::tb;
   static constexpr uint32_t mat = 6 * tb;
   static constexpr uint32_t fl = mat + BwdGeom<D>::mat;
-  static constexpr int f_red = 0, f_dot = 64, f_dqd = f_dot + 64, f_ddn = f_dqd + 64, f_an = f_ddn + 32, f_rho = f_an + 32,
-                       f_qsi = f_rho + 32, f_id = f_qsi + 32, f_end = f_id + 32;
+  static constexpr int f_red = 0, f_dot = 8 * NWB, f_dqd = f_dot + 32 * CS, f_ddn = f_dqd + 32 * CS, f_an = f_ddn + 32, f_rho = f_an + 32,
+                       f_qsi = f_rho + 32, f_id = f_qsi + 32, f_y = f_id + 32, f_end = f_y + 2 * D;
   static constexpr uint32_t smem_bytes = fl + f_end * 4 + 32;
 };
 
-// largest of N per-thread values over a CTA of 8 warps, through red[8 * N]; the caller synchronises between
+// largest of N per-thread values over a CTA of NW warps, through red[NW * N]; the caller synchronises between
 // cta_max_put and cta_max_get
+template <int NW>
 __device__ __forceinline__ void cta_max_put(float* red, int slot, float m, int warp, int lane) {
   m = warp_max_nonneg(m);
-  if (lane == 0) red[slot * 8 + warp] = m;
+  if (lane == 0) red[slot * NW + warp] = m;
 }
+template <int NW>
 __device__ __forceinline__ float cta_max_get(const float* red, int slot) {
   float m = 0.f;
 #pragma unroll
-  for (int w = 0; w < 8; ++w) m = fmaxf(m, red[slot * 8 + w]);
+  for (int w = 0; w < NW; w += 4) {
+    const float4 x = *reinterpret_cast<const float4*>(red + slot * NW + w);
+    m = fmaxf(m, fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
+  }
   return m;
 }
 __device__ __forceinline__ float max4(float m, float4 x) {
@@ -504,16 +512,16 @@ __device__ __forceinline__ float max4(float m, float4 x) {
 }
 
 template <int D, typename TIn, bool UT>
-__global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) {
+__global__ void __launch_bounds__(BwdBlockCfg<D>::NT) bwd_block_kernel(const BwdChunkParams p) {
   using Cfg = BwdBlockCfg<D>;
   using G = BwdGeom<D>;
-  constexpr int BC = kBwdBlock, KS = D / 16, NH = D / 16;   // NH: n tiles of half the columns
+  constexpr int BC = kBwdBlock, KS = D / 16, CS = Cfg::CS, NWB = Cfg::NWB, NT = Cfg::NT, NH = D / 8 / CS;   // NH: n tiles of a column group
   constexpr float kInv = 1.0f / 256.0f;
   extern __shared__ __align__(128) unsigned char smem[];
   const int blk = blockIdx.x, unit = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-  const int tg = warp & 1, h = (warp >> 1) & 1, role = warp >> 2;
+  const int tg = warp & 1, h = (warp >> 1) % CS, role = warp / (2 * CS);
   const int t0 = blk * BC, T = p.T, nt_valid = min(BC, T - t0), nchv = min(2, p.nch - 2 * blk);
   const size_t ub = size_t(unit) * p.NB + blk, ut0 = size_t(unit) * T + t0;
   const size_t tok = bwd_tok(p, unit, t0, D), ts = bwd_stride(p, D);   // the block's first token, distance between tokens
@@ -546,7 +554,7 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
     bulk_load(smem + Cfg::mat, p.Simg + ub * G::mat, G::mat, bar);
   }
   if (nchv < 2)   // the chunk that is not there reads as zeros
-    for (uint32_t i = tid; i < G::kslot / 4; i += 256)
+    for (uint32_t i = tid; i < G::kslot / 4; i += NT)
 #pragma unroll
       for (int a = 3; a < 6; ++a) sts32(sb + a * Cfg::tb + G::kslot + 4 * i, 0u);
   if (tid < BC) {
@@ -559,14 +567,14 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
   }
   __syncthreads();
   // ---- E, dE, dY as operand rows, scaled by their largest entry
-  constexpr int NG = BC * D / 4, NPT = (NG + 255) / 256;   // groups of four columns, per thread
+  constexpr int NG = BC * D / 4, NPT = (NG + NT - 1) / NT;   // groups of four columns, per thread
   float sE = 1.f, sDE = 1.f, sDY = 1.f, sZ = 1.0f;
   {
     float4 xe[NPT], xd[NPT], xy[NPT];
     float me = 0.f, md = 0.f, my = 0.f;
 #pragma unroll
     for (int i = 0; i < NPT; ++i) {
-      const int j = tid + 256 * i, t = j / (D / 4), c = j % (D / 4);
+      const int j = tid + NT * i, t = j / (D / 4), c = j % (D / 4);
       xe[i] = xd[i] = xy[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (j < NG && t < nt_valid) {
         const size_t o = tok + t * ts + 4 * c;
@@ -577,21 +585,21 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
     }
 #pragma unroll
     for (int i = 0; i < NPT; ++i) {
-      const int t = (tid + 256 * i) / (D / 4);
+      const int t = (tid + NT * i) / (D / 4);
       const float id = t < BC ? fabsf(fs[Cfg::f_id + t]) : 0.f;
       xy[i] = make_float4(xy[i].x * id, xy[i].y * id, xy[i].z * id, xy[i].w * id);
       me = max4(me, xe[i]); md = max4(md, xd[i]); my = max4(my, xy[i]);
     }
-    cta_max_put(red, 0, me, warp, lane);
-    cta_max_put(red, 1, md, warp, lane);
-    cta_max_put(red, 2, my, warp, lane);
+    cta_max_put<NWB>(red, 0, me, warp, lane);
+    cta_max_put<NWB>(red, 1, md, warp, lane);
+    cta_max_put<NWB>(red, 2, my, warp, lane);
     __syncthreads();
-    sE = pow2_scale(cta_max_get(red, 0), 10);
-    sDE = pow2_scale(cta_max_get(red, 1), 10);
-    sDY = pow2_scale(cta_max_get(red, 2), 10);
+    sE = pow2_scale(cta_max_get<NWB>(red, 0), 10);
+    sDE = pow2_scale(cta_max_get<NWB>(red, 1), 10);
+    sDY = pow2_scale(cta_max_get<NWB>(red, 2), 10);
 #pragma unroll
     for (int i = 0; i < NPT; ++i) {
-      const int j = tid + 256 * i, t = j / (D / 4), c = j % (D / 4);
+      const int j = tid + NT * i, t = j / (D / 4), c = j % (D / 4);
       if (j < NG) {
         row_store4<D>(tE, t, c, xe[i], sE);
         row_store4<D>(tDE, t, c, xd[i], sDE);
@@ -773,7 +781,10 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
       const int t = tr + 8 * hf;
       const float an = fs[Cfg::f_an + t];
       const bool floored = !(an > p.eps);
-      const float dot = floored ? 0.f : (fs[Cfg::f_dot + t] + fs[Cfg::f_dot + 32 + t]) * kInv * kInv;
+      float dot = 0.f;
+#pragma unroll
+      for (int w = 0; w < CS; ++w) dot += fs[Cfg::f_dot + 32 * w + t];
+      dot = floored ? 0.f : dot * kInv * kInv;
       const float ia = rcp_ftz_nr(an);
 #pragma unroll
       for (int nt = 0; nt < NH; ++nt) {
@@ -788,7 +799,10 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
     }
   } else if (tid < BC) {
     const float id = fs[Cfg::f_id + tid];
-    float dd = (fs[Cfg::f_dqd + tid] + fs[Cfg::f_dqd + 32 + tid]) * fs[Cfg::f_qsi + tid];
+    float dd = 0.f;
+#pragma unroll
+    for (int w = 0; w < CS; ++w) dd += fs[Cfg::f_dqd + 32 * w + tid];
+    dd *= fs[Cfg::f_qsi + tid];
     dd = id > 0.f && !(p.flags & VLA_FLAG_IDENTITY_MAP) ? -dd * id : 0.f;
     fs[Cfg::f_ddn + tid] = dd;
     if (tid < nt_valid) p.dden[ut0 + tid] = dd;
@@ -798,39 +812,42 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
   if constexpr (UT) {
 #pragma unroll
     for (int i = 0; i < NPT; ++i) {
-      const int j = tid + 256 * i, t = j / (D / 4), c = j % (D / 4);
+      const int j = tid + NT * i, t = j / (D / 4), c = j % (D / 4);
       xz[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (j < NG && t < nt_valid) xz[i] = gload4(p.zeta + (ut0 + t) * D + 4 * c);
       mz = max4(mz, xz[i]);
     }
-    cta_max_put(red, 4, mz, warp, lane);
+    cta_max_put<NWB>(red, 4, mz, warp, lane);
   }
-  cta_max_put(red, 3, mx, warp, lane);
+  cta_max_put<NWB>(red, 3, mx, warp, lane);
   __syncthreads();
-  const float sDA = pow2_scale(cta_max_get(red, 3), 10);
+  const float sDA = pow2_scale(cta_max_get<NWB>(red, 3), 10);
   if (role == 1) {   // da over dY's rows
 #pragma unroll
     for (int nt = 0; nt < NH; ++nt)
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf)
         row_pair_store<D>(tDY, tr + 8 * hf, (h * NH + nt) * 8 + 2 * c4, acc0[nt][2 * hf] * sDA, acc0[nt][2 * hf + 1] * sDA);
-  } else if (tid < D) {
+  }
+  for (int j = tid; j < 2 * D; j += NT) {   // the block's sum of dden q, 16 tokens a thread
+    const int c = j % D, t1 = j / D * 16;
     float y = 0.f;
-#pragma unroll 2
-    for (int t = 0; t < nt_valid; ++t) y = fmaf(fs[Cfg::f_ddn + t] * fs[Cfg::f_qsi + t], row_one<D>(smem + 4 * Cfg::tb, t, tid), y);
-    p.Y[ub * D + tid] = y;
+#pragma unroll 4
+    for (int t = t1; t < t1 + 16; ++t) y = fmaf(fs[Cfg::f_ddn + t] * fs[Cfg::f_qsi + t], row_one<D>(smem + 4 * Cfg::tb, t, c), y);
+    fs[Cfg::f_y + j] = y;
   }
   if constexpr (UT) {   // zeta over E's rows
-    sZ = pow2_scale(cta_max_get(red, 4), 10);
+    sZ = pow2_scale(cta_max_get<NWB>(red, 4), 10);
 #pragma unroll
     for (int i = 0; i < NPT; ++i) {
-      const int j = tid + 256 * i;
+      const int j = tid + NT * i;
       if (j < NG) row_store4<D>(tE, j / (D / 4), j % (D / 4), xz[i], sZ);
     }
   }
   __syncthreads();
-  // ---- g = A_t da_t = da A - tril(da zeta^T) zeta, columns split over up to four warps per 16 tokens
-  constexpr int NCG = D >= 32 ? 4 : 2, N3 = D / NCG / 8;
+  if (tid < D) p.Y[ub * D + tid] = fs[Cfg::f_y + tid] + fs[Cfg::f_y + D + tid];
+  // ---- g = A_t da_t = da A - tril(da zeta^T) zeta, columns split over the warps of 16 tokens
+  constexpr int NCG = D / 8 < 2 * CS ? D / 8 : 2 * CS, N3 = D / NCG / 8;
   using N3c = std::integral_constant<int, N3>;
   const int cg = warp >> 1;
   float ga[N3][4] = {};
@@ -888,9 +905,9 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
       ga[nt][2 * hf + 1] = x.y * an;
       mg = fmaxf(mg, fmaxf(fabsf(ga[nt][2 * hf]), fabsf(ga[nt][2 * hf + 1])));
     }
-  cta_max_put(red, 5, mg, warp, lane);
+  cta_max_put<NWB>(red, 5, mg, warp, lane);
   __syncthreads();
-  const float sG = pow2_scale(cta_max_get(red, 5), 10);
+  const float sG = pow2_scale(cta_max_get<NWB>(red, 5), 10);
   if (cg < NCG) {   // an g over dE's rows
 #pragma unroll
     for (int nt = 0; nt < N3; ++nt)
@@ -900,7 +917,7 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
   }
   __syncthreads();
   // ---- the block's sum of (an g) alpha^T + alpha (an g)^T
-  constexpr int MT = D / 16, PP = 8 / MT > D / 8 ? D / 8 : 8 / MT, N4 = D / 8 / PP;   // m tiles, warps per m tile, n tiles a warp
+  constexpr int MT = D / 16, PP = NWB / MT > D / 8 ? D / 8 : NWB / MT, N4 = D / 8 / PP;   // m tiles, warps per m tile, n tiles a warp
   const int mt = warp % MT, part = warp / MT;
   if (part < PP) {
     const uint32_t lm = tok_lane_m<D>(lane);
@@ -914,6 +931,7 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
     }
     const float f = pow2_inverse(sG) * kInv;
     float* dst = p.X + ub * D * D + size_t(mt * 16 + g) * D + 2 * c4;
+    float mX = 0.f;
 #pragma unroll 1
     for (int n = 0; n < N4; ++n) {
       const int nt = part * N4 + n;
@@ -926,9 +944,13 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
       float x[4] = {};
       mma3_f16_many<4>([&](int i, int lo) -> const uint32_t(&)[4] { return i < 2 ? (lo ? gl[i & 1] : gh[i & 1]) : (lo ? al[i & 1] : ah[i & 1]); },
                        [&](int i, int r) { return b[i][r]; }, [&](int) -> float* { return x; });
+#pragma unroll
+      for (int e = 0; e < 4; ++e) mX = fmaxf(mX, fabsf(x[e] * f));
       *reinterpret_cast<float2*>(dst + 8 * nt) = make_float2(x[0] * f, x[1] * f);
       *reinterpret_cast<float2*>(dst + 8 * D + 8 * nt) = make_float2(x[2] * f, x[3] * f);
     }
+    mX = warp_max_nonneg(mX);
+    if (lane == 0) atomicMax(reinterpret_cast<unsigned int*>(p.Xmax + ub), __float_as_uint(mX));
   }
   if (*abort_flag) {
     settle_copies();
@@ -937,25 +959,46 @@ __global__ void __launch_bounds__(256) bwd_block_kernel(const BwdChunkParams p) 
 }
 
 // ---------------------------------------------------------------- suffix sums over the blocks
-// Replaces every block's sum by what the later blocks (and the final state's gradient) add up to.
+// What the blocks after each one (and the final state's gradient) add up to, as operand images (in the place of
+// S's, which are done with).  An image's scale comes from the sum of the blocks' largest entries, which bounds the
+// entries of the sum: known while walking, at most the number of blocks above the true maximum.
 template <int D>
 __global__ void __launch_bounds__(256) bwd_scan_kernel(const BwdChunkParams p) {
   const int unit = blockIdx.y, i = blockIdx.x * 256 + threadIdx.x;
   constexpr int N = D * D / 4;
   if (i < N) {
-    float4* x = reinterpret_cast<float4*>(p.X + size_t(unit) * p.NB * D * D) + i;
+    const size_t ub = size_t(unit) * p.NB;
+    const float4* x = reinterpret_cast<const float4*>(p.X + ub * D * D) + i;
+    unsigned char* img = p.Simg + ub * BwdGeom<D>::mat + size_t(i / (D / 4)) * kTokRow<D> + 8 * (i % (D / 4));
+    const float* xm = p.Xmax + ub;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (p.dA_T) acc = reinterpret_cast<const float4*>(p.XT + size_t(unit) * D * D)[i];
+    float bound = 0.f;
+    if (p.dA_T) {
+      acc = reinterpret_cast<const float4*>(p.XT + size_t(unit) * D * D)[i];
+      bound = p.XTmax[unit];
+    }
     for (int b = p.NB - 1; b >= 0; b -= 8) {
       float4 v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (b - j >= 0) v[j] = x[size_t(b - j) * N];
+      float m[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j)
         if (b - j >= 0) {
-          x[size_t(b - j) * N] = acc;
+          v[j] = x[size_t(b - j) * N];
+          m[j] = xm[b - j];
+        }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (b - j >= 0) {
+          const float s = pow2_scale(bound, 10);
+          uint32_t h0, l0, h1, l1;
+          split_f16(acc.x * s, acc.y * s, h0, l0);
+          split_f16(acc.z * s, acc.w * s, h1, l1);
+          unsigned char* o = img + size_t(b - j) * BwdGeom<D>::mat;
+          *reinterpret_cast<uint2*>(o) = make_uint2(h0, h1);
+          *reinterpret_cast<uint2*>(o + 2 * D) = make_uint2(l0, l1);
+          if (i == 0) p.Xsc[ub + b - j] = pow2_inverse(s);
           acc.x += v[j].x; acc.y += v[j].y; acc.z += v[j].z; acc.w += v[j].w;
+          bound = (bound + m[j]) * 1.0000002f;   // (stays above the rounded sum)
         }
     }
   } else if (i < N + D) {
@@ -976,7 +1019,7 @@ template <int D>
 __global__ void __launch_bounds__(256) bwd_final_state_kernel(const BwdChunkParams p) {
   const size_t at = size_t(blockIdx.x) * D * D;
   const float *A = p.A_T + at, *dA = p.dA_T + at;
-  float *W = p.XT2 + at, *X = p.XT + at;
+  float *W = p.XT2 + at, *X = p.XT + at, mx = 0.f;
   for (int i = threadIdx.x; i < D * D; i += 256) {
     const int r = i / D, c = i % D;
     float s = 0.f;
@@ -989,24 +1032,28 @@ __global__ void __launch_bounds__(256) bwd_final_state_kernel(const BwdChunkPara
     float s = 0.f;
     for (int k = 0; k < D; ++k) s = fmaf(A[r * D + k], W[k * D + c], s);
     X[i] = s;
+    mx = fmaxf(mx, fabsf(s));
   }
+  mx = warp_max_nonneg(mx);
+  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned int*>(p.XTmax + blockIdx.x), __float_as_uint(mx));
 }
 
 // ---------------------------------------------------------------- per block: du, and dq, dk through norms and feature map
 template <int D, bool UT> struct BwdFinishCfg {
+  static constexpr int NWB = 8, NT = 32 * NWB;
   static constexpr uint32_t tb = BwdGeom<D>::tb;
   static constexpr uint32_t mat = (UT ? 5 : 4) * tb;   // K, alpha, Q, an g [, u]
   static constexpr uint32_t zz = mat + BwdGeom<D>::mat;                      // key sums, their gradients: [32][D] each
   static constexpr uint32_t fl = zz + 2 * kBwdBlock * D * 4;
-  static constexpr int f_red = 0, f_an = 64, f_qsi = 96, f_nrm = 128, f_ddn = 160, f_kd = 192, f_end = 192 + 4 * 32;
+  static constexpr int f_red = 0, f_an = 4 * NWB, f_qsi = f_an + 32, f_nrm = f_qsi + 32, f_ddn = f_nrm + 32, f_kd = f_ddn + 32, f_end = f_kd + 16 * NWB;
   static constexpr uint32_t smem_bytes = fl + f_end * 4 + 32;
 };
 
 template <int D, typename TIn, bool UT>
-__global__ void __launch_bounds__(256) bwd_finish_kernel(const BwdChunkParams p) {
+__global__ void __launch_bounds__(BwdFinishCfg<D, UT>::NT) bwd_finish_kernel(const BwdChunkParams p) {
   using Cfg = BwdFinishCfg<D, UT>;
   using G = BwdGeom<D>;
-  constexpr int BC = kBwdBlock, KS = D / 16;
+  constexpr int BC = kBwdBlock, KS = D / 16, NWB = Cfg::NWB, NT = Cfg::NT;
   constexpr float kInv = 1.0f / 256.0f;
   extern __shared__ __align__(128) unsigned char smem[];
   const int blk = blockIdx.x, unit = blockIdx.y;
@@ -1033,13 +1080,14 @@ __global__ void __launch_bounds__(256) bwd_finish_kernel(const BwdChunkParams p)
   if (tid == 0) {
     const size_t id = size_t(unit) * p.nch + 2 * blk;
     const uint32_t n = nchv * G::kslot;
-    mbar_arrive_expect_tx(bar, 3 * n);
+    mbar_arrive_expect_tx(bar, 3 * n + G::mat);
+    bulk_load(smem + Cfg::mat, p.Simg + ub * G::mat, G::mat, bar);   // X beyond this block
     bulk_load(smem, p.opK + id * G::kslot, n, bar);
     bulk_load(smem + Cfg::tb, p.opA + id * G::kslot, n, bar);
     bulk_load(smem + 2 * Cfg::tb, p.opQ + id * G::kslot, n, bar);
   }
   if (nchv < 2)
-    for (uint32_t i = tid; i < G::kslot / 4; i += 256)
+    for (uint32_t i = tid; i < G::kslot / 4; i += NT)
 #pragma unroll
       for (int a = 0; a < 3; ++a) sts32(sb + a * Cfg::tb + G::kslot + 4 * i, 0u);
   if (tid < BC) {
@@ -1050,20 +1098,15 @@ __global__ void __launch_bounds__(256) bwd_finish_kernel(const BwdChunkParams p)
     fs[Cfg::f_ddn + tid] = act ? p.dden[ut0 + tid] : 0.f;
   }
   __syncthreads();
-  // ---- X beyond this block, an g and u as operand images
-  constexpr int NG = BC * D / 4, NPT = (NG + 255) / 256, NM = (D * D / 4 + 255) / 256;
-  float sX, sG, sU = 256.0f;
+  // ---- an g and u as operand images
+  constexpr int NG = BC * D / 4, NPT = (NG + NT - 1) / NT;
+  float sG, sU = 256.0f;
   {
     float4 xg[NPT], xu[UT ? NPT : 1];
-    float mm = 0.f, mg = 0.f, mu = 0.f;
-#pragma unroll 4
-    for (int i = 0; i < NM; ++i) {
-      const int j = tid + 256 * i;
-      if (j < D * D / 4) mm = max4(mm, gload4(p.X + ub * D * D + 4 * j));
-    }
+    float mg = 0.f, mu = 0.f;
 #pragma unroll
     for (int i = 0; i < NPT; ++i) {
-      const int j = tid + 256 * i, t = j / (D / 4), c = j % (D / 4);
+      const int j = tid + NT * i, t = j / (D / 4), c = j % (D / 4);
       xg[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (UT) xu[i] = xg[i];
       if (j < NG && t < nt_valid) {
@@ -1075,21 +1118,14 @@ __global__ void __launch_bounds__(256) bwd_finish_kernel(const BwdChunkParams p)
       mg = max4(mg, xg[i]);
       if (UT) mu = max4(mu, xu[i]);
     }
-    cta_max_put(red, 0, mm, warp, lane);
-    cta_max_put(red, 1, mg, warp, lane);
-    if (UT) cta_max_put(red, 2, mu, warp, lane);
+    cta_max_put<NWB>(red, 1, mg, warp, lane);
+    if (UT) cta_max_put<NWB>(red, 2, mu, warp, lane);
     __syncthreads();
-    sX = pow2_scale(cta_max_get(red, 0), 10);
-    sG = pow2_scale(cta_max_get(red, 1), 10);
-    if (UT) sU = pow2_scale(cta_max_get(red, 2), 10);
-#pragma unroll 2
-    for (int i = 0; i < NM; ++i) {   // (read a second time, from L2)
-      const int j = tid + 256 * i;
-      if (j < D * D / 4) row_store4<D>(mat, j / (D / 4), j % (D / 4), gload4(p.X + ub * D * D + 4 * j), sX);
-    }
+    sG = pow2_scale(cta_max_get<NWB>(red, 1), 10);
+    if (UT) sU = pow2_scale(cta_max_get<NWB>(red, 2), 10);
 #pragma unroll
     for (int i = 0; i < NPT; ++i) {
-      const int j = tid + 256 * i;
+      const int j = tid + NT * i;
       if (j < NG) {
         row_store4<D>(tG, j / (D / 4), j % (D / 4), xg[i], sG);
         if (UT) row_store4<D>(tU, j / (D / 4), j % (D / 4), xu[i], sU);
@@ -1105,33 +1141,41 @@ __global__ void __launch_bounds__(256) bwd_finish_kernel(const BwdChunkParams p)
   __syncthreads();
   // ---- key sums up to each token, and the sums of dden q from each token on (thread = column)
   if (!ident) {
-    if (tid < D) {
-      float z = 0.f;
-#pragma unroll 2
-      for (int t = 0; t < nt_valid; ++t) {
-        if ((t & 15) == 0) z = p.zkc[(size_t(unit) * p.nch + 2 * blk + (t >> 4)) * D + tid];
-        z = fmaf(row_one<D>(smem, t, tid), fabsf(fs[Cfg::f_nrm + t]) * kInv, z);
-        zp[t * D + tid] = z;
-      }
-    } else if (tid >= 128 && tid - 128 < D) {
-      const int c = tid - 128;
-      float y = p.Y[ub * D + c];
-#pragma unroll 2
-      for (int t = nt_valid - 1; t >= 0; --t) {
-        y = fmaf(fs[Cfg::f_ddn + t] * fs[Cfg::f_qsi + t], row_one<D>(smem + 2 * Cfg::tb, t, c), y);
-        zg[t * D + c] = y;
+    // a thread takes one column of one chunk: first 2 D of them the key sums, which start from the stored ones,
+    // then as many the suffix sums, where the first chunk adds up the second one's first
+    for (int j = tid; j < 4 * D; j += NT) {
+      const int c = j % D, ch = j / D & 1, t1 = 16 * ch;
+      if (j < 2 * D) {
+        float z = t1 < nt_valid ? p.zkc[(size_t(unit) * p.nch + 2 * blk + ch) * D + c] : 0.f;
+#pragma unroll 4
+        for (int t = t1; t < t1 + 16; ++t) {
+          z = fmaf(row_one<D>(smem, t, c), fabsf(fs[Cfg::f_nrm + t]) * kInv, z);
+          zp[t * D + c] = z;
+        }
+      } else {
+        const unsigned char* Q = smem + 2 * Cfg::tb;
+        float y = p.Y[ub * D + c];
+        if (ch == 0) {
+#pragma unroll 4
+          for (int t = 31; t >= 16; --t) y = fmaf(fs[Cfg::f_ddn + t] * fs[Cfg::f_qsi + t], row_one<D>(Q, t, c), y);
+        }
+#pragma unroll 4
+        for (int t = t1 + 15; t >= t1; --t) {
+          y = fmaf(fs[Cfg::f_ddn + t] * fs[Cfg::f_qsi + t], row_one<D>(Q, t, c), y);
+          zg[t * D + c] = y;
+        }
       }
     }
   }
   // ---- du = -U X - triu(U alpha^T) (an g) - triu(U (an g)^T) alpha
-  constexpr int NCG = D >= 32 ? 4 : 2, N3 = D / NCG / 8;
+  constexpr int NCG = D / 8 < NWB / 2 ? D / 8 : NWB / 2, N3 = D / NCG / 8;
   const int tg = warp & 1, cg = warp >> 1;
   const uint32_t la = tok_lane_a<D>(lane), lb = tok_lane_b<D>(lane), lk = tok_lane_k<D>(lane);
   const uint32_t own = uint32_t(tg * 16) * kTokRow<D>;
   const int tr = tg * 16 + g;
   float du[N3][4] = {};
   if (cg < NCG) {
-    const float fx = -pow2_inverse(sX);
+    const float fx = -p.Xsc[ub];
 #pragma unroll 1
     for (int ks = 0; ks < KS; ++ks) {
       uint32_t ah[4], al[4];

@@ -21,6 +21,8 @@ struct BwdChunkParams {
   unsigned char *Simg, *Dimg;
   // g_t, gradient of den_t, per block sums of the penalty side [D, D] and of dden q [D]
   float *g, *dden, *X, *Y, *XT, *XT2;
+  // largest entries of X per block and of XT per unit; inverse scales of X's images (kept in Simg)
+  float *Xmax, *XTmax, *Xsc;
   int* status;
   int T, units, nch, NB, heads;
   uint32_t flags, wait_limit;

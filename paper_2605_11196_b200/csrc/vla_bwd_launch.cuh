@@ -24,14 +24,20 @@ int launch_bwd_chunk_t(const BwdChunkParams& p, cudaStream_t st) {
       !set_smem_once(done[2], reinterpret_cast<const void*>(block), Block::smem_bytes) ||
       !set_smem_once(done[3], reinterpret_cast<const void*>(fin), Fin::smem_bytes))
     return VLA_ERR_CUDA;
+  // (largest entries are gathered with atomicMax)
+  if (cudaMemsetAsync(p.Xmax, 0, size_t(p.units) * p.NB * 4, st) != cudaSuccess ||
+      (p.dA_T && cudaMemsetAsync(p.XTmax, 0, size_t(p.units) * 4, st) != cudaSuccess)) {
+    cudaGetLastError();
+    return VLA_ERR_CUDA;
+  }
   const long long chunks = (long long)p.units * p.nch;
   const dim3 blocks(p.NB, p.units);
   prep<<<unsigned((chunks + Prep::WPC - 1) / Prep::WPC), Prep::WPC * 32, Prep::smem_bytes, st>>>(p);
   chains<<<2 * p.units, Chain::NT, Chain::smem_bytes, st>>>(p);
   if (p.dA_T) bwd_final_state_kernel<D><<<p.units, 256, 0, st>>>(p);
-  block<<<blocks, 256, Block::smem_bytes, st>>>(p);
+  block<<<blocks, Block::NT, Block::smem_bytes, st>>>(p);
   bwd_scan_kernel<D><<<dim3((D * D / 4 + D + 255) / 256, p.units), 256, 0, st>>>(p);
-  fin<<<blocks, 256, Fin::smem_bytes, st>>>(p);
+  fin<<<blocks, Fin::NT, Fin::smem_bytes, st>>>(p);
   return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
 }
 

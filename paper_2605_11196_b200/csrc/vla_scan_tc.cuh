@@ -38,10 +38,11 @@ namespace vla {
 
 // Unrolling, as measured: the chunk loop of the four roles is straight-line code that is fetched
 // anew every chunk, so code size counts.  The Gram loops stay fully unrolled (rolled: 5 KB less,
-// 25 % slower), the prep group's passes take two steps at a time (it has time to spare), the chunk
-// loops themselves are not unrolled (twice: same work, 40 % slower).
+// 25 % slower), the prep group's passes are rolled (it has time to spare; two steps at a time: 2 KB more), the
+// chunk loops themselves are not unrolled (twice: same work, 40 % slower).  Size shows in the slowest SMs first, which
+// are what a launch takes: 148 units x 2048 tokens, 87 KB 9540 .. 10350 clk per chunk over the SMs, 79 KB 9450 .. 9990.
 constexpr int kTcGramUnroll = 4;
-constexpr int kTcPrepUnroll = 2;
+constexpr int kTcPrepUnroll = 1;
 constexpr int kTcLoopUnroll = 1;
 // ---------------------------------------------------------------- configuration
 template <typename TIn>
@@ -181,12 +182,14 @@ __global__ void __launch_bounds__(TcCfg<TIn>::NT, 1) vla_scan_tc_kernel(
   const uint32_t wait_limit = p.wait_limit ? p.wait_limit : kWaitProbeLimit;
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     // one probe costs some 170 clk even when the phase is complete, a look at the abort flag
-    // 90 more: the common case (complete) pays for the probe only
-    if (mbar_try_wait(bar, parity)) return;
-    if (*abort_flag) return;
-    if (!mbar_wait_bounded(bar, parity, wait_limit)) {
-      *abort_flag = 1;
-      if (p.status) atomicCAS(p.status, 0, int(VLA_ERR_DEVICE_TIMEOUT));
+    // 90 more: the common case (complete) pays for the probe only.  A limit that runs out is reported
+    // when the CTA ends: with the report here the two dozen waits take 5 KB more code
+    uint32_t it = 0;
+    while (!mbar_try_wait(bar, parity)) {
+      if (++it > wait_limit || *abort_flag) {
+        *abort_flag = 1;
+        break;
+      }
     }
   };
 
@@ -945,6 +948,7 @@ __global__ void __launch_bounds__(TcCfg<TIn>::NT, 1) vla_scan_tc_kernel(
 #endif
   tc_fence_before();
   __syncthreads();
+  if (tid == 0 && *abort_flag && p.status) atomicCAS(p.status, 0, int(VLA_ERR_DEVICE_TIMEOUT));
   if (tid < 32) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(Cfg::TMEM_COLS) : "memory");

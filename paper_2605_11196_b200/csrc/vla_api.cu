@@ -8,7 +8,9 @@
 
 #include <cstdio>
 
+#include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
@@ -192,8 +194,8 @@ SeqParLayout seqpar_layout(size_t units, size_t T, size_t D, size_t P) {
   L.Astart = take(N * D * D * sizeof(float));
   L.zstart = take(N * D * sizeof(float));
   L.ST2 = take(2 * N * D * D * sizeof(float));
-  L.AT2 = take(2 * N * D * D * sizeof(float));
-  L.zT2 = take(2 * N * D * sizeof(float));
+  L.AT2 = take(N * D * D * sizeof(float));
+  L.zT2 = take(N * D * sizeof(float));
   L.wn = take(units * T * D * sizeof(float));
   L.Sstart = take(N * D * D * sizeof(float));
   L.M0 = take(units * D * D * sizeof(double));
@@ -201,30 +203,42 @@ SeqParLayout seqpar_layout(size_t units, size_t T, size_t D, size_t P) {
   return L;
 }
 
-// The sequence-parallel path runs a segment and its transfer scan in one three-group CTA at
-// d <= 64, and as two CTAs at d = 128 (where two states fill the register file).
-constexpr bool seqpar_tri(int d) { return d <= 64; }
-
-// Segments per unit: as many as fill the device with 2 * units * P scans, P a divisor of the
-// number of 16-token chunks, at least kSeqparMinTokens tokens per segment.  1 = not worth cutting.
+// Segments per unit: P a divisor of the number of 16-token chunks, at least kSeqparMinTokens tokens per segment,
+// whichever takes least by the measured rates.  1 = not worth cutting.
 constexpr int kSeqparMinTokens = 64;   // shortest segment worth its Gram matrix, inversion and correction
 int seqpar_choose_segments(int units, int T, int d, int dtype) {
   if (units <= 0 || T <= 0 || T % 16 != 0 || d < 32) return 1;
-  const int resident = vla::chunk_resident_ctas(d, dtype, seqpar_tri(d));
-  const int target = resident / ((seqpar_tri(d) ? 1 : 2) * units);
+  const int resident = vla::pair_resident_segments(d, dtype), sms = vla::device_sms();
+  if (resident <= 0 || sms <= 0) return 1;
+  // us.  A chunk of 16 tokens takes `lone` to `full` as the device fills with segments, waves of them beyond that;
+  // cutting costs `start` (Gram matrices, one inversion, launches), `combine` for each step from one
+  // segment's state to the next, `invert` for each segment of the launch and `token` for each token and unit (Gram
+  // matrices, corrections).  Uncut, the pair kernel takes `whole` up to a quarter of what is resident and `full` at all of it.
+  struct Rate { double whole, lone, full, start, combine, invert, token; };
+  const Rate r = d == 32 ? Rate{1.55, 1.7, 2.55, 35, 3.0, 0.05, 2.6e-4}
+               : d == 64 ? Rate{2.0, 2.2, 3.1, 120, 5.6, 0.25, 6.3e-4}
+                         : Rate{3.9, 4.2, 4.3, 430, 20.5, 1.0, 1.2e-3};
+  // (d = 64, us by segments, 1 = uncut: 1 unit x 16384 tokens 2035, 8: 439, 16: 338, 32: 363; 16 x 4096 531, 2: 427, 4: 357,
+  // 8: 383; 60 x 8192 1187, 2: 1580; 16 x 65536 8100, 8: 3677, 16: 3115, 32: 3362.  d = 32, 4 x 16384 1562, 16: 216, 32: 198,
+  // 64: 270.  d = 128, 8 x 32768 7900, 4: 2990, 8: 3176, 16: 2954; 12 x 8192 1963, 4: 1600.)
   const int nch = T / 16;
+  const double pairs = (d == 32 ? 2.0 : d == 64 ? 1.0 : 0.5) * sms;   // uncut units resident at a time
+  auto waves = [](double n, double room, double lone, double full, double from) {   // us per chunk
+    const double whole = std::floor(n / room), rest = n / room - whole;
+    return whole * full + (rest > 0 ? lone + (full - lone) * std::max(0.0, rest - from) / (1.0 - from) : 0.0);
+  };
+  double best_us = nch * waves(units, pairs, r.whole, r.full, 0.25);
   int best = 1;
-  for (int P = 2; P <= target && P <= nch; ++P)
-    if (nch % P == 0 && T / P >= kSeqparMinTokens) best = P;
-  // Uncut, the pair kernel takes 1.6, 2.0, 3.9 us per 16 tokens (d = 32, 64, 128) whatever the number of units here.  Cut,
-  // the Gram matrices, inversions and corrections cost a start and a share per token, and a segment with its
-  // transfer scan 5.8 us (9.9) per 16 tokens, 12 with two CTAs on an SM.  (d = 64, 16 units x 4096 tokens: 517 us
-  // uncut, 413 in 8; 32 units: 521 and 625 in 4; 8 units x 1024: 136 and 206; 16 units x 65536: 8100 and 3790.)
-  const double uncut = nch * (d == 32 ? 1.6 : d == 64 ? 2.0 : 3.9);
-  const bool shared_sm = (seqpar_tri(d) ? 1LL : 2LL) * units * best > vla::device_sms();
-  const double cut = (d == 128 ? 590.0 : 180.0) + (d == 128 ? 9.9 : shared_sm ? 12.0 : 5.8) * nch / best +
-                     (d == 128 ? 4e-3 : 1.2e-3) * double(units) * T;
-  if (cut >= uncut) return 1;
+  for (int P = 2; P <= nch && T / P >= kSeqparMinTokens; ++P) {
+    if (nch % P != 0 || 3LL * units * P > 0x7fffffffLL) continue;
+    const double n = double(units) * P;
+    const double us = r.start + r.combine * P + r.invert * n + r.token * double(units) * T +
+                      nch / P * waves(n, resident, r.lone, r.full, 0.0);
+    if (us < best_us) {
+      best_us = us;
+      best = P;
+    }
+  }
   return best;
 }
 
@@ -668,7 +682,7 @@ int vla_forward_seqpar(const void* q, const void* k, const void* v, float lambda
   if (P == 1)   // nothing to cut: the plain scan
     return vla_forward(q, k, v, lambda_, B, H, T, d_k, d_v, S0, A0, out, S_T, A_T, opts, stream);
   if (T % 16 != 0 || (T / 16) % P != 0) return VLA_ERR_INVALID_ARG;
-  if (2LL * units * P > 0x7fffffffLL) return VLA_ERR_INVALID_ARG;
+  if (3LL * units * P > 0x7fffffffLL) return VLA_ERR_INVALID_ARG;
   const SeqParLayout L = seqpar_layout(size_t(units), size_t(T), size_t(d_k), size_t(P));
   if (!workspace || workspace_bytes < L.total) return VLA_ERR_INVALID_ARG;
   unsigned char* w = reinterpret_cast<unsigned char*>(
@@ -689,8 +703,8 @@ int vla_forward_seqpar(const void* q, const void* k, const void* v, float lambda
   float* AT2 = reinterpret_cast<float*>(w + L.AT2);
   float* zT2 = reinterpret_cast<float*>(w + L.zT2);
 
-  // every segment and its transfer scan as one launch of 2N units of T / P tokens: a unit's
-  // segments are consecutive blocks of its [T, d] arrays, so the inputs need no copy
+  // every segment and its transfer scan as one launch of N units of T / P tokens, three CTAs each: a
+  // unit's segments are consecutive blocks of its [T, d] arrays, so the inputs need no copy
   ScanParams p;
   p.q = q; p.k = k; p.v = v; p.u = o.u;
   p.S0 = nullptr; p.A0 = sp.Astart; p.z0 = sp.zstart;
@@ -698,8 +712,7 @@ int vla_forward_seqpar(const void* q, const void* k, const void* v, float lambda
   p.S_T = reinterpret_cast<float*>(w + L.ST2); p.A_T = AT2; p.zT = zT2;
   p.status = o.status;
   p.lambda = lambda_; p.eps = o.eps;
-  // d <= 64: N CTAs of three warp groups; d = 128: 2N CTAs, the transfer scans second
-  p.T = T / P; p.units = seqpar_tri(d_k) ? N : 2 * N; p.n_main = N; p.flags = o.flags;
+  p.T = T / P; p.units = N; p.n_main = N; p.flags = o.flags;
   p.refresh_period = 0; p.refresh_eta = 0.0f; p.step_offset = 0; p.u_is_khat = 0;
   p.stash_z = nullptr; p.stash_e = nullptr; p.stash_delta = nullptr; p.stash_zk = nullptr; p.stash_a = nullptr;
   p.heads = H;
@@ -707,8 +720,7 @@ int vla_forward_seqpar(const void* q, const void* k, const void* v, float lambda
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   rc = vla::seqpar_before_scan(d_k, o.qkv_dtype, sp, st);
   if (rc != VLA_OK) return rc;
-  rc = seqpar_tri(d_k) ? vla::launch_chunk_tri(d_k, o.qkv_dtype, p, st)
-                       : vla::launch_chunk(d_k, o.qkv_dtype, p, st);
+  rc = vla::launch_pair(d_k, o.qkv_dtype, p, nullptr, st);
   if (rc != VLA_OK) return rc;
   return vla::seqpar_after_scan(d_k, sp, A_T, o.zT, AT2, zT2, st);
 }

@@ -20,9 +20,8 @@ int launch_chunk_um_tm(const ScanParams& p, cudaStream_t st) {
   using Cfg = ChunkCfg<D, TIn, UM>;
   static_assert(Cfg::smem_bytes <= 227 * 1024, "chunk kernel exceeds the shared memory of one CTA");
   constexpr bool BAL = !(STASH && TM);
-  auto kern = vla_scan_chunk_kernel<D, TIn, false, UM, false, STASH, TM>;     // one CTA per unit
-  auto kern_bal = vla_scan_chunk_kernel<D, TIn, BAL, UM, false, STASH, TM>;   // persistent grid, units cut at chunks
-  if (TM && p.n_main > 0) return VLA_ERR_UNSUPPORTED;
+  auto kern = vla_scan_chunk_kernel<D, TIn, false, UM, STASH, TM>;     // one CTA per unit
+  auto kern_bal = vla_scan_chunk_kernel<D, TIn, BAL, UM, STASH, TM>;   // persistent grid, units cut at chunks
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            int(Cfg::smem_bytes)) != cudaSuccess ||
       cudaFuncSetAttribute(kern_bal, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -52,7 +51,7 @@ int launch_chunk_um_tm(const ScanParams& p, cudaStream_t st) {
     const int resident = sms * per_sm;
     const bool state_out = p.S_T && p.A_T && (p.zT || (p.flags & VLA_FLAG_IDENTITY_MAP));
     if (BAL && resident > 0 && p.units > resident && p.units % resident != 0 && p.T > 0 && state_out &&
-        p.units <= kSchedMaxUnits && p.n_main <= 0) {
+        p.units <= kSchedMaxUnits) {
       // the flag slot of this launch id must not still be in use by an earlier launch that may
       // overlap this one on the device (another stream): then the plain grid runs instead
       const unsigned int epoch = next_launch_epoch();
@@ -111,64 +110,6 @@ int launch_chunk_t(const ScanParams& p, cudaStream_t st) {
   return launch_chunk_um<D, TIn, kUKhat>(p, st);
 }
 
-// Three warp groups per CTA (sequence-parallel launches at d <= 64): one CTA per segment runs
-// the segment and its transfer scan on one pass of group A.  p.units CTAs, p.n_main == p.units.
-template <int D, typename TIn, int UM>
-int launch_chunk_tri_um(const ScanParams& p, cudaStream_t st) {
-  using Cfg = ChunkCfg<D, TIn, UM, true>;
-  static_assert(Cfg::smem_bytes <= 227 * 1024, "chunk kernel exceeds the shared memory of one CTA");
-  auto kern = vla_scan_chunk_kernel<D, TIn, false, UM, true>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(Cfg::smem_bytes)) != cudaSuccess) {
-    cudaGetLastError();
-    return VLA_ERR_CUDA;
-  }
-  SchedParams sp;
-  sp.balanced = 0;
-  sp.grid = p.units;
-  sp.epoch = 0;
-  kern<<<p.units, Cfg::NT, Cfg::smem_bytes, st>>>(p, sp, EmptyMaps{0});
-  note_launch("vla_scan_chunk_kernel(three groups)", D, sizeof(TIn) == 2 ? VLA_BF16 : VLA_F32, p.units, 0);
-  return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
-}
-
-template <int D, typename TIn>
-int launch_chunk_tri_t(const ScanParams& p, cudaStream_t st) {
-  if constexpr (D <= 64) {
-    if (p.refresh_period > 0) return VLA_ERR_UNSUPPORTED;
-    if (p.u) return launch_chunk_tri_um<D, TIn, kUTensor>(p, st);
-    return launch_chunk_tri_um<D, TIn, kUKhat>(p, st);
-  } else {
-    return VLA_ERR_UNSUPPORTED;
-  }
-}
-
-template <int D, typename TIn, bool TRI>
-int chunk_resident_ctas_t() {
-  using Cfg = ChunkCfg<D, TIn, kUKhat, TRI>;
-  auto kern = vla_scan_chunk_kernel<D, TIn, false, kUKhat, TRI>;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Cfg::smem_bytes));
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Cfg::NT, Cfg::smem_bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return sms * per_sm;
-}
-
-template <int D, typename TIn>
-int chunk_resident_t(bool tri) {
-  if constexpr (D <= 64) {
-    if (tri) return chunk_resident_ctas_t<D, TIn, true>();
-  }
-  return chunk_resident_ctas_t<D, TIn, false>();
-}
-
 }  // namespace vla
 
 // The entry points of one (d, input type): the forward kernels in one translation unit, the
@@ -176,10 +117,6 @@ int chunk_resident_t(bool tri) {
 #define VLA_DEFINE_CHUNK_TU(D, TIN, TAG)                                                        \
   namespace vla {                                                                               \
   int launch_chunk_##TAG(const ScanParams& p, cudaStream_t st) { return launch_chunk_t<D, TIN>(p, st); } \
-  int launch_chunk_tri_##TAG(const ScanParams& p, cudaStream_t st) {                            \
-    return launch_chunk_tri_t<D, TIN>(p, st);                                                   \
-  }                                                                                             \
-  int chunk_resident_##TAG(bool tri) { return chunk_resident_t<D, TIN>(tri); }                  \
   }
 #define VLA_DEFINE_CHUNK_STASH_TU(D, TIN, TAG)                                                  \
   namespace vla {                                                                               \

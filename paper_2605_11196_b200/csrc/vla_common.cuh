@@ -32,12 +32,12 @@ struct ScanParams {
   float refresh_eta;
   long long step_offset;     // tokens processed before this call
   int u_is_khat;             // token kernel, two-exchange path: use u = k_hat although no u was given
-  // Sequence-parallel scans (chunk kernel only).  With n_main > 0, units [n_main, units) are
-  // "transfer" scans: unit x reads q, k, u, A0, z0 of unit x - n_main, takes v = 0 and
-  // S0 = I, and writes its readout to out2 instead of out; its S_T is then the product of
-  // the segment's right-acting maps I - k_hat alpha^T.  n_main <= 0: no such units.
+  // Sequence-parallel scans (pair kernel only).  With n_main > 0 (= units) every unit, a segment started from
+  // S = 0, has a "transfer" scan beside it: the same q, k, u, A0, z0, but v = 0 and S0 = I.  It writes its
+  // readout to out2 and its final state n_main units further in S_T, where it is the product of the
+  // segment's right-acting maps I - k_hat alpha^T.  n_main <= 0: no such scans.
   int n_main;
-  float* out2;               // [units - n_main, T, D]
+  float* out2;               // [n_main, T, D]
   // Backward pass (chunk kernel, u = k_hat path): per-token z_t, e_t [units, T, D] and delta_t
   // [units, T] of the forward recurrence are left here; nullptr: not wanted.  With a stash the
   // readout may be dropped (out == nullptr).

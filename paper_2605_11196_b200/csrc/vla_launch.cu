@@ -16,8 +16,6 @@ namespace vla {
 
 #define VLA_DECLARE_CHUNK_TU(TAG)                                   \
   int launch_chunk_##TAG(const ScanParams& p, cudaStream_t st);     \
-  int launch_chunk_tri_##TAG(const ScanParams& p, cudaStream_t st); \
-  int chunk_resident_##TAG(bool tri);                               \
   int launch_chunk_stash_##TAG(const ScanParams& p, cudaStream_t st);
 VLA_DECLARE_CHUNK_TU(d32_f32)
 VLA_DECLARE_CHUNK_TU(d32_bf16)
@@ -43,19 +41,9 @@ int launch_chunk(int d, int dtype, const ScanParams& p, cudaStream_t st) {
   return VLA_ERR_UNSUPPORTED;
 }
 
-int launch_chunk_tri(int d, int dtype, const ScanParams& p, cudaStream_t st) {
-  VLA_CHUNK_DISPATCH(launch_chunk_tri, p, st);
-  return VLA_ERR_UNSUPPORTED;
-}
-
 int launch_chunk_stash(int d, int dtype, const ScanParams& p, cudaStream_t st) {
   VLA_CHUNK_DISPATCH(launch_chunk_stash, p, st);
   return VLA_ERR_UNSUPPORTED;
-}
-
-int chunk_resident_ctas(int d, int dtype, bool tri) {
-  VLA_CHUNK_DISPATCH(chunk_resident, tri);
-  return 0;
 }
 
 bool set_smem_once(std::atomic<unsigned long long>& done, const void* kern, size_t bytes) {
@@ -92,7 +80,9 @@ int device_sms() {
   return n;
 }
 
-#define VLA_DECLARE_PAIR_TU(TAG) int launch_pair_##TAG(const ScanParams& p, const PairStash* sh, cudaStream_t st);
+#define VLA_DECLARE_PAIR_TU(TAG)                                                       \
+  int launch_pair_##TAG(const ScanParams& p, const PairStash* sh, cudaStream_t st); \
+  int pair_resident_segments_##TAG();
 VLA_DECLARE_PAIR_TU(d16_f32)
 VLA_DECLARE_PAIR_TU(d16_bf16)
 VLA_DECLARE_PAIR_TU(d32_f32)
@@ -118,6 +108,26 @@ int launch_bwd_chunk(int d, int dtype, const BwdChunkParams& p, cudaStream_t st)
   if (d == 16) return dtype == VLA_F32 ? launch_bwd_chunk_d16_f32(p, st) : launch_bwd_chunk_d16_bf16(p, st);
   VLA_CHUNK_DISPATCH(launch_bwd_chunk, p, st);
   return VLA_ERR_UNSUPPORTED;
+}
+
+int pair_resident_segments(int d, int dtype) {
+  // (asked once per device, width and type: the answer costs some 10 us)
+  static std::atomic<int> known[64][3][2];
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return 0;
+  }
+  std::atomic<int>& slot = known[dev][d == 32 ? 0 : d == 64 ? 1 : 2][dtype == VLA_F32 ? 0 : 1];
+  int n = slot.load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  auto ask = [&]() {
+    VLA_CHUNK_DISPATCH(pair_resident_segments);
+    return 0;
+  };
+  n = ask();
+  slot.store(n, std::memory_order_relaxed);
+  return n;
 }
 
 int launch_pair(int d, int dtype, const ScanParams& p, const PairStash* sh, cudaStream_t st) {

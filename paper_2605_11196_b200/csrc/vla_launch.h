@@ -39,6 +39,9 @@ int launch_decode(int d, int dtype, const ScanParams& p, cudaStream_t st);
 // explicit, no refresh; sh: what a backward pass wants left behind, or nullptr.
 int launch_pair(int d, int dtype, const ScanParams& p, const PairStash* sh, cudaStream_t st);
 
+// Segments of a cut sequence that the current device holds at a time, d in {32, 64, 128}; 0 on a failure.
+int pair_resident_segments(int d, int dtype);
+
 // Chunk kernel, d in {32, 64, 128}: plain or balanced grid, chosen from the shape.
 int launch_chunk(int d, int dtype, const ScanParams& p, cudaStream_t st);
 
@@ -49,12 +52,6 @@ int launch_chunk_tc(int d, int dtype, const ScanParams& p, cudaStream_t st);
 int launch_chunk_stash(int d, int dtype, const ScanParams& p, cudaStream_t st);
 // The tensor-core form of the same (d = 128, u = k_hat, no refresh).
 int launch_chunk_tc_stash(int d, int dtype, const ScanParams& p, cudaStream_t st);
-
-// Chunk kernel with three warp groups per CTA (d in {32, 64}; sequence-parallel launches).
-int launch_chunk_tri(int d, int dtype, const ScanParams& p, cudaStream_t st);
-
-// CTAs of the chunk kernel (u = k_hat variant) that the current device holds at a time.
-int chunk_resident_ctas(int d, int dtype, bool tri);
 
 // Sequence-parallel helpers: Gram matrices + inversion before the scan, combination +
 // correction + final-state copies after it.

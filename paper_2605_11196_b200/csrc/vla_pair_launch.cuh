@@ -7,17 +7,17 @@
 
 namespace vla {
 
-template <int D, typename TIn, bool UT, bool STASH>
+template <int D, typename TIn, bool UT, bool STASH, int NS = 1>
 int launch_pair_t(const ScanParams& p, const PairStash& sh, cudaStream_t st) {
   using Cfg = PairCfg<D, TIn, UT>;
   static_assert(Cfg::smem_bytes <= 227 * 1024, "pair kernel exceeds the shared memory of one CTA");
-  if (p.units > 0x3fffffff) return VLA_ERR_INVALID_ARG;
-  auto kern = vla_scan_pair_kernel<D, TIn, UT, STASH>;
+  if (p.units > 0x7fffffff / (1 + NS)) return VLA_ERR_INVALID_ARG;
+  auto kern = vla_scan_pair_kernel<D, TIn, UT, STASH, NS>;
   static std::atomic<unsigned long long> done{0};
   if (!set_smem_once(done, reinterpret_cast<const void*>(kern), Cfg::smem_bytes)) return VLA_ERR_CUDA;
-  const int grid = STASH ? p.units : 2 * p.units;
+  const int grid = STASH ? p.units : (1 + NS) * p.units;
   kern<<<grid, Cfg::NT, Cfg::smem_bytes, st>>>(p, sh);
-  note_launch(STASH ? "vla_scan_pair_kernel(stash)" : "vla_scan_pair_kernel", D, sizeof(TIn) == 2 ? VLA_BF16 : VLA_F32,
+  note_launch(STASH ? "vla_scan_pair_kernel(stash)" : NS == 2 ? "vla_scan_pair_kernel(segments)" : "vla_scan_pair_kernel", D, sizeof(TIn) == 2 ? VLA_BF16 : VLA_F32,
               grid, 0);
   return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
 }
@@ -25,14 +25,43 @@ int launch_pair_t(const ScanParams& p, const PairStash& sh, cudaStream_t st) {
 template <int D, typename TIn>
 int launch_pair_any(const ScanParams& p, const PairStash* sh, cudaStream_t st) {
   const PairStash none = {};
+  if constexpr (D >= 32) {   // the segments of a cut sequence with their transfer scans
+    if (p.n_main > 0) return p.u ? launch_pair_t<D, TIn, true, false, 2>(p, none, st) : launch_pair_t<D, TIn, false, false, 2>(p, none, st);
+  }
   if (sh) return p.u ? launch_pair_t<D, TIn, true, true>(p, *sh, st) : launch_pair_t<D, TIn, false, true>(p, *sh, st);
   return p.u ? launch_pair_t<D, TIn, true, false>(p, none, st) : launch_pair_t<D, TIn, false, false>(p, none, st);
+}
+
+// Segments of a cut sequence (clusters of three) that the current device holds at a time; 0: cannot tell.
+template <int D, typename TIn>
+int pair_resident_segments_t() {
+  if constexpr (D >= 32) {
+    using Cfg = PairCfg<D, TIn, false>;
+    auto kern = vla_scan_pair_kernel<D, TIn, false, false, 2>;
+    static std::atomic<unsigned long long> done{0};
+    if (!set_smem_once(done, reinterpret_cast<const void*>(kern), Cfg::smem_bytes)) return 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(3);
+    cfg.blockDim = dim3(Cfg::NT);
+    cfg.dynamicSmemBytes = Cfg::smem_bytes;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 3;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess) return n;
+    cudaGetLastError();
+  }
+  return 0;
 }
 
 }  // namespace vla
 
 #define VLA_DEFINE_PAIR_TU(D, TIN, TAG)                                                          \
   namespace vla {                                                                                \
+  int pair_resident_segments_##TAG() { return pair_resident_segments_t<D, TIN>(); }              \
   int launch_pair_##TAG(const ScanParams& p, const PairStash* sh, cudaStream_t st) {             \
     return launch_pair_any<D, TIN>(p, sh, st);                                                   \
   }                                                                                              \

@@ -53,7 +53,7 @@ struct ChunkTile {
 //             which A_t k_hat_t is no longer parallel to z_t; one product with A per chunk
 enum : int { kUKhat = 0, kUTensor = 1, kUKhatGen = 2 };
 
-template <int D, typename TIn, int UM = kUKhat, bool TRI = false>
+template <int D, typename TIn, int UM = kUKhat>
 struct ChunkCfg {
   static constexpr bool GEN = UM != kUKhat;      // general path
   static constexpr bool UT = UM == kUTensor;     // a fourth input tensor
@@ -63,18 +63,15 @@ struct ChunkCfg {
   static constexpr int LPR = D / TW;             // lanes that share a row block (== TR)
   static constexpr int NV = TW / 4;              // float4 operand groups per thread
   static constexpr int NG = D;                   // threads per warp group
-  static constexpr int NGROUPS = TRI ? 3 : 2;    // A, S [, transfer scan]
+  static constexpr int NGROUPS = 2;              // A, S
   // d <= 64: group A is one or two warps, and widening the next chunk's inputs around the
-  // factorisation was an eighth to a fifth of its chain; there a warp of its own does it (not in
-  // the three-group kernel at d = 64, whose two CTAs per SM leave it no registers)
-  static constexpr bool PREPW = D == 32 || (D == 64 && !TRI);
+  // factorisation was an eighth to a fifth of its chain; there a warp of its own does it
+  static constexpr bool PREPW = D <= 64;
   static constexpr int NT = NGROUPS * D + (PREPW ? 32 : 0);   // threads per CTA
   static constexpr int NWG = D / 32;             // warps per group
   static constexpr int NIN = UT ? 4 : 3;         // q, k, v[, u]
   // raw q/k/v[/u] chunks in flight (fewer on the general path: shared memory is the limit)
-  // (the three-group kernel with 16-bit inputs keeps one stage: two of its CTAs then share an SM)
-  static constexpr int NSTAGE = TRI ? (sizeof(TIn) == 2 ? 1 : 2)
-                                    : UT ? (sizeof(TIn) == 2 ? 2 : 1) : (sizeof(TIn) == 2 ? 4 : 2);
+  static constexpr int NSTAGE = UT ? (sizeof(TIn) == 2 ? 2 : 1) : (sizeof(TIn) == 2 ? 4 : 2);
   static constexpr int RING = 2;                 // Z / Gu / HT / sc slots (group A -> group S)
   static constexpr int KRING = 3;                // widened k_hat / q_f / v / ||phi(k)|| slots
   static constexpr int CP = C + 4;               // padded row of the small C x C matrices
@@ -249,28 +246,22 @@ __device__ __forceinline__ void gram16(const float* X, const float* Y, float* G,
 // (512 units on 148 SMs: 3.46 segments of work per SM instead of 4).
 static __device__ unsigned int g_sched_flags[kSchedSlots * kSchedMaxUnits];
 
-// TRI: a third warp group runs the segment's transfer scan (S from I, v = 0; sequence-parallel
-// launches at d <= 64) next to group S, on the same products of group A.  Its readout goes to
-// out2 and its final state to S_T[n_main + unit].
 // STASH: the launch also leaves z_t, e_t, delta_t of every token in global memory (and may
 // drop the readout) for the backward pass; a separate instantiation so that the plain forward
 // kernel carries none of it.
 // TM: q, k, v, u, out are [B, T, H, d]: the 16 rows of a chunk are H * d apart, so they move as
 // one tiled TMA request per array (box d x 1 x 16 x 1 of the 4-d tensor) through the tensor maps
 // in `maps`; the head-major instantiations take an empty struct there.
-template <int D, typename TIn, bool BALANCED, int UM, bool TRI = false, bool STASH = false, bool TM = false>
-__global__ void __launch_bounds__((ChunkCfg<D, TIn, UM, TRI>::NT), (TRI && sizeof(TIn) == 2) ? 2 : 1)
+template <int D, typename TIn, bool BALANCED, int UM, bool STASH = false, bool TM = false>
+__global__ void __launch_bounds__((ChunkCfg<D, TIn, UM>::NT), 1)
 vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
                       const __grid_constant__ typename ChunkMapsArg<TM>::type maps) {
-  using Cfg = ChunkCfg<D, TIn, UM, TRI>;
-  static_assert(!TM || !TRI, "token-major tensors: not with the three-group kernel");
+  using Cfg = ChunkCfg<D, TIn, UM>;
   static_assert(!TM || (Cfg::raw_bytes + sizeof(float) * (Cfg::KRING * Cfg::kslot_floats + Cfg::RING * Cfg::slot_floats +
                                                           Cfg::a_floats + 3 * Cfg::C * D)) % 128 == 0,
                 "the out stage must be 128-byte aligned for a tiled TMA store");
-  static_assert(!TRI || (D <= 64 && !BALANCED), "three groups: d <= 64, one CTA per unit");
-  static_assert(!STASH || !TRI, "the stash: not with the three-group kernel");
   constexpr bool HAS_U = Cfg::GEN;   // general path: a_t = A_t k_hat_t formed explicitly
-  constexpr bool kUnrollMatvec = D == 64 && !TRI;
+  constexpr bool kUnrollMatvec = D == 64;
   constexpr bool UT = Cfg::UT;       // u comes from the caller's tensor
   constexpr int NIN = Cfg::NIN;
   constexpr int C = Cfg::C, TW = Cfg::TW, TR = Cfg::TR, LPR = Cfg::LPR, NV = Cfg::NV;
@@ -305,8 +296,8 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
   // shuffles inside them compile to plain shuffles.  Taken as divergent code they are several
   // times longer, and the chunk loop then overflows the instruction cache.
   const int warp_u = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);
-  const int grp = warp_u / (Cfg::NG / 32);   // 0: A, 1: S, 2: transfer scan (TRI)
-  float* sbase = abase + Cfg::a_floats + (grp == 2 ? Cfg::s_floats : 0);
+  const int grp = warp_u / (Cfg::NG / 32);   // 0: A, 1: S
+  float* sbase = abase + Cfg::a_floats;
   float* VS = sbase;                // [C][D]  B = V^T - S K^T
   float* R0s = VS + C * D;          // [C][D]
   float* Eps = R0s + C * D;         // [C][D]
@@ -368,12 +359,6 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
 #pragma unroll 1
   for (int pi = 0; get_piece<BALANCED>(sp, p.units, nch_unit, blockIdx.x, pi, pc); ++pi) {
   const int unit = pc.unit;
-  // transfer scan of a sequence-parallel launch: inputs of unit `uin`, v = 0, S0 = I
-  // TRI: the third group is the transfer scan of this very unit; otherwise transfer scans are
-  // the CTAs of units >= n_main
-  const bool pscan_cta = !TRI && p.n_main > 0 && unit >= p.n_main;
-  const bool pscan = TRI ? (grp == 2) : pscan_cta;
-  const int uin = pscan_cta ? unit - p.n_main : unit;
   const int t_begin = pc.cb * C;
   const int T = min(p.T, pc.ce * C) - t_begin;   // tokens of this piece
   const int nchunks = pc.ce - pc.cb;
@@ -390,16 +375,16 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
     const uint32_t bytes = uint32_t(n) * D * sizeof(TIn);
     TIn* dst = raw + size_t(s) * NIN * C * D;
     if constexpr (!TM) {
-      mbar_arrive_expect_tx(&full[s], (pscan_cta ? NIN - 1 : NIN) * bytes);
-      const size_t tok = size_t(uin) * size_t(p.T) + size_t(t_begin) + size_t(c) * C;
+      mbar_arrive_expect_tx(&full[s], NIN * bytes);
+      const size_t tok = size_t(unit) * size_t(p.T) + size_t(t_begin) + size_t(c) * C;
       bulk_load(dst + 0 * C * D, static_cast<const TIn*>(p.q) + tok * D, bytes, &full[s]);
       bulk_load(dst + 1 * C * D, static_cast<const TIn*>(p.k) + tok * D, bytes, &full[s]);
-      if (!pscan_cta) bulk_load(dst + 2 * C * D, static_cast<const TIn*>(p.v) + tok * D, bytes, &full[s]);
+      bulk_load(dst + 2 * C * D, static_cast<const TIn*>(p.v) + tok * D, bytes, &full[s]);
       if (UT) bulk_load(dst + 3 * C * D, static_cast<const TIn*>(p.u) + tok * D, bytes, &full[s]);
     } else {
       // [B, T, H, d] tensors: one tiled request per array; rows past T arrive as zeros and
       // count towards the bytes like any other
-      const int b = uin / p.heads, h = uin - b * p.heads, t0 = t_begin + c * C;
+      const int b = unit / p.heads, h = unit - b * p.heads, t0 = t_begin + c * C;
       mbar_arrive_expect_tx(&full[s], NIN * uint32_t(C * D * sizeof(TIn)));
       tma_load_4d(dst + 0 * C * D, &maps.q, 0, h, t0, b, &full[s]);
       tma_load_4d(dst + 1 * C * D, &maps.k, 0, h, t0, b, &full[s]);
@@ -454,8 +439,7 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
   if (!is_P) {
     // a tail piece continues from the state its head left in the caller's output buffers
     // (written by another SM: read past L1)
-    const float* src = from_handoff ? (is_A ? p.A_T : p.S_T) : (is_A ? p.A0 : (pscan ? nullptr : p.S0));
-    const int usrc = from_handoff ? unit : uin;   // a transfer-scan CTA reads the A0 of its partner
+    const float* src = from_handoff ? (is_A ? p.A_T : p.S_T) : (is_A ? p.A0 : p.S0);
 #pragma unroll
     for (int r = 0; r < TR; ++r) {
       const int row = rb * TR + r;
@@ -464,9 +448,9 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
         const int c4 = m * LPR + cg;
         float4 x;
         if (src) {
-          x = __ldcg(reinterpret_cast<const float4*>(src + (size_t(usrc) * D + row) * D) + c4);
+          x = __ldcg(reinterpret_cast<const float4*>(src + (size_t(unit) * D + row) * D) + c4);
         } else {
-          const float dg = is_A ? 1.0f / p.lambda : (pscan ? 1.0f : 0.0f);
+          const float dg = is_A ? 1.0f / p.lambda : 0.0f;
           x.x = (c4 * 4 + 0 == row) ? dg : 0.0f;
           x.y = (c4 * 4 + 1 == row) ? dg : 0.0f;
           x.z = (c4 * 4 + 2 == row) ? dg : 0.0f;
@@ -511,7 +495,7 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
         if (act) {
           kf[i] = load4(rk + tt * D, f);
           qf = load4(rq + tt * D, f);
-          if (!pscan_cta) vv = load4(rv + tt * D, f);
+          vv = load4(rv + tt * D, f);
           if (!ident) {
             kf[i].x = phi_fast(kf[i].x); kf[i].y = phi_fast(kf[i].y);
             kf[i].z = phi_fast(kf[i].z); kf[i].w = phi_fast(kf[i].w);
@@ -566,7 +550,7 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
     if (from_handoff) {
       if (p.zT) zk = __ldcg(p.zT + size_t(unit) * D + g);
     } else if (p.z0) {
-      zk = p.z0[size_t(uin) * D + g];
+      zk = p.z0[size_t(unit) * D + g];
     }
 
     // Periodic refresh (general path): ph = tokens since the last refresh boundary
@@ -885,7 +869,7 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
 
       // ---- B = V^T - S K^T and R0 = S Q^T, row g of each
       tile_matvec_chunk<TR, TW, LPR, D, C, kUnrollMatvec>(st, Kh, cg, [&](int t, float x) {
-        VS[t * D + g] = (TRI && pscan ? 0.0f : Vf[t * D + g]) - x;
+        VS[t * D + g] = Vf[t * D + g] - x;
       });
       tile_matvec_chunk<TR, TW, LPR, D, C, kUnrollMatvec>(st, Qf, cg, [&](int t, float x) { R0s[t * D + g] = x; });
       if (g == 0) bulk_wait_read<1>();  // the out stage of chunk c-2 has left shared memory
@@ -968,13 +952,12 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
       group_bar(sbar, NG);  // Eps and the out stage complete
       if (g == 0) {
         const size_t tq = size_t(t_begin) + size_t(c) * C;
-        float* odst = pscan ? p.out2 : p.out;
-        if (!STASH || odst) {   // a backward pass that only wants the stash passes no readout buffer
+        if (!STASH || p.out) {   // a backward pass that only wants the stash passes no readout buffer
           if constexpr (!TM) {
-            bulk_store(odst + (size_t(uin) * size_t(p.T) + tq) * D, ostage + size_t(c & 1) * C * D,
+            bulk_store(p.out + (size_t(unit) * size_t(p.T) + tq) * D, ostage + size_t(c & 1) * C * D,
                        uint32_t(n) * D * sizeof(float));
           } else {   // rows past T are clipped by the tensor map
-            const int b = uin / p.heads, h = uin - b * p.heads;
+            const int b = unit / p.heads, h = unit - b * p.heads;
             tma_store_4d(&maps.out, 0, h, int(tq), b, ostage + size_t(c & 1) * C * D);
           }
           bulk_commit();
@@ -995,7 +978,7 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
         const int row = rb * TR + r;
 #pragma unroll
         for (int m = 0; m < NV; ++m)
-          reinterpret_cast<float4*>(p.S_T + (size_t(TRI && pscan ? unit + p.n_main : unit) * D + row) * D)[m * LPR + cg] =
+          reinterpret_cast<float4*>(p.S_T + (size_t(unit) * D + row) * D)[m * LPR + cg] =
               make_float4(st[r][2 * m].x, st[r][2 * m].y, st[r][2 * m + 1].x, st[r][2 * m + 1].y);
       }
     }

@@ -14,6 +14,10 @@
 // S row is independent of the others.  Beside the D / 16 state warps a CTA has one warp for the
 // 16 x 16 algebra and one or two that widen the inputs (phi, k_hat, hi/lo operand rows) one chunk ahead.
 //
+// A segment of a cut sequence takes a third CTA (NS = 2): rank 2 carries the segment's transfer scan on the same
+// alpha.  d = 64, 16 units x 65536 tokens in 16 segments: scan 2.92 -> 2.2 ms against the FMA chunk kernel, where the
+// two scans shared one CTA with A (6 us of an SM per 16 tokens of a segment; three CTAs here, two on an SM: 4.7).
+
 // What bounds it: at one unit per SM pair the serial chain of rank 0 (state split, Z0, W, the
 // 16 x 16 elimination, Z, update), with many units the tensor pipe (8 clk per instruction and
 // scheduler).  Two CTAs because at d = 128 both states and their operands do not fit one SM's
@@ -86,8 +90,10 @@ __device__ __forceinline__ void tok_store4(uint32_t base, int row, int pl, float
   sts64(at + 2 * D, l0, l1);
 }
 
-template <int D, typename TIn, bool UT, bool STASH>
-__global__ void __cluster_dims__(STASH ? 1 : 2, 1, 1) __launch_bounds__((PairCfg<D, TIn, UT>::NT), (PairCfg<D, TIn, UT>::MINB))
+// NS: CTAs that carry an S.  2 (the segments of a cut sequence): rank 1 the segment from S = 0, rank 2 its
+// transfer scan (S = I, v = 0, readout to out2, final state n_main units further), one A for both.
+template <int D, typename TIn, bool UT, bool STASH, int NS>
+__global__ void __cluster_dims__(STASH ? 1 : 1 + NS, 1, 1) __launch_bounds__((PairCfg<D, TIn, UT>::NT), (PairCfg<D, TIn, UT>::MINB))
 vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
   using Cfg = PairCfg<D, TIn, UT>;
   constexpr int C = Cfg::C, NW = Cfg::NW, NPREP = Cfg::NPREP, LPT = Cfg::LPT, TPW = Cfg::TPW, NP = Cfg::NP;
@@ -97,8 +103,8 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
 
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t sb = smem_u32(smem);
-  const uint32_t rank = STASH ? 0u : blockIdx.x & 1u;   // (of the cluster; from the block index, which the compiler knows to be uniform)
-  const int unit = int(STASH ? blockIdx.x : blockIdx.x >> 1);
+  const uint32_t rank = STASH ? 0u : blockIdx.x % (1u + NS);   // (of the cluster; from the block index, which the compiler knows to be uniform)
+  const int unit = int(STASH ? blockIdx.x : blockIdx.x / (1u + NS));
   const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
   // read from lane 0 so that the compiler takes the roles as uniform over a warp
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -148,7 +154,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     mbar_init(&pfull[1], 1);
     for (int i = 0; i < RA; ++i) {
       mbar_init(&afull[i], 1);
-      mbar_init(&aempty[i], NW + 1);
+      mbar_init(&aempty[i], NS * (NW + 1));
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&gfull[i], 1);
@@ -169,7 +175,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     // together has to stay inside the SM's instruction cache.)
     const int pw = warp - NW - 1, sub = lane / LPT, pl = lane % LPT;
     const TIn* src0 = static_cast<const TIn*>(p.k) + tok0 + 4 * pl;
-    const bool two = UT || rank == 1, sums = STASH || rank == 1;   // sums: this side carries the key sum
+    const bool two = UT || rank != 0, sums = STASH || rank != 0;   // sums: this side carries the key sum
     const TIn* src1 = two ? static_cast<const TIn*>(rank ? p.q : p.u) + tok0 + 4 * pl : src0;
     float* fs = reinterpret_cast<float*>(smem + (rank ? Cfg::s_f : Cfg::a_f));
     const uint32_t base0 = sb + (rank ? Cfg::s_K : Cfg::a_K), base1 = sb + (rank ? Cfg::s_Q : Cfg::a_U);
@@ -212,7 +218,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         if (two) x = piece_f32(raw + 128);
         if (!ident) {
           k.x = phi_fast(k.x); k.y = phi_fast(k.y); k.z = phi_fast(k.z); k.w = phi_fast(k.w);
-          if (rank == 1) {
+          if (rank != 0) {
             x.x = phi_fast(x.x); x.y = phi_fast(x.y); x.z = phi_fast(x.z); x.w = phi_fast(x.w);
           }
         }
@@ -234,7 +240,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           tok_store4<D>(base1 + slot * Cfg::kslot, tt, pl, x, s);
           if (pl == 0) fs[(rank ? Cfg::sf_qs : Cfg::af_us) + slot * 16 + tt] = pow2_inverse(s);
         }
-        if (rank == 1 && pl == 0) {
+        if (rank != 0 && pl == 0) {
           fs[Cfg::sf_nrm + slot * 16 + tt] = act ? nr : 0.f;
           fs[Cfg::sf_dq + slot * 16 + tt] = dn;
         }
@@ -261,7 +267,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       arrive(&kfull[slot]);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    if (sums && p.zT && pw == 0 && sub == 0)
+    if (sums && rank < 2 && p.zT && pw == 0 && sub == 0)
       *reinterpret_cast<float4*>(p.zT + size_t(unit) * D + 4 * pl) = make_float4(zk[0], zk[1], zk[2], zk[3]);
   } else if (rank == 0 && warp == NW) {
     // ===================================================================== rank 0: elimination
@@ -358,7 +364,6 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     float* mxs = fs + Cfg::af_mx;
     const int row0 = 16 * warp;
     const uint32_t my_rows = uint32_t(row0 + g) * kVecRow + 4 * c4;
-    const uint32_t remote_A = STASH ? 0u : map_to_rank(sb + Cfg::s_A, 1);
     float st[NTILE][4];
     float sA, sAi;                   // st = sA * A
     {
@@ -425,9 +430,12 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           vec_store(stage + my_rows, al);
           fence_async_smem();
           __syncwarp();
-          if (lane == 0 && !*abort_flag)
-            bulk_to_cluster(remote_A + as * Cfg::aslot + row0 * kVecRow, stage + row0 * kVecRow, 16 * kVecRow,
-                            map_to_rank(smem_u32(&afull[as]), 1));
+          if (lane == 0 && !*abort_flag) {
+#pragma unroll
+            for (int to = 1; to <= NS; ++to)
+              bulk_to_cluster(map_to_rank(sb + Cfg::s_A, to) + as * Cfg::aslot + row0 * kVecRow, stage + row0 * kVecRow, 16 * kVecRow,
+                              map_to_rank(smem_u32(&afull[as]), to));
+          }
         }
       }
       if (c1 < nch && c1 >= 0) {
@@ -775,21 +783,24 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
         float2 x = make_float2(0.f, 0.f);
-        if (p.S0) x = *reinterpret_cast<const float2*>(p.S0 + (size_t(unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4);
+        if (NS == 2) {
+          const int row = row0 + g + 8 * hf, col = 8 * nt + 2 * c4;
+          if (rank == 2) x = make_float2(row == col ? 1.f : 0.f, row == col + 1 ? 1.f : 0.f);
+        } else if (p.S0) x = *reinterpret_cast<const float2*>(p.S0 + (size_t(unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4);
         st[nt][2 * hf] = x.x;
         st[nt][2 * hf + 1] = x.y;
       }
-    bool look = p.S0 != nullptr;
+    bool look = NS == 2 || p.S0 != nullptr;
     // this lane's four tokens of a chunk: 2 c4, 2 c4 + 1, and 8 further
     const size_t my0 = tok0 + size_t(2 * c4) * tstride + row0 + g;
     const TIn* vsrc = static_cast<const TIn*>(p.v) + my0;
-    float* odst = p.out + my0;
+    float* odst = (NS == 2 && rank == 2 ? p.out2 : p.out) + my0;
     float vn[8];
     auto fetch_v = [&](int c) {   // v^T in accumulator order: [token tile][row half * 2 + token]
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const TIn* q = vsrc + (k & 1 ? tstride : 0) + (k & 2 ? 8 * tstride : 0);
-        const bool act = c * C + 2 * c4 + (k & 1) + 4 * (k & 2) < T;
+        const bool act = c * C + 2 * c4 + (k & 1) + 4 * (k & 2) < T && (NS == 1 || rank == 1);
         vn[2 * (k & 2) + (k & 1)] = act ? load1<TIn>(q, 0) : 0.0f;
         vn[2 * (k & 2) + 2 + (k & 1)] = act ? load1<TIn>(q, 8) : 0.0f;
       }
@@ -886,7 +897,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       for (int nt = 0; nt < NTILE; ++nt)
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf)
-          *reinterpret_cast<float2*>(p.S_T + (size_t(unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
+          *reinterpret_cast<float2*>(p.S_T + (size_t(NS == 2 && rank == 2 ? unit + p.n_main : unit) * D + row0 + g + 8 * hf) * D + 8 * nt + 2 * c4) =
               make_float2(st[nt][2 * hf] * sSi, st[nt][2 * hf + 1] * sSi);
     }
   }

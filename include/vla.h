@@ -84,12 +84,12 @@ typedef enum {
   VLA_KERNEL_DECODE = 3, /* one step (T = 1) with S0, A0, S_T, A_T all given, u = k_hat, no refresh,
                            d >= 32: the states stream through shared memory once (HBM-bound);
                            VLA_ERR_UNSUPPORTED otherwise.  AUTO picks it when it applies */
-  VLA_KERNEL_CHUNK_TC = 4 /* the chunk algebra on the tensor cores (Section 3.4: the chunked recurrence
+  VLA_KERNEL_CHUNK_TC = 4, /* the chunk algebra on the tensor cores (Section 3.4: the chunked recurrence
                            is a chain of dense products): states in tensor memory, TF32 products in
                            hi/lo pairs with fp32 accumulation.  d = 128, u = k_hat, no refresh,
                            [B,H,T,d] or [B,T,H,d] tensors, T >= 1; VLA_ERR_UNSUPPORTED otherwise.  AUTO picks it
-                           where it applies (and VLA_KERNEL_CHUNK then forces the fp32-FMA form) */
-  ,VLA_KERNEL_PAIR = 5    /* the chunk algebra on warp-level tensor-core products (fp16 hi/lo operands, fp32
+                           there for more units than SM pairs */
+  VLA_KERNEL_PAIR = 5 /* the chunk algebra on warp-level tensor-core products (fp16 hi/lo operands, fp32
                            accumulation, states in registers), two CTAs per unit; every d, u = k_hat or
                            explicit, either layout; VLA_ERR_UNSUPPORTED with the refresh */
 } vla_kernel_t;

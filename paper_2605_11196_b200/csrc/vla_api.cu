@@ -215,12 +215,12 @@ int seqpar_choose_segments(int units, int T, int d, int dtype) {
   // segment's state to the next, `invert` for each segment of the launch and `token` for each token and unit (Gram
   // matrices, corrections).  Uncut, the pair kernel takes `whole` up to a quarter of what is resident and `full` at all of it.
   struct Rate { double whole, lone, full, start, combine, invert, token; };
-  const Rate r = d == 32 ? Rate{1.55, 1.7, 2.55, 35, 3.0, 0.05, 2.6e-4}
-               : d == 64 ? Rate{2.0, 2.2, 3.1, 120, 5.6, 0.25, 6.3e-4}
-                         : Rate{3.9, 4.2, 4.3, 430, 20.5, 1.0, 1.2e-3};
-  // (d = 64, us by segments, 1 = uncut: 1 unit x 16384 tokens 2035, 8: 439, 16: 338, 32: 363; 16 x 4096 531, 2: 427, 4: 357,
-  // 8: 383; 60 x 8192 1187, 2: 1580; 16 x 65536 8100, 8: 3677, 16: 3115, 32: 3362.  d = 32, 4 x 16384 1562, 16: 216, 32: 198,
-  // 64: 270.  d = 128, 8 x 32768 7900, 4: 2990, 8: 3176, 16: 2954; 12 x 8192 1963, 4: 1600.)
+  const Rate r = d == 32 ? Rate{1.55, 1.7, 2.55, 45, 1.7, 0.05, 1.8e-4}
+               : d == 64 ? Rate{2.0, 2.2, 3.1, 110, 3.8, 0.25, 4.8e-4}
+                         : Rate{3.9, 4.2, 4.3, 420, 17.0, 1.0, 1.0e-3};
+  // (d = 64, us by segments, 1 = uncut: 1 unit x 16384 tokens 2035, 8: 423, 16: 313, 32: 306; 30 x 8192 1040, 2: 942, 4: 837,
+  // 8: 850; 60 x 8192 1170, 2: 1539; 16 x 65536 8100, 8: 3500, 16: 2959, 32: 3154.  d = 32, 4 x 16384 1563, 16: 185, 32: 151,
+  // 64: 187.  d = 128, 8 x 32768 7900, 4: 2960, 8: 3126, 16: 2836; 12 x 8192 1979, 4: 1569.)
   const int nch = T / 16;
   const double pairs = (d == 32 ? 2.0 : d == 64 ? 1.0 : 0.5) * sms;   // uncut units resident at a time
   auto waves = [](double n, double room, double lone, double full, double from) {   // us per chunk

@@ -437,8 +437,8 @@ int seqpar_after_d(const SeqParParams& sp, float* A_T, float* zT, const float* A
                    cudaStream_t st) {
   const int N = sp.units * sp.P;
   const int Ls = sp.T / sp.P;
-  const size_t comb_smem = (16 + size_t(D)) * (D + 1) * sizeof(float);
-  const size_t corr_smem = (size_t(D) + 64) * (D + 4) * sizeof(float);
+  const size_t comb_smem = (16 + size_t(D)) * (D + 4) * sizeof(float);
+  const size_t corr_smem = 2 * size_t(D) * (D + 4) * sizeof(float);
   if (cudaFuncSetAttribute(seqpar_combine_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            int(comb_smem)) != cudaSuccess ||
       cudaFuncSetAttribute(seqpar_correct_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -446,20 +446,10 @@ int seqpar_after_d(const SeqParParams& sp, float* A_T, float* zT, const float* A
     cudaGetLastError();
     return VLA_ERR_CUDA;
   }
-  seqpar_combine_kernel<D><<<dim3(sp.units, D / 16), 256, comb_smem, st>>>(sp);
-  const int per_cta = kCorrectTile * kCorrectTiles;
-  seqpar_correct_kernel<D><<<dim3(N, (Ls + per_cta - 1) / per_cta), 256, corr_smem, st>>>(sp);
-  if (cudaGetLastError() != cudaSuccess) return VLA_ERR_CUDA;
-  // final A and key sum: those of each unit's last segment
-  const size_t P = size_t(sp.P);
-  if (A_T &&
-      cudaMemcpy2DAsync(A_T, size_t(D) * D * 4, AT2 + (P - 1) * D * D, P * D * D * 4, size_t(D) * D * 4,
-                        size_t(sp.units), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return VLA_ERR_CUDA;
-  if (zT && cudaMemcpy2DAsync(zT, size_t(D) * 4, zT2 + (P - 1) * D, P * D * 4, size_t(D) * 4,
-                              size_t(sp.units), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return VLA_ERR_CUDA;
-  return VLA_OK;
+  // (also copies the final A and key sum, those of each unit's last segment, out)
+  seqpar_combine_kernel<D><<<dim3(sp.units, D / 16), 256, comb_smem, st>>>(sp, A_T, zT, AT2, zT2);
+  seqpar_correct_kernel<D><<<dim3(N, (Ls + kCorrectTokens - 1) / kCorrectTokens), 256, corr_smem, st>>>(sp);
+  return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
 }
 
 }  // namespace

@@ -364,6 +364,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     float* mxs = fs + Cfg::af_mx;
     const int row0 = 16 * warp;
     const uint32_t my_rows = uint32_t(row0 + g) * kVecRow + 4 * c4;
+    const uint32_t remote_A = STASH ? 0u : map_to_rank(sb + Cfg::s_A, 1);
     float st[NTILE][4];
     float sA, sAi;                   // st = sA * A
     {
@@ -431,10 +432,11 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           fence_async_smem();
           __syncwarp();
           if (lane == 0 && !*abort_flag) {
-#pragma unroll
-            for (int to = 1; to <= NS; ++to)
-              bulk_to_cluster(map_to_rank(sb + Cfg::s_A, to) + as * Cfg::aslot + row0 * kVecRow, stage + row0 * kVecRow, 16 * kVecRow,
-                              map_to_rank(smem_u32(&afull[as]), to));
+            bulk_to_cluster(remote_A + as * Cfg::aslot + row0 * kVecRow, stage + row0 * kVecRow, 16 * kVecRow,
+                            map_to_rank(smem_u32(&afull[as]), 1));
+            if constexpr (NS == 2)
+              bulk_to_cluster(map_to_rank(sb + Cfg::s_A, 2) + as * Cfg::aslot + row0 * kVecRow, stage + row0 * kVecRow,
+                              16 * kVecRow, map_to_rank(smem_u32(&afull[as]), 2));
           }
         }
       }

@@ -25,6 +25,7 @@
 #pragma once
 
 #include "vla_common.cuh"
+#include "vla_mma.cuh"
 #include "vla_seqpar_params.h"
 
 namespace vla {
@@ -238,112 +239,160 @@ __global__ void __launch_bounds__(256) seqpar_invert_kernel(const SeqParParams p
 
 // ---- 4. states at the segment starts, in order: S_start_{j+1} = S_start_j P_j + G_j.  The rows
 // of S do not mix, so a unit is spread over D / 16 CTAs of 16 rows each: grid (units, D / 16),
-// 256 threads (thread = one row of the block, D / 16 columns); dynamic shared memory:
-// (16 + D) * (D + 1) floats.
+// 256 threads (thread = one row of the block, D / 16 columns).  A chain of P steps, each bound by P_j's way from
+// global memory: the next one is fetched into registers while a step computes (d = 32, 4 units x 16384 tokens in
+// 64 segments: the whole call 271 -> 187 us).  The unit's first CTA also copies the last segment's A and key sum out.
 template <int D>
-__global__ void __launch_bounds__(256) seqpar_combine_kernel(const SeqParParams p) {
+__global__ void __launch_bounds__(256) seqpar_combine_kernel(const SeqParParams p, float* A_T, float* zT, const float* AT2,
+                                                             const float* zT2) {
   extern __shared__ __align__(16) unsigned char seqpar_smem[];
-  constexpr int LD = D + 1, R = D / 16, RB = 16;
+  constexpr int LD = D + 4, R = D / 16, RB = 16, NF = D * D / 1024;
   float* Sc = reinterpret_cast<float*>(seqpar_smem);   // [RB][LD] current rows of S_start
   float* Pj = Sc + RB * LD;                            // [D][LD]
   const int unit = blockIdx.x, row0 = blockIdx.y * RB, tid = threadIdx.x;
   const int ty = tid >> 4, tx = tid & 15;
   const size_t N = size_t(p.units) * p.P;
-  for (int idx = tid; idx < RB * D; idx += 256)
-    Sc[(idx / D) * LD + idx % D] = p.S0 ? p.S0[(size_t(unit) * D + row0) * D + idx] : 0.0f;
-  __syncthreads();
-  for (int j = 0; j < p.P; ++j) {
+  float s[R], g[R];
+  float4 pre[NF];
+  const size_t own = size_t(row0 + ty) * D + tx * R;   // this thread's entries of a D x D matrix
+  auto fetch = [&](int j) {
     const size_t vu = size_t(unit) * p.P + j;
-    const float* G = p.ST2 + (vu * D + row0) * D;
-    const float* Pg = p.ST2 + (N + vu) * D * D;
-    float* Ss = p.Sstart + (vu * D + row0) * D;
-    for (int idx = tid; idx < RB * D; idx += 256) Ss[idx] = Sc[(idx / D) * LD + idx % D];
-    for (int idx = tid; idx < D * D; idx += 256) Pj[(idx / D) * LD + idx % D] = Pg[idx];
-    __syncthreads();
+    const float4* Pg = reinterpret_cast<const float4*>(p.ST2 + (N + vu) * D * D);
+#pragma unroll
+    for (int i = 0; i < NF; ++i) pre[i] = Pg[i * 256 + tid];
+#pragma unroll
+    for (int b = 0; b < R; ++b) g[b] = p.ST2[vu * D * D + own + b];
+  };
+  fetch(0);
+#pragma unroll
+  for (int b = 0; b < R; ++b) s[b] = p.S0 ? p.S0[size_t(unit) * D * D + own + b] : 0.0f;
+  for (int j = 0; j < p.P; ++j) {
+    float* Ss = p.Sstart + (size_t(unit) * p.P + j) * D * D + own;
     float acc[R];
 #pragma unroll
-    for (int b = 0; b < R; ++b) acc[b] = G[ty * D + tx * R + b];
+    for (int b = 0; b < R; ++b) {
+      Ss[b] = s[b];
+      Sc[ty * LD + tx * R + b] = s[b];
+      acc[b] = g[b];
+    }
+#pragma unroll
+    for (int i = 0; i < NF; ++i) {
+      const int at = 4 * (i * 256 + tid);
+      *reinterpret_cast<float4*>(&Pj[(at / D) * LD + at % D]) = pre[i];
+    }
+    __syncthreads();
+    if (j + 1 < p.P) fetch(j + 1);
 #pragma unroll 4
     for (int m = 0; m < D; ++m) {
       const float sa = Sc[ty * LD + m];
+      float pr[R];
 #pragma unroll
-      for (int b = 0; b < R; ++b) acc[b] = fmaf(sa, Pj[m * LD + tx * R + b], acc[b]);
+      for (int b = 0; b < R; b += 2) *reinterpret_cast<float2*>(pr + b) = *reinterpret_cast<const float2*>(&Pj[m * LD + tx * R + b]);
+#pragma unroll
+      for (int b = 0; b < R; ++b) acc[b] = fmaf(sa, pr[b], acc[b]);
     }
     __syncthreads();
 #pragma unroll
-    for (int b = 0; b < R; ++b) Sc[ty * LD + tx * R + b] = acc[b];
-    __syncthreads();
+    for (int b = 0; b < R; ++b) s[b] = acc[b];
   }
-  if (p.S_T)
-    for (int idx = tid; idx < RB * D; idx += 256)
-      p.S_T[(size_t(unit) * D + row0) * D + idx] = Sc[(idx / D) * LD + idx % D];
+  const size_t last = size_t(unit) * p.P + p.P - 1;
+#pragma unroll
+  for (int b = 0; b < R; ++b) {
+    if (p.S_T) p.S_T[size_t(unit) * D * D + own + b] = s[b];
+    if (A_T) A_T[size_t(unit) * D * D + own + b] = AT2[last * D * D + own + b];
+  }
+  if (zT && row0 == 0 && tid < D) zT[size_t(unit) * D + tid] = zT2[last * D + tid];
 }
 
-// ---- 5. o_t = o0_t + S_start_j w_t.  Grid (units * P, ceil(Ls / 256)): a CTA keeps S_start_j
-// in shared memory and walks four 64-token tiles of its segment; dynamic shared memory:
-// D * (D + 4) + 64 * (D + 4) floats.
-constexpr int kCorrectTile = 64;     // tokens per shared-memory tile
-constexpr int kCorrectTiles = 4;     // tiles per CTA
+// ---- 5. o_t += S_start_j w_t.  Grid (units * P, ceil(Ls / kCorrectTokens)), 8 warps; a warp takes 16 tokens at a
+// time, all D rows of S_start_j.  fp32 operands as two tf32 terms, all four products (lanes
+// take float4 pairs 2 c4, 2 c4 + 1 of every 32 columns, conflict-free at a row stride of D + 4); S_start_j is split once per CTA.
+// Bound by memory (w once, o twice): the fp32-FMA form before it waited on its shared-memory operands (335 us of the
+// 3.12 ms at d = 64, 16 units x 65536 tokens; the whole call is 2.96 ms now).
+constexpr int kCorrectTokens = 512;
 
 template <int D>
-__global__ void __launch_bounds__(256) seqpar_correct_kernel(const SeqParParams p) {
+__global__ void __launch_bounds__(256, D == 128 ? 1 : 2) seqpar_correct_kernel(const SeqParParams p) {
   extern __shared__ __align__(16) unsigned char seqpar_smem[];
-  constexpr int LD = D + 4, TBK = kCorrectTile;
-  constexpr int RW = D >= 64 ? 4 : 2;          // rows per thread: tr, tr + TRW, ...
-  constexpr int TRW = D / RW;                  // threads along the rows
-  constexpr int TTK = 256 / TRW;               // threads along the tokens
-  constexpr int TT = TBK / TTK;                // tokens per thread
-  float* Ss = reinterpret_cast<float*>(seqpar_smem);   // [D][LD]
-  float* Wb = Ss + D * LD;                              // [TBK][LD]
+  constexpr int LD = D + 4, NT = D / 8;
+  uint32_t* Sh = reinterpret_cast<uint32_t*>(seqpar_smem);   // [D][LD] upper terms
+  uint32_t* Sl = Sh + D * LD;                                // [D][LD] remainders
   const int vu = blockIdx.x, j = vu % p.P;
   if (j == 0 && !p.S0) return;                 // S_start = 0: nothing to add
   const int Ls = p.T / p.P;
-  const int tid = threadIdx.x;
-  const int tr = tid % TRW, tk = tid / TRW;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
   const float4* Sg = reinterpret_cast<const float4*>(p.Sstart + size_t(vu) * D * D);
-  for (int idx = tid; idx < D * D / 4; idx += 256)
-    *reinterpret_cast<float4*>(&Ss[(idx / (D / 4)) * LD + (idx % (D / 4)) * 4]) = Sg[idx];
-  for (int tile = 0; tile < kCorrectTiles; ++tile) {
-    const int t0 = (blockIdx.y * kCorrectTiles + tile) * TBK;
-    if (t0 >= Ls) break;                       // uniform over the CTA
-    const int nt = min(TBK, Ls - t0);
-    __syncthreads();                           // the previous tile has been consumed
-    const float4* wg = reinterpret_cast<const float4*>(p.wn + (size_t(vu) * Ls + t0) * D);
-    for (int idx = tid; idx < TBK * D / 4; idx += 256) {
-      const int t = idx / (D / 4);
-      *reinterpret_cast<float4*>(&Wb[t * LD + (idx % (D / 4)) * 4]) =
-          t < nt ? wg[idx] : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
-    float acc[TT][RW];
+  for (int idx = tid; idx < D * D / 4; idx += 256) {
+    const float4 x = Sg[idx];
+    uint4 h, l;
+    split_tf32(x.x, h.x, l.x); split_tf32(x.y, h.y, l.y); split_tf32(x.z, h.z, l.z); split_tf32(x.w, h.w, l.w);
+    const int at = (idx / (D / 4)) * LD + (idx % (D / 4)) * 4;
+    *reinterpret_cast<uint4*>(Sh + at) = h;
+    *reinterpret_cast<uint4*>(Sl + at) = l;
+  }
+  __syncthreads();
+  const int end = min(Ls, (int(blockIdx.y) + 1) * kCorrectTokens);
+#pragma unroll 1
+  for (int t0 = blockIdx.y * kCorrectTokens + warp * 16; t0 < end; t0 += 8 * 16) {
+    float acc[NT][4];
 #pragma unroll
-    for (int a = 0; a < TT; ++a)
+    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-      for (int b = 0; b < RW; ++b) acc[a][b] = 0.0f;
-#pragma unroll 2
-    for (int m = 0; m < D; m += 4) {
-      float4 sv[RW], wv[TT];
+      for (int e = 0; e < 4; ++e) acc[nt][e] = 0.0f;
+#pragma unroll 1
+    for (int c0 = 0; c0 < D; c0 += 32) {
+      uint32_t ah[4][4], al[4][4];     // [8 columns]
+      {
+        float4 x[2][2];
 #pragma unroll
-      for (int b = 0; b < RW; ++b) sv[b] = *reinterpret_cast<const float4*>(&Ss[(tr + b * TRW) * LD + m]);
+        for (int hf = 0; hf < 2; ++hf) {
+          const int t = t0 + 8 * hf + g;
+          const float4* w = reinterpret_cast<const float4*>(p.wn + (size_t(vu) * Ls + t) * D + c0) + 2 * c4;
 #pragma unroll
-      for (int a = 0; a < TT; ++a) wv[a] = *reinterpret_cast<const float4*>(&Wb[(tk * TT + a) * LD + m]);
-#pragma unroll
-      for (int a = 0; a < TT; ++a)
-#pragma unroll
-        for (int b = 0; b < RW; ++b) {
-          acc[a][b] = fmaf(wv[a].x, sv[b].x, acc[a][b]);
-          acc[a][b] = fmaf(wv[a].y, sv[b].y, acc[a][b]);
-          acc[a][b] = fmaf(wv[a].z, sv[b].z, acc[a][b]);
-          acc[a][b] = fmaf(wv[a].w, sv[b].w, acc[a][b]);
+          for (int k = 0; k < 2; ++k) x[hf][k] = t < end ? w[k] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float u0[4] = {x[0][k].x, x[0][k].y, x[1][k].x, x[1][k].y};
+          const float u1[4] = {x[0][k].z, x[0][k].w, x[1][k].z, x[1][k].w};
+          split_frag_tf32(u0, ah[2 * k], al[2 * k]);
+          split_frag_tf32(u1, ah[2 * k + 1], al[2 * k + 1]);
+        }
+      }
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        const int at = (8 * nt + g) * LD + c0 + 8 * c4;
+        uint32_t bh[8], bl[8];
+        *reinterpret_cast<uint4*>(bh) = *reinterpret_cast<const uint4*>(Sh + at);
+        *reinterpret_cast<uint4*>(bh + 4) = *reinterpret_cast<const uint4*>(Sh + at + 4);
+        *reinterpret_cast<uint4*>(bl) = *reinterpret_cast<const uint4*>(Sl + at);
+        *reinterpret_cast<uint4*>(bl + 4) = *reinterpret_cast<const uint4*>(Sl + at + 4);
+        {
+          float y[4][4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) mma_tf32_zero(y[q], al[q], bl[2 * q], bl[2 * q + 1]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) mma_tf32(y[q], al[q], bh[2 * q], bh[2 * q + 1]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) mma_tf32(y[q], ah[q], bl[2 * q], bl[2 * q + 1]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) mma_tf32(y[q], ah[q], bh[2 * q], bh[2 * q + 1]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[nt][e] += (y[0][e] + y[1][e]) + (y[2][e] + y[3][e]);
+        }
+      }
     }
-    float* og = p.out + (size_t(vu) * Ls + t0) * D;
 #pragma unroll
-    for (int a = 0; a < TT; ++a) {
-      const int t = tk * TT + a;
-      if (t < nt) {
+    for (int hf = 0; hf < 2; ++hf) {
+      const int t = t0 + 8 * hf + g;
+      if (t >= end) continue;
+      float2* o = reinterpret_cast<float2*>(p.out + (size_t(vu) * Ls + t) * D + 2 * c4);
 #pragma unroll
-        for (int b = 0; b < RW; ++b) og[size_t(t) * D + tr + b * TRW] += acc[a][b];
+      for (int nt = 0; nt < NT; ++nt) {
+        float2 x = o[4 * nt];
+        x.x += acc[nt][2 * hf];
+        x.y += acc[nt][2 * hf + 1];
+        o[4 * nt] = x;
       }
     }
   }

@@ -278,8 +278,7 @@ __global__ void __launch_bounds__(BwdChainCfg<D>::NT) bwd_chains_kernel(const Bw
     // a warp's 16 rows of S (or of its adjoint D), scaled by a power of two that follows their size
     const int row0 = 16 * warp;
     const float* init = rev ? p.dS_T : p.S0;
-    float st[NTILE][4], sc = 1.0f, sci = 1.0f, bound = 0.0f;
-    bool look = init != nullptr;
+    float st[NTILE][4], sc = 1.0f, sci = 1.0f;
 #pragma unroll
     for (int nt = 0; nt < NTILE; ++nt)
 #pragma unroll
@@ -323,24 +322,14 @@ __global__ void __launch_bounds__(BwdChainCfg<D>::NT) bwd_chains_kernel(const Bw
 #pragma unroll 1
     for (int i = 0; i < nch; ++i) {
       const int c = chunk_of(i), s = i % NS;
-      if (look) {
-        float mx = 0.f;
+      const float mx = state_max(st);
+      if (state_leaves_scale(mx)) {
+        const float r = state_rescale(sc, mx);
+        sci = pow2_inverse(sc);
 #pragma unroll
         for (int nt = 0; nt < NTILE; ++nt)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fabsf(st[nt][e]));
-        mx = warp_max_nonneg(mx);
-        bound = mx;
-        if (mx > 0.0f && (mx > 512.0f || mx < 1.0f)) {
-          const float ns = fminf(fmaxf(sc * pow2_scale(mx, 5), 7.888609e-31f), 1.2676506e30f), r = ns * sci;
-#pragma unroll
-          for (int nt = 0; nt < NTILE; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) st[nt][e] *= r;
-          sc = ns;
-          sci = pow2_inverse(ns);
-          bound = mx * r;
-        }
+          for (int e = 0; e < 4; ++e) st[nt][e] *= r;
       }
       // ---- checkpoint: S at a block's start, D at its end
       if (rev ? (i == 0 || (c & 1) == 1) : (c & 1) == 0) {
@@ -413,14 +402,13 @@ __global__ void __launch_bounds__(BwdChainCfg<D>::NT) bwd_chains_kernel(const Bw
       }
       if (i + 1 < nch) fetch(chunk_of(i + 1));
       // ---- S += E^T alpha, or D += dY^T Q - dE^T K
-      auto update = [&](float (&co)[2][4], uint32_t op, float unit_scale, float reach) {
+      auto update = [&](float (&co)[2][4], uint32_t op, float unit_scale) {
         float m = 0.f;
 #pragma unroll
         for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
           for (int e = 0; e < 4; ++e) m = fmaxf(m, fabsf(co[nt][e]));
         m = warp_max_nonneg(m);
-        bound += 16.0f * m * reach;
         const float sx = pow2_scale(m, 8), so = pow2_inverse(sx) * unit_scale;
 #pragma unroll
         for (int nt = 0; nt < 2; ++nt)
@@ -454,11 +442,10 @@ __global__ void __launch_bounds__(BwdChainCfg<D>::NT) bwd_chains_kernel(const Bw
         for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
           for (int e = 0; e < 4; ++e) co[nt][e] = pass ? y[nt][e] : ev[nt][e];
-        update(co, pass ? Qop : rev ? Kop : Aop, pass ? 1.0f : (rev ? -1.0f : 1.0f) / 256.0f, pass ? 512.0f : 1.0f);
+        update(co, pass ? Qop : rev ? Kop : Aop, pass ? 1.0f : (rev ? -1.0f : 1.0f) / 256.0f);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[s]);
-      look = !(bound <= 16384.0f) || bound < 1.0f;
     }
     float* fin = rev ? p.dS0 : nullptr;
     if (fin) {

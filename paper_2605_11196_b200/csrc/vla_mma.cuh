@@ -315,6 +315,34 @@ __device__ __forceinline__ float pow2_scale(float m, int target) {
 // its inverse
 __device__ __forceinline__ float pow2_inverse(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
 
+// The memory side's states are scaled by a power of two that keeps their largest entry, looked at for every chunk, within
+// [2^4, 2^14].  Both ends count: a state may fall at any time (large values overwritten, a large carried state), and
+// below 1 its remainders would be fp16 subnormals.  With a scale that only followed S upwards a start 1e6 above the rest of a
+// sequence left S_T wrong by 1e-3 of its size (fp32 kernels: 1e-6).  The look costs a scan 0.5 to 2 % (d = 64, 32 units x 4096
+// tokens 522 -> 525 us; d = 128, 48 x 1777 447 -> 455); a look only where products of S had become small cost more, because
+// taking those products again makes a loop of them and the loads in flight are waited for at its edge (522 -> 612 us).
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+template <int NTILE>
+__device__ __forceinline__ float state_max(const float (&st)[NTILE][4]) {
+  float m[2] = {0.f, 0.f};
+#pragma unroll
+  for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+    for (int e = 0; e < 4; e += 2) m[e >> 1] = max3(m[e >> 1], fabsf(st[nt][e]), fabsf(st[nt][e + 1]));
+  return warp_max_nonneg(fmaxf(m[0], m[1]));
+}
+__device__ __forceinline__ bool state_leaves_scale(float mx) { return mx > 16384.0f || (mx < 16.0f && mx > 0.0f); }
+// the scale that puts mx into [2^9, 2^10) (within 2^+-100); returns the factor for what is held
+__device__ __forceinline__ float state_rescale(float& scale, float mx) {
+  const float s = fminf(fmaxf(scale * pow2_scale(mx, 9), 7.888609e-31f), 1.2676506e30f), f = s * pow2_inverse(scale);
+  scale = s;
+  return f;
+}
+
 // Held back before a CTA that has given up a wait ends: its copies in flight (a few microseconds at
 // most) must land before its shared memory is handed on, and the barriers that count them are no longer
 // followed.  About 50 us.

@@ -755,31 +755,6 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
     const int row0 = 16 * warp;
     float st[NTILE][4];
     float sS = 1.0f, sSi = 1.0f;     // st = sS * S
-    float bound = 0.0f;              // largest entry of st, from above
-    auto true_max = [&]() {
-      float mx = 0.f;
-#pragma unroll
-      for (int nt = 0; nt < NTILE; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fabsf(st[nt][e]));
-      return warp_max_nonneg(mx);
-    };
-    auto rescale = [&](float mx) {
-      bound = mx;
-      if (mx > 0.0f && (mx > 512.0f || mx < 1.0f)) {
-        // (sS itself stays within 2^+-100)
-        float f = pow2_scale(mx, 5);
-        const float ns = fminf(fmaxf(sS * f, 7.888609e-31f), 1.2676506e30f);
-        f = ns * sSi;
-#pragma unroll
-        for (int nt = 0; nt < NTILE; ++nt)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) st[nt][e] *= f;
-        sS = ns;
-        sSi = pow2_inverse(ns);
-        bound = mx * f;
-      }
-    };
 #pragma unroll
     for (int nt = 0; nt < NTILE; ++nt)
 #pragma unroll
@@ -792,7 +767,6 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         st[nt][2 * hf] = x.x;
         st[nt][2 * hf + 1] = x.y;
       }
-    bool look = NS == 2 || p.S0 != nullptr;
     // this lane's four tokens of a chunk: 2 c4, 2 c4 + 1, and 8 further
     const size_t my0 = tok0 + size_t(2 * c4) * tstride + row0 + g;
     const TIn* vsrc = static_cast<const TIn*>(p.v) + my0;
@@ -814,7 +788,15 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       const int slot = c % RK, as = c % RA, gs = c & 1;
       const uint32_t Kop = sb + Cfg::s_K + slot * Cfg::kslot, Qop = sb + Cfg::s_Q + slot * Cfg::kslot;
       const uint32_t Aop = sb + Cfg::s_A + as * Cfg::aslot;
-      if (look) rescale(true_max());
+      const float mx = state_max(st);
+      if (state_leaves_scale(mx)) {
+        const float f = state_rescale(sS, mx);
+        sSi = pow2_inverse(sS);
+#pragma unroll
+        for (int nt = 0; nt < NTILE; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) st[nt][e] *= f;
+      }
       wait(&kfull[slot], (c / RK) & 1);
       // ---- P = S K^T and R = S Q^T (rows: this warp's, columns: tokens)
       float pk[2][4] = {}, rq[2][4] = {};
@@ -891,8 +873,6 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       }
       }
       arrive_cl(&aempty[as], 0);
-      bound += 16.0f * me;
-      look = !(bound <= 16384.0f) || bound < 1.0f;
     }
     if (p.S_T) {
 #pragma unroll

@@ -1,0 +1,59 @@
+"""Operand ranges of the fp16 hi/lo products (-m gpu), against the fp64 oracles: what they hold may fall
+or rise by orders of magnitude within a sequence."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2605_11196_b200 as vla
+from paper_2605_11196_b200 import workloads as W
+from parity_util import NTHREADS, run_gpu, run_oracle, to_oracle_array
+
+pytestmark = pytest.mark.gpu
+
+PAIR, IDENT = vla.VLA_KERNEL_PAIR, vla.VLA_FLAG_IDENTITY_MAP
+
+
+def _rel(x, ref):
+    x = x.detach().cpu().double().numpy()
+    assert np.all(np.isfinite(x))
+    return float(np.abs(x - ref).max() / np.abs(ref).max())
+
+
+# After a start 1e6 above the rest a sequence is left, by its end, with the fp32 kernels' own 1e-6 to 7e-6 of
+# the late values (what is left of the large ones has decayed); three times that.  A scale that does not fall with the
+# state leaves 6e-4 to 2e-3.
+FALLEN = 2e-5
+
+
+@pytest.mark.parametrize("d,T", [(16, 1024), (32, 1040), (64, 2048), (128, 3008)])
+@pytest.mark.parametrize("flags", [0, IDENT])
+def test_scale_of_S_falls_with_it(d, T, flags):
+    w = W.Workload("fall", 1, 2, d, T, "f32", 11)
+    q, k, v = W.make_inputs(w)
+    big = v.clone()
+    big[:, :, :64] *= 1e6
+    S0 = 1e6 * torch.randn((1, 2, d, d), generator=torch.Generator().manual_seed(1))
+    for vv, kw in ((big, {}), (v, {"S0": S0})):
+        ref = run_oracle(q, k, vv, 1.0, flags=flags, **kw)
+        r = run_gpu(q, k, vv, 1.0, flags=flags, kernel=PAIR, **kw)
+        assert _rel(r.S_T, ref.S_T) <= FALLEN and _rel(r.out[:, :, -64:], ref.out[:, :, -64:]) <= FALLEN
+
+
+@pytest.mark.parametrize("d,T", [(16, 1024), (64, 2048)])
+@pytest.mark.parametrize("flags", [0, IDENT])
+def test_scales_of_the_backward_chains_fall_with_them(d, T, flags):
+    """S after large early values (late dq, dk), its adjoint before large late gradients (early dv, dS0)."""
+    w = W.Workload("fall", 1, 2, d, T, "f32", 12)
+    q, k, v = W.make_inputs(w)
+    do = torch.randn((1, 2, T, d), generator=torch.Generator().manual_seed(3))
+    big_v, big_do = v.clone(), do.clone()
+    big_v[:, :, :64] *= 1e6
+    big_do[:, :, -64:] *= 1e6
+    for vv, g, names, part in ((big_v, do, ("dq", "dk"), slice(-64, None)), (v, big_do, ("dv",), slice(0, 64))):
+        a = [to_oracle_array(x)[0] for x in (q, k, vv)]
+        ref = oracle.backward(*a, 1.0, g.double().numpy(), in_dtype=oracle.F32, flags=flags, n_threads=NTHREADS)
+        got = vla.vla_backward(q.cuda(), k.cuda(), vv.cuda(), 1.0, g.cuda(), want_dA0=False, flags=flags)
+        for n in names:
+            assert _rel(getattr(got, n)[:, :, part], getattr(ref, n)[:, :, part]) <= FALLEN, n
+        assert _rel(got.dS0, ref.dS0) <= FALLEN

@@ -286,6 +286,11 @@ __device__ __forceinline__ float rcp_ftz_nr(float x) {
   const float r = rcp_ftz(x);
   return fmaf(r, fmaf(-x, r, 1.0f), r);
 }
+__device__ __forceinline__ float rsqrt_ftz_nr(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
+}
 // 1/x to within an ulp or so: hardware estimate plus one Newton step
 __device__ __forceinline__ float rcp_nr(float x) {
   const float r = rcp_approx(x);
@@ -339,12 +344,17 @@ __device__ __forceinline__ void tile16_store(float* G, int i0, int j0, const flo
 // row's own two travel by shuffle while the two pivot rows go through shared memory (1050 clk alone; one column
 // a step with the row by shuffles: 1530).  The registers rotate by two a step, so that columns s, s + 1 are always
 // m[0], m[1] of the half that holds them and the loop stays small; eight steps bring them back.
-__device__ __forceinline__ float eliminate16(float (&m)[8], int lane, float* piv, float eps) {
+// OWN: every row has its own floor of delta, eps * own[row] (own in shared memory, 8-byte aligned).
+template <bool OWN = false>
+__device__ __forceinline__ float eliminate16(float (&m)[8], int lane, float* piv, float eps, const float* own = nullptr) {
   const int r = lane & 15, h = lane >> 4;
-  float delta = 1.0f;
+  float delta = 1.0f, f0 = eps, f1 = eps;
+  if (OWN) { f0 = eps * own[0]; f1 = eps * own[1]; }
 #pragma unroll 2
   for (int s = 0; s < 16; s += 2) {
     constexpr unsigned full = 0xffffffffu;
+    float2 next = make_float2(1.0f, 1.0f);   // (a step ahead: off the chain)
+    if (OWN) next = *reinterpret_cast<const float2*>(own + ((s + 2) & 15));
     const int hs = s >> 3;
     float* rows = piv + (s & 2) * 16;   // (two buffers: one barrier a step is enough)
     const float a0 = __shfl_sync(full, m[0], s + 16 * hs);
@@ -363,8 +373,8 @@ __device__ __forceinline__ float eliminate16(float (&m)[8], int lane, float* piv
     const float r0[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
     const float r1[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
     // Algorithm 1 clamps delta at eps (delta >= 1 whenever A is positive definite)
-    const float a = fmaxf(a0, eps);
-    const float det = fmaxf(fmaf(a, d, -b * b), eps * a);
+    const float a = fmaxf(a0, f0);
+    const float det = fmaxf(fmaf(a, d, -b * b), f1 * a);
     const float idet = rcp_ftz(det), ia = rcp_ftz(a);
     const float n0 = fmaf(d, ms0, -b * ms1), n1 = fmaf(a, ms1, -b * ms0);
     const float q = r == s + 1 ? b * ia : 0.0f;     // row s + 1 loses its multiple of row s
@@ -386,6 +396,7 @@ __device__ __forceinline__ float eliminate16(float (&m)[8], int lane, float* piv
     for (int j = 0; j < 6; ++j) m[j] = fmaf(-w0, r0[j + 2], fmaf(-w1, r1[j + 2], m[j + 2]));
     m[6] = t[0];
     m[7] = t[1];
+    if (OWN) { f0 = eps * next.x; f1 = eps * next.y; }
   }
   return delta;
 }

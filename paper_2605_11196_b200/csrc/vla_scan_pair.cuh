@@ -24,9 +24,13 @@
 // registers, and below because small batches then use twice the SMs.
 //
 // Ranges of the fp16 operands (vla_mma.cuh): k_hat and alpha are unit vectors, scaled by 2^8; A <= its
-// largest diagonal entry elementwise, which never grows, scaled to 2^7 (||A k|| then stays below 2^15 at
-// d = 128) and rescaled by powers of two as it shrinks; rows of Q and u by their own power of two;
-// S and E by powers of two per warp that follow their size.
+// largest diagonal entry elementwise, which never grows, scaled to 2^7 (an entry of A k then stays below 2^12 at
+// d = 128) and rescaled by powers of two as it shrinks; rows of Q by their own power of two;
+// S and E by powers of two per warp that follow their size.  The update takes zeta = z / sqrt(delta), which
+// zeta zeta^T <= A bounds whatever u is, in both operands: z / delta in one of them ran into subnormals for small lambda.
+// An explicit u is used verbatim, of any norm: u_t = D_t u'_t with a power of two D_t that leaves 1 <= ||u'_t|| < 2
+// (norms from 2^-20 to 2^60), and everything up to zeta runs on u':  U' A U'^T + D^-2 = L' diag(delta / D^2) L'^T, Z' = L'^-1 U' A = D^-1 Z.
+// (In true units z = A u passed fp16's range at norms of 250 to 500 times the largest entry of A.)
 #pragma once
 
 #include "vla_launch.h"
@@ -59,7 +63,7 @@ struct PairCfg {
   static constexpr uint32_t a_K = 0, a_U = RK * kslot, a_Z0 = a_U + (UT ? RK * kslot : 0), a_W0 = a_Z0 + aslot,
                             a_Z = a_W0 + (UT ? aslot : 0), a_A = a_Z + aslot, a_f = a_A + RA * aslot;
   static constexpr int af_W = 0, af_Li = af_W + (UT ? 3 : 1) * PARTS * SM, af_PT = af_Li + SM, af_dl = af_PT + (UT ? 2 * SM : 0),
-                       af_n = af_dl + 32, af_mx = af_n + 2 * NW * 16, af_us = af_mx + 16, af_pv = af_us + RK * 16, af_zp = af_pv + 64, af_end = af_zp + 2 * NPREP * D;
+                       af_n = af_dl + 48, af_mx = af_n + 2 * NW * 16, af_us = af_mx + 16, af_ud = af_us + RK * 16, af_pv = af_ud + (UT ? 4 * 16 : 0), af_zp = af_pv + 64, af_end = af_zp + 2 * NPREP * D;
   // rank 1
   static constexpr uint32_t s_K = 0, s_Q = RK * kslot, s_A = 2 * RK * kslot, s_f = s_A + RA * aslot;
   static constexpr int sf_N = 0, sf_T = SM, sf_H = sf_T + 2 * SM, sf_osc = sf_H + 2 * SM, sf_nrm = sf_osc + 32,
@@ -238,7 +242,16 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         if (two) {
           const float s = pow2_scale(sqrt_ftz(qq), 8);
           tok_store4<D>(base1 + slot * Cfg::kslot, tt, pl, x, s);
-          if (pl == 0) fs[(rank ? Cfg::sf_qs : Cfg::af_us) + slot * 16 + tt] = pow2_inverse(s);
+          if (pl == 0) {
+            const float inv = pow2_inverse(s);
+            if (rank) {
+              fs[Cfg::sf_qs + slot * 16 + tt] = inv;
+            } else {   // u row -> u', and D^-2 (four slots: the elimination is done with one by the time it comes round again)
+              const float iD = pow2_inverse(fminf(fmaxf(256.0f * inv, 9.5367432e-7f), 1.1529215e18f));
+              fs[Cfg::af_us + slot * 16 + tt] = inv * iD;
+              fs[Cfg::af_ud + (c & 3) * 16 + tt] = iD * iD;
+            }
+          }
         }
         if (rank != 0 && pl == 0) {
           fs[Cfg::sf_nrm + slot * 16 + tt] = act ? nr : 0.f;
@@ -293,9 +306,11 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         m[0] = x.x; m[1] = x.y; m[2] = x.z; m[3] = x.w;
         m[4] = y.x; m[5] = y.y; m[6] = y.z; m[7] = y.w;
       }
+      const float* ud = fs + Cfg::af_ud + (c & 3) * 16;
+      const float one = UT ? ud[r] : 1.0f;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) m[j] += (8 * h + j == r) ? 1.0f : 0.0f;
-      const float delta = eliminate16(m, lane, piv, eps);
+      for (int j = 0; j < 8; ++j) m[j] += (8 * h + j == r) ? one : 0.0f;
+      const float delta = eliminate16<UT>(m, lane, piv, eps, ud);   // (explicit u: delta / D^2)
       {
         float x[8];
 #pragma unroll
@@ -304,27 +319,31 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         o[0] = make_float4(x[0], x[1], x[2], x[3]);
         o[1] = make_float4(x[4], x[5], x[6], x[7]);
         if (h == 0) {
-          dl[r] = delta;
           dl[16 + r] = rcp_ftz_nr(delta);
+          dl[32 + r] = rsqrt_ftz_nr(delta);
         }
       }
       named_arrive(4, (NW + 1) * 32);   // L^-1 and delta are written
-      if (STASH && h == 0 && c * C + r < T) sh.delta[size_t(unit) * T + c * C + r] = delta;
+      if (STASH && h == 0 && c * C + r < T) sh.delta[size_t(unit) * T + c * C + r] = UT ? delta * pow2_inverse(one) : delta;
       if constexpr (UT) {
-        // N = L^-1 X, X[s][t] = u_s . A k_t;  PT[t][s] = N[s][t] / delta_s for s <= t
+        // N = L^-1 X, X[s][t] = u'_s . A k_t;  PT[t][s] = N[s][t] / delta_s for s <= t
         // (X and PT alternate between two buffers: the state warps may be a chunk ahead here)
         const float* X = fs + Cfg::af_W + (1 + (c & 1)) * PARTS * SM;
         float* PT = fs + Cfg::af_PT + (c & 1) * SM;
-        float n[2][4] = {};
+        uint32_t ah[2][4], al[2][4];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const float2 la = *reinterpret_cast<const float2*>(Li + g * LD + 8 * j + 2 * c4);
           const float2 lb = *reinterpret_cast<const float2*>(Li + (g + 8) * LD + 8 * j + 2 * c4);
           const float lt[4] = {la.x, la.y, lb.x, lb.y};
-          uint32_t ah[4], al[4];
-          split_frag_tf32(lt, ah, al);
+          split_frag_tf32(lt, ah[j], al[j]);
+        }
+        const float i0 = dl[16 + g], i1 = dl[24 + g];
+#pragma unroll 1
+        for (int nt = 0; nt < 2; ++nt) {   // (rolled: code size)
+          float n[4] = {};
 #pragma unroll
-          for (int nt = 0; nt < 2; ++nt) {
+          for (int j = 0; j < 2; ++j) {
             float b0 = 0.f, b1 = 0.f;
 #pragma unroll
             for (int q = 0; q < PARTS; ++q) {
@@ -335,23 +354,20 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
             split_tf32(b0, bh0, bl0);
             split_tf32(b1, bh1, bl1);
             float x[4];
-            mma_tf32_zero(x, al, bl0, bl1);
-            mma_tf32(x, al, bh0, bh1);
-            mma_tf32(x, ah, bl0, bl1);
-            mma_tf32(x, ah, bh0, bh1);
+            mma_tf32_zero(x, al[j], bl0, bl1);
+            mma_tf32(x, al[j], bh0, bh1);
+            mma_tf32(x, ah[j], bl0, bl1);
+            mma_tf32(x, ah[j], bh0, bh1);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) n[nt][e] += x[e];
+            for (int e = 0; e < 4; ++e) n[e] += x[e];
           }
-        }
-        const float i0 = dl[16 + g], i1 = dl[24 + g];
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const int t = 8 * nt + 2 * c4 + e;
-            PT[t * LD + g] = g <= t ? n[nt][e] * i0 : 0.0f;
-            PT[t * LD + g + 8] = g + 8 <= t ? n[nt][2 + e] * i1 : 0.0f;
+            PT[t * LD + g] = g <= t ? n[e] * i0 : 0.0f;
+            PT[t * LD + g + 8] = g + 8 <= t ? n[2 + e] * i1 : 0.0f;
           }
+        }
         arrive(&pfull[c & 1]);
       }
     }
@@ -402,12 +418,17 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         const float* q = np + (c2 & 1) * NW * 16;
         const int as = c2 % RA;
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
+        for (int nt = 0; nt < 2; ++nt) {
+          float2 s2 = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int w = 0; w < NW; ++w) {
+            const float2 x = *reinterpret_cast<const float2*>(q + w * 16 + 8 * nt + 2 * c4);
+            s2.x += x.x;
+            s2.y += x.y;
+          }
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
-            float n2 = 0.f;
-#pragma unroll
-            for (int w = 0; w < NW; ++w) n2 += q[w * 16 + 8 * nt + 2 * c4 + e];
+            const float n2 = e ? s2.y : s2.x;
             const float an = fmaxf(sqrt_ftz(n2), eps), sc = rcp_ftz_nr(an);
             al[nt][e] = a2[nt][e] * sc;
             al[nt][2 + e] = a2[nt][2 + e] * sc;
@@ -424,6 +445,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
             al[nt][e] *= kUnit;
             al[nt][2 + e] *= kUnit;
           }
+        }
         if (bad && (p.flags & VLA_FLAG_CHECK_FINITE) && p.status) atomicCAS(p.status, 0, int(VLA_ERR_NONFINITE));
         if constexpr (!STASH) {
           if (c2 >= RA) wait(&aempty[as], (c2 / RA - 1) & 1);   // (the staged rows have been copied too, then)
@@ -471,13 +493,13 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         for (int e = 0; e < 4; ++e) a2[nt][e] = a1[nt][e];
     };
     float sz1 = 0.f;
-    // scale of z / delta in the update of A: 2^10 / sqrt(sA), rounded to a power of two
+    // scale of zeta in the update of A: 2^7 / sqrt(sA), rounded to a power of two.  |zeta| <= sqrt(max A) < 2^4 / sqrt(sA) and
+    // it carries sA already, so the operand stays below 2^11
     float sy, sAy;
     auto set_sy = [&]() {
       const int e = 127 - int(__float_as_uint(sA) >> 23);   // sA = 2^-e
-      const int k = 10 + (e >> 1);
-      sy = __uint_as_float(uint32_t(127 + k) << 23);
-      sAy = sAi * pow2_inverse(sy);
+      sy = __uint_as_float(uint32_t(134 + (e >> 1)) << 23);
+      sAy = (e & 1) ? -1.0f / 8192.0f : -1.0f / 16384.0f;   // -1 / (sA sy^2)
     };
     set_sy();
     if (nch > 0) wait(&kfull[0], 0);
@@ -570,46 +592,38 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       // kept near the top of fp16's range, or the remainders would run into its subnormals
       const bool look = (c & 7) == 7 || c < D / 4;
       if (look) {
-        float mx = 0.f;
-#pragma unroll
-        for (int nt = 0; nt < NTILE; ++nt)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fabsf(st[nt][e]));
-        mx = warp_max_nonneg(mx);
+        const float mx = state_max(st);
         if (lane == 0) mxs[warp] = mx;
       }
       named_sync(4, (NW + 1) * 32);   // L^-1
       // ---- Z^T = Z0^T L^-T
       float z[2][4] = {};
       small_product<LD>(z, z0, Li, lane);
-      vec_store(sb + Cfg::a_Z + my_rows, z);
       uint32_t yh[4], yl[4];
       {
         float y[2][4];
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
+        for (int nt = 0; nt < 2; ++nt) {
+          const float2 id2 = *reinterpret_cast<const float2*>(dl + 16 + 8 * nt + 2 * c4);
+          const float2 rs2 = *reinterpret_cast<const float2*>(dl + 32 + 8 * nt + 2 * c4);
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            const float idl = dl[16 + 8 * nt + 2 * c4 + (e & 1)];
-            y[nt][e] = -z[nt][e] * idl;
-            if (!UT) a1[nt][e] = -y[nt][e] * sAi;   // u = k_hat: a_t = z_t / delta_t
-            else { z1[nt][e] = z[nt][e]; w1[nt][e] = w0[nt][e]; }
+            const int s = 8 * nt + 2 * c4 + (e & 1);
+            y[nt][e] = z[nt][e] * (e & 1 ? rs2.y : rs2.x);
             if (STASH && UT) {
-              const int t = c * C + 8 * nt + 2 * c4 + (e & 1);
-              if (t < T) sh.zeta[(size_t(unit) * T + t) * D + row0 + g + 8 * (e >> 1)] = z[nt][e] * sAi * sqrt_ftz(idl);
+              if (c * C + s < T) sh.zeta[(size_t(unit) * T + c * C + s) * D + row0 + g + 8 * (e >> 1)] = y[nt][e] * sAi;
             }
+            y[nt][e] *= sy;
+            if (!UT) a1[nt][e] = z[nt][e] * (e & 1 ? id2.y : id2.x) * sAi;   // u = k_hat: a_t = z_t / delta_t
+            else { z1[nt][e] = z[nt][e]; w1[nt][e] = w0[nt][e]; }
           }
+        }
         sz1 = sAi;
-        // z / delta may lie far below z: scaled up on its own, or its remainders would be fp16 subnormals
-        // (|z / delta| <= sqrt(max A) / 2 whatever u is, so sy * y stays below 2^14)
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) y[nt][e] *= sy;
+        vec_store(sb + Cfg::a_Z + my_rows, y);
         split_frag(y[0], y[1], yh, yl);
       }
       named_sync(1, NW * 32);
-      // ---- A <- A - Z^T diag(1/delta) Z
+      // ---- A <- A - sum zeta zeta^T
 #pragma unroll
       for (int nt = 0; nt < NTILE; nt += NB) {
         uint32_t b[NB][4];

@@ -57,3 +57,36 @@ def test_scales_of_the_backward_chains_fall_with_them(d, T, flags):
         for n in names:
             assert _rel(getattr(got, n)[:, :, part], getattr(ref, n)[:, :, part]) <= FALLEN, n
         assert _rel(got.dS0, ref.dS0) <= FALLEN
+
+
+# An explicit u is used verbatim, whatever its norm.  While fewer tokens than dimensions have come, A keeps directions of its first
+# size beside ones shrunk by (1 + |u|^2 / lambda), and the fp32 kernels stay within 1e-4 (A_T, S_T) of the oracle; three times that.
+VERBATIM = 3e-4
+
+
+@pytest.mark.parametrize("d", [16, 32, 64, 128])
+@pytest.mark.parametrize("norm", [1e-3, 30.0, 1e3, 1e5, 1e10, "mixed"])
+def test_explicit_u_of_any_norm(d, norm):
+    w = W.Workload("norm", 1, 2, d, d - 3, "f32", 13)
+    q, k, v = W.make_inputs(w)
+    u = W.make_u(w, 1.0)
+    # mixed: every token its own norm between 1e-3 and 1e4
+    u = u * (10.0 ** (7 * torch.rand(u.shape[:-1] + (1,), generator=torch.Generator().manual_seed(2)) - 3) if norm == "mixed" else norm)
+    for lam in (1.0, 0.01):
+        for flags in (0, IDENT):
+            ref = run_oracle(q, k, v, lam, u=u, flags=flags)
+            r = run_gpu(q, k, v, lam, u=u, flags=flags, kernel=PAIR)
+            for n in ("out", "S_T", "A_T"):
+                assert _rel(getattr(r, n), getattr(ref, n)) <= VERBATIM, (n, lam, flags)
+
+
+@pytest.mark.parametrize("d", [32, 128])
+@pytest.mark.parametrize("lam", [1e-6, 1e-10, 1e-14])
+def test_small_lambda(d, lam):
+    """A starts at 1 / lambda: its update's two operands are of one size however large the ratio is (z / delta alone was lost
+    in subnormals: A_T wrong by 8e-4 at 1e-14, the fp32 kernels by 5e-6 at d = 32, 8e-5 at d = 128; three times these)."""
+    w = W.Workload("lam", 1, 2, d, d - 3, "f32", 14)
+    q, k, v = W.make_inputs(w)
+    ref = run_oracle(q, k, v, lam, flags=IDENT)
+    r = run_gpu(q, k, v, lam, flags=IDENT, kernel=PAIR)
+    assert _rel(r.A_T, ref.A_T) <= (1.5e-5 if d == 32 else 2.5e-4)

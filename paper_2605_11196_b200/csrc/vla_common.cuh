@@ -401,6 +401,41 @@ __device__ __forceinline__ float eliminate16(float (&m)[8], int lane, float* piv
   return delta;
 }
 
+// ... of a matrix of any size: pivots above 1e18 (explicit u of norm 1e9 and more) would overflow in the 2 x 2 determinant, so
+// rows and columns are brought to diagonals of order one by powers of two first, and back afterwards.  piv: 80 floats.
+__device__ __forceinline__ float eliminate16_any(float (&m)[8], int lane, float* piv, float eps) {
+  constexpr unsigned full = 0xffffffffu;
+  const int r = lane & 15, h = lane >> 4;
+  float* own = piv + 64;
+  float big = 0.f, dr = 0.f;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    big = fmaxf(big, fabsf(m[j]));
+    dr = 8 * h + j == r ? m[j] : dr;
+  }
+  const bool far = __any_sync(full, big > 1e18f);
+  float er = 1.0f;
+  if (far) {
+    dr = fmaxf(__shfl_sync(full, dr, r + 16 * (r >> 3)), 1.0f);
+    er = __uint_as_float((127u - ((__float_as_uint(dr) >> 23) - 127u) / 2u) << 23);   // 2^-floor(log2(dr) / 2)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m[j] = m[j] * er * __shfl_sync(full, er, 8 * h + j);
+  }
+  if (h == 0) own[r] = er * er;
+  __syncwarp();
+  float delta = eliminate16<true>(m, lane, piv, eps, own);
+  if (far) {
+    const float ie = 1.0f / er;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float ec = __shfl_sync(full, er, 8 * h + j);
+      m[j] = 8 * h + j < r ? m[j] * ec * ie : m[j] * ie * (1.0f / ec);
+    }
+    delta *= ie * ie;
+  }
+  return delta;
+}
+
 // Reduce-scatter of 16 values over a full warp: lanes 2t and 2t+1 end with the sum of v[t].
 __device__ __forceinline__ float warp_reduce_scatter16(float (&v)[16], int lane) {
 #pragma unroll

@@ -649,7 +649,7 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
         }
         __syncwarp();
         // (the pivot rows pass through an array that is free by now)
-        const float delta = eliminate16(m, lane, HAS_U ? PTs : Ws, eps);
+        const float delta = UT ? eliminate16_any(m, lane, PTs, eps) : eliminate16(m, lane, HAS_U ? PTs : Ws, eps);
         *reinterpret_cast<float4*>(Ls + r * CP + h * 8) = make_float4(m[0], m[1], m[2], m[3]);
         *reinterpret_cast<float4*>(Ls + r * CP + h * 8 + 4) = make_float4(m[4], m[5], m[6], m[7]);
         if (h == 0) {

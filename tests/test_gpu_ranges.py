@@ -90,3 +90,17 @@ def test_small_lambda(d, lam):
     ref = run_oracle(q, k, v, lam, flags=IDENT)
     r = run_gpu(q, k, v, lam, flags=IDENT, kernel=PAIR)
     assert _rel(r.A_T, ref.A_T) <= (1.5e-5 if d == 32 else 2.5e-4)
+
+
+@pytest.mark.parametrize("d", [32, 64, 128])
+@pytest.mark.parametrize("norm", [1e5, 1e10, 1e12])
+def test_explicit_u_of_any_norm_on_the_chunk_kernel(d, norm):
+    """The fp32 chunk kernel (and with it the periodic refresh): pivots far beyond the square root of fp32's range."""
+    w = W.Workload("norm", 1, 2, d, d - 3, "f32", 13)
+    q, k, v = W.make_inputs(w)
+    u = W.make_u(w, norm)
+    for lam, refresh in ((1.0, None), (0.01, None), (1.0, (2 * d, 1e-3, 0))):
+        ref = run_oracle(q, k, v, lam, u=u, refresh=refresh)
+        r = run_gpu(q, k, v, lam, u=u, kernel=vla.VLA_KERNEL_CHUNK, refresh=refresh)
+        for n in ("out", "S_T", "A_T", "z_T"):
+            assert _rel(getattr(r, n), getattr(ref, n)) <= VERBATIM, (n, lam)

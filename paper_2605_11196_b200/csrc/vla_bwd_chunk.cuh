@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(BwdBlockCfg<D>::NT) bwd_block_kernel(const Bwd
   constexpr int BC = kBwdBlock, KS = D / 16, CS = Cfg::CS, NWB = Cfg::NWB, NT = Cfg::NT, NH = D / 8 / CS;   // NH: n tiles of a column group
   constexpr float kInv = 1.0f / 256.0f;
   extern __shared__ __align__(128) unsigned char smem[];
-  const int blk = blockIdx.x, unit = blockIdx.y;
+  const int unit = blockIdx.x / p.NB, blk = blockIdx.x - unit * p.NB;
   const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int tg = warp & 1, h = (warp >> 1) % CS, role = warp / (2 * CS);
@@ -951,8 +951,8 @@ __global__ void __launch_bounds__(BwdBlockCfg<D>::NT) bwd_block_kernel(const Bwd
 // entries of the sum: known while walking, at most the number of blocks above the true maximum.
 template <int D>
 __global__ void __launch_bounds__(256) bwd_scan_kernel(const BwdChunkParams p) {
-  const int unit = blockIdx.y, i = blockIdx.x * 256 + threadIdx.x;
-  constexpr int N = D * D / 4;
+  constexpr int N = D * D / 4, CTAS = (N + D + 255) / 256;   // of a unit
+  const int unit = blockIdx.x / CTAS, i = (blockIdx.x - unit * CTAS) * 256 + threadIdx.x;
   if (i < N) {
     const size_t ub = size_t(unit) * p.NB;
     const float4* x = reinterpret_cast<const float4*>(p.X + ub * D * D) + i;
@@ -1043,7 +1043,7 @@ __global__ void __launch_bounds__(BwdFinishCfg<D, UT>::NT) bwd_finish_kernel(con
   constexpr int BC = kBwdBlock, KS = D / 16, NWB = Cfg::NWB, NT = Cfg::NT;
   constexpr float kInv = 1.0f / 256.0f;
   extern __shared__ __align__(128) unsigned char smem[];
-  const int blk = blockIdx.x, unit = blockIdx.y;
+  const int unit = blockIdx.x / p.NB, blk = blockIdx.x - unit * p.NB;
   const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c4 = lane & 3;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int t0 = blk * BC, T = p.T, nt_valid = min(BC, T - t0), nchv = min(2, p.nch - 2 * blk);

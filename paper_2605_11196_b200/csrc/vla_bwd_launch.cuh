@@ -30,14 +30,16 @@ int launch_bwd_chunk_t(const BwdChunkParams& p, cudaStream_t st) {
     cudaGetLastError();
     return VLA_ERR_CUDA;
   }
-  const long long chunks = (long long)p.units * p.nch;
-  const dim3 blocks(p.NB, p.units);
+  // (units in the grid's x, which may pass 65535; a unit's blocks are neighbours in it)
+  const long long chunks = (long long)p.units * p.nch, blocks = (long long)p.units * p.NB;
+  constexpr int kScanCtas = (D * D / 4 + D + 255) / 256;
+  if (chunks > 0x7fffffffLL || (long long)p.units * kScanCtas > 0x7fffffffLL) return VLA_ERR_INVALID_ARG;
   prep<<<unsigned((chunks + Prep::WPC - 1) / Prep::WPC), Prep::WPC * 32, Prep::smem_bytes, st>>>(p);
   chains<<<2 * p.units, Chain::NT, Chain::smem_bytes, st>>>(p);
   if (p.dA_T) bwd_final_state_kernel<D><<<p.units, 256, 0, st>>>(p);
-  block<<<blocks, Block::NT, Block::smem_bytes, st>>>(p);
-  bwd_scan_kernel<D><<<dim3((D * D / 4 + D + 255) / 256, p.units), 256, 0, st>>>(p);
-  fin<<<blocks, Fin::NT, Fin::smem_bytes, st>>>(p);
+  block<<<unsigned(blocks), Block::NT, Block::smem_bytes, st>>>(p);
+  bwd_scan_kernel<D><<<unsigned(p.units) * kScanCtas, 256, 0, st>>>(p);
+  fin<<<unsigned(blocks), Fin::NT, Fin::smem_bytes, st>>>(p);
   return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
 }
 

@@ -251,9 +251,13 @@ size_t vla_seqpar_workspace_bytes(int B, int H, int T, int d_k, int segments);
  * which must then be non-NULL; d in {32, 64, 128}); the periodic refresh of opts (d in
  * {32, 64, 128}); VLA_FLAG_TOKEN_MAJOR (d in {32, 64, 128}); anything else returns
  * VLA_ERR_UNSUPPORTED.  `workspace` is a
- * DEVICE buffer of at least vla_backward_workspace_bytes(B, H, T, d_k) bytes (per token: z_t,
- * e_t, delta_t of the forward and three vectors the two reverse scans exchange; the final
- * states), owned by the caller and free for reuse once the work enqueued on `stream` has completed.
+ * DEVICE buffer of at least vla_backward_workspace_bytes(B, H, T, d_k) bytes, owned by the caller and free for
+ * reuse once the work enqueued on `stream` has completed.
+ *
+ * Two forms of the pass: the chunked one, several times faster, and with dA0 or the refresh the token-level one.  The
+ * workspace serves either.  The chunked form takes its units in groups whose part stays below 4 GiB, or below what the
+ * token-level form needs for the whole batch (seven fp32 vectors and a few words per token, two matrices per unit) where that is
+ * more; so the answer is at most the larger of the two, but for a single unit that is above them by itself.
  */
 int vla_backward(const void* q, const void* k, const void* v, float lambda_,
                  int B, int H, int T, int d_k, int d_v,

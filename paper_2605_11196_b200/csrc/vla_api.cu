@@ -285,13 +285,24 @@ BwdLayout bwd_layout(size_t T, size_t d) {
   return L;
 }
 size_t bwd_unit_bytes(size_t T, size_t d) { return bwd_layout(T, d).total; }
-// Units per pass.  The chains of a pass run one CTA per unit, so all units go at once while the workspace stays
-// below 4 GiB; beyond that groups of at least one unit per SM take turns in it ([B,T,H,d] tensors: whole
-// batch entries).
-size_t bwd_group(size_t units, size_t H, size_t T, size_t d) {
-  const size_t fits = (size_t(4) << 30) / bwd_unit_bytes(T, d), want = fits > 148 ? fits : 148;
-  if (units <= want) return units;
-  return H >= want ? H : want / H * H;
+// Units per pass, at most.  All at once while their workspace stays below 4 GiB, or below what the token-level scans
+// take for the whole batch where that is more (their form of the pass needs it anyway); beyond that groups take turns
+// in it, which leaves chains of few units idle SMs but keeps the bound.  Only a single unit may be above it.
+constexpr size_t kBwdWorkspace = size_t(4) << 30;
+size_t bwd_units(size_t units, size_t T, size_t d) {
+  const size_t one = bwd_unit_bytes(T, d), scans = backward_scans_bytes(units, T, d);
+  const size_t fits = (scans > kBwdWorkspace ? scans : kBwdWorkspace) / one;
+  return fits < 1 ? 1 : fits < units ? fits : units;
+}
+// The number taken from u0 on: groups of one size as far as they go.  [B,T,H,d] tensors are cut at batch entries, or
+// within one where not even that fits.
+size_t bwd_group(size_t u0, size_t units, size_t H, size_t most, bool token_major) {
+  auto even = [](size_t n, size_t at_most) { const size_t g = (n + at_most - 1) / at_most; return (n + g - 1) / g; };
+  size_t n;
+  if (!token_major) n = even(units, most);
+  else if (most >= H) n = even(units / H, most / H) * H;
+  else return std::min(even(H, most), H - u0 % H);
+  return std::min(n, units - u0);
 }
 
 // One event per (device, flag slot) of the balanced schedule, recorded behind the launch that
@@ -310,11 +321,12 @@ int backward_chunked(const void* q, const void* k, const void* v, float lambda_,
                      unsigned char* w, cudaStream_t st) {
   const size_t es = o.qkv_dtype == VLA_F32 ? 4 : 2, Tz = size_t(T), dd = size_t(d);
   const BwdLayout L = bwd_layout(Tz, dd);
-  const size_t group = bwd_group(size_t(units), size_t(H), Tz, dd);
-  for (size_t u0 = 0; u0 < size_t(units); u0 += group) {
-    const size_t n = size_t(units) - u0 < group ? size_t(units) - u0 : group;
-    // (a [B,T,H,d] group starts at a batch entry, so unit u0's tokens start at u0 T d in both layouts)
-    const size_t tok = u0 * Tz * dd, sq = u0 * dd * dd;
+  const bool token_major = (o.flags & VLA_FLAG_TOKEN_MAJOR) != 0;
+  const size_t most = bwd_units(size_t(units), Tz, dd), Hz = size_t(H);
+  for (size_t u0 = 0, n; u0 < size_t(units); u0 += n) {
+    n = bwd_group(u0, size_t(units), Hz, most, token_major);
+    // unit u0's first token (a [B,T,H,d] group that starts within a batch entry also ends there)
+    const size_t tok = (token_major ? u0 / Hz * Hz * Tz + u0 % Hz : u0 * Tz) * dd, sq = u0 * dd * dd;
     auto in = [&](const void* p) { return p ? static_cast<const void*>(static_cast<const unsigned char*>(p) + tok * es) : nullptr; };
     auto at = [](auto* p, size_t off) { return p ? p + off : p; };
     auto ws = [&](size_t off) { return w + off * n; };
@@ -727,10 +739,9 @@ int vla_forward_seqpar(const void* q, const void* k, const void* v, float lambda
 
 size_t vla_backward_workspace_bytes(int B, int H, int T, int d_k) {
   if (B < 0 || H < 0 || T < 0 || d_k <= 0) return 0;
-  const size_t units = size_t(B) * size_t(H);
-  const size_t one = bwd_unit_bytes(size_t(T), size_t(d_k)), group = bwd_group(units, size_t(H), size_t(T), size_t(d_k));
-  const size_t scans = backward_scans_bytes(units, size_t(T), size_t(d_k));
-  return one * group + 256 > scans ? one * group + 256 : scans;
+  const size_t units = size_t(B) * size_t(H), Tz = size_t(T), dz = size_t(d_k);
+  const size_t chunked = bwd_unit_bytes(Tz, dz) * bwd_units(units, Tz, dz) + 256, scans = backward_scans_bytes(units, Tz, dz);
+  return chunked > scans ? chunked : scans;
 }
 
 int vla_backward(const void* q, const void* k, const void* v, float lambda_, int B, int H, int T,

@@ -24,3 +24,27 @@ def test_more_units_than_a_grids_second_dimension(B, H, T, d):
         q, k, v, do, dS, dA = [y[s].contiguous() for y in x + [dS_T, dA_T]]
         _same(a, s, vla.vla_backward(q, k, v, 1.0, do, dS_T=dS, dA_T=dA, want_dA0=False))
     assert int(a.status.item()) == 0
+
+
+@pytest.mark.parametrize("tm,B,H", [(False, 1, 61), (True, 12, 5), (True, 1, 61), (True, 2, 61)])
+def test_groups_of_either_layout(tm, B, H):
+    """T = 8192, d = 128: 94 MB a unit, so 60 units pass 4 GiB and take turns: whole batch entries, and parts of one
+    where a single entry is too large.  Explicit u, carried states and state gradients, the last units of every group."""
+    T, d = 8192, 128
+    g = torch.Generator(device="cuda").manual_seed(2)
+    rnd = lambda *s: torch.randn(s, generator=g, device="cuda")
+    seq = (B, T, H, d) if tm else (B, H, T, d)
+    q, k, v, u = [rnd(*seq).bfloat16() for _ in range(4)]
+    u = torch.nn.functional.normalize(u.float(), dim=-1).bfloat16()
+    do, S0, dS_T, dA_T, z0, dz_T = rnd(*seq), rnd(B, H, d, d), rnd(B, H, d, d), rnd(B, H, d, d), 5 + rnd(B, H, d).abs(), rnd(B, H, d)
+    h = 0.05 * rnd(B, H, d, d)
+    A0 = (h @ h.transpose(-1, -2) + 0.5 * torch.eye(d, device="cuda")).contiguous()
+    flags = vla.VLA_FLAG_TOKEN_MAJOR if tm else 0
+    a = vla.vla_backward(q, k, v, 1.0, do, u=u, S0=S0, A0=A0, z0=z0, dS_T=dS_T, dA_T=dA_T, dz_T=dz_T, flags=flags, want_dA0=False)
+    assert int(a.status.item()) == 0
+    for b, hh in [(0, 0), (B - 1, H - 1), (B // 2, H // 2), (0, H - 1), (B - 1, 0)]:
+        c = lambda x: x[b:b + 1, :, hh:hh + 1].contiguous() if tm and x.dim() == 4 and x.shape[1] == T else x[b:b + 1, hh:hh + 1].contiguous()
+        own = vla.vla_backward(c(q), c(k), c(v), 1.0, c(do), u=c(u), S0=c(S0), A0=c(A0), z0=c(z0), dS_T=c(dS_T), dA_T=c(dA_T),
+                               dz_T=c(dz_T), flags=flags, want_dA0=False)
+        for n in ("dq", "dk", "dv", "du", "dS0", "dz0"):
+            assert torch.equal(c(getattr(a, n)), getattr(own, n)), (n, b, hh)

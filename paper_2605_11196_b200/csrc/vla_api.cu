@@ -294,6 +294,11 @@ size_t bwd_units(size_t units, size_t T, size_t d) {
   const size_t fits = (scans > kBwdWorkspace ? scans : kBwdWorkspace) / one;
   return fits < 1 ? 1 : fits < units ? fits : units;
 }
+// Either form's arrays come first, then a word per unit (PairStash::far).
+size_t backward_far_offset(size_t units, size_t T, size_t d) {
+  const size_t chunked = bwd_unit_bytes(T, d) * bwd_units(units, T, d), scans = backward_scans_bytes(units, T, d);
+  return round256(chunked > scans ? chunked : scans);
+}
 // The number taken from u0 on: groups of one size as far as they go.  [B,T,H,d] tensors are cut at batch entries, or
 // within one where not even that fits.
 size_t bwd_group(size_t u0, size_t units, size_t H, size_t most, bool token_major) {
@@ -318,7 +323,7 @@ thread_local LaunchNote g_last_launch = {"", 0, 0, 0, 0};
 int backward_chunked(const void* q, const void* k, const void* v, float lambda_, int H, int T, int d, int units,
                      const float* S0, const float* A0, const float* d_out, const float* dS_T, const float* dA_T,
                      const float* dz_T, float* dq, float* dk, float* dv, float* dS0, float* dz0, const vla_opts_t& o,
-                     unsigned char* w, cudaStream_t st) {
+                     unsigned char* w, int* far, cudaStream_t st) {
   const size_t es = o.qkv_dtype == VLA_F32 ? 4 : 2, Tz = size_t(T), dd = size_t(d);
   const BwdLayout L = bwd_layout(Tz, dd);
   const bool token_major = (o.flags & VLA_FLAG_TOKEN_MAJOR) != 0;
@@ -337,7 +342,7 @@ int backward_chunked(const void* q, const void* k, const void* v, float lambda_,
     vla::PairStash sh;
     sh.alpha = wf(L.alpha); sh.zeta = wf(L.zeta); sh.zkc = wf(L.zkc);
     sh.delta = wf(L.scal); sh.an = sh.delta + scal;
-    sh.Aimg = ws(L.Aimg); sh.Asc = wf(L.sc); sh.ck = 2;
+    sh.Aimg = ws(L.Aimg); sh.Asc = wf(L.sc); sh.ck = 2; sh.far = at(far, u0);
     ScanParams f = {};
     f.q = in(q); f.k = in(k); f.v = in(v); f.u = in(o.u);
     f.A0 = at(A0, sq); f.z0 = at(o.z0, u0 * dd);
@@ -740,8 +745,7 @@ int vla_forward_seqpar(const void* q, const void* k, const void* v, float lambda
 size_t vla_backward_workspace_bytes(int B, int H, int T, int d_k) {
   if (B < 0 || H < 0 || T < 0 || d_k <= 0) return 0;
   const size_t units = size_t(B) * size_t(H), Tz = size_t(T), dz = size_t(d_k);
-  const size_t chunked = bwd_unit_bytes(Tz, dz) * bwd_units(units, Tz, dz) + 256, scans = backward_scans_bytes(units, Tz, dz);
-  return chunked > scans ? chunked : scans;
+  return backward_far_offset(units, Tz, dz) + round256(units * sizeof(int)) + 256;
 }
 
 int vla_backward(const void* q, const void* k, const void* v, float lambda_, int B, int H, int T,
@@ -772,8 +776,21 @@ int vla_backward(const void* q, const void* k, const void* v, float lambda_, int
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // The chunked form: everything but the refresh (M_t is no longer a plain sum there) and the gradient of A0,
   // which is taken entry by entry through the recurrence and needs its adjoint of A
-  if (T > 0 && o.refresh_period <= 0 && !dA0)
-    return backward_chunked(q, k, v, lambda_, H, T, d_k, units, S0, A0, d_out, dS_T, dA_T, dz_T, dq, dk, dv, dS0, dz0, o, w, st);
+  int* far = nullptr;
+  if (T > 0 && o.refresh_period <= 0 && !dA0) {
+    // It forms du_t = -X_t u_t from a sum over later tokens, which cancels delta_t-fold where u_t shrank A a lot: du was wrong
+    // by 2e-7 delta of its size (delta 1e3: 2e-4, as the token-level form at T = 1000; 1e6, an explicit u of norm 1000: 0.4).  Units in
+    // which some delta passes kFarDelta are gone over again by the token-level form, where the arguments allow such a delta.
+    if (o.u || A0 || lambda_ * (vla::kFarDelta - 1.0f) < 1.0f) {
+      far = reinterpret_cast<int*>(w + backward_far_offset(size_t(units), size_t(T), size_t(d_k)));
+      if (cudaMemsetAsync(far, 0, size_t(units) * sizeof(int), st) != cudaSuccess) {
+        cudaGetLastError();
+        return VLA_ERR_CUDA;
+      }
+    }
+    rc = backward_chunked(q, k, v, lambda_, H, T, d_k, units, S0, A0, d_out, dS_T, dA_T, dz_T, dq, dk, dv, dS0, dz0, o, w, far, st);
+    if (rc != VLA_OK || !far) return rc;
+  }
   const size_t vec = round256(size_t(units) * T * d_k * sizeof(float));
   const size_t mat = round256(size_t(units) * d_k * d_k * sizeof(float));
   const size_t sca = round256(size_t(units) * T * sizeof(float));
@@ -793,7 +810,7 @@ int vla_backward(const void* q, const void* k, const void* v, float lambda_, int
     p.d_out = d_out; p.dS_T = dS_T; p.dA_T = dA_T; p.dz_T = dz_T;
     p.dq = dq; p.dk = dk; p.dv = dv; p.dS0 = dS0; p.dA0 = dA0; p.dz0 = dz0;
     p.zst = zst; p.est = est; p.dst = dst; p.zkc = zkcw;
-    p.status = o.status; p.lambda = lambda_; p.eps = o.eps; p.T = T; p.units = units; p.flags = o.flags;
+    p.status = o.status; p.lambda = lambda_; p.eps = o.eps; p.T = T; p.units = units; p.flags = o.flags; p.only = far;
     return vla::launch_backward(d_k, o.qkv_dtype, p, st);
   }
   // 1. the forward recurrence on the chunk kernel, leaving z_t, e_t, delta_t and the final states
@@ -815,8 +832,9 @@ int vla_backward(const void* q, const void* k, const void* v, float lambda_, int
   f.stash_z = zst; f.stash_e = est; f.stash_delta = dst; f.stash_zk = zkcw; f.stash_a = general ? astw : nullptr;
   f.heads = H;
   f.wait_limit = o.wait_probe_limit;
+  f.only = far;
   // d = 128, u = k_hat, no refresh: the tensor-core form of the chunk kernel leaves the same stash
-  if (chunk_tc_covers(f, d_k)) rc = vla::launch_chunk_tc_stash(d_k, o.qkv_dtype, f, st);
+  if (!far && chunk_tc_covers(f, d_k)) rc = vla::launch_chunk_tc_stash(d_k, o.qkv_dtype, f, st);
   else rc = vla::launch_chunk_stash(d_k, o.qkv_dtype, f, st);
   if (rc != VLA_OK) return rc;
   // 2. the S-side and A-side reverse scans
@@ -829,6 +847,7 @@ int vla_backward(const void* q, const void* k, const void* v, float lambda_, int
   p.general = general ? 1 : 0;
   p.heads = H;
   p.progress = progw;
+  p.only = far;
   p.refresh_period = o.refresh_period; p.refresh_eta = o.refresh_eta; p.step_offset = o.step_offset;
   return vla::launch_backward_split(d_k, o.qkv_dtype, p, st);
 }

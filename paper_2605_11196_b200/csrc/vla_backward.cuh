@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(256) vla_backward_token_kernel(const BackwardP
   float* gz = gzbuf;    // dL/d(key sum), carried by the closing warp
 
   const int unit = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (p.only && !p.only[unit]) return;
   const int ty = tid >> 4, tx = tid & 15;
   const int row0 = ty * R, col0 = tx * R;
   const bool ident = (p.flags & VLA_FLAG_IDENTITY_MAP) != 0;

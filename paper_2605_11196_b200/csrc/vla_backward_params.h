@@ -26,6 +26,7 @@ struct BackwardParams {
   float* est;           // workspace [units, T, D]  e_t
   float* dst;           // workspace [units, T]     delta_t
   float* zkc;           // workspace [units, ceil(T / 16), D]  key sum after each 16 tokens
+  const int* only;      // [units]: units whose word is 0 are left out; nullptr: none is
   int* status;
   float lambda;
   float eps;
@@ -65,6 +66,7 @@ struct BackwardSplitParams {
   float* dz0;           // [units, D] or nullptr
   int* progress;             // [units + 1], zero on entry: per unit the tokens (from the end) whose S-side
                              // vectors are out; the last word hands out the CTAs' tickets
+  const int* only;      // [units]: units whose word is 0 are left out; nullptr: none is
   int* status;
   float eps;
   int T;

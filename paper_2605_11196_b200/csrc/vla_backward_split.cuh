@@ -943,6 +943,7 @@ vla_backward_sa_kernel(const BackwardSplitParams p) {
   if (threadIdx.x == 0) *ticket_s = atomicAdd(p.progress + p.units, 1);   // the word after the units' own
   __syncthreads();
   const int ticket = *ticket_s;
+  if (p.only && !p.only[ticket < p.units ? ticket : ticket - p.units]) return;
   if (ticket < p.units) vla_backward_s_body<D, TIn, UX>(p, ticket, smem_raw);
   else vla_backward_a_body<D, TIn, UX>(p, ticket - p.units, smem_raw);
 }

@@ -39,7 +39,7 @@ int launch_chunk_um_tm(const ScanParams& p, cudaStream_t st) {
   // Not while the stream is being captured into a CUDA graph: the hand-over flags are keyed by a
   // launch number drawn here, on the host, and every replay of the graph would carry the same one.
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
+  if (p.only || cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
     cudaGetLastError();
     capture = cudaStreamCaptureStatusActive;
   }
@@ -77,8 +77,9 @@ int launch_chunk_um_tm(const ScanParams& p, cudaStream_t st) {
   } else {
     kern<<<sp.grid, Cfg::NT, Cfg::smem_bytes, st>>>(p, sp, maps);
   }
-  note_launch(STASH ? "vla_scan_chunk_kernel(stash)" : "vla_scan_chunk_kernel", D, sizeof(TIn) == 2 ? VLA_BF16 : VLA_F32,
-              sp.grid, sp.balanced);
+  if (!p.only)
+    note_launch(STASH ? "vla_scan_chunk_kernel(stash)" : "vla_scan_chunk_kernel", D, sizeof(TIn) == 2 ? VLA_BF16 : VLA_F32,
+                sp.grid, sp.balanced);
   return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
 }
 

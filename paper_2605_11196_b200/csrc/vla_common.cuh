@@ -52,6 +52,8 @@ struct ScanParams {
   // Failed probes after which a device-side wait gives up and reports VLA_ERR_DEVICE_TIMEOUT
   // (0: the library's default, kWaitProbeLimit).
   uint32_t wait_limit = 0;
+  // With a stash, one CTA per unit: units whose word is 0 are left out (nullptr: none is).
+  const int* only = nullptr;
 #ifdef VLA_SECTION_TIMERS
   long long* dbg;      // debug builds only: per-section clock64 totals of unit 0
 #endif

@@ -270,6 +270,8 @@ vla_scan_chunk_kernel(const ScanParams p, const SchedParams sp,
   static_assert(TR == LPR, "row ownership after the reduce-scatter needs TR == D/TW");
   static_assert(C == 16, "the small-matrix code is written for 16-token chunks");
 
+  if (STASH && p.only && !p.only[blockIdx.x]) return;
+
   extern __shared__ __align__(128) unsigned char smem[];
   TIn* raw = reinterpret_cast<TIn*>(smem);
   float* fbase = reinterpret_cast<float*>(smem + Cfg::raw_bytes);

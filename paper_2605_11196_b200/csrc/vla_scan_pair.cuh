@@ -324,7 +324,11 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         }
       }
       named_arrive(4, (NW + 1) * 32);   // L^-1 and delta are written
-      if (STASH && h == 0 && c * C + r < T) sh.delta[size_t(unit) * T + c * C + r] = UT ? delta * pow2_inverse(one) : delta;
+      if (STASH && h == 0 && c * C + r < T) {
+        const float dt = UT ? delta * pow2_inverse(one) : delta;
+        sh.delta[size_t(unit) * T + c * C + r] = dt;
+        if (sh.far && !(dt <= kFarDelta)) sh.far[unit] = 1;
+      }
       if constexpr (UT) {
         // N = L^-1 X, X[s][t] = u'_s . A k_t;  PT[t][s] = N[s][t] / delta_s for s <= t
         // (X and PT alternate between two buffers: the state warps may be a chunk ahead here)

@@ -104,3 +104,44 @@ def test_explicit_u_of_any_norm_on_the_chunk_kernel(d, norm):
         r = run_gpu(q, k, v, lam, u=u, kernel=vla.VLA_KERNEL_CHUNK, refresh=refresh)
         for n in ("out", "S_T", "A_T", "z_T"):
             assert _rel(getattr(r, n), getattr(ref, n)) <= VERBATIM, (n, lam)
+
+
+@pytest.mark.parametrize("d", [32, 64, 128])
+@pytest.mark.parametrize("norm", [100.0, 1e3, 1e5, 1e10])
+@pytest.mark.parametrize("tm", [False, True])
+def test_gradients_with_explicit_u_of_any_norm(d, norm, tm):
+    """du of a u that shrank A a lot cancels in the chunked form, which leaves such units to the token-level one (bound as
+    above).  The other units of the call (norm 1 / sqrt(d)) keep the chunked form's accuracy."""
+    w = W.Workload("norm", 2, 2, d, d - 3, "f32", 13)
+    q, k, v = W.make_inputs(w)
+    u = W.make_u(w, d ** -0.5)
+    u[:, 1] *= norm * d ** 0.5
+    do = torch.randn(q.shape, generator=torch.Generator().manual_seed(3))
+    lay = (lambda x: x.transpose(1, 2).contiguous()) if tm else (lambda x: x)
+    for lam in (1.0, 0.01):
+        ref = oracle.backward(q.numpy(), k.numpy(), v.numpy(), lam, do.double().numpy(), u=u.numpy(), in_dtype=oracle.F32, n_threads=NTHREADS)
+        got = vla.vla_backward(lay(q).cuda(), lay(k).cuda(), lay(v).cuda(), lam, lay(do).cuda(), u=lay(u).cuda(), want_dA0=False,
+                               flags=vla.VLA_FLAG_TOKEN_MAJOR if tm else 0)
+        assert int(got.status.item()) == 0
+        for h, tol in ((0, 5e-5), (1, VERBATIM)):
+            for n in ("dq", "dk", "dv", "du"):
+                assert _rel(lay(getattr(got, n))[:, h], getattr(ref, n)[:, h]) <= tol, (n, h, lam)
+            assert _rel(got.dS0[:, h], ref.dS0[:, h]) <= tol
+
+
+@pytest.mark.parametrize("d", [16, 32, 64, 128])
+def test_gradients_at_small_lambda_and_after_a_large_A0(d):
+    """u = k_hat, while A still has directions of its first size: lambda = 1e-5, and carried states of that size in half of the
+    units.  No further from the oracle than three times the token-level form (1e-6 where that is exact to rounding)."""
+    w = W.Workload("lam", 1, 4, d, d - 3, "f32", 14)
+    q, k, v = W.make_inputs(w)
+    do = torch.randn(q.shape, generator=torch.Generator().manual_seed(3))
+    A0 = torch.eye(d).repeat(1, 4, 1, 1) * torch.tensor([1.0, 1e5, 1.0, 1e5]).view(1, 4, 1, 1)
+    for lam, kw in ((1e-5, {}), (1.0, {"A0": A0})):
+        ref = oracle.backward(q.numpy(), k.numpy(), v.numpy(), lam, do.double().numpy(), in_dtype=oracle.F32, n_threads=NTHREADS,
+                              **{a: x.double().numpy() for a, x in kw.items()})
+        dev = {a: x.cuda() for a, x in kw.items()}
+        got = vla.vla_backward(q.cuda(), k.cuda(), v.cuda(), lam, do.cuda(), want_dA0=False, **dev)
+        tok = vla.vla_backward(q.cuda(), k.cuda(), v.cuda(), lam, do.cuda(), **dev)
+        for n in ("dq", "dk", "dv"):
+            assert _rel(getattr(got, n), getattr(ref, n)) <= 3 * max(_rel(getattr(tok, n), getattr(ref, n)), 1e-6), n

@@ -5,7 +5,8 @@
 //
 // Every entry returns None for anything but well-formed CUDA arguments on the ordinary path; the caller
 // then takes the Python path, which raises the proper errors.  A library status other than VLA_OK comes back as
-// an int.
+// an int.  Whatever throws in between (a tensor subclass that answers for its sizes in Python, an allocation, a
+// saved-tensor hook) leaves as the Python exception torch makes of it.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -14,6 +15,7 @@
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAGraphsC10Utils.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -147,6 +149,7 @@ PyObject* wrap(const Tensor& t) {
 // forward(q, k, v, lam, u, S0, A0, z0, flags, eps, out, S_T, A_T, z_T, status, want_status, kernel, workspace, probes)
 // -> (out, S_T, A_T, z_T, status) | None | status code
 PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
   Tensor q, k, v, u, S0, A0, z0, out, S_T, A_T, z_T, status, ws;
   double lam = 0, eps = 0;
   int64_t flags = 0, kernel = 0, probes = 0;
@@ -170,7 +173,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
       !is_or_none(out, seq, kF32, dev) || !is_or_none(S_T, st4, kF32, dev) || !is_or_none(A_T, st4, kF32, dev) ||
       !is_or_none(z_T, vec, kF32, dev) || (status.defined() && !(status.is_cuda() && status.scalar_type() == at::kInt)))
     Py_RETURN_NONE;
-  try {
+  {
     at::AutoDispatchBelowADInplaceOrView guard;
     c10::cuda::OptionalCUDAGuard on;
     if (c10::cuda::current_device() != dev.index()) on.set_device(dev);
@@ -193,9 +196,6 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int rc = vla_forward(raw(q), raw(k), raw(v), float(lam), int(s.B), int(s.H), int(s.T), int(s.d), int(s.d), f32(S0),
                                f32(A0), f32(out), f32(S_T), f32(A_T), &o, stream.stream());
     if (rc != VLA_OK) return PyLong_FromLong(rc);
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
   }
   PyObject* r = PyTuple_New(5);
   if (!r) return nullptr;
@@ -205,6 +205,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   PyTuple_SET_ITEM(r, 3, wrap(z_T));
   PyTuple_SET_ITEM(r, 4, wrap(status));
   return r;
+  END_HANDLE_TH_ERRORS
 }
 
 // ---------------------------------------------------------------- the scan under autograd
@@ -276,6 +277,7 @@ struct Scan : public torch::autograd::Function<Scan> {
 
 // scan(q, k, v, lam, u, S0, A0, z0, flags, eps, status) -> (out, S_T, A_T, z_T) | None | status code
 PyObject* scan(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
   Tensor q, k, v, u, S0, A0, z0, status;
   double lam = 0, eps = 0;
   int64_t flags = 0;
@@ -297,14 +299,12 @@ PyObject* scan(PyObject*, PyObject* const* a, Py_ssize_t n) {
     r = Scan::apply(q, k, v, opt(u), opt(S0), opt(A0), opt(z0), status, lam, flags, eps);
   } catch (const Failed& f) {
     return PyLong_FromLong(f.code);
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
   }
   PyObject* t = PyTuple_New(4);
   if (!t) return nullptr;
   for (int i = 0; i < 4; ++i) PyTuple_SET_ITEM(t, i, wrap(r[i]));
   return t;
+  END_HANDLE_TH_ERRORS
 }
 
 PyMethodDef methods[] = {

@@ -141,6 +141,17 @@ bool real_arg(PyObject* o, double* x) {
   }
   return false;
 }
+// Without Python's global lock: a launch may wait (a full launch queue, cudaMalloc), and other threads go on meanwhile.
+class Unlocked {
+ public:
+  Unlocked() : state_(PyEval_SaveThread()) {}
+  ~Unlocked() { PyEval_RestoreThread(state_); }
+  Unlocked(const Unlocked&) = delete;
+  Unlocked& operator=(const Unlocked&) = delete;
+
+ private:
+  PyThreadState* state_;
+};
 PyObject* wrap(const Tensor& t) {
   if (!t.defined()) Py_RETURN_NONE;
   return THPVariable_Wrap(t);
@@ -173,7 +184,9 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
       !is_or_none(out, seq, kF32, dev) || !is_or_none(S_T, st4, kF32, dev) || !is_or_none(A_T, st4, kF32, dev) ||
       !is_or_none(z_T, vec, kF32, dev) || (status.defined() && !(status.is_cuda() && status.scalar_type() == at::kInt)))
     Py_RETURN_NONE;
+  int rc = VLA_OK;
   {
+    Unlocked threads;
     at::AutoDispatchBelowADInplaceOrView guard;
     c10::cuda::OptionalCUDAGuard on;
     if (c10::cuda::current_device() != dev.index()) on.set_device(dev);
@@ -193,10 +206,10 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
       o.workspace = ws.data_ptr();
       o.workspace_bytes = size_t(ws.numel());
     }
-    const int rc = vla_forward(raw(q), raw(k), raw(v), float(lam), int(s.B), int(s.H), int(s.T), int(s.d), int(s.d), f32(S0),
-                               f32(A0), f32(out), f32(S_T), f32(A_T), &o, stream.stream());
-    if (rc != VLA_OK) return PyLong_FromLong(rc);
+    rc = vla_forward(raw(q), raw(k), raw(v), float(lam), int(s.B), int(s.H), int(s.T), int(s.d), int(s.d), f32(S0),
+                     f32(A0), f32(out), f32(S_T), f32(A_T), &o, stream.stream());
   }
+  if (rc != VLA_OK) return PyLong_FromLong(rc);
   PyObject* r = PyTuple_New(5);
   if (!r) return nullptr;
   PyTuple_SET_ITEM(r, 0, wrap(out));
@@ -296,6 +309,7 @@ PyObject* scan(PyObject*, PyObject* const* a, Py_ssize_t n) {
   torch::autograd::variable_list r;
   try {
     auto opt = [](const Tensor& t) { return t.defined() ? OptTensor(t) : OptTensor(); };
+    Unlocked threads;
     r = Scan::apply(q, k, v, opt(u), opt(S0), opt(A0), opt(z0), status, lam, flags, eps);
   } catch (const Failed& f) {
     return PyLong_FromLong(f.code);

@@ -330,6 +330,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         if (sh.far && !(dt <= kFarDelta)) sh.far[unit] = 1;
       }
       if constexpr (UT) {
+        __syncwarp();   // (the other lanes' rows of L^-1 and their delta: the arrival above orders them for the others only)
         // N = L^-1 X, X[s][t] = u'_s . A k_t;  PT[t][s] = N[s][t] / delta_s for s <= t
         // (X and PT alternate between two buffers: the state warps may be a chunk ahead here)
         const float* X = fs + Cfg::af_W + (1 + (c & 1)) * PARTS * SM;

@@ -342,7 +342,7 @@ int backward_chunked(const void* q, const void* k, const void* v, float lambda_,
     vla::PairStash sh;
     sh.alpha = wf(L.alpha); sh.zeta = wf(L.zeta); sh.zkc = wf(L.zkc);
     sh.delta = wf(L.scal); sh.an = sh.delta + scal;
-    sh.Aimg = ws(L.Aimg); sh.Asc = wf(L.sc); sh.ck = 2; sh.far = at(far, u0);
+    sh.Aimg = ws(L.Aimg); sh.Asc = wf(L.sc); sh.far = at(far, u0);
     ScanParams f = {};
     f.q = in(q); f.k = in(k); f.v = in(v); f.u = in(o.u);
     f.A0 = at(A0, sq); f.z0 = at(o.z0, u0 * dd);

@@ -19,14 +19,14 @@ struct BwdChunkParams;
 // What the backward pass asks the pair kernel's rank 0 for (STASH instantiations: one CTA per unit, no
 // rank 1).  Per token: alpha_t [units, T, D], zeta_t = z_t / sqrt(delta_t) (explicit u only), delta_t and
 // an_t = max(||a_t||, eps) [units, T].  Per chunk: the key sum at its start [units, chunks, D].  Per block of
-// `ck` chunks: A at its start as an operand image (token-row layout, D rows) and the image's scale.  Per unit, if wanted: a
+// kStashBlock chunks: A at its start as an operand image (token-row layout, D rows) and the image's scale.  Per unit, if wanted: a
 // word set when some delta_t passes kFarDelta.
 constexpr float kFarDelta = 1024.0f;
+constexpr int kStashBlock = 2;
 struct PairStash {
   float *alpha, *zeta, *delta, *an, *zkc, *Asc;
   unsigned char* Aimg;
   int* far;
-  int ck;
 };
 }
 

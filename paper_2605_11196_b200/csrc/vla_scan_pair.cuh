@@ -3,16 +3,16 @@
 // states in registers.  A cluster of two CTAs works on one (batch, head) unit:
 //
 //   rank 0 carries A.   Z0^T = A K^T;  W = K Z0 + I = L diag(delta) L^T;  Z = L^-1 Z0;
-//                       A <- A - Z^T diag(1/delta) Z;  alpha_t = sc_t z_t -> rank 1
+//                       A <- A - Z^T diag(1/delta) Z;  alpha_t = z_t / ||z_t|| -> rank 1
 //   rank 1 carries S.   P = S K^T, R = S Q^T;  E = Tm (V - P), Tm = (I + stril(K alpha^T))^-1;
 //                       O = R + tril(Q alpha^T) E;  S <- S + E^T alpha
 //
 // (explicit u: Z0 = A U^T, W = U Z0, W0 = A K^T, N = L^-1 (U W0), a = W0 - tril(N^T diag(1/delta)) Z,
 // alpha = a / ||a||.)  A warp owns 16 rows of a state as accumulator tiles; an accumulator tile is also
 // the A operand of the next product, so a chunk's chain K -> Z0 -> Z -> A stays in one warp's
-// registers except for two exchanges over shared memory (Z0 for W, Z for the update); every
+// registers except for two exchanges over shared memory (Z0 for W, zeta for the update); every
 // S row is independent of the others.  Beside the D / 16 state warps a CTA has one warp for the
-// 16 x 16 algebra and one or two that widen the inputs (phi, k_hat, hi/lo operand rows) one chunk ahead.
+// 16 x 16 algebra and one to three that widen the inputs (phi, k_hat, hi/lo operand rows) one chunk ahead.
 //
 // A segment of a cut sequence takes a third CTA (NS = 2): rank 2 carries the segment's transfer scan on the same
 // alpha.  d = 64, 16 units x 65536 tokens in 16 segments: scan 2.92 -> 2.2 ms against the FMA chunk kernel, where the
@@ -45,7 +45,8 @@ struct PairCfg {
   static constexpr int NPREP = D == 128 ? 3 : D == 64 ? 2 : 1;   // widening warps
   static constexpr int NT = (NW + 1 + NPREP) * 32;
   // CTAs per SM the registers are cut for.  d = 64: two hide one another's chains (128 units x 1024 tokens 355 -> 203 us,
-  // 256 units 657 -> 392) and cost one unit 2 % (128 registers instead of 192)
+  // 256 units 657 -> 392) and cost one unit 2 % (128 registers instead of 192).  At d = 64 and 128 the cap is reached: 8 to 150
+  // bytes a thread are spilled, most with explicit u
   static constexpr int MINB = D == 64 ? 2 : 1;
   static constexpr int LPT = D / 4;                         // lanes per token in the widening pass
   static constexpr int TPW = 32 / LPT;                      // tokens per warp pass
@@ -513,8 +514,8 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       const bool live = c < nch;
       const int slot = c % RK;
       const uint32_t Kop = sb + Cfg::a_K + slot * Cfg::kslot, Uop = UT ? sb + Cfg::a_U + slot * Cfg::kslot : Kop;
-      if (STASH && live && c % sh.ck == 0) {
-        const size_t blk = size_t(unit) * ((nch + sh.ck - 1) / sh.ck) + c / sh.ck;
+      if (STASH && live && c % kStashBlock == 0) {
+        const size_t blk = size_t(unit) * ((nch + kStashBlock - 1) / kStashBlock) + c / kStashBlock;
         unsigned char* dst = sh.Aimg + blk * (D * kTokRow<D>) + size_t(row0 + g) * kTokRow<D> + 4 * c4;
 #pragma unroll
         for (int nt = 0; nt < NTILE; ++nt)

@@ -21,7 +21,7 @@
 //
 // All of it is exact algebra; it costs about half more arithmetic than the plain scan (one A for both scans) and
 // makes P times as many clusters, which is what a long sequence with few (batch, head) units needs.  16 units x 65536
-// tokens at d = 64: 8.1 ms uncut, 3.1 in 16 segments (3.8 with both scans in one CTA of the FMA chunk kernel).
+// tokens at d = 64: 8.1 ms uncut, 2.96 in 16 segments (3.8 with both scans in one CTA of the FMA chunk kernel).
 #pragma once
 
 #include "vla_common.cuh"

@@ -170,7 +170,9 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
       !tensor_arg(a[12], &A_T) || !tensor_arg(a[13], &z_T) || !tensor_arg(a[14], &status) || !int_arg(a[16], &kernel) ||
       !int_arg(a[18], &probes))
     Py_RETURN_NONE;
-  const bool want_status = a[15] == Py_True;
+  const int want = PyObject_IsTrue(a[15]);   // (any truth value, as in Python)
+  if (want < 0) return nullptr;
+  const bool want_status = want != 0;
   const bool auto_ws = a[17] == Py_True;
   if (!auto_ws && a[17] != Py_None && a[17] != Py_False && !(tensor_arg(a[17], &ws) && ws.is_cuda())) Py_RETURN_NONE;
   Shape s;

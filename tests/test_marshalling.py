@@ -63,3 +63,13 @@ def test_other_threads_go_on_while_the_launch_queue_is_full(train):
     t.join()
     torch.cuda.synchronize()
     assert longest < 0.25 * a.elapsed_time(b) * 1e-3, (longest, a.elapsed_time(b))
+
+
+@pytest.mark.gpu
+def test_want_status_takes_any_truth_value():
+    import paper_2605_11196_b200 as vla
+    x = torch.randn((1, 1, 1, 32), device="cuda")
+    for yes in (True, 1, "yes"):
+        assert vla.vla_forward(x, x, x, 1.0, want_status=yes).status is not None
+    for no in (False, 0, None):
+        assert vla.vla_forward(x, x, x, 1.0, want_status=no).status is None

@@ -502,13 +502,17 @@ def main():
                               hbm_frac=alg_bytes_per_token(ww.d, ib) * ww.tokens / (ms * 1e-3) / 1e9 / hbm_peak,
                               unit_limited_frac_bound=min(ww.units, n_sm) / n_sm)
             qd2, kd2, vd2 = q2.to(dev), k2.to(dev), v2.to(dev)
-            # backward pass: forward recomputed inside (chunk kernel leaving the per-token stash),
-            # both reverse scans as one launch, the dA0 kernel
+            # backward pass with the gradient of A0 (token-level: forward recomputed by the chunk kernel leaving the
+            # per-token stash, both reverse scans as one launch, the dA0 kernel), and without it: the chunked form, which
+            # is what autograd runs (A pass, prep, chains, block, scan, finish)
             if name in ("mid", "recall"):
                 go3 = torch.randn((ww.B, ww.H, ww.T, ww.d), device=dev)
                 ms = timed_ms(lambda: vla.vla_backward(qd2, kd2, vd2, ww.lam, go3, stream=stream), stream, dev, 1, 3, fl)
                 per[name + "_backward"] = entry(ww, ms, gpu_launches_per_step=3,
                                                 forward_ms=per[name]["ms"], ratio_to_forward=ms / per[name]["ms"])
+                ms = timed_ms(lambda: vla.vla_backward(qd2, kd2, vd2, ww.lam, go3, want_dA0=False, stream=stream), stream, dev, 1, 3, fl)
+                per[name + "_backward_chunked"] = entry(ww, ms, gpu_launches_per_step=6,
+                                                        forward_ms=per[name]["ms"], ratio_to_forward=ms / per[name]["ms"])
                 del go3
             # fewer units than SMs: with scratch memory the plain call cuts each sequence into
             # segments that are scanned concurrently (twice the arithmetic, P times the CTAs)
@@ -536,6 +540,8 @@ def main():
         ms = timed_ms(lambda: vla.vla_backward(qd, kd, vd, w.lam, go_h, workspace=wsb, stream=stream), stream, dev, 1, 2)
         per[w.name + "_backward"] = entry(w, ms, gpu_launches_per_step=3, forward_ms=launch_ms,
                                           ratio_to_forward=ms / launch_ms)
+        ms = timed_ms(lambda: vla.vla_backward(qd, kd, vd, w.lam, go_h, workspace=wsb, want_dA0=False, stream=stream), stream, dev, 1, 2)
+        per[w.name + "_backward_chunked"] = entry(w, ms, forward_ms=launch_ms, ratio_to_forward=ms / launch_ms)
         uu = W.make_u(w, w.d ** -0.5).to(dev)      # explicit penalty directions u = unit / sqrt(d_h)
         ms = timed_ms(lambda: vla.vla_backward(qd, kd, vd, w.lam, go_h, u=uu, workspace=wsb, stream=stream), stream, dev, 1, 2)
         per[w.name + "_backward_explicit_u"] = entry(w, ms, gpu_launches_per_step=3)

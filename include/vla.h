@@ -226,9 +226,9 @@ int vla_forward_seqpar(const void* q, const void* k, const void* v, float lambda
                        const vla_opts_t* opts, int segments,
                        void* workspace, size_t workspace_bytes, void* stream);
 
-/* Segments per unit that vla_forward_seqpar picks on the current device for this problem:
-   enough to fill the GPU with 2 * B * H * segments concurrent scans, at least 256 tokens each;
-   1 when cutting does not pay (or the shape is not covered). */
+/* Segments per unit that vla_forward_seqpar picks on the current device for this problem: the divisor of
+   T / 16 that takes least by measured rates, at least 64 tokens each; 1 when cutting does not pay (or
+   the shape is not covered). */
 int vla_seqpar_segments(int B, int H, int T, int d_k, int qkv_dtype);
 
 /* Device bytes vla_forward_seqpar needs for `segments` >= 1 (0 on a bad argument). */

@@ -108,6 +108,30 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return false;
 }
 
+// The same wait, giving up when `limit` probes have failed or another warp has given up (the 32-bit word at `flag` in shared
+// memory, which is set then).  One loop in place: written in C++ its second half is laid out at the end of the kernel, and
+// the jumps there and back cost instruction cache lines.
+__device__ __forceinline__ void mbar_wait_flagged(uint32_t bar, uint32_t parity, uint32_t limit, uint32_t flag) {
+  asm volatile(
+      "{\n"
+      "  .reg .pred p, q;\n"
+      "  .reg .u32 n, a;\n"
+      "  mov.u32 n, 0;\n"
+      "PROBE:\n"
+      "  mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n"
+      "  @p bra DONE;\n"
+      "  ld.volatile.shared.u32 a, [%3];\n"
+      "  add.u32 n, n, 1;\n"
+      "  setp.gt.u32 q, n, %2;\n"
+      "  setp.ne.or.u32 q, a, 0, q;\n"
+      "  @!q bra PROBE;\n"
+      "  st.volatile.shared.u32 [%3], 1;\n"
+      "DONE:\n"
+      "}\n" ::"r"(bar),
+      "r"(parity), "r"(limit), "r"(flag)
+      : "memory");
+}
+
 // global -> shared bulk copy, completion counted in bytes on `bar`.
 // dst, src 16-byte aligned; bytes a multiple of 16.  No multicast.
 __device__ __forceinline__ void bulk_load(void* smem_dst, const void* gmem_src, uint32_t bytes,
@@ -241,6 +265,21 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   return *reinterpret_cast<float2*>(&rd);
 }
 
+__device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
+  unsigned long long ra, rb, rd;
+  ra = *reinterpret_cast<unsigned long long*>(&a);
+  rb = *reinterpret_cast<unsigned long long*>(&b);
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
+  return *reinterpret_cast<float2*>(&rd);
+}
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+  unsigned long long ra, rb, rd;
+  ra = *reinterpret_cast<unsigned long long*>(&a);
+  rb = *reinterpret_cast<unsigned long long*>(&b);
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
+  return *reinterpret_cast<float2*>(&rd);
+}
+
 __device__ __forceinline__ void group_bar(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
@@ -258,10 +297,11 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // Fast elementwise helpers of the prep pass (relative error ~1e-6, far inside the parity bound).
 // Branch-free: both sides are evaluated and selected, so a warp never diverges here.
 __device__ __forceinline__ float phi_fast(float x) {
-  const float xm = x > 0.0f ? 0.0f : x;   // keeps a NaN (fminf would drop it)
-  float e;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(xm * 1.4426950408889634f));
-  return x > 0.0f ? x + 1.0f : e;
+  float lo, hi, e;   // x + 1 = max(x, 0) + 2^0 above zero, 0 + e^x below: both exact sums (.NaN: a NaN stays one)
+  asm("min.NaN.f32 %0, %1, 0f00000000;" : "=f"(lo) : "f"(x));
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(hi) : "f"(x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(lo * 1.4426950408889634f));
+  return hi + e;
 }
 __device__ __forceinline__ float sqrt_approx(float x) {
   float r;

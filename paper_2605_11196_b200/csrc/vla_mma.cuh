@@ -55,8 +55,12 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], uint32_t addr) {
 // two values -> packed fp16 pair of their rounded parts and of the remainders (x0 in the low half)
 __device__ __forceinline__ void split_f16(float x0, float x1, uint32_t& hi, uint32_t& lo) {
   asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(x1), "f"(x0));
-  const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hi));
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(x1 - h.y), "f"(x0 - h.x));
+  float r0, r1;   // x - hi, exact; one mixed-precision FMA instead of a conversion and a subtraction
+  asm("{\n.reg .b16 h0, h1, m;\nmov.b16 m, 0xbc00;\nmov.b32 {h0, h1}, %2;\n"
+      "fma.rn.f32.f16 %0, h0, m, %3;\nfma.rn.f32.f16 %1, h1, m, %4;\n}"
+      : "=f"(r0), "=f"(r1)
+      : "r"(hi), "f"(x0), "f"(x1));
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(r1), "f"(r0));
 }
 // hi: the upper 19 bits (a NaN stays one); lo: the remainder, rounded where the tensor core cuts it
 __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
@@ -81,6 +85,24 @@ __device__ __forceinline__ void split_frag_tf32(const float (&t)[4], uint32_t (&
   split_tf32(t[3], hi[3], lo[3]);
 }
 
+// acc += x, acc += s x: accumulator tiles two values an instruction
+__device__ __forceinline__ void tile_add(float* acc, const float (&x)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; e += 2) {
+    const float2 r = fadd2(make_float2(acc[e], acc[e + 1]), make_float2(x[e], x[e + 1]));
+    acc[e] = r.x;
+    acc[e + 1] = r.y;
+  }
+}
+__device__ __forceinline__ void tile_fma(float* acc, const float (&x)[4], float s) {
+#pragma unroll
+  for (int e = 0; e < 4; e += 2) {
+    const float2 r = ffma2(make_float2(x[e], x[e + 1]), make_float2(s, s), make_float2(acc[e], acc[e + 1]));
+    acc[e] = r.x;
+    acc[e + 1] = r.y;
+  }
+}
+
 // N independent products of one K step, acc[i] += A[i] B[i] as lo*hi + hi*lo + hi*hi from zero, added
 // in fp32.  A warp issues in order and an mma's result takes 21 clk, so the three dependent
 // instructions of one product are spread over the others' (at 8 clk apiece three products hide it).
@@ -95,9 +117,7 @@ __device__ __forceinline__ void mma3_f16_many(FA a, FB b, FC acc) {
 #pragma unroll
   for (int i = 0; i < N; ++i) mma_f16(x[i], a(i, 0), b(i, 0), b(i, 1));
 #pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc(i)[e] += x[i][e];
+  for (int i = 0; i < N; ++i) tile_add(acc(i), x[i]);
 }
 // ... with the result scaled: acc[i] += s A[i] B[i]
 template <int N, typename FA, typename FB, typename FC>
@@ -110,9 +130,7 @@ __device__ __forceinline__ void mma3_f16_scaled(FA a, FB b, FC acc, float s) {
 #pragma unroll
   for (int i = 0; i < N; ++i) mma_f16(x[i], a(i, 0), b(i, 0), b(i, 1));
 #pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc(i)[e] = fmaf(x[i][e], s, acc(i)[e]);
+  for (int i = 0; i < N; ++i) tile_fma(acc(i), x[i], s);
 }
 // out (16 x 16 as two tiles) += X M^T for a small row-major M[n][k] (16 x 16 fp32, row stride LD) and
 // X in accumulator tiles (16 x 16).  M[n][k] is taken as 0 for n < 8 <= k (lower triangular matrices).
@@ -204,7 +222,7 @@ __device__ __forceinline__ void unit_lower_inverse16(float* Tm, float* N, int la
   __syncwarp();
   // lane: row g of the lower left block, columns 2 c, 2 c + 1
   float2 y = make_float2(0.f, 0.f);
-#pragma unroll
+#pragma unroll 4
   for (int k = 0; k < 8; ++k) {
     const float nk = N[(8 + g) * LD + k];
     const float2 tk = *reinterpret_cast<const float2*>(Tm + k * LD + 2 * c);
@@ -214,7 +232,7 @@ __device__ __forceinline__ void unit_lower_inverse16(float* Tm, float* N, int la
   *reinterpret_cast<float2*>(N + 8 + g * LD + 2 * c) = y;
   __syncwarp();
   float2 z = make_float2(0.f, 0.f);
-#pragma unroll
+#pragma unroll 4
   for (int k = 0; k < 8; ++k) {
     const float tk = Tm[(8 + g) * LD + 8 + k];
     const float2 yk = *reinterpret_cast<const float2*>(N + 8 + k * LD + 2 * c);
@@ -287,6 +305,9 @@ __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
 __device__ __forceinline__ void sts64(uint32_t addr, uint32_t v0, uint32_t v1) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(v0), "r"(v1) : "memory");
 }
+__device__ __forceinline__ void sts128(uint32_t addr, const uint32_t (&v)[4]) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
 // a warp's 16 x 16 accumulator (rows g, g + 8; columns = tokens) into vector rows; base: row g's address + 4 c4
 __device__ __forceinline__ void vec_store(uint32_t base, const float (&x)[2][4]) {
 #pragma unroll
@@ -297,6 +318,16 @@ __device__ __forceinline__ void vec_store(uint32_t base, const float (&x)[2][4])
       split_f16(x[nt][2 * r], x[nt][2 * r + 1], hi, lo);
       sts32(base + r * 8 * kVecRow + nt * 16, hi);
       sts32(base + r * 8 * kVecRow + nt * 16 + 32, lo);
+    }
+}
+// ... from its A operand (split_frag of the same accumulator)
+__device__ __forceinline__ void vec_store_frag(uint32_t base, const uint32_t (&hi)[4], const uint32_t (&lo)[4]) {
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      sts32(base + r * 8 * kVecRow + nt * 16, hi[r + 2 * nt]);
+      sts32(base + r * 8 * kVecRow + nt * 16 + 32, lo[r + 2 * nt]);
     }
 }
 

@@ -18,6 +18,13 @@
 // alpha.  d = 64, 16 units x 65536 tokens in 16 segments: scan 2.92 -> 2.2 ms against the FMA chunk kernel, where the
 // two scans shared one CTA with A (6 us of an SM per 16 tokens of a segment; three CTAs here, two on an SM: 4.7).
 
+// Widening: eight columns a lane, so that a token's norms are two to four shuffle rounds and a warp takes twice the tokens at a
+// time.  With four the widening warps of rank 1 set the pace of every d >= 32 (d = 64: 2830 of 3560 clk per chunk).
+//
+// Instruction cache: an SM holds CTAs of one rank only (measured: a cluster's ranks lie on the two SMs of a TPC), and runs straight
+// code from 32 KB of cache at one instruction a clock, beyond that at 2.1 (and all SMs of a GPC share what is beyond).  So each
+// rank has its own copy of the widening code, small loops stay rolled, and values go through two-wide instructions.
+//
 // What bounds it: at one unit per SM pair the serial chain of rank 0 (state split, Z0, W, the
 // 16 x 16 elimination, Z, update), with many units the tensor pipe (8 clk per instruction and
 // scheduler).  Two CTAs because at d = 128 both states and their operands do not fit one SM's
@@ -33,6 +40,8 @@
 // (In true units z = A u passed fp16's range at norms of 250 to 500 times the largest entry of A.)
 #pragma once
 
+#include <type_traits>
+
 #include "vla_launch.h"
 #include "vla_mma.cuh"
 
@@ -42,17 +51,18 @@ template <int D, typename TIn, bool UT>
 struct PairCfg {
   static constexpr int C = 16;
   static constexpr int NW = D / 16;                         // state warps
-  static constexpr int NPREP = D == 128 ? 3 : D == 64 ? 2 : 1;   // widening warps
+  static constexpr int NPREP = D >= 64 ? 2 : 1;             // widening warps
   static constexpr int NT = (NW + 1 + NPREP) * 32;
   // CTAs per SM the registers are cut for.  d = 64: two hide one another's chains (128 units x 1024 tokens 355 -> 203 us,
   // 256 units 657 -> 392) and cost one unit 2 % (128 registers instead of 192).  At d = 64 and 128 the cap is reached: 8 to 150
   // bytes a thread are spilled, most with explicit u
   static constexpr int MINB = D == 64 ? 2 : 1;
-  static constexpr int LPT = D / 4;                         // lanes per token in the widening pass
+  static constexpr int LPT = D / 8;                         // lanes per token in the widening pass
   static constexpr int TPW = 32 / LPT;                      // tokens per warp pass
-  static constexpr int NP = (C + TPW * NPREP - 1) / (TPW * NPREP);   // passes per chunk
-  static constexpr uint32_t piece = 4 * sizeof(TIn);        // bytes of a lane's four columns
-  static constexpr uint32_t raw_stage = 2 * NPREP * NP * 32 * piece;   // both tensors of a chunk as the lanes take them
+  static constexpr int NP = C / (TPW * NPREP);              // passes per chunk
+  static_assert(C % (TPW * NPREP) == 0, "a widening pass takes whole tokens of one chunk");
+  static constexpr int PB = 8 * sizeof(TIn) / 16;           // 16-byte pieces of a lane's eight columns
+  static constexpr uint32_t raw_stage = 2 * NPREP * NP * PB * 512;   // both tensors of a chunk as the lanes take them
   static constexpr int RK = 2, RA = 4;                      // input and alpha slots
   static constexpr int LD = 20;                             // row of a small matrix
   static constexpr int SM = C * LD;
@@ -76,23 +86,40 @@ struct PairCfg {
   static constexpr size_t smem_bytes = bars + NBAR * 8 + 16;
 };
 
-// global -> shared, 16 or 8 bytes, zeros when !act (each lane reads back only what it copied itself)
-template <int BYTES>
+// global -> shared, 16 bytes, zeros when !act (each lane reads back only what it copied itself)
 __device__ __forceinline__ void copy_piece(uint32_t dst, const void* src, bool act) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(BYTES), "r"(act ? BYTES : 0) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(act ? 16 : 0) : "memory");
 }
-__device__ __forceinline__ float4 piece_f32(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float4 piece_f32(const uint16_t* p) { return load4(p, 0); }
+// a lane's eight columns back from its pieces, 512 bytes apart
+__device__ __forceinline__ void piece_f32(const unsigned char* at, float (&x)[8], const float*) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const float4 y = *reinterpret_cast<const float4*>(at + 512 * i);
+    x[4 * i] = y.x; x[4 * i + 1] = y.y; x[4 * i + 2] = y.z; x[4 * i + 3] = y.w;
+  }
+}
+__device__ __forceinline__ void piece_f32(const unsigned char* at, float (&x)[8], const uint16_t*) {
+  const uint4 y = *reinterpret_cast<const uint4*>(at);
+  const uint32_t w[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    x[2 * i] = __uint_as_float(w[i] << 16);
+    x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+  }
+}
 
-// four consecutive columns of a token row, scaled, as hi/lo operand entries
+// eight consecutive columns of a token row, scaled, as hi/lo operand entries
 template <int D>
-__device__ __forceinline__ void tok_store4(uint32_t base, int row, int pl, float4 x, float s) {
-  uint32_t h0, l0, h1, l1;
-  split_f16(x.x * s, x.y * s, h0, l0);
-  split_f16(x.z * s, x.w * s, h1, l1);
-  const uint32_t at = base + uint32_t(row) * kTokRow<D> + 8 * pl;
-  sts64(at, h0, h1);
-  sts64(at + 2 * D, l0, l1);
+__device__ __forceinline__ void tok_store8(uint32_t base, int row, int pl, const float (&x)[8], float s) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 y = fmul2(make_float2(x[2 * i], x[2 * i + 1]), make_float2(s, s));
+    split_f16(y.x, y.y, h[i], l[i]);
+  }
+  const uint32_t at = base + uint32_t(row) * kTokRow<D> + 16 * pl;
+  sts128(at, h);
+  sts128(at + 2 * D, l);
 }
 
 // NS: CTAs that carry an S.  2 (the segments of a cut sequence): rank 1 the segment from S = 0, rank 2 its
@@ -101,10 +128,11 @@ template <int D, typename TIn, bool UT, bool STASH, int NS>
 __global__ void __cluster_dims__(STASH ? 1 : 1 + NS, 1, 1) __launch_bounds__((PairCfg<D, TIn, UT>::NT), (PairCfg<D, TIn, UT>::MINB))
 vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
   using Cfg = PairCfg<D, TIn, UT>;
-  constexpr int C = Cfg::C, NW = Cfg::NW, NPREP = Cfg::NPREP, LPT = Cfg::LPT, TPW = Cfg::TPW, NP = Cfg::NP;
+  constexpr int C = Cfg::C, NW = Cfg::NW, NPREP = Cfg::NPREP, LPT = Cfg::LPT, TPW = Cfg::TPW, NP = Cfg::NP, PB = Cfg::PB;
   constexpr int RK = Cfg::RK, RA = Cfg::RA, LD = Cfg::LD, SM = Cfg::SM, PARTS = Cfg::PARTS, NJOB = Cfg::NJOB;
   constexpr int NTILE = D / 8, KS = D / 16, NB = NTILE < 4 ? NTILE : 4;
   constexpr float kUnit = 256.0f, kUnitInv = 1.0f / 256.0f;   // scale of unit-vector operands
+  constexpr float kLam = 16384.0f, kLamInv = 1.0f / 16384.0f; // ... of diag(delta)^-1/2 L^-1
 
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t sb = smem_u32(smem);
@@ -130,15 +158,9 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + Cfg::NBAR);
 
   // Bounded wait; a limit that runs out is reported when the CTA ends.
-  const uint32_t probes = p.wait_limit == 0 ? kWaitProbeLimit : p.wait_limit;
+  const uint32_t probes = p.wait_limit == 0 ? kWaitProbeLimit : p.wait_limit, abort_at = sb + Cfg::bars + Cfg::NBAR * 8;
   auto wait = [&](uint64_t* bar, int parity) {
-    uint32_t it = 0;
-    while (!mbar_try_wait(bar, uint32_t(parity))) {
-      if (++it > probes || *abort_flag) {
-        *abort_flag = 1;
-        break;
-      }
-    }
+    mbar_wait_flagged(smem_u32(bar), uint32_t(parity), probes, abort_at);
   };
   auto arrive = [&](uint64_t* bar) {   // one arrival per warp
     __syncwarp();
@@ -173,116 +195,159 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
   const uint32_t lane_ta = tok_lane_a<D>(lane), lane_tb = tok_lane_b<D>(lane), lane_vb = vec_lane_b(lane), lane_vt = vec_lane_bt(lane), lane_vn = vec_lane_bt1(lane);
   const size_t tok0 = token_offset(p, unit, 0, D), tstride = token_stride(p, D);
 
-  if (warp > NW) {
-    // ===================================================================== widening warps
-    // A lane takes four columns of a token at a time, through a staging ring that only it reads; the
-    // copies of chunk c + 1 are in flight while chunk c is widened.  (Rolled loops: all warps' code
-    // together has to stay inside the SM's instruction cache.)
-    const int pw = warp - NW - 1, sub = lane / LPT, pl = lane % LPT;
-    const TIn* src0 = static_cast<const TIn*>(p.k) + tok0 + 4 * pl;
-    const bool two = UT || rank != 0, sums = STASH || rank != 0;   // sums: this side carries the key sum
-    const TIn* src1 = two ? static_cast<const TIn*>(rank ? p.q : p.u) + tok0 + 4 * pl : src0;
-    float* fs = reinterpret_cast<float*>(smem + (rank ? Cfg::s_f : Cfg::a_f));
-    const uint32_t base0 = sb + (rank ? Cfg::s_K : Cfg::a_K), base1 = sb + (rank ? Cfg::s_Q : Cfg::a_U);
-    auto stage = [&](int c, int ps) {   // byte offset of this lane's pieces (the second tensor's follows at + 32 pieces)
-      return Cfg::raw + (c & 1) * Cfg::raw_stage + uint32_t((ps * NPREP + pw) * 64 + lane) * Cfg::piece;
-    };
-    auto fetch = [&](int c) {
+  // ======================================================================= widening warps (both ranks)
+  // A lane takes eight columns of a token at a time, through a staging ring that only it reads; the
+  // copies of chunk c + 1 are in flight while chunk c is widened.
+  auto widen = [&](auto r1) {
+  constexpr bool R1 = decltype(r1)::value;   // rank 1 and 2: keys and queries; rank 0: keys [and u]
+  const int pw = warp - NW - 1, sub = lane / LPT, pl = lane % LPT;
+  const TIn* src0 = static_cast<const TIn*>(p.k) + tok0 + 8 * pl;
+  constexpr bool two = UT || R1, sums = STASH || R1;   // sums: this side carries the key sum
+  const TIn* src1 = two ? static_cast<const TIn*>(R1 ? p.q : p.u) + tok0 + 8 * pl : src0;
+  float* fs = reinterpret_cast<float*>(smem + (R1 ? Cfg::s_f : Cfg::a_f));
+  const uint32_t base0 = sb + (R1 ? Cfg::s_K : Cfg::a_K), base1 = sb + (R1 ? Cfg::s_Q : Cfg::a_U);
+  auto stage = [&](int c, int ps) {   // byte offset of this lane's pieces (the second tensor's PB pieces follow the first's)
+    return Cfg::raw + (c & 1) * Cfg::raw_stage + uint32_t(ps * NPREP + pw) * (2 * PB * 512) + uint32_t(lane) * 16;
+  };
+  auto fetch = [&](int c) {
 #pragma unroll 1
-      for (int ps = 0; ps < NP; ++ps) {
-        const int t = c * C + (ps * NPREP + pw) * TPW + sub;
-        const bool act = t < T && (C % (TPW * NPREP) == 0 || (ps * NPREP + pw) * TPW < C);
-        const size_t off = act ? size_t(t) * tstride : 0;
-        copy_piece<Cfg::piece>(sb + stage(c, ps), src0 + off, act);
-        if (two) copy_piece<Cfg::piece>(sb + stage(c, ps) + 32 * Cfg::piece, src1 + off, act);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    float zk[4] = {0.f, 0.f, 0.f, 0.f};
-    if (sums && p.z0) {
+    for (int ps = 0; ps < NP; ++ps) {
+      const int t = c * C + (ps * NPREP + pw) * TPW + sub;
+      const bool act = t < T;
+      const size_t off = act ? size_t(t) * tstride : 0;
+      const uint32_t at = sb + stage(c, ps);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) zk[e] = p.z0[size_t(unit) * D + 4 * pl + e];
+      for (int i = 0; i < PB; ++i) {
+        copy_piece(at + 512 * i, src0 + off + i * (8 / PB), act);
+        if (two) copy_piece(at + 512 * (PB + i), src1 + off + i * (8 / PB), act);
+      }
     }
-    if (nch > 0) fetch(0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float zk[8] = {};
+  if (sums && p.z0) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) zk[e] = p.z0[size_t(unit) * D + 8 * pl + e];
+  }
+  if (nch > 0) fetch(0);
 #pragma unroll 1
-    for (int c = 0; c < nch; ++c) {
-      const int slot = c % RK;
-      fetch(c + 1);   // (past the end: zeros)
-      if (STASH && pw == 0 && sub == 0)
-        *reinterpret_cast<float4*>(sh.zkc + (size_t(unit) * nch + c) * D + 4 * pl) = make_float4(zk[0], zk[1], zk[2], zk[3]);
-      if (c >= RK) wait(&kfree[slot], (c / RK - 1) & 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-      float ks[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-      for (int ps = 0; ps < NP; ++ps) {
-        const int tt = (ps * NPREP + pw) * TPW + sub;
-        if (C % (TPW * NPREP) != 0 && tt >= C) break;   // (uniform over the warp: one token a pass there)
-        const bool act = c * C + tt < T;
-        const TIn* raw = reinterpret_cast<const TIn*>(smem + stage(c, ps));
-        float4 k = piece_f32(raw), x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (two) x = piece_f32(raw + 128);
-        if (!ident) {
-          k.x = phi_fast(k.x); k.y = phi_fast(k.y); k.z = phi_fast(k.z); k.w = phi_fast(k.w);
-          if (rank != 0) {
-            x.x = phi_fast(x.x); x.y = phi_fast(x.y); x.z = phi_fast(x.z); x.w = phi_fast(x.w);
-          }
-        }
-        if (!act) k = x = make_float4(0.f, 0.f, 0.f, 0.f);
-        float ss = fmaf(k.x, k.x, fmaf(k.y, k.y, fmaf(k.z, k.z, k.w * k.w)));
-        float qq = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
-        float dn = fmaf(x.x, zk[0], fmaf(x.y, zk[1], fmaf(x.z, zk[2], x.w * zk[3])));
-        ks[0] += k.x; ks[1] += k.y; ks[2] += k.z; ks[3] += k.w;
-#pragma unroll
-        for (int off = LPT / 2; off >= 1; off >>= 1) {
-          ss += __shfl_xor_sync(0xffffffffu, ss, off);
-          qq += __shfl_xor_sync(0xffffffffu, qq, off);
-          dn += __shfl_xor_sync(0xffffffffu, dn, off);
-        }
-        const float nr = fmaxf(sqrt_ftz(ss), eps);   // max(||phi(k)||, eps)
-        tok_store4<D>(base0 + slot * Cfg::kslot, tt, pl, k, rcp_ftz_nr(nr) * kUnit);
-        if (two) {
-          const float s = pow2_scale(sqrt_ftz(qq), 8);
-          tok_store4<D>(base1 + slot * Cfg::kslot, tt, pl, x, s);
-          if (pl == 0) {
-            const float inv = pow2_inverse(s);
-            if (rank) {
-              fs[Cfg::sf_qs + slot * 16 + tt] = inv;
-            } else {   // u row -> u', and D^-2 (four slots: the elimination is done with one by the time it comes round again)
-              const float iD = pow2_inverse(fminf(fmaxf(256.0f * inv, 9.5367432e-7f), 1.1529215e18f));
-              fs[Cfg::af_us + slot * 16 + tt] = inv * iD;
-              fs[Cfg::af_ud + (c & 3) * 16 + tt] = iD * iD;
-            }
-          }
-        }
-        if (rank != 0 && pl == 0) {
-          fs[Cfg::sf_nrm + slot * 16 + tt] = act ? nr : 0.f;
-          fs[Cfg::sf_dq + slot * 16 + tt] = dn;
-        }
-      }
-      if (sums && !ident) {   // the key sum after this chunk
-#pragma unroll
-        for (int off = LPT; off < 32; off <<= 1)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) ks[e] += __shfl_xor_sync(0xffffffffu, ks[e], off);
-        if constexpr (NPREP > 1) {
-          float* zp = fs + (STASH ? Cfg::af_zp : Cfg::sf_zp) + (c & 1) * NPREP * D;
-          if (sub == 0) *reinterpret_cast<float4*>(zp + pw * D + 4 * pl) = make_float4(ks[0], ks[1], ks[2], ks[3]);
-          named_sync(2, NPREP * 32);
-          ks[0] = ks[1] = ks[2] = ks[3] = 0.f;
-#pragma unroll
-          for (int w = 0; w < NPREP; ++w) {
-            const float4 y = *reinterpret_cast<const float4*>(zp + w * D + 4 * pl);
-            ks[0] += y.x; ks[1] += y.y; ks[2] += y.z; ks[3] += y.w;
-          }
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) zk[e] += ks[e];
-      }
-      arrive(&kfull[slot]);
+  for (int c = 0; c < nch; ++c) {
+    const int slot = c % RK;
+    fetch(c + 1);   // (past the end: zeros)
+    if (STASH && pw == 0 && sub == 0) {
+      float4* o = reinterpret_cast<float4*>(sh.zkc + (size_t(unit) * nch + c) * D + 8 * pl);
+      o[0] = make_float4(zk[0], zk[1], zk[2], zk[3]);
+      o[1] = make_float4(zk[4], zk[5], zk[6], zk[7]);
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    if (sums && rank < 2 && p.zT && pw == 0 && sub == 0)
-      *reinterpret_cast<float4*>(p.zT + size_t(unit) * D + 4 * pl) = make_float4(zk[0], zk[1], zk[2], zk[3]);
+    if (c >= RK) wait(&kfree[slot], (c / RK - 1) & 1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    float ks[8] = {};
+#pragma unroll 1
+    for (int ps = 0; ps < NP; ++ps) {
+      const int tt = (ps * NPREP + pw) * TPW + sub;
+      const bool act = c * C + tt < T;
+      const unsigned char* raw = smem + stage(c, ps);
+      float k[8], x[8] = {};
+      piece_f32(raw, k, src0);
+      if (two) piece_f32(raw + 512 * PB, x, src0);
+      if (!ident) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) k[e] = phi_fast(k[e]);
+        if constexpr (R1) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) x[e] = phi_fast(x[e]);
+        }
+      }
+      // (a token past the end came in as zeros: its key row and its share of the key sum are zeros too; what its query,
+      // phi(0) = 1, gives is not stored)
+      const float on = act ? 1.0f : 0.0f;
+      float2 ss2 = make_float2(0.f, 0.f), qq2 = ss2, dn2 = ss2;
+#pragma unroll
+      for (int e = 0; e < 8; e += 2) {
+        const float2 k2 = make_float2(k[e], k[e + 1]), x2 = make_float2(x[e], x[e + 1]);
+        ss2 = ffma2(k2, k2, ss2);
+        if (two) qq2 = ffma2(x2, x2, qq2);
+        if (R1) dn2 = ffma2(x2, make_float2(zk[e], zk[e + 1]), dn2);
+        if (sums) {
+          const float2 s2 = ffma2(make_float2(on, on), k2, make_float2(ks[e], ks[e + 1]));
+          ks[e] = s2.x;
+          ks[e + 1] = s2.y;
+        }
+      }
+      float ss = ss2.x + ss2.y, qq = qq2.x + qq2.y, dn = dn2.x + dn2.y;
+#pragma unroll
+      for (int off = LPT / 2; off >= 1; off >>= 1) {
+        ss += __shfl_xor_sync(0xffffffffu, ss, off);
+        if (two) qq += __shfl_xor_sync(0xffffffffu, qq, off);
+        if (R1) dn += __shfl_xor_sync(0xffffffffu, dn, off);
+      }
+      const float nr = fmaxf(sqrt_ftz(ss), eps);   // max(||phi(k)||, eps)
+      tok_store8<D>(base0 + slot * Cfg::kslot, tt, pl, k, rcp_ftz_nr(nr) * (on * kUnit));
+      if constexpr (two) {
+        const float s = pow2_scale(sqrt_ftz(qq), 8);
+        tok_store8<D>(base1 + slot * Cfg::kslot, tt, pl, x, s);
+        if (pl == 0) {
+          const float inv = pow2_inverse(s);
+          if constexpr (R1) {
+            fs[Cfg::sf_qs + slot * 16 + tt] = inv;
+          } else {   // u row -> u', and D^-2 (four slots: the elimination is done with one by the time it comes round again)
+            const float iD = pow2_inverse(fminf(fmaxf(256.0f * inv, 9.5367432e-7f), 1.1529215e18f));
+            fs[Cfg::af_us + slot * 16 + tt] = inv * iD;
+            fs[Cfg::af_ud + (c & 3) * 16 + tt] = iD * iD;
+          }
+        }
+      }
+      if (R1 && pl == 0) {
+        fs[Cfg::sf_nrm + slot * 16 + tt] = act ? nr : 0.f;
+        fs[Cfg::sf_dq + slot * 16 + tt] = dn;
+      }
+    }
+    if (sums && !ident) {
+      // the key sum after this chunk: over the tokens a warp took at a time by halving (a lane ends with KN
+      // columns), over the warps and back to eight columns a lane through shared memory
+      constexpr int KN = TPW >= 8 ? 1 : 8 / TPW;
+      int col = 0;
+#pragma unroll
+      for (int off = 16, n = 8; off >= LPT; off >>= 1) {
+        n >>= 1;
+        if (n >= 1) {
+          const bool up = (lane & off) != 0;
+#pragma unroll
+          for (int e = 0; e < n; ++e) {
+            const float send = up ? ks[e] : ks[e + n], keep = up ? ks[e + n] : ks[e];
+            ks[e] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+          }
+          if (up) col += n;
+        } else {
+          ks[0] += __shfl_xor_sync(0xffffffffu, ks[0], off);
+        }
+      }
+      float* zp = fs + (STASH ? Cfg::af_zp : Cfg::sf_zp) + (c & 1) * NPREP * D;
+#pragma unroll
+      for (int e = 0; e < KN; ++e) zp[pw * D + 8 * pl + col + e] = ks[e];   // (d = 16: two lanes, one value)
+      if constexpr (NPREP > 1) named_sync(2, NPREP * 32);
+      else __syncwarp();
+#pragma unroll
+      for (int w = 0; w < NPREP; ++w) {
+        const float4* y = reinterpret_cast<const float4*>(zp + w * D + 8 * pl);
+        const float4 y0 = y[0], y1 = y[1];
+        const float y8[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) zk[e] += y8[e];
+      }
+    }
+    arrive(&kfull[slot]);
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (sums && rank < 2 && p.zT && pw == 0 && sub == 0) {
+    float4* o = reinterpret_cast<float4*>(p.zT + size_t(unit) * D + 8 * pl);
+    o[0] = make_float4(zk[0], zk[1], zk[2], zk[3]);
+    o[1] = make_float4(zk[4], zk[5], zk[6], zk[7]);
+  }
+  };
+  // (the roles of a rank stand together: that is the code an SM runs)
+  if (rank == 0 && warp > NW) {
+    widen(std::false_type{});
   } else if (rank == 0 && warp == NW) {
     // ===================================================================== rank 0: elimination
     // I + W = L diag(delta) L^T in place (eliminate16): lane (r, h) holds row r, columns 8 h .. 8 h + 7.
@@ -316,12 +381,38 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         float x[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) x[j] = 8 * h + j < r ? m[j] : (8 * h + j == r ? 1.0f : 0.0f);
-        float4* o = reinterpret_cast<float4*>(Li + r * LD + 8 * h);
-        o[0] = make_float4(x[0], x[1], x[2], x[3]);
-        o[1] = make_float4(x[4], x[5], x[6], x[7]);
-        if (h == 0) {
-          dl[16 + r] = rcp_ftz_nr(delta);
-          dl[32 + r] = rsqrt_ftz_nr(delta);
+        if constexpr (UT) {
+          float4* o = reinterpret_cast<float4*>(Li + r * LD + 8 * h);
+          o[0] = make_float4(x[0], x[1], x[2], x[3]);
+          o[1] = make_float4(x[4], x[5], x[6], x[7]);
+          if (h == 0) {
+            dl[16 + r] = rcp_ftz_nr(delta);
+            dl[32 + r] = rsqrt_ftz_nr(delta);
+          }
+        } else {
+          // diag(delta)^-1/2 L^-1, whose rows are no longer than 1 (I + W >= I), as an operand.  They may be as short as
+          // 1 / sqrt(delta): past 2^-15 (lambda below 1e-9) each row gets a power of two of its own
+          const float rs = rsqrt_ftz_nr(delta);
+          float f = rs * kLam, fi = kLamInv;
+          if (__any_sync(0xffffffffu, delta > 1e9f)) {
+            float mx = 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) mx = fmaxf(mx, fabsf(x[j]));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+            const float own = pow2_scale(mx * rs, 0);
+            f *= own;
+            fi *= pow2_inverse(own);
+          }
+          uint32_t hi[4], lo[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) split_f16(x[2 * j] * f, x[2 * j + 1] * f, hi[j], lo[j]);
+          const uint32_t at = smem_u32(Li) + r * kVecRow + 16 * h;
+          sts128(at, hi);
+          sts128(at + 32, lo);
+          if (h == 0) {
+            dl[16 + r] = fi;
+            dl[32 + r] = rs;
+          }
         }
       }
       named_arrive(4, (NW + 1) * 32);   // L^-1 and delta are written
@@ -508,13 +599,34 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       sAy = (e & 1) ? -1.0f / 8192.0f : -1.0f / 16384.0f;   // -1 / (sA sy^2)
     };
     set_sy();
-    if (nch > 0) wait(&kfull[0], 0);
-#pragma unroll 1
-    for (int c = 0; c < nch + 2; ++c) {   // (the last two rounds only pass on the last two chunks' alpha)
-      const bool live = c < nch;
-      const int slot = c % RK;
+    // Z0^T = A U^T (rows: this warp's state rows, columns: tokens), with an explicit u also A K^T, of the chunk in a
+    // slot: K steps ks .. ks + KB - 1
+    constexpr int KB = (KS >= 2 && !UT) ? 2 : 1;   // K steps whose products are interleaved
+    float z0[2][4], w0[2][4];
+    auto clear_z0 = [&]() {
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) z0[nt][e] = w0[nt][e] = 0.f;
+    };
+    auto product = [&](int ks, int slot) {
       const uint32_t Kop = sb + Cfg::a_K + slot * Cfg::kslot, Uop = UT ? sb + Cfg::a_U + slot * Cfg::kslot : Kop;
-      if (STASH && live && c % kStashBlock == 0) {
+      uint32_t ah[KB][4], al[KB][4], bh[2][4], bl[2][4];   // UT: operand 0 is U, 1 is K; else K step
+#pragma unroll
+      for (int i = 0; i < KB; ++i) split_frag(st[2 * (ks + i)], st[2 * (ks + i) + 1], ah[i], al[i]);
+#pragma unroll
+      for (int i = 0; i < (UT ? 2 : KB); ++i) {
+        tok_frag<D>(bh[i], (i == 0 || !UT ? Uop : Kop) + lane_tb, ks + (UT ? 0 : i), false);
+        tok_frag<D>(bl[i], (i == 0 || !UT ? Uop : Kop) + lane_tb, ks + (UT ? 0 : i), true);
+      }
+      // product i: operand (K step, or U / K) i >> 1, token tile i & 1
+      mma3_f16_many<UT ? 4 : 2 * KB>(
+          [&](int i, int lo) -> const uint32_t(&)[4] { return lo ? al[UT ? 0 : i >> 1] : ah[UT ? 0 : i >> 1]; },
+          [&](int i, int r) { return (r & 2) ? bl[i >> 1][2 * (i & 1) + (r & 1)] : bh[i >> 1][2 * (i & 1) + (r & 1)]; },
+          [&](int i) -> float* { return UT && i >= 2 ? w0[i & 1] : z0[i & 1]; });
+    };
+    auto stash_state = [&](int c) {   // A before chunk c as an operand image
+      if (STASH && c < nch && c % kStashBlock == 0) {
         const size_t blk = size_t(unit) * ((nch + kStashBlock - 1) / kStashBlock) + c / kStashBlock;
         unsigned char* dst = sh.Aimg + blk * (D * kTokRow<D>) + size_t(row0 + g) * kTokRow<D> + 4 * c4;
 #pragma unroll
@@ -528,26 +640,21 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           }
         if (tid == 0) sh.Asc[blk] = sAi;
       }
-      // ---- Z0^T = A U^T (rows: this warp's state rows, columns: tokens), with an explicit u also A K^T
-      float z0[2][4] = {}, w0[2][4] = {};
+    };
+    clear_z0();
+    if (nch > 0) {
+      wait(&kfull[0], 0);
+#pragma unroll
+      for (int ks = 0; ks < KS; ks += KB) product(ks, 0);
+      stash_state(0);
+    }
+#pragma unroll 1
+    for (int c = 0; c < nch + 2; ++c) {   // (the last two rounds only pass on the last two chunks' alpha)
+      const bool live = c < nch;
+      const int slot = c % RK;
+      const uint32_t Uop = sb + (UT ? Cfg::a_U : Cfg::a_K) + slot * Cfg::kslot;
+      uint32_t zh[4], zl[4];
       if (live) {
-      constexpr int KB = (KS >= 2 && !UT) ? 2 : 1;   // K steps whose products are interleaved
-#pragma unroll
-      for (int ks = 0; ks < KS; ks += KB) {
-        uint32_t ah[KB][4], al[KB][4], bh[2][4], bl[2][4];   // UT: operand 0 is U, 1 is K; else K step
-#pragma unroll
-        for (int i = 0; i < KB; ++i) split_frag(st[2 * (ks + i)], st[2 * (ks + i) + 1], ah[i], al[i]);
-#pragma unroll
-        for (int i = 0; i < (UT ? 2 : KB); ++i) {
-          tok_frag<D>(bh[i], (i == 0 || !UT ? Uop : Kop) + lane_tb, ks + (UT ? 0 : i), false);
-          tok_frag<D>(bl[i], (i == 0 || !UT ? Uop : Kop) + lane_tb, ks + (UT ? 0 : i), true);
-        }
-        // product i: operand (K step, or U / K) i >> 1, token tile i & 1
-        mma3_f16_many<UT ? 4 : 2 * KB>(
-            [&](int i, int lo) -> const uint32_t(&)[4] { return lo ? al[UT ? 0 : i >> 1] : ah[UT ? 0 : i >> 1]; },
-            [&](int i, int r) { return (r & 2) ? bl[i >> 1][2 * (i & 1) + (r & 1)] : bh[i >> 1][2 * (i & 1) + (r & 1)]; },
-            [&](int i) -> float* { return UT && i >= 2 ? w0[i & 1] : z0[i & 1]; });
-      }
       const float* us = fs + Cfg::af_us + slot * 16;
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt)
@@ -556,7 +663,8 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           z0[nt][e] *= UT ? us[8 * nt + 2 * c4 + (e & 1)] : kUnitInv;
           w0[nt][e] *= kUnitInv;
         }
-      vec_store(sb + Cfg::a_Z0 + my_rows, z0);
+      split_frag(z0[0], z0[1], zh, zl);
+      vec_store_frag(sb + Cfg::a_Z0 + my_rows, zh, zl);
       if (UT) vec_store(sb + Cfg::a_W0 + my_rows, w0);
       named_sync(1, NW * 32);
       // ---- W = U Z0 [and X = U W0], one 16 x 8 tile a job, the contraction split over PARTS warps
@@ -602,50 +710,77 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         if (lane == 0) mxs[warp] = mx;
       }
       named_sync(4, (NW + 1) * 32);   // L^-1
-      // ---- Z^T = Z0^T L^-T
-      float z[2][4] = {};
-      small_product<LD>(z, z0, Li, lane);
+      // ---- Z^T = Z0^T L^-T;  zeta = z / sqrt(delta)
       uint32_t yh[4], yl[4];
       {
         float y[2][4];
+        if constexpr (UT) {
+          float z[2][4] = {};
+          small_product<LD>(z, z0, Li, lane);
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          const float2 id2 = *reinterpret_cast<const float2*>(dl + 16 + 8 * nt + 2 * c4);
-          const float2 rs2 = *reinterpret_cast<const float2*>(dl + 32 + 8 * nt + 2 * c4);
+          for (int nt = 0; nt < 2; ++nt) {
+            const float2 rs2 = *reinterpret_cast<const float2*>(dl + 32 + 8 * nt + 2 * c4);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int s = 8 * nt + 2 * c4 + (e & 1);
-            y[nt][e] = z[nt][e] * (e & 1 ? rs2.y : rs2.x);
-            if (STASH && UT) {
-              if (c * C + s < T) sh.zeta[(size_t(unit) * T + c * C + s) * D + row0 + g + 8 * (e >> 1)] = y[nt][e] * sAi;
+            for (int e = 0; e < 4; ++e) {
+              const int s = 8 * nt + 2 * c4 + (e & 1);
+              y[nt][e] = z[nt][e] * (e & 1 ? rs2.y : rs2.x);
+              if (STASH && c * C + s < T)
+                sh.zeta[(size_t(unit) * T + c * C + s) * D + row0 + g + 8 * (e >> 1)] = y[nt][e] * sAi;
+              y[nt][e] *= sy;
+              z1[nt][e] = z[nt][e];
+              w1[nt][e] = w0[nt][e];
             }
-            y[nt][e] *= sy;
-            if (!UT) a1[nt][e] = z[nt][e] * (e & 1 ? id2.y : id2.x) * sAi;   // u = k_hat: a_t = z_t / delta_t
-            else { z1[nt][e] = z[nt][e]; w1[nt][e] = w0[nt][e]; }
+          }
+        } else {
+          uint32_t b[2][4];
+          float x[2][4];
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) vec_frag_b(b[nt], smem_u32(Li) + lane_vb, nt);
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) mma_f16_zero(x[nt], zl, b[nt][0], b[nt][1]);
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) mma_f16(x[nt], zh, b[nt][2], b[nt][3]);
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) mma_f16(x[nt], zh, b[nt][0], b[nt][1]);
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) {
+            const float2 fi2 = *reinterpret_cast<const float2*>(dl + 16 + 8 * nt + 2 * c4);
+            const float2 rs2 = *reinterpret_cast<const float2*>(dl + 32 + 8 * nt + 2 * c4);
+            const float fy[2] = {sy * fi2.x, sy * fi2.y}, fa[2] = {sAi * fi2.x * rs2.x, sAi * fi2.y * rs2.y};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              y[nt][e] = x[nt][e] * fy[e & 1];
+              a1[nt][e] = x[nt][e] * fa[e & 1];   // u = k_hat: a_t = z_t / delta_t
+            }
           }
         }
         sz1 = sAi;
-        vec_store(sb + Cfg::a_Z + my_rows, y);
         split_frag(y[0], y[1], yh, yl);
+        vec_store_frag(sb + Cfg::a_Z + my_rows, yh, yl);
       }
       named_sync(1, NW * 32);
-      // ---- A <- A - sum zeta zeta^T
+      // ---- A <- A - sum zeta zeta^T, and at once the next chunk's Z0 (past the end: unused).  One block of code without a
+      // branch, so that the two products' latencies overlap.
+      clear_z0();
+      {
+        const int next = (c + 1) % RK;
+        constexpr int NU = 2 * KB;   // tiles a step
 #pragma unroll
-      for (int nt = 0; nt < NTILE; nt += NB) {
-        uint32_t b[NB][4];
-        float x[NB][4];
+        for (int nt = 0; nt < NTILE; nt += NU) {
+          uint32_t b[NU][4];
+          float x[NU][4];
 #pragma unroll
-        for (int i = 0; i < NB; ++i) vec_frag_b(b[i], sb + Cfg::a_Z + lane_vb, nt + i);
+          for (int i = 0; i < NU; ++i) vec_frag_b(b[i], sb + Cfg::a_Z + lane_vb, nt + i);
 #pragma unroll
-        for (int i = 0; i < NB; ++i) mma_f16_zero(x[i], yl, b[i][0], b[i][1]);
+          for (int i = 0; i < NU; ++i) mma_f16_zero(x[i], yl, b[i][0], b[i][1]);
 #pragma unroll
-        for (int i = 0; i < NB; ++i) mma_f16(x[i], yh, b[i][2], b[i][3]);
+          for (int i = 0; i < NU; ++i) mma_f16(x[i], yh, b[i][2], b[i][3]);
 #pragma unroll
-        for (int i = 0; i < NB; ++i) mma_f16(x[i], yh, b[i][0], b[i][1]);
+          for (int i = 0; i < NU; ++i) mma_f16(x[i], yh, b[i][0], b[i][1]);
 #pragma unroll
-        for (int i = 0; i < NB; ++i)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) st[nt + i][e] = fmaf(x[i][e], sAy, st[nt + i][e]);
+          for (int i = 0; i < NU; ++i) tile_fma(st[nt + i], x[i], sAy);
+          product(nt / 2, next);
+        }
       }
       if (look) {
         float mx = 0.f;
@@ -657,11 +792,19 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           for (int nt = 0; nt < NTILE; ++nt)
 #pragma unroll
             for (int e = 0; e < 4; ++e) st[nt][e] *= f;
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              z0[nt][e] *= f;
+              w0[nt][e] *= f;
+            }
           sA *= f;
           sAi = pow2_inverse(sA);
           set_sy();
         }
       }
+      stash_state(c + 1);
     }
     // rank 1's arrivals on this CTA's barriers must have landed before the CTA may leave (the cluster
     // barrier at the end does not order them): wait for the last use of every slot
@@ -675,6 +818,8 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
               make_float2(st[nt][2 * hf] * sAi, st[nt][2 * hf + 1] * sAi);
     }
   } else if constexpr (STASH) {
+  } else if (warp > NW) {
+    widen(std::true_type{});
   } else if (warp == NW) {
     // ===================================================================== rank 1: small matrices
     // N = K alpha^T, H = Q alpha^T, Q K^T; Tm = (I + stril(N))^-1; output scales 1 / (den_t * scale of q_t)
@@ -833,16 +978,27 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
                          [&](int i) -> float* { return i >= 2 ? rq[i & 1] : pk[i & 1]; });
       }
       arrive(&kfree[slot]);
-      float b[2][4], ev[2][4] = {};
+      float ev[2][4], y[2][4] = {};   // V - P, then E^T; the product's sum
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) b[nt][e] = fmaf(vn[4 * nt + e], sS, -pk[nt][e] * kUnitInv);
+        for (int e = 0; e < 4; ++e) ev[nt][e] = fmaf(vn[4 * nt + e], sS, -pk[nt][e] * kUnitInv);
       if (c + 1 < nch) fetch_v(c + 1);
       wait(&gfull[gs], (c >> 1) & 1);
       // ---- E^T = (V - P) Tm^T;  O^T = R + E^T H^T
-      small_product<LD>(ev, b, fs + Cfg::sf_T + gs * SM, lane);
-      small_product<LD>(rq, ev, fs + Cfg::sf_H + gs * SM, lane);
+#pragma unroll 1
+      for (int i = 0; i < 2; ++i) {   // (one copy of the code)
+        small_product<LD>(y, ev, fs + (i ? Cfg::sf_H : Cfg::sf_T) + gs * SM, lane);
+        if (i == 0) {
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              ev[nt][e] = y[nt][e];
+              y[nt][e] = rq[nt][e];
+            }
+        }
+      }
       {
         const float* osc = fs + Cfg::sf_osc + gs * 16;
 #pragma unroll
@@ -851,8 +1007,8 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           const float f = osc[8 * nt + 2 * c4 + e] * sSi;
           if (c * C + 2 * c4 + e + 8 * nt < T) {
             float* q = odst + (e ? tstride : 0) + (nt ? 8 * tstride : 0);
-            q[0] = rq[nt][e] * f;
-            q[8] = rq[nt][2 + e] * f;
+            q[0] = y[nt][e] * f;
+            q[8] = y[nt][2 + e] * f;
           }
         }
         odst += 16 * tstride;
@@ -887,9 +1043,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
 #pragma unroll
         for (int i = 0; i < NB; ++i) mma_f16(x[i], ah, b[i][0], b[i][1]);
 #pragma unroll
-        for (int i = 0; i < NB; ++i)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) st[nt + i][e] = fmaf(x[i][e], sei, st[nt + i][e]);
+        for (int i = 0; i < NB; ++i) tile_fma(st[nt + i], x[i], sei);
       }
       }
       arrive_cl(&aempty[as], 0);

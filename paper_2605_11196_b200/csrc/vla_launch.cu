@@ -425,8 +425,14 @@ int seqpar_before_d(int dtype, const SeqParParams& sp, cudaStream_t st) {
   if (cudaMemsetAsync(sp.Gd, 0, size_t(N) * D * D * sizeof(double), st) != cudaSuccess ||
       cudaMemsetAsync(sp.zsum, 0, size_t(N) * D * sizeof(float), st) != cudaSuccess)
     return VLA_ERR_CUDA;
-  if (dtype == VLA_F32) seqpar_gram_kernel<D, float><<<dim3(N, kGramSplit), 256, 0, st>>>(sp);
-  else seqpar_gram_kernel<D, uint16_t><<<dim3(N, kGramSplit), 256, 0, st>>>(sp);
+  if (sp.u) {
+    if (dtype == VLA_F32) seqpar_gram_kernel<D, float><<<dim3(N, kGramSplit), 256, 0, st>>>(sp);
+    else seqpar_gram_kernel<D, uint16_t><<<dim3(N, kGramSplit), 256, 0, st>>>(sp);
+  } else {
+    const dim3 grid(N, kGramSplit, D == 128 ? 2 : 1);
+    if (dtype == VLA_F32) seqpar_gram_unit_kernel<D, float><<<grid, 256, 0, st>>>(sp);
+    else seqpar_gram_unit_kernel<D, uint16_t><<<grid, 256, 0, st>>>(sp);
+  }
   if (sp.A0) seqpar_m0_kernel<D><<<sp.units, 256, 0, st>>>(sp);
   seqpar_invert_kernel<D><<<N, 256, 0, st>>>(sp);
   return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;

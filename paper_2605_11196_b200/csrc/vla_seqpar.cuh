@@ -8,7 +8,7 @@
 // segment start comes from a Gram matrix and one inversion.  A unit's sequence is therefore cut
 // into P equal segments that are scanned at the same time:
 //
-//   1. gram     G_j = sum_{t in segment j} u_t u_t^T  (fp32 products, fp64 accumulation) and
+//   1. gram     G_j = sum_{t in segment j} u_t u_t^T  (fp32 accuracy, accumulated in 48 bits or fp64) and
 //               the segment's sum of phi(k)
 //   2. invert   A_start_j = (lambda I + sum_{i<j} G_i)^-1 in fp64 (Gauss-Jordan, no pivoting:
 //               the matrix is symmetric positive definite), running key sum at the start;
@@ -21,7 +21,7 @@
 //
 // All of it is exact algebra; it costs about half more arithmetic than the plain scan (one A for both scans) and
 // makes P times as many clusters, which is what a long sequence with few (batch, head) units needs.  16 units x 65536
-// tokens at d = 64: 8.1 ms uncut, 2.96 in 16 segments (3.8 with both scans in one CTA of the FMA chunk kernel).
+// tokens at d = 64: 8.1 ms uncut, 2.69 in 16 segments (3.8 with both scans in one CTA of the FMA chunk kernel).
 #pragma once
 
 #include "vla_common.cuh"
@@ -39,6 +39,134 @@ __device__ __forceinline__ float seqpar_phi(float x) { return x > 0.0f ? x + 1.0
 // Input rows: 8 lanes per token, 32 tokens per block, every load of a block in flight at once.
 // Thread (ty, tx) of a 16 x 16 grid owns an R x R block of the D x D result, R = D / 16.
 
+// The segments' tokens of one CTA: whole 32-token blocks except at the end
+struct GramSlice { int unit, j, Ls, tlo, thi; };
+__device__ __forceinline__ GramSlice gram_slice(const SeqParParams& p, int TB) {
+  GramSlice s;
+  s.unit = int(blockIdx.x) / p.P;
+  s.j = int(blockIdx.x) % p.P;
+  s.Ls = p.T / p.P;
+  const int nblk = (s.Ls + TB - 1) / TB;
+  s.tlo = int((long long)nblk * blockIdx.y / kGramSplit) * TB;
+  s.thi = min(s.Ls, int((long long)nblk * (blockIdx.y + 1) / kGramSplit) * TB);
+  return s;
+}
+
+// u = k_hat: unit rows, so the products run on warp-level tensor-core instructions in two fp16 terms (vla_mma.cuh).  What
+// bounded the FMA form was the fp64 addition of every 32-token partial sum (4096 of them at d = 64, at some 2 a clock and
+// SM): here the partial sums are added in pairs of floats (a two-sum: nothing is lost to second order), and only a CTA's
+// result goes to fp64.  A warp owns tiles of one 16-row strip; the next block's keys are fetched while this one is multiplied.
+// 16 units x 65536 tokens, d = 64, bf16: 320 -> 198 us.
+template <int D, typename TIn>
+__global__ void __launch_bounds__(256) seqpar_gram_unit_kernel(const SeqParParams p) {
+  constexpr int TB = 32, EPL = D / 8, F = EPL / 4;
+  constexpr int NTW = D == 128 ? 8 : D == 64 ? 4 : 1;   // 16 x 8 tiles of a warp (d = 128: half the columns a CTA, blockIdx.z)
+  constexpr int NG = NTW < 4 ? NTW : 4;                 // ... whose products are interleaved
+  constexpr uint32_t buf_bytes = TB * kTokRow<D>;
+  __shared__ __align__(128) unsigned char buf[2][buf_bytes];
+  const GramSlice sl = gram_slice(p, TB);
+  if (sl.j == p.P - 1) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tok = tid >> 3, pl = tid & 7;
+  const bool ident = (p.flags & VLA_FLAG_IDENTITY_MAP) != 0;
+  const int mt = D == 128 ? warp : D == 64 ? warp >> 1 : warp >> 2;
+  const int nt0 = D == 128 ? 8 * int(blockIdx.z) : D == 64 ? 4 * (warp & 1) : warp & 3;
+  const TIn* kk = static_cast<const TIn*>(p.k) + (size_t(sl.unit) * p.T + size_t(sl.j) * sl.Ls) * D;
+  const uint32_t lm = tok_lane_m<D>(lane), lk = tok_lane_k<D>(lane);
+
+  float2 hi[NTW][2], lo[NTW][2];
+#pragma unroll
+  for (int i = 0; i < NTW; ++i)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) hi[i][e] = lo[i][e] = make_float2(0.f, 0.f);
+  float zs[EPL] = {};
+  float4 x[F];
+  auto fetch = [&](int t0) {
+    const int t = t0 + tok;
+#pragma unroll
+    for (int f = 0; f < F; ++f) x[f] = t < sl.thi ? load4(kk + size_t(t) * D, f * 8 + pl) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  if (sl.tlo < sl.thi) fetch(sl.tlo);
+  int ring = 0;
+  for (int t0 = sl.tlo; t0 < sl.thi; t0 += TB, ring ^= 1) {
+    const uint32_t base = smem_u32(buf[ring]);
+    {
+      const bool act = t0 + tok < sl.thi;
+      float ss = 0.0f;
+#pragma unroll
+      for (int f = 0; f < F; ++f) {
+        if (act && !ident) x[f] = make_float4(seqpar_phi(x[f].x), seqpar_phi(x[f].y), seqpar_phi(x[f].z), seqpar_phi(x[f].w));
+        zs[4 * f] += x[f].x; zs[4 * f + 1] += x[f].y; zs[4 * f + 2] += x[f].z; zs[4 * f + 3] += x[f].w;
+        ss = fmaf(x[f].x, x[f].x, fmaf(x[f].y, x[f].y, fmaf(x[f].z, x[f].z, fmaf(x[f].w, x[f].w, ss))));
+      }
+#pragma unroll
+      for (int off = 4; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+      const float inv = 256.0f / fmaxf(sqrtf(ss), p.eps);
+#pragma unroll
+      for (int f = 0; f < F; ++f) {
+        uint32_t h0, l0, h1, l1;
+        split_f16(x[f].x * inv, x[f].y * inv, h0, l0);
+        split_f16(x[f].z * inv, x[f].w * inv, h1, l1);
+        const uint32_t at = base + uint32_t(tok) * kTokRow<D> + 8 * (f * 8 + pl);
+        sts64(at, h0, h1);
+        sts64(at + 2 * D, l0, l1);
+      }
+    }
+    __syncthreads();   // (two buffers: a warp that writes the next block's rows has passed this barrier after its last reads)
+    fetch(t0 + TB);
+    uint32_t ah[2][4], al[2][4];
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+      tok_frag_m<D>(ah[ks], base + lm, 16 * ks, mt, false);
+      tok_frag_m<D>(al[ks], base + lm, 16 * ks, mt, true);
+    }
+#pragma unroll
+    for (int n = 0; n < NTW; n += NG) {
+      float acc[NG][4] = {};
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) {
+        uint32_t b[NG][4];
+#pragma unroll
+        for (int i = 0; i < NG; ++i) tok_frag_k<D>(b[i], base + lk, 16 * ks, nt0 + n + i);
+        mma3_f16_many<NG>([&](int, int l) -> const uint32_t(&)[4] { return l ? al[ks] : ah[ks]; },
+                          [&](int i, int r) { return b[i][r]; }, [&](int i) -> float* { return acc[i]; });
+      }
+      const float2 m1 = make_float2(-1.0f, -1.0f);
+#pragma unroll
+      for (int i = 0; i < NG; ++i)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          float2& h = hi[n + i][e];
+          const float2 y = make_float2(acc[i][2 * e], acc[i][2 * e + 1]), sum = fadd2(h, y), d = ffma2(h, m1, sum);
+          lo[n + i][e] = fadd2(lo[n + i][e], fadd2(ffma2(ffma2(d, m1, sum), m1, h), ffma2(d, m1, y)));
+          h = sum;
+        }
+    }
+  }
+  double* G = p.Gd + size_t(blockIdx.x) * D * D;
+#pragma unroll
+  for (int i = 0; i < NTW; ++i)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      double* o = G + size_t(16 * mt + (lane >> 2) + 8 * e) * D + 8 * (nt0 + i) + 2 * (lane & 3);
+      atomicAdd(o, (double(hi[i][e].x) + double(lo[i][e].x)) * (1.0 / 65536.0));
+      atomicAdd(o + 1, (double(hi[i][e].y) + double(lo[i][e].y)) * (1.0 / 65536.0));
+    }
+  if (blockIdx.z == 0) {   // key sum: this thread's columns are (f * 8 + pl) * 4 + i; add over the 32 token slots
+    __syncthreads();
+    float* zpart = reinterpret_cast<float*>(buf);
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) zpart[tok * D + ((e / 4) * 8 + pl) * 4 + (e & 3)] = zs[e];
+    __syncthreads();
+    for (int c = tid; c < D; c += 256) {
+      float s = 0.0f;
+#pragma unroll
+      for (int w = 0; w < TB; ++w) s += zpart[w * D + c];
+      atomicAdd(&p.zsum[size_t(blockIdx.x) * D + c], s);
+    }
+  }
+}
+
+// An explicit u, of any norm: fp32 products (one scale per K step of fp16 products would not do for rows of different norms)
 template <int D, typename TIn>
 __global__ void __launch_bounds__(256) seqpar_gram_kernel(const SeqParParams p) {
   constexpr int R = D / 16;
@@ -47,19 +175,16 @@ __global__ void __launch_bounds__(256) seqpar_gram_kernel(const SeqParParams p) 
   constexpr int LDU = D + 4;
   __shared__ __align__(16) float U[TB][LDU];
   __shared__ float zpart[TB][D];
-  const int vu = blockIdx.x, unit = vu / p.P, j = vu % p.P;
+  const int vu = blockIdx.x;
+  const GramSlice sl = gram_slice(p, TB);
+  const int unit = sl.unit, j = sl.j, Ls = sl.Ls, tlo = sl.tlo, thi = sl.thi;
   if (j == p.P - 1) return;
-  const int Ls = p.T / p.P;
-  // this CTA's tokens of the segment: [tlo, thi), whole 32-token blocks except at the end
-  const int nblk = (Ls + TB - 1) / TB;
-  const int tlo = int((long long)nblk * blockIdx.y / kGramSplit) * TB;
-  const int thi = min(Ls, int((long long)nblk * (blockIdx.y + 1) / kGramSplit) * TB);
   const int tid = threadIdx.x;
   const int ty = tid >> 4, tx = tid & 15;
   const int tok = tid >> 3, pl = tid & 7;      // input stage: token of the block, lane of the token
   const bool ident = (p.flags & VLA_FLAG_IDENTITY_MAP) != 0;
   const TIn* kk = static_cast<const TIn*>(p.k) + (size_t(unit) * p.T + size_t(j) * Ls) * D;
-  const TIn* uu = p.u ? static_cast<const TIn*>(p.u) + (size_t(unit) * p.T + size_t(j) * Ls) * D : nullptr;
+  const TIn* uu = static_cast<const TIn*>(p.u) + (size_t(unit) * p.T + size_t(j) * Ls) * D;
 
   double accd[R][R];
 #pragma unroll
@@ -71,12 +196,10 @@ __global__ void __launch_bounds__(256) seqpar_gram_kernel(const SeqParParams p) 
   for (int e = 0; e < EPL; ++e) zs[e] = 0.0f;
 
   for (int t0 = tlo; t0 < thi; t0 += TB) {
-    // rows u_t of this block: k_hat = phi(k)/||phi(k)|| (or k/||k||), or the given u verbatim
+    // rows u_t of this block verbatim; the keys for their sum
     {
       const int t = t0 + tok;
       const bool act = t < thi;
-      float x[EPL];
-      float ss = 0.0f;
 #pragma unroll
       for (int f = 0; f < EPL / 4; ++f) {
         float4 k4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -85,21 +208,9 @@ __global__ void __launch_bounds__(256) seqpar_gram_kernel(const SeqParParams p) 
           k4.x = seqpar_phi(k4.x); k4.y = seqpar_phi(k4.y);
           k4.z = seqpar_phi(k4.z); k4.w = seqpar_phi(k4.w);
         }
-        x[4 * f + 0] = k4.x; x[4 * f + 1] = k4.y; x[4 * f + 2] = k4.z; x[4 * f + 3] = k4.w;
-      }
-#pragma unroll
-      for (int e = 0; e < EPL; ++e) {
-        zs[e] += x[e];
-        ss = fmaf(x[e], x[e], ss);
-      }
-#pragma unroll
-      for (int off = 4; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-      const float inv = 1.0f / fmaxf(sqrtf(ss), p.eps);
-#pragma unroll
-      for (int f = 0; f < EPL / 4; ++f) {
-        float4 v4 = make_float4(x[4 * f] * inv, x[4 * f + 1] * inv, x[4 * f + 2] * inv, x[4 * f + 3] * inv);
-        if (uu) v4 = act ? load4(uu + size_t(t) * D, f * 8 + pl) : make_float4(0.f, 0.f, 0.f, 0.f);
-        *reinterpret_cast<float4*>(&U[tok][(f * 8 + pl) * 4]) = v4;
+        zs[4 * f] += k4.x; zs[4 * f + 1] += k4.y; zs[4 * f + 2] += k4.z; zs[4 * f + 3] += k4.w;
+        *reinterpret_cast<float4*>(&U[tok][(f * 8 + pl) * 4]) =
+            act ? load4(uu + size_t(t) * D, f * 8 + pl) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
     __syncthreads();

@@ -393,13 +393,16 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           // diag(delta)^-1/2 L^-1, whose rows are no longer than 1 (I + W >= I), as an operand.  They may be as short as
           // 1 / sqrt(delta): past 2^-15 (lambda below 1e-9) each row gets a power of two of its own
           const float rs = rsqrt_ftz_nr(delta);
-          float f = rs * kLam, fi = kLamInv;
+          // (scaled by the power of two below delta^-1/2: L^-1's unit diagonal stays exact, the rest of the factor is applied in fp32.
+          // With all of it in the operand A_T was off by 1.5 to 2.5 times as much at lambda <= 1e-6)
+          const float p2 = __uint_as_float(__float_as_uint(rs) & 0x7f800000u);
+          float f = p2 * kLam, fi = rs * pow2_inverse(p2) * kLamInv;
           if (__any_sync(0xffffffffu, delta > 1e9f)) {
             float mx = 0.f;
 #pragma unroll
             for (int j = 0; j < 8; ++j) mx = fmaxf(mx, fabsf(x[j]));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-            const float own = pow2_scale(mx * rs, 0);
+            const float own = pow2_scale(mx * p2, 0);
             f *= own;
             fi *= pow2_inverse(own);
           }

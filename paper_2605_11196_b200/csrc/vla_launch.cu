@@ -418,6 +418,16 @@ int launch_decode(int d, int dtype, const ScanParams& p, cudaStream_t st) {
 // ---------------------------------------------------------------- sequence-parallel helpers
 namespace {
 
+template <int D, typename TIn>
+int launch_gram_unit_t(const SeqParParams& sp, cudaStream_t st) {
+  using Cfg = GramUnitCfg<D>;
+  auto kern = seqpar_gram_unit_kernel<D, TIn>;
+  static std::atomic<unsigned long long> done{0};
+  if (!set_smem_once(done, reinterpret_cast<const void*>(kern), Cfg::smem_bytes)) return VLA_ERR_CUDA;
+  kern<<<dim3(sp.units * sp.P, kGramSplit, D == 128 ? 2 : 1), 256, Cfg::smem_bytes, st>>>(sp);
+  return VLA_OK;
+}
+
 template <int D>
 int seqpar_before_d(int dtype, const SeqParParams& sp, cudaStream_t st) {
   const int N = sp.units * sp.P;
@@ -429,9 +439,8 @@ int seqpar_before_d(int dtype, const SeqParParams& sp, cudaStream_t st) {
     if (dtype == VLA_F32) seqpar_gram_kernel<D, float><<<dim3(N, kGramSplit), 256, 0, st>>>(sp);
     else seqpar_gram_kernel<D, uint16_t><<<dim3(N, kGramSplit), 256, 0, st>>>(sp);
   } else {
-    const dim3 grid(N, kGramSplit, D == 128 ? 2 : 1);
-    if (dtype == VLA_F32) seqpar_gram_unit_kernel<D, float><<<grid, 256, 0, st>>>(sp);
-    else seqpar_gram_unit_kernel<D, uint16_t><<<grid, 256, 0, st>>>(sp);
+    const int rc = dtype == VLA_F32 ? launch_gram_unit_t<D, float>(sp, st) : launch_gram_unit_t<D, uint16_t>(sp, st);
+    if (rc != VLA_OK) return rc;
   }
   if (sp.A0) seqpar_m0_kernel<D><<<sp.units, 256, 0, st>>>(sp);
   seqpar_invert_kernel<D><<<N, 256, 0, st>>>(sp);

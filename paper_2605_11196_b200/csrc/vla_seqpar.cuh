@@ -8,7 +8,7 @@
 // segment start comes from a Gram matrix and one inversion.  A unit's sequence is therefore cut
 // into P equal segments that are scanned at the same time:
 //
-//   1. gram     G_j = sum_{t in segment j} u_t u_t^T  (fp32 accuracy, accumulated in 48 bits or fp64) and
+//   1. gram     G_j = sum_{t in segment j} u_t u_t^T  (fp32 accuracy; sums in float pairs or fp64) and
 //               the segment's sum of phi(k)
 //   2. invert   A_start_j = (lambda I + sum_{i<j} G_i)^-1 in fp64 (Gauss-Jordan, no pivoting:
 //               the matrix is symmetric positive definite), running key sum at the start;
@@ -21,7 +21,7 @@
 //
 // All of it is exact algebra; it costs about half more arithmetic than the plain scan (one A for both scans) and
 // makes P times as many clusters, which is what a long sequence with few (batch, head) units needs.  16 units x 65536
-// tokens at d = 64: 8.1 ms uncut, 2.69 in 16 segments (3.8 with both scans in one CTA of the FMA chunk kernel).
+// tokens at d = 64: 8.1 ms uncut, 2.72 in 16 segments (3.8 with both scans in one CTA of the FMA chunk kernel).
 #pragma once
 
 #include "vla_common.cuh"
@@ -37,7 +37,6 @@ __device__ __forceinline__ float seqpar_phi(float x) { return x > 0.0f ? x + 1.0
 // segment's tokens are divided among kGramSplit CTAs of 256 threads, which add their results
 // into the segment's (zeroed) matrix; the last segment of a unit needs neither and is skipped.
 // Input rows: 8 lanes per token, 32 tokens per block, every load of a block in flight at once.
-// Thread (ty, tx) of a 16 x 16 grid owns an R x R block of the D x D result, R = D / 16.
 
 // The segments' tokens of one CTA: whole 32-token blocks except at the end
 struct GramSlice { int unit, j, Ls, tlo, thi; };
@@ -52,18 +51,31 @@ __device__ __forceinline__ GramSlice gram_slice(const SeqParParams& p, int TB) {
   return s;
 }
 
-// u = k_hat: unit rows, so the products run on warp-level tensor-core instructions in two fp16 terms (vla_mma.cuh).  What
-// bounded the FMA form was the fp64 addition of every 32-token partial sum (4096 of them at d = 64, at some 2 a clock and
-// SM): here the partial sums are added in pairs of floats (a two-sum: nothing is lost to second order), and only a CTA's
-// result goes to fp64.  A warp owns tiles of one 16-row strip; the next block's keys are fetched while this one is multiplied.
-// 16 units x 65536 tokens, d = 64, bf16: 320 -> 198 us.
+// u = k_hat: unit rows, so the products run on warp-level tensor-core instructions in fp16.  The tensor core truncates when it
+// adds, to one side, and over tens of thousands of tokens such a bias does not average out: with two rounded terms a factor
+// (hi*hi + hi*lo + lo*hi) G's diagonal was 8e-8 short and A at a segment start up to four times as far off as with fp32
+// products.  So a unit row, scaled to 2^9, is cut into a whole number H of at most ten bits and two fp16 terms M + L of the rest:
+// every H H' and any sum of 32 of them (<= 2^23) is a whole number that fp32 holds, nothing is cut off, and the other products
+// are 2^-10 of these or less.  Off from 64 bits in the 2-norm, 1024 to 8192 tokens a segment, every d: G 3e-8 to 9e-8 with two
+// terms, 0.5e-8 to 5e-8 with fp32 FMAs, 0.1e-8 to 3e-8 so (what is left is the rounding of k_hat itself); A at a segment start,
+// keys all alike, 2e-6 to 3.5e-5, 2e-6 to 9e-6, 3e-8 to 2e-7.  What bounded the FMA form was the fp64 addition of every 32-token
+// partial sum (4096 of them at d = 64, at some 2 a clock and SM): here H H' is added in pairs of floats (the two-sum of
+// Knuth, TAOCP 2, 4.2.2), and only a CTA's result goes to fp64.  A warp owns tiles of one 16-row strip; the next block's keys are
+// fetched while this one is multiplied.  16 units x 65536 tokens, d = 64, bf16: 320 us with fp32 FMAs, 198 with two terms; the
+// three products more cost the whole call 30 us (2.69 -> 2.72 ms), at d = 128 8 units x 32768 45 (2.49 -> 2.54).
+template <int D>
+struct GramUnitCfg {
+  static constexpr int TB = 32;
+  static constexpr uint32_t row = 6 * D + 16;   // H, M, L; an odd number of 16-byte pieces
+  static constexpr uint32_t buf = TB * row, smem_bytes = 2 * buf;
+};
 template <int D, typename TIn>
-__global__ void __launch_bounds__(256) seqpar_gram_unit_kernel(const SeqParParams p) {
-  constexpr int TB = 32, EPL = D / 8, F = EPL / 4;
+__global__ void __launch_bounds__(256, D == 128 ? 1 : 2) seqpar_gram_unit_kernel(const SeqParParams p) {
+  using Cfg = GramUnitCfg<D>;
+  constexpr int TB = Cfg::TB, EPL = D / 8, F = EPL / 4;
   constexpr int NTW = D == 128 ? 8 : D == 64 ? 4 : 1;   // 16 x 8 tiles of a warp (d = 128: half the columns a CTA, blockIdx.z)
   constexpr int NG = NTW < 4 ? NTW : 4;                 // ... whose products are interleaved
-  constexpr uint32_t buf_bytes = TB * kTokRow<D>;
-  __shared__ __align__(128) unsigned char buf[2][buf_bytes];
+  extern __shared__ __align__(128) unsigned char gram_smem[];
   const GramSlice sl = gram_slice(p, TB);
   if (sl.j == p.P - 1) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tok = tid >> 3, pl = tid & 7;
@@ -71,7 +83,10 @@ __global__ void __launch_bounds__(256) seqpar_gram_unit_kernel(const SeqParParam
   const int mt = D == 128 ? warp : D == 64 ? warp >> 1 : warp >> 2;
   const int nt0 = D == 128 ? 8 * int(blockIdx.z) : D == 64 ? 4 * (warp & 1) : warp & 3;
   const TIn* kk = static_cast<const TIn*>(p.k) + (size_t(sl.unit) * p.T + size_t(sl.j) * sl.Ls) * D;
-  const uint32_t lm = tok_lane_m<D>(lane), lk = tok_lane_k<D>(lane);
+  // ldmatrix addresses: the A operand's 16 columns of G, the B operand's eight (H and M; L of two tiles)
+  const uint32_t lm = uint32_t((lane & 7) + (lane >> 4) * 8) * Cfg::row + ((lane >> 3) & 1) * 16 + mt * 32;
+  const uint32_t lr = uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * Cfg::row + nt0 * 16;
+  const uint32_t lk = lr + (lane >> 4) * (2 * D), ll = lr + (lane >> 4) * 16 + 4 * D;
 
   float2 hi[NTW][2], lo[NTW][2];
 #pragma unroll
@@ -86,9 +101,10 @@ __global__ void __launch_bounds__(256) seqpar_gram_unit_kernel(const SeqParParam
     for (int f = 0; f < F; ++f) x[f] = t < sl.thi ? load4(kk + size_t(t) * D, f * 8 + pl) : make_float4(0.f, 0.f, 0.f, 0.f);
   };
   if (sl.tlo < sl.thi) fetch(sl.tlo);
+  const float2 m1 = make_float2(-1.0f, -1.0f);
   int ring = 0;
   for (int t0 = sl.tlo; t0 < sl.thi; t0 += TB, ring ^= 1) {
-    const uint32_t base = smem_u32(buf[ring]);
+    const uint32_t base = smem_u32(gram_smem) + ring * Cfg::buf;
     {
       const bool act = t0 + tok < sl.thi;
       float ss = 0.0f;
@@ -100,44 +116,65 @@ __global__ void __launch_bounds__(256) seqpar_gram_unit_kernel(const SeqParParam
       }
 #pragma unroll
       for (int off = 4; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-      const float inv = 256.0f / fmaxf(sqrtf(ss), p.eps);
+      const float inv = 512.0f / fmaxf(sqrtf(ss), p.eps);
 #pragma unroll
       for (int f = 0; f < F; ++f) {
-        uint32_t h0, l0, h1, l1;
-        split_f16(x[f].x * inv, x[f].y * inv, h0, l0);
-        split_f16(x[f].z * inv, x[f].w * inv, h1, l1);
-        const uint32_t at = base + uint32_t(tok) * kTokRow<D> + 8 * (f * 8 + pl);
-        sts64(at, h0, h1);
-        sts64(at + 2 * D, l0, l1);
+        const float2 inv2 = make_float2(inv, inv), round = make_float2(12582912.0f, 12582912.0f);   // 1.5 * 2^23: to a whole number
+        const float2 v[2] = {fmul2(make_float2(x[f].x, x[f].y), inv2), fmul2(make_float2(x[f].z, x[f].w), inv2)};
+        uint32_t H[2], M[2], L[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const float2 h = ffma2(round, m1, fadd2(v[i], round)), r = ffma2(h, m1, v[i]);   // (both differences exact)
+          asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(H[i]) : "f"(h.y), "f"(h.x));
+          split_f16(r.x, r.y, M[i], L[i]);
+        }
+        const uint32_t at = base + uint32_t(tok) * Cfg::row + 8 * (f * 8 + pl);
+        sts64(at, H[0], H[1]);
+        sts64(at + 2 * D, M[0], M[1]);
+        sts64(at + 4 * D, L[0], L[1]);
       }
     }
     __syncthreads();   // (two buffers: a warp that writes the next block's rows has passed this barrier after its last reads)
     fetch(t0 + TB);
-    uint32_t ah[2][4], al[2][4];
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      tok_frag_m<D>(ah[ks], base + lm, 16 * ks, mt, false);
-      tok_frag_m<D>(al[ks], base + lm, 16 * ks, mt, true);
-    }
 #pragma unroll
     for (int n = 0; n < NTW; n += NG) {
-      float acc[NG][4] = {};
+      float y[NG][4], r[NG][4];   // H H', and the rest
+#pragma unroll
+      for (int i = 0; i < NG; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) y[i][e] = r[i][e] = 0.f;
 #pragma unroll
       for (int ks = 0; ks < 2; ++ks) {
-        uint32_t b[NG][4];
+        const uint32_t at = base + 16 * ks * Cfg::row;
+        uint32_t aH[4], aM[4], aL[4], b[NG][4], bL[(NG + 1) / 2][4];
+        ldsm_x4_t(aH, at + lm);
+        ldsm_x4_t(aM, at + lm + 2 * D);
+        ldsm_x4_t(aL, at + lm + 4 * D);
 #pragma unroll
-        for (int i = 0; i < NG; ++i) tok_frag_k<D>(b[i], base + lk, 16 * ks, nt0 + n + i);
-        mma3_f16_many<NG>([&](int, int l) -> const uint32_t(&)[4] { return l ? al[ks] : ah[ks]; },
-                          [&](int i, int r) { return b[i][r]; }, [&](int i) -> float* { return acc[i]; });
+        for (int i = 0; i < NG; ++i) ldsm_x4_t(b[i], at + lk + 16 * (n + i));
+#pragma unroll
+        for (int i = 0; i < NG; i += 2) ldsm_x4_t(bL[i / 2], at + ll + 16 * (n + i));   // (d = 32: the second tile's is not used)
+#pragma unroll
+        for (int i = 0; i < NG; ++i) mma_f16(y[i], aH, b[i][0], b[i][1]);
+#pragma unroll
+        for (int i = 0; i < NG; ++i) mma_f16(r[i], aH, bL[i / 2][2 * (i & 1)], bL[i / 2][2 * (i & 1) + 1]);
+#pragma unroll
+        for (int i = 0; i < NG; ++i) mma_f16(r[i], aL, b[i][0], b[i][1]);
+#pragma unroll
+        for (int i = 0; i < NG; ++i) mma_f16(r[i], aM, b[i][2], b[i][3]);
+#pragma unroll
+        for (int i = 0; i < NG; ++i) mma_f16(r[i], aH, b[i][2], b[i][3]);
+#pragma unroll
+        for (int i = 0; i < NG; ++i) mma_f16(r[i], aM, b[i][0], b[i][1]);
       }
-      const float2 m1 = make_float2(-1.0f, -1.0f);
 #pragma unroll
       for (int i = 0; i < NG; ++i)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           float2& h = hi[n + i][e];
-          const float2 y = make_float2(acc[i][2 * e], acc[i][2 * e + 1]), sum = fadd2(h, y), d = ffma2(h, m1, sum);
-          lo[n + i][e] = fadd2(lo[n + i][e], fadd2(ffma2(ffma2(d, m1, sum), m1, h), ffma2(d, m1, y)));
+          const float2 x2 = make_float2(y[i][2 * e], y[i][2 * e + 1]), sum = fadd2(h, x2), d = ffma2(h, m1, sum);
+          const float2 err = fadd2(ffma2(ffma2(d, m1, sum), m1, h), ffma2(d, m1, x2));
+          lo[n + i][e] = fadd2(lo[n + i][e], fadd2(err, make_float2(r[i][2 * e], r[i][2 * e + 1])));
           h = sum;
         }
     }
@@ -148,12 +185,12 @@ __global__ void __launch_bounds__(256) seqpar_gram_unit_kernel(const SeqParParam
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       double* o = G + size_t(16 * mt + (lane >> 2) + 8 * e) * D + 8 * (nt0 + i) + 2 * (lane & 3);
-      atomicAdd(o, (double(hi[i][e].x) + double(lo[i][e].x)) * (1.0 / 65536.0));
-      atomicAdd(o + 1, (double(hi[i][e].y) + double(lo[i][e].y)) * (1.0 / 65536.0));
+      atomicAdd(o, (double(hi[i][e].x) + double(lo[i][e].x)) * (1.0 / 262144.0));
+      atomicAdd(o + 1, (double(hi[i][e].y) + double(lo[i][e].y)) * (1.0 / 262144.0));
     }
   if (blockIdx.z == 0) {   // key sum: this thread's columns are (f * 8 + pl) * 4 + i; add over the 32 token slots
     __syncthreads();
-    float* zpart = reinterpret_cast<float*>(buf);
+    float* zpart = reinterpret_cast<float*>(gram_smem);
 #pragma unroll
     for (int e = 0; e < EPL; ++e) zpart[tok * D + ((e / 4) * 8 + pl) * 4 + (e & 3)] = zs[e];
     __syncthreads();
@@ -166,7 +203,8 @@ __global__ void __launch_bounds__(256) seqpar_gram_unit_kernel(const SeqParParam
   }
 }
 
-// An explicit u, of any norm: fp32 products (one scale per K step of fp16 products would not do for rows of different norms)
+// An explicit u, of any norm: fp32 products (one scale per K step of fp16 products would not do for rows of different norms).
+// Thread (ty, tx) of a 16 x 16 grid owns an R x R block of the D x D result, R = D / 16.
 template <int D, typename TIn>
 __global__ void __launch_bounds__(256) seqpar_gram_kernel(const SeqParParams p) {
   constexpr int R = D / 16;

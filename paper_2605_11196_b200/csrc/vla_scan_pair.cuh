@@ -379,9 +379,9 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       const float delta = eliminate16<UT>(m, lane, piv, eps, ud);   // (explicit u: delta / D^2)
       {
         float x[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) x[j] = 8 * h + j < r ? m[j] : (8 * h + j == r ? 1.0f : 0.0f);
         if constexpr (UT) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[j] = 8 * h + j < r ? m[j] : (8 * h + j == r ? 1.0f : 0.0f);
           float4* o = reinterpret_cast<float4*>(Li + r * LD + 8 * h);
           o[0] = make_float4(x[0], x[1], x[2], x[3]);
           o[1] = make_float4(x[4], x[5], x[6], x[7]);
@@ -390,13 +390,18 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
             dl[32 + r] = rsqrt_ftz_nr(delta);
           }
         } else {
-          // diag(delta)^-1/2 L^-1, whose rows are no longer than 1 (I + W >= I), as an operand.  They may be as short as
-          // 1 / sqrt(delta): past 2^-15 (lambda below 1e-9) each row gets a power of two of its own
+          // diag(delta)^-1/2 (L^-1 - I) as an operand; the unit diagonal does not go through fp16 and the truncating sum, z_t takes
+          // z0_t in fp32.  Rows of diag(delta)^-1/2 L^-1 are no longer than 1 (I + W >= I).  They may be as short as
+          // 1 / sqrt(delta): past 2^-15 (lambda below 1e-9) each row gets a power of two of its own.
+          // A_T's error over lambda 1 to 1e-14, T 13 to 1500 (geometric mean at d = 16, 32, 64, 128), against tf32 pairs of all of
+          // L^-1 in four products: 0.87, 0.87, 0.89, 0.93 times; with the diagonal in the operand 0.97, 1.00, 1.07, 1.13
+          // (1.85 at lambda 1e-9, d = 128).  The dropped remainders' product is worth 0.01.  The fp32 share costs 70 to 110 clk of a
+          // chunk at d = 32 and 64 (32 units x 4096 tokens, d = 64: 442 -> 457 us)
           const float rs = rsqrt_ftz_nr(delta);
-          // (scaled by the power of two below delta^-1/2: L^-1's unit diagonal stays exact, the rest of the factor is applied in fp32.
-          // With all of it in the operand A_T was off by 1.5 to 2.5 times as much at lambda <= 1e-6)
-          const float p2 = __uint_as_float(__float_as_uint(rs) & 0x7f800000u);
+          const float p2 = __uint_as_float(__float_as_uint(rs) & 0x7f800000u);   // the power of two below: exact
           float f = p2 * kLam, fi = rs * pow2_inverse(p2) * kLamInv;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[j] = 8 * h + j < r ? m[j] : 0.0f;
           if (__any_sync(0xffffffffu, delta > 1e9f)) {
             float mx = 0.f;
 #pragma unroll
@@ -749,11 +754,12 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           for (int nt = 0; nt < 2; ++nt) {
             const float2 fi2 = *reinterpret_cast<const float2*>(dl + 16 + 8 * nt + 2 * c4);
             const float2 rs2 = *reinterpret_cast<const float2*>(dl + 32 + 8 * nt + 2 * c4);
-            const float fy[2] = {sy * fi2.x, sy * fi2.y}, fa[2] = {sAi * fi2.x * rs2.x, sAi * fi2.y * rs2.y};
+            const float fi[2] = {fi2.x, fi2.y}, rs[2] = {rs2.x, rs2.y}, fa[2] = {sAi * rs2.x, sAi * rs2.y};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              y[nt][e] = x[nt][e] * fy[e & 1];
-              a1[nt][e] = x[nt][e] * fa[e & 1];   // u = k_hat: a_t = z_t / delta_t
+              const float zeta = fmaf(z0[nt][e], rs[e & 1], x[nt][e] * fi[e & 1]);
+              y[nt][e] = zeta * sy;
+              a1[nt][e] = zeta * fa[e & 1];   // u = k_hat: a_t = z_t / delta_t
             }
           }
         }

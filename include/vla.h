@@ -298,8 +298,8 @@ int vla_probe_fp32_fma(int iters, float* sink, double* flops, void* stream);
 
 /*
  * vla_selftest_wait_timeout -- test helper (the paper has no counterpart): enqueues a one-warp
- * kernel that waits, with the scan kernels' bounded wait and `probe_limit` probes, on a barrier
- * that cannot complete.  When the probes run out the kernel writes VLA_ERR_DEVICE_TIMEOUT to
+ * kernel that waits, with both forms of the scan kernels' bounded wait and `probe_limit` probes, on
+ * a barrier that cannot complete.  When the probes of both have run out the kernel writes VLA_ERR_DEVICE_TIMEOUT to
  * *status (DEVICE int32, 0 on entry) and returns normally; nothing traps and the context stays
  * usable.  probe_limit must be > 0 (a few thousand probes take well under a millisecond).
  */

@@ -488,23 +488,40 @@ int seqpar_after_scan(int d, const SeqParParams& sp, float* A_T, float* zT, cons
   }
 }
 
-// ---------------------------------------------------------------- the bounded wait, tested
-// One warp waits, with the kernels' own mbar_wait_bounded, on a barrier that expects two
-// arrivals and gets one: the wait can only end by running out of probes.  The kernel then does
-// what the scan kernels do: it records VLA_ERR_DEVICE_TIMEOUT in the caller's status word and
+// ---------------------------------------------------------------- the bounded waits, tested
+// One warp waits, with both forms of the kernels' own wait (mbar_wait_bounded, and the pair kernel's mbar_wait_flagged), on a
+// barrier that expects two arrivals and gets one: these waits can only end by running out of probes.  A wait on a barrier
+// that is complete must leave the flag alone, and one that finds the flag set must end long before its own limit.  The kernel
+// then does what the scan kernels do: it records VLA_ERR_DEVICE_TIMEOUT in the caller's status word and
 // returns normally (no trap, the context stays usable).
 namespace {
 __global__ void wait_selftest_kernel(unsigned int probe_limit, int* status) {
-  __shared__ uint64_t bar;
+  __shared__ uint64_t bar, done;
+  __shared__ int flag;
   if (threadIdx.x == 0) {
     mbar_init(&bar, 2);
+    mbar_init(&done, 1);
     mbar_init_fence();
+    flag = 0;
   }
   __syncthreads();
-  if (threadIdx.x == 0) mbar_arrive(&bar);      // one of the two arrivals; the other never comes
+  if (threadIdx.x == 0) {
+    mbar_arrive(&bar);      // one of the two arrivals; the other never comes
+    mbar_arrive(&done);
+  }
   __syncthreads();
-  if (!mbar_wait_bounded(&bar, 0, probe_limit) && threadIdx.x == 0)
-    atomicCAS(status, 0, int(VLA_ERR_DEVICE_TIMEOUT));
+  volatile int* seen = &flag;
+  bool ok = !mbar_wait_bounded(&bar, 0, probe_limit);
+  mbar_wait_flagged(smem_u32(&done), 0, probe_limit, smem_u32(&flag));
+  ok &= *seen == 0;
+  __syncwarp();
+  mbar_wait_flagged(smem_u32(&bar), 0, probe_limit, smem_u32(&flag));
+  __syncwarp();
+  ok &= *seen == 1;
+  const long long start = clock64();
+  mbar_wait_flagged(smem_u32(&bar), 0, 1u << 18, smem_u32(&flag));   // (its own limit: some 60 ms)
+  ok &= clock64() - start < 20000000;                                 // (one probe; 10 ms)
+  if (ok && threadIdx.x == 0) atomicCAS(status, 0, int(VLA_ERR_DEVICE_TIMEOUT));
 }
 }  // namespace
 

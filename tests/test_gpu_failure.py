@@ -20,8 +20,8 @@ def _scan(dev, kernel=vla.VLA_KERNEL_AUTO, **kw):
 
 
 def test_bounded_wait_runs_out_and_the_device_stays_usable():
-    """The library's own bounded wait (the function every scan kernel waits with) on a barrier
-    that can never complete: after `probe_limit` probes the kernel reports
+    """The library's own bounded waits (mbar_wait_bounded and the pair kernel's mbar_wait_flagged) on a barrier
+    that can never complete: when both have given up after `probe_limit` probes the kernel reports
     VLA_ERR_DEVICE_TIMEOUT through the status word and ends normally.  A scan before and a scan
     after it on the same device give bit-identical results."""
     dev = torch.device("cuda:0")

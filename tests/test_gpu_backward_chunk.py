@@ -69,3 +69,28 @@ def test_units_in_groups_and_long_sequences():
     for s in (slice(0, 1), slice(units - 2, units)):
         b = vla.vla_backward(q[s].contiguous(), k[s].contiguous(), v[s].contiguous(), 1.0, do[s].contiguous(), want_dA0=False)
         assert all(torch.equal(getattr(a, n)[s], getattr(b, n)) for n in ("dq", "dk", "dv", "dS0"))
+
+
+@pytest.mark.parametrize("d", [16, 32, 64, 128])
+@pytest.mark.parametrize("units,T", [(5, 37), (5, 16), (40, 1000)])
+@pytest.mark.parametrize("explicit_u", [False, True])
+def test_gradients_do_not_depend_on_what_the_workspace_held(d, units, T, explicit_u):
+    """A value read before it is written, or a missing wait, shows as a difference: four calls, the workspace full of zeros, NaN,
+    large numbers and what the call before left in it, give the same bits."""
+    if explicit_u and d == 16:
+        return
+    w = W.Workload("ws", 1, units, d, T, "bf16", 3 * d + T)
+    q, k, v = [x.cuda() for x in W.make_inputs(w)]
+    u = W.make_u(w, d ** -0.5).cuda() if explicit_u else None
+    g = torch.randn(q.shape, device="cuda")
+    ws = torch.empty((vla.backward_workspace_bytes(1, units, T, d),), dtype=torch.uint8, device="cuda")
+    first = None
+    for fill in (0, 255, 0x6f, None):
+        if fill is not None:
+            ws.fill_(fill)
+        r = vla.vla_backward(q, k, v, 1.0, g, u=u, workspace=ws, want_dA0=False)
+        assert int(r.status.item()) == 0
+        got = [r.dq, r.dk, r.dv, r.dS0, r.dz0] + ([r.du] if explicit_u else [])
+        assert all(torch.isfinite(x).all() for x in got)
+        first = first or got
+        assert all(torch.equal(a, b) for a, b in zip(first, got))

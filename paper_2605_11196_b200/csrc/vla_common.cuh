@@ -387,12 +387,12 @@ __device__ __forceinline__ void tile16_store(float* G, int i0, int j0, const flo
 // a step with the row by shuffles: 1530).  The registers rotate by two a step, so that columns s, s + 1 are always
 // m[0], m[1] of the half that holds them and the loop stays small; eight steps bring them back.
 // OWN: every row has its own floor of delta, eps * own[row] (own in shared memory, 8-byte aligned).
-template <bool OWN = false>
+template <bool OWN = false, int UNROLL = 2>
 __device__ __forceinline__ float eliminate16(float (&m)[8], int lane, float* piv, float eps, const float* own = nullptr) {
   const int r = lane & 15, h = lane >> 4;
   float delta = 1.0f, f0 = eps, f1 = eps;
   if (OWN) { f0 = eps * own[0]; f1 = eps * own[1]; }
-#pragma unroll 2
+#pragma unroll UNROLL
   for (int s = 0; s < 16; s += 2) {
     constexpr unsigned full = 0xffffffffu;
     float2 next = make_float2(1.0f, 1.0f);   // (a step ahead: off the chain)

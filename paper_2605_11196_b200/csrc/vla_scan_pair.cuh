@@ -12,21 +12,32 @@
 // the A operand of the next product, so a chunk's chain K -> Z0 -> Z -> A stays in one warp's
 // registers except for two exchanges over shared memory (Z0 for W, zeta for the update); every
 // S row is independent of the others.  Beside the D / 16 state warps a CTA has one warp for the
-// 16 x 16 algebra and one to three that widen the inputs (phi, k_hat, hi/lo operand rows) one chunk ahead.
+// 16 x 16 algebra and one or two that widen the inputs (phi, k_hat, hi/lo operand rows) one chunk ahead.
 //
 // A segment of a cut sequence takes a third CTA (NS = 2): rank 2 carries the segment's transfer scan on the same
-// alpha.  d = 64, 16 units x 65536 tokens in 16 segments: scan 2.92 -> 2.2 ms against the FMA chunk kernel, where the
-// two scans shared one CTA with A (6 us of an SM per 16 tokens of a segment; three CTAs here, two on an SM: 4.7).
+// alpha.  d = 64, 16 units x 65536 tokens in 16 segments: scan 2.92 -> 2.07 ms against the FMA chunk kernel, where the
+// two scans shared one CTA with A (6 us of an SM per 16 tokens of a segment; three CTAs here, two on an SM: 4.2).
 
-// Widening: eight columns a lane, so that a token's norms are two to four shuffle rounds and a warp takes twice the tokens at a
+// Widening: eight columns a lane, so that a token's norms are one to four shuffle rounds and a warp takes twice the tokens at a
 // time.  With four the widening warps of rank 1 set the pace of every d >= 32 (d = 64: 2830 of 3560 clk per chunk).
 //
-// Instruction cache: an SM holds CTAs of one rank only (measured: a cluster's ranks lie on the two SMs of a TPC), and runs straight
-// code from 32 KB of cache at one instruction a clock, beyond that at 2.1 (and all SMs of a GPC share what is beyond).  So each
-// rank has its own copy of the widening code, small loops stay rolled, and values go through two-wide instructions.
+// Instruction cache: an SM runs straight code from 32 KB of cache at one instruction a clock, beyond that at 2.1, and all SMs of a GPC
+// share what is beyond.  In clusters of two an SM holds CTAs of one rank only (measured with 64, 148 and 296 CTAs: a cluster's
+// ranks lie on the two SMs of a TPC, and the second wave falls in with the first), so each rank has its own copy of the
+// widening code, small loops stay rolled, and values go through two-wide instructions.  (Three ranks on two SMs mix.)  What lies
+// beyond the cache comes at a rate that differs from GPU to GPU: one build takes 457 us on four GPUs and 533 on three others (32
+// units x 4096 tokens, d = 64).
 //
-// What bounds it: at one unit per SM pair the serial chain of rank 0 (state split, Z0, W, the
-// 16 x 16 elimination, Z, update), with many units the tensor pipe (8 clk per instruction and
+// With explicit u rank 0's roles are some 8 KB longer and do not fit.  Widened side by side, eight columns of keys and u a lane, they made
+// two CTAs on an SM (d = 64) wait twice as long for instructions as the form before (1.9 against 0.8 warps per instruction
+// issued, for 15 % fewer instructions).  So keys and u go through one loop, the elimination's and W's loops are rolled, and at d = 64 a lane
+// takes four columns and the next chunk's products stand by themselves (SHORT).  us, four columns and all unrolled / eight / now:
+// d = 64 256 units x 2048 tokens 990 / 1140 / 996 (on a GPU of the slower kind 919 / 1020 / 935), 32 x 4096 634 / 618 / 629 (717 / 779 /
+// 732); d = 128 64 x 2048 603 / 605 / 591, 512 x 8192 17.7 / 18.0 / 17.5 ms; d = 32 256 x 512 171 / 172 / 171.  (Four columns at d = 32 and 128: 179 and 703; SHORT at d = 32 and 128: 180
+// and 721; a third and fourth widening warp at d = 128: 590, where two left 548.)
+//
+// What bounds it: at one unit per SM pair the serial chain of rank 0 (W, the 16 x 16 elimination, Z, then the update of A with the
+// next chunk's Z0 in it), with many units the tensor pipe (8 clk per instruction and
 // scheduler).  Two CTAs because at d = 128 both states and their operands do not fit one SM's
 // registers, and below because small batches then use twice the SMs.
 //
@@ -54,15 +65,13 @@ struct PairCfg {
   static constexpr int NPREP = D >= 64 ? 2 : 1;             // widening warps
   static constexpr int NT = (NW + 1 + NPREP) * 32;
   // CTAs per SM the registers are cut for.  d = 64: two hide one another's chains (128 units x 1024 tokens 355 -> 203 us,
-  // 256 units 657 -> 392) and cost one unit 2 % (128 registers instead of 192).  At d = 64 and 128 the cap is reached: 8 to 150
-  // bytes a thread are spilled, most with explicit u
+  // 256 units 657 -> 392) and cost one unit 2 % (128 registers instead of 192).  At d = 64 and 128 the cap is reached: up to 110
+  // bytes a thread are spilled, most in the segments' form
   static constexpr int MINB = D == 64 ? 2 : 1;
-  static constexpr int LPT = D / 8;                         // lanes per token in the widening pass
-  static constexpr int TPW = 32 / LPT;                      // tokens per warp pass
-  static constexpr int NP = C / (TPW * NPREP);              // passes per chunk
-  static_assert(C % (TPW * NPREP) == 0, "a widening pass takes whole tokens of one chunk");
-  static constexpr int PB = 8 * sizeof(TIn) / 16;           // 16-byte pieces of a lane's eight columns
-  static constexpr uint32_t raw_stage = 2 * NPREP * NP * PB * 512;   // both tensors of a chunk as the lanes take them
+  // rank 0 at d = 64 with explicit u: shorter code (head of this file)
+  static constexpr bool SHORT = UT && D == 64;
+  static constexpr int columns(bool r1) { return SHORT && !r1 ? 4 : 8; }   // that a widening lane takes at a time
+  static constexpr uint32_t raw_stage = 2 * C * D * sizeof(TIn);   // both tensors of a chunk as the lanes take them
   static constexpr int RK = 2, RA = 4;                      // input and alpha slots
   static constexpr int LD = 20;                             // row of a small matrix
   static constexpr int SM = C * LD;
@@ -86,40 +95,54 @@ struct PairCfg {
   static constexpr size_t smem_bytes = bars + NBAR * 8 + 16;
 };
 
-// global -> shared, 16 bytes, zeros when !act (each lane reads back only what it copied itself)
+// global -> shared, 16 or 8 bytes, zeros when !act (each lane reads back only what it copied itself)
+template <int BYTES>
 __device__ __forceinline__ void copy_piece(uint32_t dst, const void* src, bool act) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(act ? 16 : 0) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(BYTES), "r"(act ? BYTES : 0) : "memory");
 }
-// a lane's eight columns back from its pieces, 512 bytes apart
-__device__ __forceinline__ void piece_f32(const unsigned char* at, float (&x)[8], const float*) {
+// a lane's columns back from its pieces (16-byte pieces lie 512 bytes apart)
+template <int CPL>
+__device__ __forceinline__ void piece_f32(const unsigned char* at, float (&x)[CPL], const float*) {
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < CPL / 4; ++i) {
     const float4 y = *reinterpret_cast<const float4*>(at + 512 * i);
     x[4 * i] = y.x; x[4 * i + 1] = y.y; x[4 * i + 2] = y.z; x[4 * i + 3] = y.w;
   }
 }
-__device__ __forceinline__ void piece_f32(const unsigned char* at, float (&x)[8], const uint16_t*) {
-  const uint4 y = *reinterpret_cast<const uint4*>(at);
-  const uint32_t w[4] = {y.x, y.y, y.z, y.w};
+template <int CPL>
+__device__ __forceinline__ void piece_f32(const unsigned char* at, float (&x)[CPL], const uint16_t*) {
+  uint32_t w[CPL / 2];
+  if constexpr (CPL == 8) {
+    const uint4 y = *reinterpret_cast<const uint4*>(at);
+    w[0] = y.x; w[1] = y.y; w[2] = y.z; w[3] = y.w;
+  } else {
+    const uint2 y = *reinterpret_cast<const uint2*>(at);
+    w[0] = y.x; w[1] = y.y;
+  }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < CPL / 2; ++i) {
     x[2 * i] = __uint_as_float(w[i] << 16);
     x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
   }
 }
 
-// eight consecutive columns of a token row, scaled, as hi/lo operand entries
-template <int D>
-__device__ __forceinline__ void tok_store8(uint32_t base, int row, int pl, const float (&x)[8], float s) {
-  uint32_t h[4], l[4];
+// CPL consecutive columns of a token row, scaled, as hi/lo operand entries
+template <int D, int CPL>
+__device__ __forceinline__ void tok_store(uint32_t base, int row, int pl, const float (&x)[CPL], float s) {
+  uint32_t h[CPL / 2], l[CPL / 2];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < CPL / 2; ++i) {
     const float2 y = fmul2(make_float2(x[2 * i], x[2 * i + 1]), make_float2(s, s));
     split_f16(y.x, y.y, h[i], l[i]);
   }
-  const uint32_t at = base + uint32_t(row) * kTokRow<D> + 16 * pl;
-  sts128(at, h);
-  sts128(at + 2 * D, l);
+  const uint32_t at = base + uint32_t(row) * kTokRow<D> + 2 * CPL * pl;
+  if constexpr (CPL == 8) {
+    sts128(at, h);
+    sts128(at + 2 * D, l);
+  } else {
+    sts64(at, h[0], h[1]);
+    sts64(at + 2 * D, l[0], l[1]);
+  }
 }
 
 // NS: CTAs that carry an S.  2 (the segments of a cut sequence): rank 1 the segment from S = 0, rank 2 its
@@ -128,7 +151,7 @@ template <int D, typename TIn, bool UT, bool STASH, int NS>
 __global__ void __cluster_dims__(STASH ? 1 : 1 + NS, 1, 1) __launch_bounds__((PairCfg<D, TIn, UT>::NT), (PairCfg<D, TIn, UT>::MINB))
 vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
   using Cfg = PairCfg<D, TIn, UT>;
-  constexpr int C = Cfg::C, NW = Cfg::NW, NPREP = Cfg::NPREP, LPT = Cfg::LPT, TPW = Cfg::TPW, NP = Cfg::NP, PB = Cfg::PB;
+  constexpr int C = Cfg::C, NW = Cfg::NW, NPREP = Cfg::NPREP;
   constexpr int RK = Cfg::RK, RA = Cfg::RA, LD = Cfg::LD, SM = Cfg::SM, PARTS = Cfg::PARTS, NJOB = Cfg::NJOB;
   constexpr int NTILE = D / 8, KS = D / 16, NB = NTILE < 4 ? NTILE : 4;
   constexpr float kUnit = 256.0f, kUnitInv = 1.0f / 256.0f;   // scale of unit-vector operands
@@ -196,154 +219,178 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
   const size_t tok0 = token_offset(p, unit, 0, D), tstride = token_stride(p, D);
 
   // ======================================================================= widening warps (both ranks)
-  // A lane takes eight columns of a token at a time, through a staging ring that only it reads; the
+  // A lane takes CPL columns of a token at a time, through a staging ring that only it reads; the
   // copies of chunk c + 1 are in flight while chunk c is widened.
   auto widen = [&](auto r1) {
-  constexpr bool R1 = decltype(r1)::value;   // rank 1 and 2: keys and queries; rank 0: keys [and u]
-  const int pw = warp - NW - 1, sub = lane / LPT, pl = lane % LPT;
-  const TIn* src0 = static_cast<const TIn*>(p.k) + tok0 + 8 * pl;
-  constexpr bool two = UT || R1, sums = STASH || R1;   // sums: this side carries the key sum
-  const TIn* src1 = two ? static_cast<const TIn*>(R1 ? p.q : p.u) + tok0 + 8 * pl : src0;
-  float* fs = reinterpret_cast<float*>(smem + (R1 ? Cfg::s_f : Cfg::a_f));
-  const uint32_t base0 = sb + (R1 ? Cfg::s_K : Cfg::a_K), base1 = sb + (R1 ? Cfg::s_Q : Cfg::a_U);
-  auto stage = [&](int c, int ps) {   // byte offset of this lane's pieces (the second tensor's PB pieces follow the first's)
-    return Cfg::raw + (c & 1) * Cfg::raw_stage + uint32_t(ps * NPREP + pw) * (2 * PB * 512) + uint32_t(lane) * 16;
-  };
-  auto fetch = [&](int c) {
+    constexpr bool R1 = decltype(r1)::value;   // rank 1 and 2: keys and queries; rank 0: keys [and u]
+    constexpr bool two = UT || R1, sums = STASH || R1;   // sums: this side carries the key sum
+    constexpr int CPL = Cfg::columns(R1), LPT = D / CPL, TPW = 32 / LPT, NP = C / (TPW * NPREP);   // lanes a token, tokens a pass, passes
+    static_assert(C % (TPW * NPREP) == 0, "a widening pass takes whole tokens of one chunk");
+    constexpr int BYTES = CPL * sizeof(TIn), PIECE = BYTES < 16 ? BYTES : 16, PB = BYTES / PIECE;   // a lane's columns, in pieces
+    const int pw = warp - NW - 1, sub = lane / LPT, pl = lane % LPT;
+    const TIn* src0 = static_cast<const TIn*>(p.k) + tok0 + CPL * pl;
+    const TIn* src1 = two ? static_cast<const TIn*>(R1 ? p.q : p.u) + tok0 + CPL * pl : src0;
+    float* fs = reinterpret_cast<float*>(smem + (R1 ? Cfg::s_f : Cfg::a_f));
+    const uint32_t base0 = sb + (R1 ? Cfg::s_K : Cfg::a_K), base1 = sb + (R1 ? Cfg::s_Q : Cfg::a_U);
+    auto stage = [&](int c, int ps) {   // byte offset of this lane's pieces (the second tensor's PB pieces follow the first's)
+      return Cfg::raw + (c & 1) * Cfg::raw_stage + uint32_t(ps * NPREP + pw) * (2 * 32 * BYTES) + uint32_t(lane) * PIECE;
+    };
+    auto fetch = [&](int c) {
 #pragma unroll 1
-    for (int ps = 0; ps < NP; ++ps) {
-      const int t = c * C + (ps * NPREP + pw) * TPW + sub;
-      const bool act = t < T;
-      const size_t off = act ? size_t(t) * tstride : 0;
-      const uint32_t at = sb + stage(c, ps);
+      for (int ps = 0; ps < NP; ++ps) {
+        const int t = c * C + (ps * NPREP + pw) * TPW + sub;
+        const bool act = t < T;
+        const size_t off = act ? size_t(t) * tstride : 0;
+        const uint32_t at = sb + stage(c, ps);
 #pragma unroll
-      for (int i = 0; i < PB; ++i) {
-        copy_piece(at + 512 * i, src0 + off + i * (8 / PB), act);
-        if (two) copy_piece(at + 512 * (PB + i), src1 + off + i * (8 / PB), act);
+        for (int i = 0; i < PB; ++i) {
+          copy_piece<PIECE>(at + 32 * PIECE * i, src0 + off + i * (CPL / PB), act);
+          if (two) copy_piece<PIECE>(at + 32 * PIECE * (PB + i), src1 + off + i * (CPL / PB), act);
+        }
       }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  float zk[8] = {};
-  if (sums && p.z0) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) zk[e] = p.z0[size_t(unit) * D + 8 * pl + e];
-  }
-  if (nch > 0) fetch(0);
-#pragma unroll 1
-  for (int c = 0; c < nch; ++c) {
-    const int slot = c % RK;
-    fetch(c + 1);   // (past the end: zeros)
-    if (STASH && pw == 0 && sub == 0) {
-      float4* o = reinterpret_cast<float4*>(sh.zkc + (size_t(unit) * nch + c) * D + 8 * pl);
-      o[0] = make_float4(zk[0], zk[1], zk[2], zk[3]);
-      o[1] = make_float4(zk[4], zk[5], zk[6], zk[7]);
-    }
-    if (c >= RK) wait(&kfree[slot], (c / RK - 1) & 1);
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    float ks[8] = {};
-#pragma unroll 1
-    for (int ps = 0; ps < NP; ++ps) {
-      const int tt = (ps * NPREP + pw) * TPW + sub;
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float zk[CPL] = {}, ks[CPL];   // key sum before the chunk, this lane's share of the chunk's
+    // (a token past the end came in as zeros: its key row and its share of the key sum are zeros too; what its query,
+    // phi(0) = 1, gives is not stored)
+    // rank 1: keys and queries side by side, one round of shuffles for both
+    auto both = [&](const unsigned char* raw, int c, int slot, int tt) {
       const bool act = c * C + tt < T;
-      const unsigned char* raw = smem + stage(c, ps);
-      float k[8], x[8] = {};
+      const float on = act ? 1.0f : 0.0f;
+      float k[CPL], x[CPL];
       piece_f32(raw, k, src0);
-      if (two) piece_f32(raw + 512 * PB, x, src0);
+      piece_f32(raw + 32 * BYTES, x, src0);
       if (!ident) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) k[e] = phi_fast(k[e]);
-        if constexpr (R1) {
+        for (int e = 0; e < CPL; ++e) k[e] = phi_fast(k[e]);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) x[e] = phi_fast(x[e]);
-        }
+        for (int e = 0; e < CPL; ++e) x[e] = phi_fast(x[e]);
       }
-      // (a token past the end came in as zeros: its key row and its share of the key sum are zeros too; what its query,
-      // phi(0) = 1, gives is not stored)
-      const float on = act ? 1.0f : 0.0f;
       float2 ss2 = make_float2(0.f, 0.f), qq2 = ss2, dn2 = ss2;
 #pragma unroll
-      for (int e = 0; e < 8; e += 2) {
+      for (int e = 0; e < CPL; e += 2) {
         const float2 k2 = make_float2(k[e], k[e + 1]), x2 = make_float2(x[e], x[e + 1]);
         ss2 = ffma2(k2, k2, ss2);
-        if (two) qq2 = ffma2(x2, x2, qq2);
-        if (R1) dn2 = ffma2(x2, make_float2(zk[e], zk[e + 1]), dn2);
-        if (sums) {
-          const float2 s2 = ffma2(make_float2(on, on), k2, make_float2(ks[e], ks[e + 1]));
-          ks[e] = s2.x;
-          ks[e + 1] = s2.y;
-        }
+        qq2 = ffma2(x2, x2, qq2);
+        dn2 = ffma2(x2, make_float2(zk[e], zk[e + 1]), dn2);
+        const float2 s2 = ffma2(make_float2(on, on), k2, make_float2(ks[e], ks[e + 1]));
+        ks[e] = s2.x;
+        ks[e + 1] = s2.y;
       }
       float ss = ss2.x + ss2.y, qq = qq2.x + qq2.y, dn = dn2.x + dn2.y;
 #pragma unroll
       for (int off = LPT / 2; off >= 1; off >>= 1) {
         ss += __shfl_xor_sync(0xffffffffu, ss, off);
-        if (two) qq += __shfl_xor_sync(0xffffffffu, qq, off);
-        if (R1) dn += __shfl_xor_sync(0xffffffffu, dn, off);
+        qq += __shfl_xor_sync(0xffffffffu, qq, off);
+        dn += __shfl_xor_sync(0xffffffffu, dn, off);
       }
       const float nr = fmaxf(sqrt_ftz(ss), eps);   // max(||phi(k)||, eps)
-      tok_store8<D>(base0 + slot * Cfg::kslot, tt, pl, k, rcp_ftz_nr(nr) * (on * kUnit));
-      if constexpr (two) {
-        const float s = pow2_scale(sqrt_ftz(qq), 8);
-        tok_store8<D>(base1 + slot * Cfg::kslot, tt, pl, x, s);
-        if (pl == 0) {
-          const float inv = pow2_inverse(s);
-          if constexpr (R1) {
-            fs[Cfg::sf_qs + slot * 16 + tt] = inv;
-          } else {   // u row -> u', and D^-2 (four slots: the elimination is done with one by the time it comes round again)
-            const float iD = pow2_inverse(fminf(fmaxf(256.0f * inv, 9.5367432e-7f), 1.1529215e18f));
-            fs[Cfg::af_us + slot * 16 + tt] = inv * iD;
-            fs[Cfg::af_ud + (c & 3) * 16 + tt] = iD * iD;
-          }
-        }
-      }
-      if (R1 && pl == 0) {
+      tok_store<D>(base0 + slot * Cfg::kslot, tt, pl, k, rcp_ftz_nr(nr) * (on * kUnit));
+      const float s = pow2_scale(sqrt_ftz(qq), 8);
+      tok_store<D>(base1 + slot * Cfg::kslot, tt, pl, x, s);
+      if (pl == 0) {
+        fs[Cfg::sf_qs + slot * 16 + tt] = pow2_inverse(s);
         fs[Cfg::sf_nrm + slot * 16 + tt] = act ? nr : 0.f;
         fs[Cfg::sf_dq + slot * 16 + tt] = dn;
       }
-    }
-    if (sums && !ident) {
-      // the key sum after this chunk: over the tokens a warp took at a time by halving (a lane ends with KN
-      // columns), over the warps and back to eight columns a lane through shared memory
-      constexpr int KN = TPW >= 8 ? 1 : 8 / TPW;
-      int col = 0;
+    };
+    // rank 0: keys, then u, one copy of the code for both (it waits less for these warps than for instructions)
+    auto each = [&](const unsigned char* raw, int c, int slot, int tt) {
+      const float on = c * C + tt < T ? 1.0f : 0.0f;
+#pragma unroll 1
+      for (int i = 0; i < (UT ? 2 : 1); ++i) {
+        float x[CPL];
+        piece_f32(raw + 32 * BYTES * i, x, src0);
+        if (i == 0 && !ident) {
 #pragma unroll
-      for (int off = 16, n = 8; off >= LPT; off >>= 1) {
-        n >>= 1;
-        if (n >= 1) {
-          const bool up = (lane & off) != 0;
+          for (int e = 0; e < CPL; ++e) x[e] = phi_fast(x[e]);
+        }
+        float2 ss2 = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int e = 0; e < n; ++e) {
-            const float send = up ? ks[e] : ks[e + n], keep = up ? ks[e + n] : ks[e];
-            ks[e] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        for (int e = 0; e < CPL; e += 2) {
+          const float2 x2 = make_float2(x[e], x[e + 1]);
+          ss2 = ffma2(x2, x2, ss2);
+          if (sums && (!UT || i == 0)) {
+            const float2 s2 = ffma2(make_float2(on, on), x2, make_float2(ks[e], ks[e + 1]));
+            ks[e] = s2.x;
+            ks[e + 1] = s2.y;
           }
-          if (up) col += n;
-        } else {
-          ks[0] += __shfl_xor_sync(0xffffffffu, ks[0], off);
+        }
+        float ss = ss2.x + ss2.y;
+#pragma unroll
+        for (int off = LPT / 2; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+        const float n = sqrt_ftz(ss);
+        // k_hat = phi(k) / max(||phi(k)||, eps), or a row of u with a power of two of its own
+        const float s = !UT || i == 0 ? rcp_ftz_nr(fmaxf(n, eps)) * (on * kUnit) : pow2_scale(n, 8);
+        tok_store<D>((UT && i ? base1 : base0) + slot * Cfg::kslot, tt, pl, x, s);
+        if (UT && i == 1 && pl == 0) {   // u row -> u', and D^-2 (four slots: the elimination is done with one by the time it comes round again)
+          const float inv = pow2_inverse(s), iD = pow2_inverse(fminf(fmaxf(256.0f * inv, 9.5367432e-7f), 1.1529215e18f));
+          fs[Cfg::af_us + slot * 16 + tt] = inv * iD;
+          fs[Cfg::af_ud + (c & 3) * 16 + tt] = iD * iD;
         }
       }
-      float* zp = fs + (STASH ? Cfg::af_zp : Cfg::sf_zp) + (c & 1) * NPREP * D;
+    };
+    auto store_sum = [&](float* row) {
 #pragma unroll
-      for (int e = 0; e < KN; ++e) zp[pw * D + 8 * pl + col + e] = ks[e];   // (d = 16: two lanes, one value)
-      if constexpr (NPREP > 1) named_sync(2, NPREP * 32);
-      else __syncwarp();
+      for (int e = 0; e < CPL; e += 4) *reinterpret_cast<float4*>(row + CPL * pl + e) = make_float4(zk[e], zk[e + 1], zk[e + 2], zk[e + 3]);
+    };
+    if (sums && p.z0) {
 #pragma unroll
-      for (int w = 0; w < NPREP; ++w) {
-        const float4* y = reinterpret_cast<const float4*>(zp + w * D + 8 * pl);
-        const float4 y0 = y[0], y1 = y[1];
-        const float y8[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) zk[e] += y8[e];
-      }
+      for (int e = 0; e < CPL; ++e) zk[e] = p.z0[size_t(unit) * D + CPL * pl + e];
     }
-    arrive(&kfull[slot]);
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  if (sums && rank < 2 && p.zT && pw == 0 && sub == 0) {
-    float4* o = reinterpret_cast<float4*>(p.zT + size_t(unit) * D + 8 * pl);
-    o[0] = make_float4(zk[0], zk[1], zk[2], zk[3]);
-    o[1] = make_float4(zk[4], zk[5], zk[6], zk[7]);
-  }
+    if (nch > 0) fetch(0);
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) {
+      const int slot = c % RK;
+      fetch(c + 1);   // (past the end: zeros)
+      if (STASH && pw == 0 && sub == 0) store_sum(sh.zkc + (size_t(unit) * nch + c) * D);
+      if (c >= RK) wait(&kfree[slot], (c / RK - 1) & 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+#pragma unroll
+      for (int e = 0; e < CPL; ++e) ks[e] = 0.f;
+#pragma unroll 1
+      for (int ps = 0; ps < NP; ++ps) {
+        const int tt = (ps * NPREP + pw) * TPW + sub;
+        if constexpr (R1) both(smem + stage(c, ps), c, slot, tt);
+        else each(smem + stage(c, ps), c, slot, tt);
+      }
+      if (sums && !ident) {
+        // the key sum after this chunk: over the tokens a warp took at a time by halving (a lane ends with KN
+        // columns), over the warps and back to CPL columns a lane through shared memory
+        constexpr int KN = TPW >= CPL ? 1 : CPL / TPW;
+        int col = 0;
+#pragma unroll
+        for (int off = 16, n = CPL; off >= LPT; off >>= 1) {
+          n >>= 1;
+          if (n >= 1) {
+            const bool up = (lane & off) != 0;
+#pragma unroll
+            for (int e = 0; e < n; ++e) {
+              const float send = up ? ks[e] : ks[e + n], keep = up ? ks[e + n] : ks[e];
+              ks[e] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
+            if (up) col += n;
+          } else {
+            ks[0] += __shfl_xor_sync(0xffffffffu, ks[0], off);
+          }
+        }
+        float* zp = fs + (STASH ? Cfg::af_zp : Cfg::sf_zp) + (c & 1) * NPREP * D;
+#pragma unroll
+        for (int e = 0; e < KN; ++e) zp[pw * D + CPL * pl + col + e] = ks[e];   // (d = 16: two lanes, one value)
+        if constexpr (NPREP > 1) named_sync(2, NPREP * 32);
+        else __syncwarp();
+#pragma unroll
+        for (int w = 0; w < NPREP; ++w)
+#pragma unroll
+          for (int e = 0; e < CPL; e += 4) {
+            const float4 y = *reinterpret_cast<const float4*>(zp + w * D + CPL * pl + e);
+            zk[e] += y.x; zk[e + 1] += y.y; zk[e + 2] += y.z; zk[e + 3] += y.w;
+          }
+      }
+      arrive(&kfull[slot]);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (sums && rank < 2 && p.zT && pw == 0 && sub == 0) store_sum(p.zT + size_t(unit) * D);
   };
   // (the roles of a rank stand together: that is the code an SM runs)
   if (rank == 0 && warp > NW) {
@@ -376,7 +423,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       const float one = UT ? ud[r] : 1.0f;
 #pragma unroll
       for (int j = 0; j < 8; ++j) m[j] += (8 * h + j == r) ? one : 0.0f;
-      const float delta = eliminate16<UT>(m, lane, piv, eps, ud);   // (explicit u: delta / D^2)
+      const float delta = eliminate16<UT, UT ? 1 : 2>(m, lane, piv, eps, ud);   // (explicit u: delta / D^2)
       {
         float x[8];
         if constexpr (UT) {
@@ -649,11 +696,14 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         if (tid == 0) sh.Asc[blk] = sAi;
       }
     };
-    clear_z0();
+    auto all_products = [&](int slot) {
+      clear_z0();
+#pragma unroll
+      for (int ks = 0; ks < KS; ks += KB) product(ks, slot);
+    };
     if (nch > 0) {
       wait(&kfull[0], 0);
-#pragma unroll
-      for (int ks = 0; ks < KS; ks += KB) product(ks, 0);
+      if constexpr (!Cfg::SHORT) all_products(0);
       stash_state(0);
     }
 #pragma unroll 1
@@ -663,6 +713,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       const uint32_t Uop = sb + (UT ? Cfg::a_U : Cfg::a_K) + slot * Cfg::kslot;
       uint32_t zh[4], zl[4];
       if (live) {
+      if constexpr (Cfg::SHORT) all_products(slot);
       const float* us = fs + Cfg::af_us + slot * 16;
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt)
@@ -683,7 +734,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         constexpr int K2 = KS / PARTS < 2 ? 1 : 2;
         const uint32_t src = sb + (job >= 2 ? Cfg::a_W0 : Cfg::a_Z0) + lane_vn + (job & 1) * 16 + part * (KS / PARTS) * 16 * kVecRow;
         const uint32_t rows = Uop + lane_ta + part * (KS / PARTS) * 32;
-#pragma unroll
+#pragma unroll (UT ? 1 : KS)   // (explicit u: code size)
         for (int k2 = 0; k2 < KS / PARTS; k2 += K2) {
           uint32_t ah[K2][4], al[K2][4], b[K2][4];
 #pragma unroll
@@ -711,7 +762,8 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       }
       if (c + 1 < nch) wait(&kfull[(c + 1) % RK], ((c + 1) / RK) & 1);
       // A shrinks as tokens come, by up to 1 / lambda within the first d of them, by 1 / t later: its operands are
-      // kept near the top of fp16's range, or the remainders would run into its subnormals
+      // kept near the top of fp16's range, or the remainders would run into its subnormals.  (The next chunk's A K^T is
+      // formed before the rescale and scaled after it: its operands lag one chunk more)
       const bool look = (c & 7) == 7 || c < D / 4;
       if (look) {
         const float mx = state_max(st);
@@ -770,10 +822,10 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
       named_sync(1, NW * 32);
       // ---- A <- A - sum zeta zeta^T, and at once the next chunk's Z0 (past the end: unused).  One block of code without a
       // branch, so that the two products' latencies overlap.
-      clear_z0();
+      if constexpr (!Cfg::SHORT) clear_z0();
       {
         const int next = (c + 1) % RK;
-        constexpr int NU = 2 * KB;   // tiles a step
+        constexpr int NU = Cfg::SHORT ? NB : 2 * KB;   // tiles a step
 #pragma unroll
         for (int nt = 0; nt < NTILE; nt += NU) {
           uint32_t b[NU][4];
@@ -788,7 +840,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           for (int i = 0; i < NU; ++i) mma_f16(x[i], yh, b[i][0], b[i][1]);
 #pragma unroll
           for (int i = 0; i < NU; ++i) tile_fma(st[nt + i], x[i], sAy);
-          product(nt / 2, next);
+          if constexpr (!Cfg::SHORT) product(nt / 2, next);
         }
       }
       if (look) {

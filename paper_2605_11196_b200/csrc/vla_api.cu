@@ -89,11 +89,13 @@ bool chunk_tc_covers(const ScanParams& p, int d) {
 bool pair_covers(const ScanParams& p) { return p.refresh_period <= 0 && p.n_main <= 0 && p.units <= 0x3fffffff; }
 
 // Where it is the library's choice.  Below d = 128 everywhere but for very short sequences, which the token
-// kernel does without a cluster's start: few units, us at T = 8, 16, 32 (d = 64): token 8.4, 13.4, 24.6, pair
-// 8.2, 8.2, 11.1; more units than fit at once (1024): 33, 57, 107 and 63, 63, 90; d = 32: 12, 19, 35 and 31, 31, 43.  At
-// d = 128 the tensor-memory kernel keeps what is short (below seven chunks the clusters' start costs
-// what the shorter chain saves) and, with u = k_hat, more units than SM pairs (one SM per unit there:
-// 48 units x 1777 tokens 0.59 against 0.44 ms, 128 x 2048 0.69 against 1.02 ms).
+// kernel does without a cluster's start: few units, us at T = 8, 16, 24 (d = 64): token 10.3, 14.8, 20.9, pair
+// 10.1, 9.8, 12.5; more units than fit at once (1024) at T = 16, 24, 36: 58, 85, 123 and 64, 89, 107; d = 32 at T = 24, 36, 48: 29, 42,
+// 53 and 42, 50, 51 (d = 16: 19, 25, 31 and 29, 34, 34).  At d = 128 the tensor-memory kernel keeps, with u = k_hat, more units than SM
+// pairs (one SM per unit there: 75 units at T = 128, 512: 58, 188 against 76, 231 us; 74 units 58, 188 against 44, 142), and what is
+// short.  (That line, T = 96, comes from an earlier pair kernel: one wave of today's is ahead from T = 9 on, 1 unit at T = 9, 48, 96: 14.6,
+// 23.0, 33.2 against 18.8, 29.1, 45.5 us, 74 units 14.8, 24.9, 35.9 against 18.7, 29.2, 45.8; with explicit u, against the FMA
+// chunk kernel, 512 units at T = 48, 96: 187, 285 against 217, 379.)
 bool pair_pays_off(const ScanParams& p, int d) {
   const long long sms = vla::device_sms();
   const long long resident = d == 16 ? 6 : d == 32 ? 4 : d == 64 ? 2 : 1;   // CTAs per SM
@@ -218,9 +220,13 @@ int seqpar_choose_segments(int units, int T, int d, int dtype) {
   const Rate r = d == 32 ? Rate{1.55, 1.7, 2.55, 45, 1.7, 0.05, 1.8e-4}
                : d == 64 ? Rate{2.0, 2.2, 3.1, 110, 3.8, 0.25, 4.8e-4}
                          : Rate{3.9, 4.2, 4.3, 420, 17.0, 1.0, 1.0e-3};
-  // (d = 64, us by segments, 1 = uncut: 1 unit x 16384 tokens 2035, 8: 423, 16: 313, 32: 306; 30 x 8192 1040, 2: 942, 4: 837,
-  // 8: 850; 60 x 8192 1170, 2: 1539; 16 x 65536 8100, 8: 3500, 16: 2959, 32: 3154.  d = 32, 4 x 16384 1563, 16: 185, 32: 151,
-  // 64: 187.  d = 128, 8 x 32768 7900, 4: 2960, 8: 3126, 16: 2836; 12 x 8192 1979, 4: 1569.)
+  // (The rates are those of the GPUs and kernels on which a chunk took longest; how many segments are best moves little with them.
+  // With today's kernels, over 50 shapes up to 65536 tokens and 400 units, the choice took at most 1.03 times the best divisor's time
+  // with u = k_hat, 1.05 with an explicit u but for one (64 units x 4096, d = 32: 472 us in 8, 401 uncut).
+  // us by segments, 1 = uncut: d = 64, 1 unit x 16384 tokens 1688, 8: 382, 16: 297, 32: 304; 30 x 8192 920, 2: 880, 4: 788,
+  // 8: 796; 60 x 8192 1270, 2: 1363; 16 x 65536 7181, 8: 3216, 16: 2727, 32: 2881.  d = 32, 4 x 16384 1141, 16: 168, 32: 146,
+  // 64: 182; 128 x 4096 441, 2: 571.  d = 128, 8 x 32768 6690, 4: 2655, 8: 2815, 16: 2544; 12 x 8192 1684, 2: 1367, 8: 1404; 24 x 8192
+  // 1688, 4: 2064.)
   const int nch = T / 16;
   const double pairs = (d == 32 ? 2.0 : d == 64 ? 1.0 : 0.5) * sms;   // uncut units resident at a time
   auto waves = [](double n, double room, double lone, double full, double from) {   // us per chunk

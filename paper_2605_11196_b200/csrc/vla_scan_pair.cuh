@@ -25,8 +25,8 @@
 // share what is beyond.  In clusters of two an SM holds CTAs of one rank only (measured with 64, 148 and 296 CTAs: a cluster's
 // ranks lie on the two SMs of a TPC, and the second wave falls in with the first), so each rank has its own copy of the
 // widening code, small loops stay rolled, and values go through two-wide instructions.  (Three ranks on two SMs mix.)  What lies
-// beyond the cache comes at a rate that differs from GPU to GPU: one build takes 457 us on four GPUs and 533 on three others (32
-// units x 4096 tokens, d = 64).
+// beyond the cache comes at a rate that differs from GPU to GPU: one build takes 442 us on five GPUs, 462 on one and 518 on three
+// (32 units x 4096 tokens, d = 64).
 //
 // With explicit u rank 0's roles are some 8 KB longer and do not fit.  Widened side by side, eight columns of keys and u a lane, they made
 // two CTAs on an SM (d = 64) wait twice as long for instructions as the form before (1.9 against 0.8 warps per instruction
@@ -439,17 +439,19 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         } else {
           // diag(delta)^-1/2 (L^-1 - I) as an operand; the unit diagonal does not go through fp16 and the truncating sum, z_t takes
           // z0_t in fp32.  Rows of diag(delta)^-1/2 L^-1 are no longer than 1 (I + W >= I).  They may be as short as
-          // 1 / sqrt(delta): past 2^-15 (lambda below 1e-9) each row gets a power of two of its own.
+          // 1 / sqrt(delta): past delta = 1e6 (lambda below 1e-6) each row gets a power of two of its own, before its remainders run into
+          // subnormals.
           // A_T's error over lambda 1 to 1e-14, T 13 to 1500 (geometric mean at d = 16, 32, 64, 128), against tf32 pairs of all of
-          // L^-1 in four products: 0.87, 0.87, 0.89, 0.93 times; with the diagonal in the operand 0.97, 1.00, 1.07, 1.13
-          // (1.85 at lambda 1e-9, d = 128).  The dropped remainders' product is worth 0.01.  The fp32 share costs 70 to 110 clk of a
-          // chunk at d = 32 and 64 (32 units x 4096 tokens, d = 64: 442 -> 457 us)
+          // L^-1 in four products: 0.87, 0.86, 0.88, 0.92 times; with the diagonal in the operand 0.97, 1.00, 1.07, 1.13
+          // (1.85 at lambda 1e-9, d = 128); with the rows' powers of two from delta = 1e9 on only, 1.05 to 1.26 at lambda 1e-9, d >= 64.  The dropped remainders' product is worth 0.01.  The fp32 share costs 50 clk of a
+          // chunk at d = 64 (32 units x 4096 tokens: 442 -> 449 us, another GPU 462 -> 472; 457 with one value an instruction), nothing at
+          // the other d
           const float rs = rsqrt_ftz_nr(delta);
           const float p2 = __uint_as_float(__float_as_uint(rs) & 0x7f800000u);   // the power of two below: exact
           float f = p2 * kLam, fi = rs * pow2_inverse(p2) * kLamInv;
 #pragma unroll
           for (int j = 0; j < 8; ++j) x[j] = 8 * h + j < r ? m[j] : 0.0f;
-          if (__any_sync(0xffffffffu, delta > 1e9f)) {
+          if (__any_sync(0xffffffffu, delta > 1e6f)) {
             float mx = 0.f;
 #pragma unroll
             for (int j = 0; j < 8; ++j) mx = fmaxf(mx, fabsf(x[j]));
@@ -794,6 +796,7 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
         } else {
           uint32_t b[2][4];
           float x[2][4];
+          const float sAz = sAi * pow2_inverse(sy);
 #pragma unroll
           for (int nt = 0; nt < 2; ++nt) vec_frag_b(b[nt], smem_u32(Li) + lane_vb, nt);
 #pragma unroll
@@ -806,12 +809,15 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           for (int nt = 0; nt < 2; ++nt) {
             const float2 fi2 = *reinterpret_cast<const float2*>(dl + 16 + 8 * nt + 2 * c4);
             const float2 rs2 = *reinterpret_cast<const float2*>(dl + 32 + 8 * nt + 2 * c4);
-            const float fi[2] = {fi2.x, fi2.y}, rs[2] = {rs2.x, rs2.y}, fa[2] = {sAi * rs2.x, sAi * rs2.y};
+            // (two values an instruction; the powers of two sy and sAi change no bit wherever they are applied)
+            const float2 sy2 = make_float2(sy, sy), fy = fmul2(fi2, sy2), ry = fmul2(rs2, sy2), fa = fmul2(rs2, make_float2(sAz, sAz));
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float zeta = fmaf(z0[nt][e], rs[e & 1], x[nt][e] * fi[e & 1]);
-              y[nt][e] = zeta * sy;
-              a1[nt][e] = zeta * fa[e & 1];   // u = k_hat: a_t = z_t / delta_t
+            for (int e = 0; e < 4; e += 2) {
+              const float2 w = ffma2(make_float2(z0[nt][e], z0[nt][e + 1]), ry, fmul2(make_float2(x[nt][e], x[nt][e + 1]), fy)), a = fmul2(w, fa);
+              y[nt][e] = w.x;
+              y[nt][e + 1] = w.y;
+              a1[nt][e] = a.x;   // u = k_hat: a_t = z_t / delta_t
+              a1[nt][e + 1] = a.y;
             }
           }
         }

@@ -442,10 +442,10 @@ vla_scan_pair_kernel(const ScanParams p, const PairStash sh) {
           // 1 / sqrt(delta): past delta = 1e6 (lambda below 1e-6) each row gets a power of two of its own, before its remainders run into
           // subnormals.
           // A_T's error over lambda 1 to 1e-14, T 13 to 1500 (geometric mean at d = 16, 32, 64, 128), against tf32 pairs of all of
-          // L^-1 in four products: 0.87, 0.86, 0.88, 0.92 times; with the diagonal in the operand 0.97, 1.00, 1.07, 1.13
-          // (1.85 at lambda 1e-9, d = 128); with the rows' powers of two from delta = 1e9 on only, 1.05 to 1.26 at lambda 1e-9, d >= 64.  The dropped remainders' product is worth 0.01.  The fp32 share costs 50 clk of a
-          // chunk at d = 64 (32 units x 4096 tokens: 442 -> 449 us, another GPU 462 -> 472; 457 with one value an instruction), nothing at
-          // the other d
+          // L^-1 in four products: 0.87, 0.86, 0.88, 0.92 times; with the diagonal in the operand 0.97, 1.00, 1.07, 1.13 (1.85 at
+          // lambda 1e-9, d = 128); with the rows' powers of two only from delta = 1e9 on, 1.05 to 1.26 at lambda 1e-9, d >= 64.  The
+          // dropped remainders' product is worth 0.01.  The fp32 share costs 50 clk of a chunk at d = 64 (32 units x 4096 tokens: 442 ->
+          // 449 us, another GPU 462 -> 472; 457 with one value an instruction), nothing at the other d
           const float rs = rsqrt_ftz_nr(delta);
           const float p2 = __uint_as_float(__float_as_uint(rs) & 0x7f800000u);   // the power of two below: exact
           float f = p2 * kLam, fi = rs * pow2_inverse(p2) * kLamInv;

@@ -33,8 +33,9 @@
 // issued, for 15 % fewer instructions).  So keys and u go through one loop, the elimination's and W's loops are rolled, and at d = 64 a lane
 // takes four columns and the next chunk's products stand by themselves (SHORT).  us, four columns and all unrolled / eight / now:
 // d = 64 256 units x 2048 tokens 990 / 1140 / 996 (on a GPU of the slower kind 919 / 1020 / 935), 32 x 4096 634 / 618 / 629 (717 / 779 /
-// 732); d = 128 64 x 2048 603 / 605 / 591, 512 x 8192 17.7 / 18.0 / 17.5 ms; d = 32 256 x 512 171 / 172 / 171.  (Four columns at d = 32 and 128: 179 and 703; SHORT at d = 32 and 128: 180
-// and 721; a third and fourth widening warp at d = 128: 590, where two left 548.)
+// 732); d = 128 64 x 2048 603 / 605 / 591, 512 x 8192 17.7 / 18.0 / 17.5 ms, one unit x 2048 560 / 516 / 535; d = 32 256 x 512
+// 171 / 172 / 171.  (Four columns at d = 32 and 128: 179 and 703; SHORT there: 183 and 721; four widening warps at d = 128: 590, where
+// two left 548.)
 //
 // What bounds it: at one unit per SM pair the serial chain of rank 0 (W, the 16 x 16 elimination, Z, then the update of A with the
 // next chunk's Z0 in it), with many units the tensor pipe (8 clk per instruction and
